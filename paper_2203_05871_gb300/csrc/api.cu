@@ -66,9 +66,10 @@ int release_slots(mpdo_ctx* c) {
     void* ptrs[] = {c->d_thetap, c->d_W,    c->d_Z,     c->d_Yk,    c->d_snorm, c->d_desc,  c->d_cta,
                     c->d_sync,   c->d_sweeps, c->d_pre_ok, c->d_W0,  c->d_E,     c->d_Q,     c->d_W32,
                     c->d_U32,    c->d_gemm,  c->d_copy,  c->d_oz_as, c->d_oz_bs, c->d_oz_ea, c->d_oz_eb,
-                    c->d_oz};
+                    c->d_oz,     c->d_refine};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    c->d_refine = nullptr;
     c->d_thetap = c->d_W = c->d_Z = c->d_Yk = c->d_snorm = nullptr;
     c->d_W0 = c->d_E = c->d_Q = nullptr;
     c->d_W32 = c->d_U32 = nullptr;
@@ -102,8 +103,8 @@ int alloc_slots(mpdo_ctx* c, int want) {
     release_slots(c);
     const size_t mat = (size_t)c->ld * c->ld;
     size_t per_slot_bytes = (3 * mat + (size_t)c->cap * c->ld + 2 * c->ld) * sizeof(double);
-    if (c->mixed) {
-        c->oz_slot_bytes = oz_slice_bytes(c->ld, c->ld, c->oz_bf16);
+    if (c->precond) {
+        c->oz_slot_bytes = oz_slice_bytes(c->ld, c->ld, c->oz_bf16, c->oz_s);
         per_slot_bytes += 3 * mat * sizeof(double) + 2 * mat * sizeof(float) + 2 * c->oz_slot_bytes +
                           2 * oz_exp_ints(c->ld) * sizeof(int);
     }
@@ -131,7 +132,8 @@ int alloc_slots(mpdo_ctx* c, int want) {
     CU(cudaMallocHost((void**)&c->h_cta, sizeof(int) * 3 * (2 * gcap + s)));
     CU(dalloc(&c->d_copy, (size_t)4 * s));
     CU(cudaMallocHost((void**)&c->h_copy, sizeof(Copy2D) * 4 * s));
-    if (c->mixed) {
+    if (c->precond) {
+        CU(dalloc(&c->d_refine, (size_t)s));
         CU(dalloc(&c->d_W0, (size_t)s * mat));
         CU(dalloc(&c->d_E, (size_t)s * mat));
         CU(dalloc(&c->d_Q, (size_t)s * mat));
@@ -265,21 +267,47 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.jb = tuned_block_rows(c, d.cl, d.cr, false, jacobi_block_rows(d.L, d.c, 8));
     d.jb32 = tuned_block_rows(c, d.cl, d.cr, true, jacobi_block_rows_f32(d.L, d.c));
     d.sweeps_out = c->d_sweeps + s;
-    d.pre_ok = c->mixed ? c->d_pre_ok + s : nullptr;
+    d.pre_ok = c->precond ? c->d_pre_ok + s : nullptr;
+    d.rf = refine_on(c) ? c->d_refine + s : nullptr;
     d.forced_k = 0;
     d.full_svd = c->full_svd ? 1 : 0;
     d.tape_V = nullptr;
     d.tape_s = nullptr;
-    d.W0 = c->mixed ? c->d_W0 + (size_t)s * mat : d.W;
-    d.W32 = c->mixed ? c->d_W32 + (size_t)s * mat : nullptr;
-    d.U32 = c->mixed ? c->d_U32 + (size_t)s * mat : nullptr;
-    d.E = c->mixed ? c->d_E + (size_t)s * mat : nullptr;
-    d.Q = c->mixed ? c->d_Q + (size_t)s * mat : nullptr;
+    d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
+    d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
+    d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
+    d.E = c->precond ? c->d_E + (size_t)s * mat : nullptr;
+    d.Q = c->precond ? c->d_Q + (size_t)s * mat : nullptr;
     d.Zinit = nullptr;
-    d.oz_as = c->mixed ? c->d_oz_as + (size_t)s * c->oz_slot_bytes : nullptr;
-    d.oz_bs = c->mixed ? c->d_oz_bs + (size_t)s * c->oz_slot_bytes : nullptr;
-    d.oz_ea = c->mixed ? c->d_oz_ea + (size_t)s * oz_exp_ints(ld) : nullptr;
-    d.oz_eb = c->mixed ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
+    d.oz_as = c->precond ? c->d_oz_as + (size_t)s * c->oz_slot_bytes : nullptr;
+    d.oz_bs = c->precond ? c->d_oz_bs + (size_t)s * c->oz_slot_bytes : nullptr;
+    d.oz_ea = c->precond ? c->d_oz_ea + (size_t)s * oz_exp_ints(ld) : nullptr;
+    d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
+}
+
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st) {
+    const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
+    auto oz = [&](int kind) {
+        return launch_oz_ops(d_desc, nops, kind, c->d_oz, c->cap, c->oz_bf16, c->oz_s, timeout_ns, st);
+    };
+    // E = U U^T - I (~1e-6), then one orthogonalisation step: second order
+    // (Q = U - E U / 2, defect 3 E^2 / 4) on the mixed path, third order (defect
+    // 5 E^3 / 8, below FP64 rounding) on the FP64 path
+    std::vector<int> kinds = {OZ_E, OZ_Q, OZ_W};
+    if (!c->mixed) kinds = {OZ_E, OZ_T, OZ_Q3, OZ_W};
+    for (int kind : kinds) {
+        const cudaError_t e = oz(kind);
+        if (e != cudaSuccess) return e;
+    }
+    if (!refine_on(c)) return cudaSuccess;
+    // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
+    const double tol = fp64_jacobi_tol(c);
+    const bool can = c->oz_s == 7 || tol >= 1e-12;
+    return launch_refine(d_desc, nops, c->d_oz, c->cap, c->oz_bf16, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
+}
+
+int svd_products_kernels(const mpdo_ctx* c) {
+    return (c->mixed ? 9 : 12) + (refine_on(c) ? kRefineKernels : 0);
 }
 
 int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* forced, const TapeSlot* tape,
@@ -332,7 +360,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     ProfScope p_merge(c, K_MERGE);
     if (c->mixed) {
-        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, c->d_oz, cap, c->oz_bf16, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, c->d_oz, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
         CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
     } else {
         CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
@@ -436,22 +464,19 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         }
     }
     double fl_gemm = 0.0;
-    if (c->mixed) {
+    if (c->precond) {
         // FP32 preconditioning Jacobi on (W32 | U32)
         ProfScope p_j32(c, K_JACOBI32);
         int rc = run_jacobi(true, 1);
         if (rc) return rc;
         p_j32.stop();
-        // E = U U^T - I, Q = U - E U / 2 (one Newton-Schulz step), W = Q W0, all
-        // FP64-accurate tensor-core products (oz_gemm.cu)
+        // Q from U32, W = Q W0 and the rows' refinement: FP64-accurate tensor-core products
         for (int s = 0; s < nops; ++s) {
             const OpDesc& d = c->h_desc[s];
             fl_gemm += 2.0 * d.c * d.c * d.c * 2 + 2.0 * d.c * d.c * d.L;
         }
         ProfScope p_gemm(c, K_GEMM);
-        CU(launch_oz_ops(c->d_desc, nops, OZ_E, c->d_oz, cap, c->oz_bf16, timeout_ns, c->st));
-        CU(launch_oz_ops(c->d_desc, nops, OZ_Q, c->d_oz, cap, c->oz_bf16, timeout_ns, c->st));
-        CU(launch_oz_ops(c->d_desc, nops, OZ_W, c->d_oz, cap, c->oz_bf16, timeout_ns, c->st));
+        CU(launch_svd_products(c, c->d_desc, nops, c->st));
         p_gemm.stop();
     }
     ProfScope p_jac(c, K_JACOBI);
@@ -465,7 +490,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     p_tr.stop();
     ProfScope p_rec(c, K_RECON);
     if (c->mixed)
-        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, c->d_oz, cap, c->oz_bf16, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, c->d_oz, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
     else
         CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
     p_rec.stop();
@@ -497,9 +522,9 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     prof_collect(c, K_MERGE, fl_merge, c->mixed ? 4 : 1);
     prof_collect(c, K_QR, qr_flops_chunk, qr_kernels_chunk);
     prof_collect(c, K_JACOBI, fl_svd, 1);
-    if (c->mixed) {
+    if (c->precond) {
         prof_collect(c, K_JACOBI32, 0.0, 1);
-        prof_collect(c, K_GEMM, fl_gemm, 9);
+        prof_collect(c, K_GEMM, fl_gemm, svd_products_kernels(c));
     }
     prof_collect(c, K_TRUNC, 0.0, 1);
     prof_collect(c, K_RECON, fl_rec, c->mixed ? 3 : 1);
@@ -620,7 +645,9 @@ int mpdo_init(mpdo_ctx** out, const mpdo_config* cfg, void* cuda_stream) {
     if (!c) return fail(MPDO_ENOMEM, "host allocation failed");
     c->dev = dev;
     c->mixed = cfg->precision != MPDO_FP64;
-    c->oz_bf16 = cfg->precision == MPDO_MIXED_BF16X3;
+    c->oz_bf16 = cfg->precision != MPDO_MIXED_TF32;
+    c->oz_s = c->mixed ? 6 : 7;
+    c->precond = c->mixed || cfg->jacobi_max_sweeps >= kRefineMinSweeps;
     c->cfg = *cfg;
     c->st = (cudaStream_t)cuda_stream;
     c->N = cfg->n_qubits;

@@ -63,4 +63,36 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// The kk-th largest of v[0..c), c <= NMAX (non-negative), by bisection on the
+// bit pattern (non-negative doubles order like their bits).  Called by every
+// thread of a CTA of NT threads; every thread returns the same value.
+template <int NT, int NMAX>
+__device__ double kth_largest(const double* v, int c, int kk) {
+    constexpr int kPer = (NMAX + NT - 1) / NT;
+    __shared__ int s_cnt[NT / 32];
+    unsigned long long key[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int j = threadIdx.x + i * NT;
+        key[i] = j < c ? (unsigned long long)__double_as_longlong(fmax(__ldcg(v + j), 0.0)) : 0ull;
+    }
+    unsigned long long x = 0ull;
+    for (int bit = 62; bit >= 0; --bit) {
+        const unsigned long long cand = x | (1ull << bit);
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) n += key[i] >= cand;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = n;
+        __syncthreads();
+        int tot = 0;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) tot += s_cnt[w];
+        __syncthreads();
+        if (tot >= kk) x = cand;
+    }
+    return __longlong_as_double((long long)x);
+}
+
 }  // namespace mpdo
+

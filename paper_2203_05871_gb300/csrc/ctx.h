@@ -87,7 +87,10 @@ struct mpdo_ctx {
     int* d_sweeps = nullptr;      // [slots] Jacobi sweeps of the last chunk
     int* d_pre_ok = nullptr;      // [slots] mixed path: the FP32 pass ended by its off-orthogonality rule
     bool mixed = false;           // mixed-precision SVD (FP32 preconditioning + FP64 finish)
-    bool oz_bf16 = false;         // mixed path: tensor-core slices in bf16 (MPDO_MIXED_BF16X3), else tf32
+    bool precond = false;         // SVD with FP32 preconditioning and Gram-matrix refinement (mixed and FP64 paths)
+    bool oz_bf16 = false;         // tensor-core slices in bf16 (MPDO_MIXED_BF16X3, FP64 path), else tf32
+    int oz_s = 6;                 // slices per operand of the SVD's products: 6 (mixed path), 7 (FP64 path)
+    mpdo::RefineOp* d_refine = nullptr;   // [slots]
     unsigned char *d_oz_as = nullptr, *d_oz_bs = nullptr;   // [slots] slice blocks of the tensor-core products
     int *d_oz_ea = nullptr, *d_oz_eb = nullptr;             // [slots][4 chi_cap] their exponents
     mpdo::OzProblem* d_oz = nullptr;                        // [slots] problems of one launch
@@ -210,6 +213,18 @@ inline double precond_rho(const mpdo_ctx* c) { return c->cfg.precond_rho > 0.0 ?
 inline double fp64_jacobi_tol(const mpdo_ctx* c) {
     return (c->cfg.jacobi_tol <= 0.0 && c->mixed && !c->full_svd) ? kMixedFinishTol : c->cfg.jacobi_tol;
 }
+
+// With a sweep limit under this every SVD is left to the Jacobi passes alone (FP64
+// path: the FP64 pass alone), whose sweeps the limit counts; the other stages
+// take the place of a handful of them.
+constexpr int kRefineMinSweeps = 16;
+inline bool refine_on(const mpdo_ctx* c) { return c->precond && c->cfg.jacobi_max_sweeps >= kRefineMinSweeps; }
+
+// The stages between the FP32 preconditioning pass and the FP64 Jacobi pass:
+// Q, the orthogonalised U32, W = Q W0, and the refinement of W's rows.
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st);
+// kernels one launch_svd_products issues
+int svd_products_kernels(const mpdo_ctx* c);
 
 int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* forced, const TapeSlot* tape,
               bool log_ranks);

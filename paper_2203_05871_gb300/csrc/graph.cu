@@ -68,7 +68,7 @@ __device__ int plan_ctas(const double* work, const int* cap, int nops, int R, in
 constexpr int kMaxChunk = 1024;
 
 __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops, const int* dims, int N, int Rj,
-                                                         int Rq, int* cta64, int* cta32, int* ctaqr, int mixed,
+                                                         int Rq, int* cta64, int* cta32, int* ctaqr, int precond,
                                                          const int* jb_table, int chi_cap, int* error) {
     __shared__ double work[kMaxChunk];
     __shared__ int cap[kMaxChunk];
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
         cap[s] = jacobi_pairs_per_round(d.c, d.jb);
     }
     bad |= plan_ctas(work, cap, nops, Rj, cta64);
-    if (mixed) {
+    if (precond) {
         for (int s = 0; s < nops; ++s) cap[s] = jacobi_pairs_per_round(descs[s].c, descs[s].jb32);
         bad |= plan_ctas(work, cap, nops, Rj, cta32);
     }
@@ -168,12 +168,12 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
         for (auto& ch : L) {
             const int nops = ch.nops;
             plan_chunk_kernel<<<1, 256, 0, st>>>(ch.d_desc, nops, c->d_dims, c->N, g->Rj, g->Rq, ch.d_cta64,
-                                                 ch.d_cta32, ch.d_ctaqr, c->mixed ? 1 : 0, c->d_jb_table, cap,
+                                                 ch.d_cta32, ch.d_ctaqr, c->precond ? 1 : 0, c->d_jb_table, cap,
                                                  g->d_error);
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
             if (c->mixed) {
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, c->d_oz, cap, c->oz_bf16, timeout_ns, st));
+                CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, c->d_oz, cap, c->oz_bf16, c->oz_s, timeout_ns, st));
                 CU(launch_gate_weight(ch.d_desc, nops, cap, st));
             } else {
                 CU(launch_merge_gate(ch.d_desc, nops, cap, st));
@@ -185,20 +185,18 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             else
                 CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
                              timeout_ns, ld, st));
-            if (c->mixed) {
+            if (c->precond) {
                 CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
                 CU(launch_jacobi(ch.d_desc, nops, ch.d_cta32, ch.d_cta32 + g->Rj, ch.d_cta32 + 2 * g->Rj, c->d_sync,
                                  g->Rj, kMaxSweepsCap / 2, 0.0, timeout_ns, ld, true, st, precond_rho(c)));
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_E, c->d_oz, cap, c->oz_bf16, timeout_ns, st));
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_Q, c->d_oz, cap, c->oz_bf16, timeout_ns, st));
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_W, c->d_oz, cap, c->oz_bf16, timeout_ns, st));
+                CU(launch_svd_products(c, ch.d_desc, nops, st));
             }
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
             CU(launch_jacobi(ch.d_desc, nops, ch.d_cta64, ch.d_cta64 + g->Rj, ch.d_cta64 + 2 * g->Rj, c->d_sync, g->Rj,
                              c->cfg.jacobi_max_sweeps, fp64_jacobi_tol(c), timeout_ns, ld, false, st, precond_rho(c)));
             CU(launch_truncate(ch.d_desc, nops, cap, st));
             if (c->mixed)
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, c->d_oz, cap, c->oz_bf16, timeout_ns, st));
+                CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, c->d_oz, cap, c->oz_bf16, c->oz_s, timeout_ns, st));
             else
                 CU(launch_reconstruct(ch.d_desc, nops, cap, st));
             klog_kernel<<<(nops + 127) / 128, 128, 0, st>>>(ch.d_desc, nops, c->n_ops, g->d_klog);
@@ -232,7 +230,7 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
             CU(dalloc(&ch.d_desc, (size_t)nops));
             CU(dalloc(&ch.d_cta64, (size_t)2 * g->Rj + nops));
             CU(dalloc(&ch.d_ctaqr, (size_t)2 * g->Rq + nops));
-            if (c->mixed) CU(dalloc(&ch.d_cta32, (size_t)2 * g->Rj + nops));
+            if (c->precond) CU(dalloc(&ch.d_cta32, (size_t)2 * g->Rj + nops));
             CU(cudaMemcpyAsync(ch.d_desc, h.data(), sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
             CU(cudaStreamSynchronize(c->st));
             g->chunks[li].push_back(ch);

@@ -36,6 +36,7 @@ std::string build_schedule(int n, const std::vector<int>& bi, const std::vector<
 // All pointers are device pointers.  Matrices in the workspace are row-major
 // with leading dimension ld = 4 * chi_cap.
 // ---------------------------------------------------------------------------
+struct RefineOp;
 struct OpDesc {
     int b;             // instance
     int op;            // op index within the step (for the rank log)
@@ -74,6 +75,7 @@ struct OpDesc {
     int* pre_ok;       // mixed path: 1 when the FP32 pass ended with every pair orthogonal to ~1e-6
                        // (its last sweep rotated by at most 1e-3); written by that pass, read by
                        // the FP64 pass (or nullptr)
+    RefineOp* rf;      // state of the Gram-matrix refinement (refine.cu), or nullptr without it
     int forced_k;      // > 0: truncation rank imposed (replay of a recorded run)
     int full_svd;      // 1: orthogonalise every pair of rows (the adjoint needs all singular vectors)
     double* tape_V;    // adjoint recompute: all c sorted right singular vectors (c x n), or nullptr
@@ -176,6 +178,8 @@ struct OzOperand {
     long long rs, ks;
     int mode, cr, cap;
     const int* gather;   // row gather (mode 0), or nullptr
+    const double* kn;    // element (r, k) is multiplied by 2^(ksgn e_k), 2^e_k ~ sqrt(kn[k]) (f64 views), or nullptr
+    int ksgn;
 };
 // C = alpha A B + beta D (- I), C and D row-major (f64 or f32); row i of C and D
 // is row c_gather[i] of their storage when c_gather is set
@@ -189,6 +193,7 @@ struct OzProblem {
     double alpha, beta;
     const void* D;
     int ldd, d_f32, sub_identity;
+    int sym;             // C (f64, no gather) is symmetric: tiles below the diagonal are mirrored, not computed
     void *as, *bs;       // slice blocks of A and B
     int *ea, *eb;        // row / column exponents
     int Mt, Nt, Kt;      // tiles (128 rows, 64 columns, 64 bytes of K)
@@ -201,23 +206,52 @@ __host__ __device__ inline void oz_set_tiles(OzProblem& p, bool bf16) {
     p.Nt = (p.N + 63) / 64;
     p.Kt = (p.K + KT - 1) / KT;
 }
-size_t oz_slice_bytes(int rows, int K, bool bf16);   // slice blocks of an operand of rows x K
+size_t oz_slice_bytes(int rows, int K, bool bf16, int S);   // slice blocks of an operand of rows x K
 size_t oz_exp_ints(int rows);                          // its exponent array (rows rounded up to a tile)
 void oz_tiles(OzProblem& p, bool bf16);
 cudaError_t oz_prepare();
 // slices both operands of count problems, then multiplies; max_m / max_n /
 // max_rows_sliced bound the grids (CTAs outside a problem's tiles return)
+// S slices per operand: 6 (error 2^-46 of the row and column maxima per term) or
+// 7 (2^-54, an FP64 product's level; bf16 slices only)
 cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
-                           unsigned long long timeout_ns, cudaStream_t st);
+                           int S, unsigned long long timeout_ns, cudaStream_t st);
 
 // The mixed path's tensor-core products of a chunk of ops, built on the
 // device from the op descriptors (so the host-planned and the graph step
 // share them): kind OZ_MERGE Theta = A B (then launch_gate_weight applies the
 // gate and the left weights), OZ_RECON B_p' = Theta' Yk^T, OZ_E E = U U^T - I,
-// OZ_Q Q = U - E U / 2, OZ_W W = Q W0.  probs: scratch for nops problems.
-enum { OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4 };
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16,
+// OZ_Q Q = U - E U / 2, OZ_W W = Q W0; OZ_T T = U - 3 E U / 4 then OZ_Q3
+// Q = U - E T / 2 (third-order orthogonalisation); OZ_G G = W W^T and OZ_R3,
+// OZ_R2, OZ_R1 the refinement's rotation (refine.cu).  probs: scratch for nops problems.
+enum { OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T = 5, OZ_Q3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
+       OZ_R1 = 10 };
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16, int S,
                           unsigned long long timeout_ns, cudaStream_t st);
+// ---------------------------------------------------------------------------
+// Refinement of nearly orthogonal rows through their Gram matrix (refine.cu)
+// ---------------------------------------------------------------------------
+enum { kRefineActive = 0, kRefineDone = 1, kRefineLeft = 2 };
+struct RefineOp {
+    int state;        // kRefineActive; kRefineDone: every needed pair is orthogonal to tol (the Jacobi
+                      // pass has nothing to do); kRefineLeft: the Jacobi pass finishes the op
+    int order;        // terms of this iteration's rotation (0: none)
+    unsigned rho2;    // largest g^2 / (a b) of a needed pair (float bits)
+    int far;          // a needed pair's angle is beyond the expansion
+    unsigned row1;    // largest absolute row sum of X (float bits)
+    double thr;       // pairs of rows whose squared norms are both below it are not needed
+    double floor2;    // squared norm of a numerically zero row
+};
+// The iterations of a chunk: W's rows, as orthogonal as the FP32 pass left them, are
+// rotated until every needed pair is orthogonal to tol (state kRefineDone) or the
+// op is left to the Jacobi pass.  Scratch: d.E (G), d.Q (X), d.W0, d.snorm.
+// tol_in as for launch_jacobi; can_finish = false: never kRefineDone.
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, OzProblem* probs, int chi_cap, bool bf16, int S,
+                          double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
+constexpr int kRefineIters = 3;
+// kernels of one launch_refine
+constexpr int kRefineKernels = 1 + kRefineIters * (3 + 3 * 4);
+
 // Theta' = G Theta in place in thetap and theta~ = lambda_l Theta' (column-major, Acm)
 cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st);
 

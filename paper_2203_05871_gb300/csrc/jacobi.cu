@@ -677,36 +677,6 @@ __device__ int block_pair_reg(const RegCtx& C, float* W, float* Z, int ld, int c
     return rot;
 }
 
-// The kk-th largest of v[0..c) (non-negative), by bisection on the bit
-// pattern (non-negative doubles order like their bits).  Called by every
-// thread of a CTA of kThreads<double>; every thread returns the same value.
-constexpr int kSelPer = (4 * kMaxChi + kThreads<double> - 1) / kThreads<double>;
-__device__ double kth_largest(const double* v, int c, int kk) {
-    __shared__ int s_cnt[kWarps<double>];
-    unsigned long long key[kSelPer];
-#pragma unroll
-    for (int i = 0; i < kSelPer; ++i) {
-        const int j = threadIdx.x + i * kThreads<double>;
-        key[i] = j < c ? (unsigned long long)__double_as_longlong(fmax(__ldcg(v + j), 0.0)) : 0ull;
-    }
-    unsigned long long x = 0ull;
-    for (int bit = 62; bit >= 0; --bit) {
-        const unsigned long long cand = x | (1ull << bit);
-        int n = 0;
-#pragma unroll
-        for (int i = 0; i < kSelPer; ++i) n += key[i] >= cand;
-        n = __reduce_add_sync(0xffffffffu, n);
-        if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = n;
-        __syncthreads();
-        int tot = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps<double>; ++w) tot += s_cnt[w];
-        __syncthreads();
-        if (tot >= kk) x = cand;
-    }
-    return __longlong_as_double((long long)x);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kThreads<T>, 1) jacobi_kernel(const OpDesc* descs, const int* cta_op, const int* cta_rank,
                                                        const int* group, unsigned* sync, int max_sweeps,
@@ -719,6 +689,7 @@ __global__ void __launch_bounds__(kThreads<T>, 1) jacobi_kernel(const OpDesc* de
     const int g = cta_rank[blockIdx.x];
     const int G = group[op];
     const OpDesc& d = descs[op];
+    if (!kF32 && d.rf && d.rf->state == kRefineDone) return;   // finished by the refinement (refine.cu)
     unsigned* sw = sync + (size_t)op * kSyncWords;
     const int c = d.c, L = d.L;
     int b = kF32 ? d.jb32 : d.jb;
@@ -876,7 +847,7 @@ __global__ void __launch_bounds__(kThreads<T>, 1) jacobi_kernel(const OpDesc* de
                 // the threshold is fixed when the gate first opens, so that a row
                 // near it keeps its side (a row changing side later would bring its
                 // unprocessed pairs back and cost another sweep)
-                if (s_conv && C.thr == 0.0) C.thr = kth_largest(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
+                if (s_conv && C.thr == 0.0) C.thr = kth_largest<kThreads<double>, 4 * kMaxChi>(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
                 __syncthreads();
             }
             // The block pairs of a sweep go to the op's CTAs through a shared

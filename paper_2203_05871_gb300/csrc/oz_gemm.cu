@@ -61,19 +61,20 @@ namespace mpdo {
 
 namespace {
 
-constexpr int kS = 6;                  // slices per operand
-constexpr int kPairs = 21;             // (t, u) with t + u <= 5
-constexpr int kLevels = 6;             // one accumulator per level t + u
+// S slices per operand (6 or 7): S (S + 1) / 2 slice pairs (t, u) with
+// t + u < S, one accumulator per level t + u
+
 constexpr int kTileM = 128;            // rows of A (and of C) per tile
 constexpr int kTileN = 64;             // columns of B (and of C) per tile
 constexpr int kBlockA = kTileM * 64;   // bytes of one slice block of A (8 KB)
 constexpr int kBlockB = kTileN * 64;   // of B (4 KB)
-constexpr int kStageBytes = kS * (kBlockA + kBlockB);   // A and B slices of one k tile
-constexpr int kStages = 3;
+__host__ __device__ constexpr int stage_bytes(int S) { return S * (kBlockA + kBlockB); }   // A and B slices of one k tile
+__host__ __device__ constexpr int stages_of(int S) { return S == 6 ? 3 : 2; }               // 216 KB / 168 KB of shared memory
 constexpr int kRangeK = 256;           // K values between accumulator drains
 constexpr int kThreads = 320;
-constexpr int kSmem = kStages * kStageBytes + 1024;
-static_assert(kLevels * kTileN <= 512, "accumulators exceed tensor memory");
+__host__ __device__ constexpr int smem_of(int S) { return stages_of(S) * stage_bytes(S) + 1024; }
+static_assert(7 * kTileN <= 512, "accumulators exceed tensor memory");
+static_assert(smem_of(6) <= 227 * 1024 && smem_of(7) <= 227 * 1024, "the ring exceeds shared memory");
 static_assert(kTileM == 128 && kTileN == 64, "oz_set_tiles (internal.h) assumes 128 x 64 tiles");
 constexpr int LBO = 128, SBO = 512;
 
@@ -157,15 +158,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ int pair_t(int p) {   // pairs in order of level: (0,0) (0,1)(1,0) (0,2)(1,1)(2,0) ...
-    constexpr int T[kPairs] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3, 0, 1, 2, 3, 4, 0, 1, 2, 3, 4, 5};
-    return T[p];
-}
-__device__ __forceinline__ int pair_u(int p) {
-    constexpr int U[kPairs] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0, 4, 3, 2, 1, 0, 5, 4, 3, 2, 1, 0};
-    return U[p];
-}
-
 // index of element (r, k) of an operand view
 __device__ __forceinline__ size_t oz_index(const OzOperand& X, int r, int k) {
     if (X.mode == 1) return ((size_t)k * 4 + (size_t)(r / X.cr)) * X.cap + (r % X.cr);
@@ -180,8 +172,18 @@ __device__ __forceinline__ size_t oz_index(const OzOperand& X, int r, int k) {
 // Bit pattern of element (r, k), zero-extended (f32 views: 32 bits).
 __device__ __forceinline__ unsigned long long oz_bits(const OzOperand& X, int r, int k) {
     const size_t i = oz_index(X, r, k);
-    return X.f32 ? (unsigned long long)__float_as_uint(static_cast<const float*>(X.base)[i])
-                 : (unsigned long long)__double_as_longlong(static_cast<const double*>(X.base)[i]);
+    if (X.f32) return (unsigned long long)__float_as_uint(static_cast<const float*>(X.base)[i]);
+    unsigned long long v = (unsigned long long)__double_as_longlong(static_cast<const double*>(X.base)[i]);
+    if (X.kn) {   // exponent shift; zeros and non-finite values stay, what would leave the range goes to 0
+        const int ek = (int)(((unsigned)__double2hiint(X.kn[k]) >> 20) & 0x7ff);
+        const int E = (int)((v >> 52) & 0x7ff);
+        if (ek != 0 && E != 0 && E != 0x7ff) {
+            const int En = E + X.ksgn * ((ek - 1023) >> 1);
+            v = En > 0 && En < 0x7ff ? (v & 0x800fffffffffffffull) | ((unsigned long long)En << 52)
+                                     : (En <= 0 ? 0ull : 0x7ff8000000000000ull);
+        }
+    }
+    return v;
 }
 
 // |x| as an unsigned key that orders like |x| within one storage type
@@ -209,8 +211,9 @@ __device__ __forceinline__ int key_exponent(unsigned long long key, bool f32) {
     return e;
 }
 
-// X = round(x 2^(47 - e)) for a finite x = +-m 2^p of a row with exponent e
-// (|x| < 2^e, so |X| <= 2^47), ties away from zero
+// X = round(x 2^(8S - 1 - e)) for a finite x = +-m 2^p of a row with exponent e
+// (|x| < 2^e, so |X| <= 2^(8S - 1)), ties away from zero
+template <int S>
 __device__ __forceinline__ long long fixed_of(unsigned long long bits, bool f32, int e) {
     bool neg;
     unsigned long long m;
@@ -236,12 +239,12 @@ __device__ __forceinline__ long long fixed_of(unsigned long long bits, bool f32,
             p = -1074;
         }
     }
-    const int sh = p + 47 - e;
+    const int sh = p + (8 * S - 1) - e;
     long long X;
     if (m == 0)
         X = 0;
     else if (sh >= 0)
-        X = (long long)(m << (sh < 63 ? sh : 63));   // m 2^sh < 2^47: no bits leave
+        X = (long long)(m << (sh < 63 ? sh : 63));   // m 2^sh < 2^(8S - 1): no bits leave
     else if (sh <= -62)
         X = 0;
     else
@@ -249,11 +252,11 @@ __device__ __forceinline__ long long fixed_of(unsigned long long bits, bool f32,
     return neg ? -X : X;
 }
 
-// The slices of G consecutive fixed-point values X[0..G) (|X| <= 2^47):
-// balanced base-256 digits X = sum_t sigma_t 2^(8(5 - t)), |sigma_t| <= 128,
+// The S slices of G consecutive fixed-point values X[0..G) (|X| <= 2^(8S - 1)):
+// balanced base-256 digits X = sum_t sigma_t 2^(8(S - 1 - t)), |sigma_t| <= 128,
 // from the lowest digit up; stored as sigma_t 2^-8t, 16 bytes per slice.
 // nan: the row has a non-finite entry, every slice is NaN.
-template <int G, bool kBf16>
+template <int G, bool kBf16, int kS>
 __device__ __forceinline__ void slice_group(const long long* X, bool nan, uint4* out /* [kS] */) {
     int sig[kS][G];
 #pragma unroll
@@ -291,7 +294,7 @@ __device__ __forceinline__ void slice_group(const long long* X, bool nan, uint4*
 // Strided views (a transposed operand, the right site of a merge): a block
 // takes 32 consecutive rows, lane = row and warp = a slice of the K range, so
 // that the 32 lanes of a load read 32 neighbouring rows at one k (coalesced).
-template <bool kBf16>
+template <bool kBf16, int kS>
 __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int Kt, unsigned char* out, int* ex,
                                  int tile, int Rt) {
     constexpr int esize = kBf16 ? 2 : 4;
@@ -322,10 +325,10 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int K
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const int k = g0 + g;
-            x[g] = (live && !bad && k < K) ? fixed_of(oz_bits(X, r, k), f32, e) : 0;
+            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
         }
         uint4 sl[kS];
-        slice_group<G, kBf16>(x, bad && live, sl);
+        slice_group<G, kBf16, kS>(x, bad && live, sl);
         const int kt = g0 / KT, kk = g0 % KT;
 #pragma unroll
         for (int t = 0; t < kS; ++t) {
@@ -338,7 +341,7 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int K
 // grid (row groups of 8, 2 = A | B, problems).  Views whose rows are
 // contiguous (ks == 1) take one warp per row, lanes along k; the others 32 rows
 // per block (slice_rows_tiled), the blocks past rows / 32 returning at once.
-template <bool kBf16>
+template <bool kBf16, int kS>
 __global__ void __launch_bounds__(256) oz_slice_kernel(const OzProblem* probs) {
     constexpr int esize = kBf16 ? 2 : 4;
     constexpr int G = 16 / esize;          // values per 16-byte store
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const OzProblem* probs) {
     if (!(X.mode == 0 && X.ks == 1)) {
         const int r0 = blockIdx.x * 32;
         if (r0 >= Rt * tile) return;   // uniform over the block (Rt * tile is a multiple of 32)
-        slice_rows_tiled<kBf16>(X, r0, R, K, Kt, out, ex, tile, Rt);
+        slice_rows_tiled<kBf16, kS>(X, r0, R, K, Kt, out, ex, tile, Rt);
         return;
     }
     const int r = blockIdx.x * 8 + warp;
@@ -386,10 +389,10 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const OzProblem* probs) {
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const int k = g0 + g;
-            x[g] = (live && !bad && k < K) ? fixed_of(oz_bits(X, r, k), f32, e) : 0;
+            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
         }
         uint4 sl[kS];
-        slice_group<G, kBf16>(x, bad && live, sl);
+        slice_group<G, kBf16, kS>(x, bad && live, sl);
         const int kt = g0 / KT, kk = g0 % KT;
 #pragma unroll
         for (int t = 0; t < kS; ++t) {
@@ -399,21 +402,22 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const OzProblem* probs) {
     }
 }
 
-// barriers: full[kStages], empty[kStages], accumulators full, accumulators drained, final
-constexpr int kBarFull = 0, kBarEmpty = kStages, kBarAccFull = 2 * kStages, kBarAccEmpty = 2 * kStages + 1,
-              kBarFinal = 2 * kStages + 2;
-
-template <bool kBf16>
+template <bool kBf16, int kS>
 __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const OzProblem* probs,
                                                                unsigned long long timeout_ns) {
     constexpr int esize = kBf16 ? 2 : 4;
     constexpr int KT = kt_elems(esize);
     constexpr int kRangeTiles = kRangeK / KT;
+    constexpr int kLevels = kS, kStages = stages_of(kS), kStageBytes = stage_bytes(kS);
+    // barriers: full[kStages], empty[kStages], accumulators full, accumulators drained, final
+    constexpr int kBarFull = 0, kBarEmpty = kStages, kBarAccFull = 2 * kStages, kBarAccEmpty = 2 * kStages + 1,
+                  kBarFinal = 2 * kStages + 2;
     extern __shared__ __align__(1024) unsigned char smem[];
     const OzProblem& P = probs[blockIdx.z];
     const int N = P.Ndyn ? *P.Ndyn : P.N;
     const int mt = blockIdx.y, nt = blockIdx.x;
     if (mt * kTileM >= P.M || nt * kTileN >= N) return;
+    if (P.sym && (nt + 1) * kTileN <= mt * kTileM) return;   // mirrored from above the diagonal
     const int Kt = P.Kt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -496,16 +500,18 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const OzProblem* p
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 const uint32_t st = smem_u32(smem + (size_t)s * kStageBytes);
 #pragma unroll
-                for (int p = 0; p < kPairs; ++p) {
-                    const int t = pair_t(p), u = pair_u(p);
-                    const int lvl = t + u;
+                for (int lvl = 0; lvl < kLevels; ++lvl) {
                     const uint32_t d = tmem + (uint32_t)(lvl * kTileN);
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const uint32_t off = q * 2 * LBO;
-                        mma(kBf16, d, smem_desc(st + t * kBlockA + off), smem_desc(st + kS * kBlockA + u * kBlockB + off),
-                            id, first[lvl] ? 0u : 1u);
-                        first[lvl] = false;
+                    for (int t = 0; t <= lvl; ++t) {
+                        const int u = lvl - t;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const uint32_t off = q * 2 * LBO;
+                            mma(kBf16, d, smem_desc(st + t * kBlockA + off),
+                                smem_desc(st + kS * kBlockA + u * kBlockB + off), id, first[lvl] ? 0u : 1u);
+                            first[lvl] = false;
+                        }
                     }
                 }
                 commit(smem_u32(bar + kBarEmpty + s));   // frees the stage once these MMAs have read it
@@ -534,9 +540,9 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const OzProblem* p
             }
             asm volatile("tcgen05.fence::after_thread_sync;");
             // level d holds n_d 2^-8d with n_d an integer (exact for d <= 3;
-            // levels 4 and 5 are rounded to the nearest 2^-32 and 2^-40):
-            // the range's sum is S 2^-40 with the integer
-            // S = sum_d n_d 2^(8 (5 - d)), |S| < 2^63, formed in int64 and
+            // higher levels are rounded to the nearest 2^-8d): the range's
+            // sum is S 2^-40 with the integer S = sum_d n_d 2^(8 (5 - d)),
+            // |S| < 2^63 (level 6 rounded to that unit), formed in int64 and
             // converted once (integer arithmetic instead of twelve FP64
             // operations per element).  A NaN slice reaches level 0.
 #pragma unroll
@@ -551,12 +557,14 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const OzProblem* p
                     const float scale = __int_as_float((127 + 8 * lvl) << 23);   // 2^8d
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const long long n = __float2int_rn(v[i] * scale);
+                        const int n = __float2int_rn(v[i] * scale);
                         if (lvl == 0) {
                             S[i] = n;
                             nan |= (v[i] != v[i]) ? 1u << i : 0u;
-                        } else {
+                        } else if (lvl < 6) {
                             S[i] = S[i] * 256 + n;
+                        } else {
+                            S[i] += (n + 128) >> 8;   // level 6 in units of 2^-40
                         }
                     }
                 }
@@ -590,6 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const OzProblem* p
                         static_cast<float*>(P.C)[ci] = (float)v;
                     else
                         static_cast<double*>(P.C)[ci] = v;
+                    if (P.sym && j > i) static_cast<double*>(P.C)[(size_t)j * P.ldc + i] = v;
                 }
             }
         }
@@ -609,10 +618,10 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
     const int ld = 4 * cap;
     OzProblem P{};
     auto rowmajor = [](const void* base, int f32, long long ld_) {   // (r, k) at r * ld + k
-        return OzOperand{base, f32, ld_, 1, 0, 1, 1, nullptr};
+        return OzOperand{base, f32, ld_, 1, 0, 1, 1, nullptr, nullptr, 0};
     };
     auto colmajor = [](const void* base, int f32, long long ld_) {   // (r, k) at k * ld + r
-        return OzOperand{base, f32, 1, ld_, 0, 1, 1, nullptr};
+        return OzOperand{base, f32, 1, ld_, 0, 1, 1, nullptr, nullptr, 0};
     };
     switch (kind) {
         case OZ_MERGE:   // Theta[(l, s1), (s2, r)] = sum_m A[(l, s1), m] B[m, (s2, r)]
@@ -620,7 +629,7 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
             P.K = d.cm;
             P.N = 4 * d.cr;
             P.A = rowmajor(d.A, d.site_f32, cap);
-            P.B = OzOperand{d.B, d.site_f32, 0, 0, 1, d.cr, cap, nullptr};
+            P.B = OzOperand{d.B, d.site_f32, 0, 0, 1, d.cr, cap, nullptr, nullptr, 0};
             P.C = d.thetap;
             P.ldc = ld;
             break;
@@ -642,19 +651,54 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
             P.C = d.E;
             P.ldc = ld;
             P.sub_identity = 1;
+            P.sym = 1;
             break;
         case OZ_Q:       // Q = U - E U / 2
+        case OZ_T:       // T = U - 3 E U / 4 (in W, free until OZ_W)
+        case OZ_Q3:      // Q = U - E T / 2
             P.M = P.N = P.K = d.c;
             P.A = rowmajor(d.E, 0, ld);
-            P.B = colmajor(d.U32, 1, ld);
-            P.C = d.Q;
+            P.B = kind == OZ_Q3 ? colmajor(d.W, 0, ld) : colmajor(d.U32, 1, ld);
+            P.C = kind == OZ_T ? d.W : d.Q;
             P.ldc = ld;
-            P.alpha = -0.5;
+            P.alpha = kind == OZ_T ? -0.75 : -0.5;
             P.beta = 1.0;
             P.D = d.U32;
             P.ldd = ld;
             P.d_f32 = 1;
             break;
+        case OZ_G:       // G = W W^T (refinement, while the op takes part in it)
+            if (d.rf->state != kRefineActive) break;
+            P.M = P.N = d.c;
+            P.K = d.L;
+            P.A = rowmajor(d.W, 0, ld);
+            P.B = rowmajor(d.W, 0, ld);
+            P.C = d.E;
+            P.ldc = ld;
+            P.alpha = 1.0;
+            P.sym = 1;
+            break;
+        case OZ_R3:      // T1 = X W / 8 + W / 2                     (order 3)
+        case OZ_R2:      // T1 = X T1 + W, or X W / 2 + W            (order 3, 2)
+        case OZ_R1: {    // W  = X T1 + W, or X W + W                (order >= 2, 1)
+            const int order = d.rf->order;
+            if (order < (kind == OZ_R3 ? 3 : kind == OZ_R2 ? 2 : 1)) break;
+            P.M = P.K = d.c;
+            P.N = d.L;
+            P.A = rowmajor(d.Q, 0, ld);
+            const bool fromT = (kind == OZ_R2 && order == 3) || (kind == OZ_R1 && order >= 2);
+            P.B = colmajor(fromT ? d.W0 : d.W, 0, ld);
+            P.A.kn = P.B.kn = d.snorm;   // squared row norms of W: X_ik |w_k| times w_k / |w_k|
+            P.A.ksgn = 1;
+            P.B.ksgn = -1;
+            P.C = kind == OZ_R1 ? d.W : d.W0;
+            P.ldc = ld;
+            P.D = d.W;
+            P.ldd = ld;
+            P.alpha = kind == OZ_R3 ? 0.125 : (kind == OZ_R2 && order == 2 ? 0.5 : 1.0);
+            P.beta = kind == OZ_R3 ? 0.5 : 1.0;
+            break;
+        }
         default:         // OZ_W: W = Q W0
             P.M = d.c;
             P.N = d.L;
@@ -665,10 +709,7 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
             P.ldc = ld;
             break;
     }
-    if (kind != OZ_Q) {
-        P.alpha = 1.0;
-        P.beta = 0.0;
-    }
+    if (kind == OZ_MERGE || kind == OZ_RECON || kind == OZ_E || kind == OZ_W) P.alpha = 1.0;
     P.as = d.oz_as;
     P.bs = d.oz_bs;
     P.ea = d.oz_ea;
@@ -706,14 +747,14 @@ __global__ void __launch_bounds__(256) gate_weight_kernel(const OpDesc* descs, i
 
 }  // namespace
 
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16,
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16, int S,
                           unsigned long long timeout_ns, cudaStream_t st) {
     if (nops <= 0) return cudaSuccess;
     oz_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, kind, probs, chi_cap, bf16 ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int big = 4 * chi_cap;
-    return launch_oz_gemm(probs, nops, big, big, big, bf16, timeout_ns, st);
+    return launch_oz_gemm(probs, nops, big, big, big, bf16, S, timeout_ns, st);
 }
 
 cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st) {
@@ -723,11 +764,11 @@ cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cuda
     return cudaGetLastError();
 }
 
-size_t oz_slice_bytes(int rows, int K, bool bf16) {
+size_t oz_slice_bytes(int rows, int K, bool bf16, int S) {
     // room for either operand: ceil(rows / 128) tiles of 8 KB cover ceil(rows / 64) of 4 KB
     const int KT = kt_elems(bf16 ? 2 : 4);
     const size_t Rt = (rows + kTileM - 1) / kTileM, Kt = (K + KT - 1) / KT;
-    return (size_t)kS * Rt * Kt * kBlockA;
+    return (size_t)S * Rt * Kt * kBlockA;
 }
 
 size_t oz_exp_ints(int rows) { return (size_t)((rows + kTileM - 1) / kTileM) * kTileM; }
@@ -735,29 +776,36 @@ size_t oz_exp_ints(int rows) { return (size_t)((rows + kTileM - 1) / kTileM) * k
 void oz_tiles(OzProblem& p, bool bf16) { oz_set_tiles(p, bf16); }
 
 cudaError_t oz_prepare() {
-    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(oz_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<true, 6>, a, smem_of(6));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<false, 6>, a, smem_of(6));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<true, 7>, a, smem_of(7));
+    return e;
 }
 
-cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced,
-                           bool bf16, unsigned long long timeout_ns, cudaStream_t st) {
-    if (count <= 0) return cudaSuccess;
+namespace {
+
+template <bool kBf16, int S>
+cudaError_t launch_oz(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced,
+                      unsigned long long timeout_ns, cudaStream_t st) {
     const int mt = (max_m + kTileM - 1) / kTileM, nt = (max_n + kTileN - 1) / kTileN;
     const int rows = ((max_rows_sliced + kTileM - 1) / kTileM) * kTileM;
-    dim3 sg((rows + 7) / 8, 2, count);
-    if (bf16)
-        oz_slice_kernel<true><<<sg, 256, 0, st>>>(d_probs);
-    else
-        oz_slice_kernel<false><<<sg, 256, 0, st>>>(d_probs);
-    cudaError_t e = cudaGetLastError();
+    oz_slice_kernel<kBf16, S><<<dim3((rows + 7) / 8, 2, count), 256, 0, st>>>(d_probs);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 g(nt, mt, count);
-    if (bf16)
-        oz_gemm_kernel<true><<<g, kThreads, kSmem, st>>>(d_probs, timeout_ns);
-    else
-        oz_gemm_kernel<false><<<g, kThreads, kSmem, st>>>(d_probs, timeout_ns);
+    oz_gemm_kernel<kBf16, S><<<dim3(nt, mt, count), kThreads, smem_of(S), st>>>(d_probs, timeout_ns);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
+                           int S, unsigned long long timeout_ns, cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    if (S == 7)   // bf16 slices only
+        return launch_oz<true, 7>(d_probs, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
+    return bf16 ? launch_oz<true, 6>(d_probs, count, max_m, max_n, max_rows_sliced, timeout_ns, st)
+                : launch_oz<false, 6>(d_probs, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
 }
 
 namespace {
@@ -772,11 +820,11 @@ __global__ void gemm_desc_oz_kernel(const GemmDesc* descs, int count, OzScratch 
     P.N = d.N;
     P.K = d.K;
     // A (M x K): stored M x K, or K x M when a_trans
-    P.A = d.a_trans ? OzOperand{d.A, d.a_f32, 1, d.lda, 0, 1, 1, nullptr}
-                    : OzOperand{d.A, d.a_f32, d.lda, 1, 0, 1, 1, nullptr};
+    P.A = d.a_trans ? OzOperand{d.A, d.a_f32, 1, d.lda, 0, 1, 1, nullptr, nullptr, 0}
+                    : OzOperand{d.A, d.a_f32, d.lda, 1, 0, 1, 1, nullptr, nullptr, 0};
     // column j of B (K x N) as a row of K values: stored K x N, or N x K when b_trans
-    P.B = d.b_trans ? OzOperand{d.B, d.b_f32, d.ldb, 1, 0, 1, 1, nullptr}
-                    : OzOperand{d.B, d.b_f32, 1, d.ldb, 0, 1, 1, nullptr};
+    P.B = d.b_trans ? OzOperand{d.B, d.b_f32, d.ldb, 1, 0, 1, 1, nullptr, nullptr, 0}
+                    : OzOperand{d.B, d.b_f32, 1, d.ldb, 0, 1, 1, nullptr, nullptr, 0};
     P.C = d.C;
     P.ldc = d.ldc;
     P.alpha = d.alpha;
@@ -801,12 +849,12 @@ cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max
     if (count <= 0) return cudaSuccess;
     // every operand must fit its slot
     const int big = max_m > max_n ? max_m : max_n;
-    if (oz_slice_bytes(big, max_k, bf16) > scr.slot_bytes || oz_exp_ints(big) > scr.exp_ints)
+    if (oz_slice_bytes(big, max_k, bf16, 6) > scr.slot_bytes || oz_exp_ints(big) > scr.exp_ints)
         return cudaErrorInvalidValue;
     gemm_desc_oz_kernel<<<(count + 127) / 128, 128, 0, st>>>(d_desc, count, scr, bf16 ? 1 : 0);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_oz_gemm(scr.probs, count, max_m, max_n, big, bf16, timeout_ns, st);
+    return launch_oz_gemm(scr.probs, count, max_m, max_n, big, bf16, 6, timeout_ns, st);
 }
 
 }  // namespace mpdo
@@ -833,13 +881,13 @@ extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const
     P.M = M;
     P.N = N;
     P.K = K;
-    P.A = OzOperand{A, 0, lda, 1, 0, 1, 1, nullptr};
-    P.B = OzOperand{B, 0, 1, ldb, 0, 1, 1, nullptr};
+    P.A = OzOperand{A, 0, lda, 1, 0, 1, 1, nullptr, nullptr, 0};
+    P.B = OzOperand{B, 0, 1, ldb, 0, 1, 1, nullptr, nullptr, 0};
     P.C = C;
     P.ldc = ldc;
     P.alpha = 1.0;
     oz_tiles(P, bf16);
-    const size_t sa = oz_slice_bytes(M, K, bf16), sb = oz_slice_bytes(N, K, bf16);
+    const size_t sa = oz_slice_bytes(M, K, bf16, 6), sb = oz_slice_bytes(N, K, bf16, 6);
     unsigned char* buf = nullptr;
     const size_t ia = oz_exp_ints(M), ib = oz_exp_ints(N);
     const size_t bytes = sa + sb + sizeof(int) * (ia + ib) + sizeof(OzProblem) + 256;
@@ -856,7 +904,7 @@ extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const
         (reinterpret_cast<uintptr_t>(P.eb + ib) + 255) & ~static_cast<uintptr_t>(255));
     e = oz_prepare();
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_p, &P, sizeof(P), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_oz_gemm(d_p, 1, M, N, M > N ? M : N, bf16, 4000000000ull, st);
+    if (e == cudaSuccess) e = launch_oz_gemm(d_p, 1, M, N, M > N ? M : N, bf16, 6, 4000000000ull, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(buf);
     if (e != cudaSuccess) {

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(QT, 1) qr_kernel(const OpDesc* descs, const in
                 const double alpha = x0 > 0.0 ? -nrm : nrm;
                 s_v0 = x0 - alpha;
                 const double vtv = 2.0 * alpha * (alpha - x0);
-                s_beta = (ss == 0.0 || !(vtv > 0.0)) ? 0.0 : 2.0 / vtv;
+                s_beta = (ss == 0.0 || !(vtv > 1e-280)) ? 0.0 : 2.0 / vtv;   // 2 / vtv stays finite
                 if (g == 0) rdiag[j] = (ss == 0.0) ? x0 : alpha;
             }
         }

@@ -304,7 +304,7 @@ __global__ void qrb_prep_kernel(const OpDesc* descs, int nops, int k0, int nb, i
         P.N = jb;
         P.K = mp;
         P.A = trail;
-        P.B = OzOperand{s.V, 0, ld, 1, 0, 1, 1, nullptr};
+        P.B = OzOperand{s.V, 0, ld, 1, 0, 1, 1, nullptr, nullptr, 0};
         P.C = s.Wt;
         P.ldc = kMaxNb;
         P.alpha = 1.0;
@@ -312,8 +312,8 @@ __global__ void qrb_prep_kernel(const OpDesc* descs, int nops, int k0, int nb, i
         P.M = np;
         P.N = mp;
         P.K = jb;
-        P.A = OzOperand{s.W2t, 0, kMaxNb, 1, 0, 1, 1, nullptr};
-        P.B = OzOperand{s.V, 0, 1, ld, 0, 1, 1, nullptr};   // (i, t) = V[t][i]
+        P.A = OzOperand{s.W2t, 0, kMaxNb, 1, 0, 1, 1, nullptr, nullptr, 0};
+        P.B = OzOperand{s.V, 0, 1, ld, 0, 1, 1, nullptr, nullptr, 0};   // (i, t) = V[t][i]
         P.C = d.Acm + k0;
         P.ldc = ld;
         P.c_gather = s.perm + k0 + jb;
@@ -421,12 +421,12 @@ cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzPro
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         qrb_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, k0, nb, 0, probs, ld, bf16 ? 1 : 0);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        if ((e = launch_oz_gemm(probs, nops, ld, nb, ld, bf16, timeout_ns, st)) != cudaSuccess) break;
+        if ((e = launch_oz_gemm(probs, nops, ld, nb, ld, bf16, 6, timeout_ns, st)) != cudaSuccess) break;
         qrb_wt_kernel<<<dim3((ld * kMaxNb + 255) / 256, nops), 256, 0, st>>>(d_desc, k0, nb, ld);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         qrb_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, k0, nb, 1, probs, ld, bf16 ? 1 : 0);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        if ((e = launch_oz_gemm(probs, nops, ld, ld, ld, bf16, timeout_ns, st)) != cudaSuccess) break;
+        if ((e = launch_oz_gemm(probs, nops, ld, ld, ld, bf16, 6, timeout_ns, st)) != cudaSuccess) break;
         qrb_norms_kernel<<<dim3((ld + 63) / 64, nops), 256, 0, st>>>(d_desc, k0, nb, ld);
         e = cudaGetLastError();
     }

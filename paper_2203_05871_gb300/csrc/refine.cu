@@ -1,0 +1,207 @@
+// Finish of the preconditioned SVD: all pairs of rows at once, through their
+// Gram matrix.
+//
+// After the FP32 preconditioning pass and its FP64-accurate application the c
+// rows of W are orthogonal to ~1e-6 of their norms.  The FP64 Jacobi sweeps that
+// used to finish them read every pair of rows with FP64 FMAs, of which GB300
+// issues two per SM and clock.  One iteration here instead
+//   1. forms G = W W^T as a tensor-core product (oz_gemm.cu; every row and
+//      column scaled by its own exponent, so G_ij is accurate relative to
+//      |w_i| |w_j| however graded the rows are),
+//   2. takes the Jacobi angle theta_ij of every pair that is not orthogonal to
+//      tol, X_ij = -theta_ij (antisymmetric), and
+//   3. turns all rows by the rotation W <- P(X) W, P(X) = I + X + X^2/2 + X^3/8.
+// P(X) P(X)^T = I - X^6/64 + ..., and with the terms through X^2 or X only it is
+// I + X^4/4 or I - X^2: each iteration takes the fewest terms whose defect is
+// below its tolerance.  The residual after an iteration is of second order
+// (angle times off-orthogonality), so two iterations finish a typical op.
+// In P(X) W the product X W scales column k of X by |w_k| and row k of W by its
+// inverse (exponents only), so a row is accurate relative to its own norm.
+//
+// An op ends in state kRefineDone when a Gram matrix shows every needed pair at
+// tol, or when the predicted residual is under a tenth of it; the FP64 Jacobi
+// pass then returns at once.  Everything the expansion does not cover (a pair
+// whose angle is too large: nearly equal singular values that are not yet
+// separated; a non-finite entry) leaves the op to the Jacobi pass, which starts
+// from the rows as they are.  Needed pairs, zero rows and tol are the Jacobi
+// pass's (jacobi.cu): two rows that the truncation discards need not be
+// orthogonal to one another, a row of norm <= eps |W|_F is set to zero.
+#include <float.h>
+#include <mpdo.h>
+
+#include "coop.cuh"
+#include "internal.h"
+
+namespace mpdo {
+
+namespace {
+
+constexpr int NT = 256;
+
+__global__ void refine_init_kernel(const OpDesc* descs, int nops) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= nops) return;
+    RefineOp& r = *descs[s].rf;
+    r.state = descs[s].c > 1 ? kRefineActive : kRefineLeft;
+    r.order = 0;
+    r.rho2 = 0u;
+    r.row1 = 0u;
+    r.far = 0;
+    r.thr = 0.0;
+    r.floor2 = 0.0;
+}
+
+// squared row norms and their inverse roots from G's diagonal, the zero floor
+// (rows at or under it are set to zero) and the discard threshold, fixed once open
+__global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, int ld) {
+    const OpDesc& d = descs[blockIdx.x];
+    RefineOp& r = *d.rf;
+    if (r.state != kRefineActive) return;
+    const int c = d.c;
+    double* a = d.snorm;
+    double* inv = d.snorm + ld;
+    __shared__ double red[NT / 32], s_floor2;
+    double f = 0.0;
+    for (int i = threadIdx.x; i < c; i += NT) {
+        const double v = d.E[(size_t)i * ld + i];
+        a[i] = v;
+        f += v;
+    }
+    f = warp_sum(f);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = f;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < NT / 32; ++w) t += red[w];
+        s_floor2 = DBL_EPSILON * DBL_EPSILON * t;
+    }
+    __syncthreads();
+    const double floor2 = s_floor2;
+    for (int i = threadIdx.x; i < c; i += NT) inv[i] = a[i] > floor2 ? 1.0 / sqrt(a[i]) : 0.0;
+    for (int i = threadIdx.x; i < c; i += NT)
+        if (a[i] <= floor2 && a[i] != 0.0)   // rare: numerically zero rows
+            for (int k = 0; k < d.L; ++k) d.W[(size_t)i * ld + k] = 0.0;
+    const int kk = d.chi_max + max(16, d.chi_max / 8);
+    const bool settled = r.order > 0 ? __uint_as_float(r.rho2) <= 1e-8f : (d.pre_ok && *d.pre_ok == 1);
+    double thr = r.thr;
+    __syncthreads();
+    if (thr == 0.0 && settled && !d.full_svd && kk < c) thr = kth_largest<NT, 4 * kMaxChi>(a, c, kk);
+    if (threadIdx.x == 0) {
+        r.thr = thr;
+        r.floor2 = floor2;
+        r.rho2 = 0u;
+        r.row1 = 0u;
+        r.far = 0;
+    }
+}
+
+// X from G, one warp per row; the largest g^2 / (a b) of a needed pair, the
+// largest absolute row sum of X (a bound of its norm), and whether an angle
+// was too large for the expansion
+__global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int ld, double tol_in, float tcap) {
+    const OpDesc& d = descs[blockIdx.y];
+    RefineOp& r = *d.rf;
+    const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= d.c || r.state != kRefineActive) return;
+    const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
+    const double* a = d.snorm;
+    const double* inv = d.snorm + ld;
+    const double ai = a[i], vi = inv[i], thr = r.thr;
+    const bool dead = vi == 0.0, low = ai < thr;
+    float rho = 0.0f, sum = 0.0f;
+    int far = 0;
+    for (int j = lane; j < d.c; j += 32) {
+        const double aj = a[j], vj = inv[j];
+        double x = 0.0;
+        if (j != i && !dead && vj != 0.0 && !(low && aj < thr)) {
+            const double v = vi * vj;
+            const float q = (float)(d.E[(size_t)i * ld + j] * v);   // g / (|w_i| |w_j|)
+            rho = !(fabsf(q) <= rho) ? fabsf(q) : rho;              // a NaN stays
+            if (fabsf(q) > tol) {
+                const float zeta = (float)((aj - ai) * v) / (2.0f * q);
+                const float t = fabsf(zeta) > 1e18f   // a row far below the other (zeta^2 leaves FP32's range)
+                                    ? 0.5f / zeta
+                                    : copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
+                if (fabsf(t) <= tcap) {
+                    const float th = t * fmaf(-t * t, 1.0f / 3.0f, 1.0f);   // atan t
+                    x = -(double)th;
+                    sum += fabsf(th);
+                } else {
+                    far = 1;
+                }
+            }
+        }
+        d.Q[(size_t)i * ld + j] = x;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float v = __shfl_xor_sync(0xffffffffu, rho, o);
+        rho = !(v <= rho) ? v : rho;
+    }
+    sum = warp_sum(sum);
+    far = __any_sync(0xffffffffu, far);
+    if (lane == 0) {
+        atomicMax(&r.rho2, __float_as_uint(fabsf(rho * rho)));
+        atomicMax(&r.row1, __float_as_uint(sum));
+        if (far) atomicOr(&r.far, 1);
+    }
+}
+
+__global__ void refine_decide_kernel(const OpDesc* descs, int nops, double tol_in, int can_finish, float defect,
+                                     int last) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= nops) return;
+    const OpDesc& d = descs[s];
+    RefineOp& r = *d.rf;
+    r.order = 0;
+    if (r.state != kRefineActive) return;
+    if (d.sweeps_out) *d.sweeps_out += 1;
+    const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
+    const float rho = sqrtf(__uint_as_float(r.rho2)), x = __uint_as_float(r.row1);
+    if (rho <= tol) {
+        r.state = can_finish ? kRefineDone : kRefineLeft;
+        return;
+    }
+    const float x2 = x * x;
+    if (x2 <= defect)
+        r.order = 1;
+    else if (0.25f * x2 * x2 <= defect)
+        r.order = 2;
+    else if (x2 * x2 * x2 <= 64.0f * defect)
+        r.order = 3;
+    else {
+        r.state = kRefineLeft;   // beyond the expansion (or not finite)
+        return;
+    }
+    if (!r.far && 2.0f * rho * x <= 0.1f * tol)
+        r.state = can_finish ? kRefineDone : kRefineLeft;   // after this rotation
+    else if (last)
+        r.state = kRefineLeft;
+}
+
+}  // namespace
+
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, OzProblem* probs, int chi_cap, bool bf16, int S,
+                          double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st) {
+    if (nops <= 0) return cudaSuccess;
+    const int ld = 4 * chi_cap, g = (nops + 127) / 128;
+    // defect of the rotation's orthogonality: FP64 rounding with 7 slices, the
+    // level of 6 slices' products otherwise; the largest single angle follows
+    const float defect = S == 7 ? 1e-17f : 1e-13f, tcap = S == 7 ? 2e-3f : 1e-2f;
+    refine_init_kernel<<<g, 128, 0, st>>>(d_desc, nops);
+    for (int it = 0; it < kRefineIters; ++it) {
+        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, probs, chi_cap, bf16, S, timeout_ns, st);
+        if (e != cudaSuccess) return e;
+        refine_diag_kernel<<<nops, NT, 0, st>>>(d_desc, ld);
+        refine_x_kernel<<<dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st>>>(d_desc, ld, tol_in, tcap);
+        refine_decide_kernel<<<g, 128, 0, st>>>(d_desc, nops, tol_in, can_finish ? 1 : 0, defect,
+                                                it == kRefineIters - 1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        for (int kind : {OZ_R3, OZ_R2, OZ_R1})
+            if ((e = launch_oz_ops(d_desc, nops, kind, probs, chi_cap, bf16, S, timeout_ns, st)) != cudaSuccess)
+                return e;
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace mpdo

@@ -113,9 +113,9 @@ extern "C" int mpdo_autotune(mpdo_ctx* c, const int* classes, int n_classes, int
             const size_t mat = (size_t)ld * ld;
             d.thetap = c->d_thetap + (size_t)s * mat;
             d.W = c->d_W + (size_t)s * mat;
-            d.W0 = c->mixed ? c->d_W0 + (size_t)s * mat : d.W;
-            d.W32 = c->mixed ? c->d_W32 + (size_t)s * mat : nullptr;
-            d.U32 = c->mixed ? c->d_U32 + (size_t)s * mat : nullptr;
+            d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
+            d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
+            d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
             d.snorm = c->d_snorm + (size_t)s * 2 * ld;
             d.status = d_status;
             d.sweeps_out = c->d_sweeps + s;
