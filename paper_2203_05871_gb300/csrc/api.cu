@@ -66,10 +66,11 @@ int release_slots(mpdo_ctx* c) {
     void* ptrs[] = {c->d_thetap, c->d_W,    c->d_Z,     c->d_Yk,    c->d_snorm, c->d_desc,  c->d_cta,
                     c->d_sync,   c->d_sweeps, c->d_pre_ok, c->d_W0,  c->d_E,     c->d_Q,     c->d_W32,
                     c->d_U32,    c->d_gemm,  c->d_copy,  c->d_oz_as, c->d_oz_bs, c->d_oz_ea, c->d_oz_eb,
-                    c->d_oz,     c->d_refine};
+                    c->d_oz,     c->d_refine, c->d_D32};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     c->d_refine = nullptr;
+    c->d_D32 = nullptr;
     c->d_thetap = c->d_W = c->d_Z = c->d_Yk = c->d_snorm = nullptr;
     c->d_W0 = c->d_E = c->d_Q = nullptr;
     c->d_W32 = c->d_U32 = nullptr;
@@ -126,14 +127,15 @@ int alloc_slots(mpdo_ctx* c, int want) {
     c->h_sweeps.assign(s, 0);
     CU(dalloc(&c->d_desc, (size_t)s));
     const int gcap = std::max(std::max(c->jacobi_resident, c->qr_resident), s);
-    CU(dalloc(&c->d_cta, (size_t)3 * (2 * gcap + s)));
+    CU(dalloc(&c->d_cta, (size_t)4 * (2 * gcap + s)));
     CU(dalloc(&c->d_sync, jacobi_sync_words(s)));
     CU(cudaMallocHost((void**)&c->h_desc, sizeof(OpDesc) * s));
-    CU(cudaMallocHost((void**)&c->h_cta, sizeof(int) * 3 * (2 * gcap + s)));
+    CU(cudaMallocHost((void**)&c->h_cta, sizeof(int) * 4 * (2 * gcap + s)));
     CU(dalloc(&c->d_copy, (size_t)4 * s));
     CU(cudaMallocHost((void**)&c->h_copy, sizeof(Copy2D) * 4 * s));
     if (c->precond) {
         CU(dalloc(&c->d_refine, (size_t)s));
+        CU(dalloc(&c->d_D32, (size_t)s * jacobi32_diag_floats(c->ld)));
         CU(dalloc(&c->d_W0, (size_t)s * mat));
         CU(dalloc(&c->d_E, (size_t)s * mat));
         CU(dalloc(&c->d_Q, (size_t)s * mat));
@@ -187,7 +189,7 @@ int plan_jacobi(mpdo_ctx* c, const OpDesc* h, int nops, bool fp32, int* hbase, i
     total = 0;
     for (int s = 0; s < nops; ++s) {
         const OpDesc& d = h[s];
-        const int pairs = jacobi_pairs_per_round(d.c, fp32 ? d.jb32 : d.jb);
+        const int pairs = jacobi_pairs_per_round(d.c, fp32 ? kJacobiB32 : d.jb);
         int g = (int)std::floor((double)R * work[s] / std::max(wsum, 1.0));
         g = std::max(1, std::min(pairs, g));
         const int passes = (pairs + g - 1) / g;      // block pairs per CTA per round
@@ -264,8 +266,7 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.status = c->d_status + b;
     d.max_disc = c->d_maxdisc + b;
     d.rank_log = nullptr;
-    d.jb = tuned_block_rows(c, d.cl, d.cr, false, jacobi_block_rows(d.L, d.c, 8));
-    d.jb32 = tuned_block_rows(c, d.cl, d.cr, true, jacobi_block_rows_f32(d.L, d.c));
+    d.jb = tuned_block_rows(c, d.cl, d.cr, jacobi_block_rows(d.L, d.c, 8));
     d.sweeps_out = c->d_sweeps + s;
     d.pre_ok = c->precond ? c->d_pre_ok + s : nullptr;
     d.rf = refine_on(c) ? c->d_refine + s : nullptr;
@@ -276,6 +277,7 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
     d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
     d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
+    d.D32 = c->precond ? c->d_D32 + (size_t)s * jacobi32_diag_floats(ld) : nullptr;
     d.E = c->precond ? c->d_E + (size_t)s * mat : nullptr;
     d.Q = c->precond ? c->d_Q + (size_t)s * mat : nullptr;
     d.Zinit = nullptr;
@@ -285,20 +287,27 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
 }
 
-cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st) {
+cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
-    auto oz = [&](int kind) {
-        return launch_oz_ops(d_desc, nops, kind, c->d_oz, c->cap, c->oz_bf16, c->oz_s, timeout_ns, st);
-    };
     // E = U U^T - I (~1e-6), then one orthogonalisation step: second order
     // (Q = U - E U / 2, defect 3 E^2 / 4) on the mixed path, third order (defect
     // 5 E^3 / 8, below FP64 rounding) on the FP64 path
     std::vector<int> kinds = {OZ_E, OZ_Q, OZ_W};
     if (!c->mixed) kinds = {OZ_E, OZ_T, OZ_Q3, OZ_W};
     for (int kind : kinds) {
-        const cudaError_t e = oz(kind);
+        const cudaError_t e =
+            launch_oz_ops(d_desc, nops, first + kind, c->d_oz, c->cap, c->oz_bf16, c->oz_s, timeout_ns, st);
         if (e != cudaSuccess) return e;
     }
+    return cudaSuccess;
+}
+
+int orthogonalise_kernels(const mpdo_ctx* c) { return c->mixed ? 9 : 12; }
+
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st) {
+    const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
+    const cudaError_t e = launch_orthogonalise(c, d_desc, nops, 0, st);
+    if (e != cudaSuccess) return e;
     if (!refine_on(c)) return cudaSuccess;
     // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
     const double tol = fp64_jacobi_tol(c);
@@ -307,7 +316,7 @@ cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cud
 }
 
 int svd_products_kernels(const mpdo_ctx* c) {
-    return (c->mixed ? 9 : 12) + (refine_on(c) ? kRefineKernels : 0);
+    return orthogonalise_kernels(c) + (refine_on(c) ? kRefineKernels : 0);
 }
 
 int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* forced, const TapeSlot* tape,
@@ -398,55 +407,66 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         return MPDO_OK;
     };
     CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, c->st));
-    // Householder QR of every theta~ (R's rows go to W0)
+    // QR of every theta~: its rows turned and graded go to W0
     {
-        const int R = c->qr_resident;
-        const int QW = qr_threads() / 32;
-        double wsum = 0.0;
-        for (double w : qwork) wsum += w;
-        std::vector<int> G(nops, 1);
-        int total = 0;
-        for (int s = 0; s < nops; ++s) {
-            const OpDesc& d = c->h_desc[s];
-            const int need = std::max(1, (d.n + QW - 1) / QW);
-            int g = (int)std::floor((double)R * qwork[s] / std::max(wsum, 1.0));
-            G[s] = std::max(1, std::min(need, g));
-            total += G[s];
-        }
-        while (total > R) {
-            int arg = (int)(std::max_element(G.begin(), G.end()) - G.begin());
-            if (G[arg] <= 1) return fail(MPDO_ECAPACITY, "more ops in flight than co-resident QR CTAs");
-            G[arg]--;
-            total--;
-        }
-        int* hbase = c->h_cta + (size_t)2 * (2 * gcap + c->slots);
-        int* dbase = c->d_cta + (size_t)2 * (2 * gcap + c->slots);
-        // fault injection (host side): leave out the last CTA of the first op that
-        // has two or more, while its group still counts it, so that the op's first
-        // barrier cannot complete and its CTAs give up after barrier_timeout_ms
-        int drop_op = -1;
-        if (c->inject == MPDO_FAULT_DROP_CTA)
-            for (int s = 0; s < nops && drop_op < 0; ++s)
-                if (G[s] >= 2) drop_op = s;
-        const int launched = total - (drop_op >= 0 ? 1 : 0);
-        int t = 0;
-        for (int s = 0; s < nops; ++s) {
-            hbase[2 * launched + s] = G[s];
-            const int run = G[s] - (s == drop_op ? 1 : 0);
-            for (int g = 0; g < run; ++g, ++t) {
-                hbase[t] = s;
-                hbase[launched + t] = g;
+        const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap);
+        // ops of the FP32 QR (q32) or of the FP64 column QR, each launch with all
+        // co-resident CTAs shared in proportion to the work
+        auto plan_qr = [&](bool q32, int slot, int& total, int*& dbase) -> int {
+            std::vector<int> G(nops, 0);
+            double wsum = 0.0;
+            auto takes = [&](int s) { return (c->precond && qr32_takes(c->h_desc[s].m, c->h_desc[s].n)) == q32; };
+            for (int s = 0; s < nops; ++s)
+                if (takes(s)) wsum += qwork[s];
+            const int R = q32 ? c->qr32_resident : c->qr_resident, QW = qr_threads() / 32;
+            total = 0;
+            for (int s = 0; s < nops; ++s) {
+                if (!takes(s)) continue;
+                const OpDesc& d = c->h_desc[s];
+                const int need = q32 ? qr32_max_ctas(d.m) : std::max(1, (d.n + QW - 1) / QW);
+                const int g = (int)std::floor((double)R * qwork[s] / std::max(wsum, 1.0));
+                G[s] = std::max(1, std::min(need, g));
+                total += G[s];
             }
-        }
-        if (drop_op >= 0) c->inject = 0;
-        total = launched;
+            while (total > R) {
+                int arg = (int)(std::max_element(G.begin(), G.end()) - G.begin());
+                if (G[arg] <= 1) return fail(MPDO_ECAPACITY, "more ops in flight than co-resident QR CTAs");
+                G[arg]--;
+                total--;
+            }
+            int* hbase = c->h_cta + (size_t)slot * (2 * gcap + c->slots);
+            dbase = c->d_cta + (size_t)slot * (2 * gcap + c->slots);
+            // fault injection (host side): leave out the last CTA of the first op that
+            // has two or more, while its group still counts it, so that the op's first
+            // barrier cannot complete and its CTAs give up after barrier_timeout_ms
+            int drop_op = -1;
+            if (c->inject == MPDO_FAULT_DROP_CTA)
+                for (int s = 0; s < nops && drop_op < 0; ++s)
+                    if (G[s] >= 2) drop_op = s;
+            const int launched = total - (drop_op >= 0 ? 1 : 0);
+            int t = 0;
+            for (int s = 0; s < nops; ++s) {
+                hbase[2 * launched + s] = G[s];
+                const int run = G[s] - (s == drop_op ? 1 : 0);
+                for (int g = 0; g < run; ++g, ++t) {
+                    hbase[t] = s;
+                    hbase[launched + t] = g;
+                }
+            }
+            if (drop_op >= 0) c->inject = 0;
+            total = launched;
+            if (total == 0) return MPDO_OK;
+            CU(cudaMemcpyAsync(dbase, hbase, sizeof(int) * (2 * total + nops), cudaMemcpyHostToDevice, c->st));
+            CU(cudaMemsetAsync(c->d_sync, 0, sizeof(unsigned) * jacobi_sync_words_per_op() * nops, c->st));
+            return MPDO_OK;
+        };
         double fl_qr = 0.0;
         for (int s = 0; s < nops; ++s) {
             const OpDesc& d = c->h_desc[s];
             fl_qr += 4.0 * d.m * d.n * d.c - 2.0 * (d.m + d.n) * d.c * d.c + 4.0 / 3.0 * d.c * d.c * d.c;
         }
         qr_flops_chunk = fl_qr;
-        if (c->mixed && c->cfg.qr_blocked && qrb_fits(cap)) {
+        if (blocked) {
             // mixed path: blocked QR, trailing updates on the tensor cores
             int r_max = 1;
             for (int s = 0; s < nops; ++s) r_max = std::max(r_max, c->h_desc[s].c);
@@ -455,11 +475,18 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
             p_qr.stop();
             qr_kernels_chunk = qrb_kernels(cap, r_max);
         } else {
-            CU(cudaMemcpyAsync(dbase, hbase, sizeof(int) * (2 * total + nops), cudaMemcpyHostToDevice, c->st));
-            CU(cudaMemsetAsync(c->d_sync, 0, sizeof(unsigned) * jacobi_sync_words_per_op() * nops, c->st));
             ProfScope p_qr(c, K_QR);
-            CU(launch_qr(c->d_desc, dbase, dbase + total, dbase + 2 * total, c->d_sync, total, timeout_ns, ld,
-                         c->st));
+            int total = 0, *db = nullptr;
+            int rc = plan_qr(false, 2, total, db);
+            if (rc) return rc;
+            qr_kernels_chunk = total > 0;
+            CU(launch_qr(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
+            if ((rc = plan_qr(true, 3, total, db))) return rc;
+            if (total > 0) {
+                CU(launch_qr32(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
+                CU(launch_orthogonalise(c, c->d_desc, nops, OZ_FIRST, c->st));
+                qr_kernels_chunk += 1 + orthogonalise_kernels(c);
+            }
             p_qr.stop();
         }
     }
@@ -686,7 +713,8 @@ int mpdo_init(mpdo_ctx** out, const mpdo_config* cfg, void* cuda_stream) {
         fail(MPDO_ECUDA, std::string("tensor-core kernel set-up: ") + cudaGetErrorString(e));
         return bail(MPDO_ECUDA);
     }
-    if ((e = qr_max_resident(&c->qr_resident)) != cudaSuccess || c->qr_resident < 1) {
+    if ((e = qr_max_resident(&c->qr_resident)) != cudaSuccess || c->qr_resident < 1 ||
+        (e = qr32_max_resident(&c->qr32_resident)) != cudaSuccess || c->qr32_resident < 1) {
         fail(MPDO_ECUDA, std::string("occupancy query: ") + cudaGetErrorString(e));
         return bail(MPDO_ECUDA);
     }

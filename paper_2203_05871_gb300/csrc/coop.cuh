@@ -12,6 +12,8 @@ namespace mpdo {
 // [8 + s] rotations and [8 + kMaxSweepsCap + s] largest off-orthogonality in Jacobi
 // sweep s, then one version per Jacobi row block (at most 4 kMaxChi blocks)
 constexpr int kSyncWords = 8 + 2 * kMaxSweepsCap + 4 * kMaxChi;
+constexpr int kSwQueue = 2;   // words 2, 3: the Jacobi block-pair counters of alternate sweeps
+constexpr int kSwVer = 8 + 2 * kMaxSweepsCap;   // the versions
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -23,6 +25,34 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
+}
+
+__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Wait (thread 0) until row blocks P and Q (those < nb) have left round R - 1,
+// i.e. their versions reached R; bounded by timeout_ns, after which the op's
+// abort flag is raised.  Returns 0 if it gave up.
+__device__ inline int wait_blocks(const unsigned* ver, int P, int Q, int nb, unsigned R, unsigned* abort_flag,
+                           unsigned long long timeout_ns) {
+    const unsigned long long t0 = globaltimer_ns();
+    for (;;) {
+        const bool okP = P >= nb || ld_acquire(ver + P) >= R;
+        const bool okQ = Q >= nb || ld_acquire(ver + Q) >= R;
+        if (okP && okQ) return 1;
+        if (ld_acquire(abort_flag) != 0u) return 0;
+        if (globaltimer_ns() - t0 > timeout_ns) {
+            atomicExch(abort_flag, 1u);
+            return 0;
+        }
+        __nanosleep(32);
+    }
+}
+
+// player in place x of a circle tournament of cp players at a step
+__device__ __forceinline__ int tour_player(int x, int step, int cp) {
+    return x == 0 ? 0 : 1 + ((x - 1 + step) % (cp - 1));
 }
 
 // Barrier of the G CTAs working on one op; returns false if it gave up.
@@ -94,5 +124,33 @@ __device__ double kth_largest(const double* v, int c, int kk) {
     return __longlong_as_double((long long)x);
 }
 
-}  // namespace mpdo
+// The same for c float values val(j) (non-negative): 31 counting rounds.
+template <int NT, int NMAX, class F>
+__device__ float kth_largest_f(F val, int c, int kk) {
+    constexpr int kPer = (NMAX + NT - 1) / NT;
+    __shared__ int s_cnt[2][NT / 32];
+    unsigned key[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int j = threadIdx.x + i * NT;
+        key[i] = j < c ? __float_as_uint(fmaxf(val(j), 0.0f)) : 0u;
+    }
+    unsigned x = 0u;
+    for (int bit = 30; bit >= 0; --bit) {
+        const unsigned cand = x | (1u << bit);
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) n += key[i] >= cand;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if ((threadIdx.x & 31) == 0) s_cnt[bit & 1][threadIdx.x >> 5] = n;
+        __syncthreads();
+        int tot = 0;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) tot += s_cnt[bit & 1][w];
+        if (tot >= kk) x = cand;
+    }
+    __syncthreads();
+    return __uint_as_float(x);
+}
 
+}  // namespace mpdo

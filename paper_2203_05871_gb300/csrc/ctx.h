@@ -96,7 +96,7 @@ struct mpdo_ctx {
     mpdo::OzProblem* d_oz = nullptr;                        // [slots] problems of one launch
     size_t oz_slot_bytes = 0;
     double *d_W0 = nullptr, *d_E = nullptr, *d_Q = nullptr;
-    float *d_W32 = nullptr, *d_U32 = nullptr;
+    float *d_W32 = nullptr, *d_U32 = nullptr, *d_D32 = nullptr;
     mpdo::GemmDesc* d_gemm = nullptr;
     mpdo::GemmDesc* h_gemm = nullptr;   // pinned, [3][slots]
     mpdo::Copy2D* d_copy = nullptr;     // [4][slots] tape copies of a chunk
@@ -109,7 +109,7 @@ struct mpdo_ctx {
     int *d_cta = nullptr, *h_cta = nullptr;   // [3][grid cap]: op, rank, then group [slots]
     unsigned* d_sync = nullptr;
     int jacobi_resident = 0;
-    int qr_resident = 0;
+    int qr_resident = 0, qr32_resident = 0;
     // measurement
     double *d_wstack = nullptr, *d_part = nullptr;   // all-pairs propagation scratch
     double *d_envL = nullptr, *d_envR = nullptr, *d_full = nullptr, *d_one_a = nullptr, *d_one_b = nullptr,
@@ -128,7 +128,7 @@ struct mpdo_ctx {
     long long gen = 0;            // bumped whenever the state changes (step, set_state, build_gates)
     long long layout = 0;         // bumped whenever the op list or the workspaces change (build_gates)
     mpdo::GraphState* graph = nullptr;
-    // autotuned Jacobi rows per block: [(chi_l * (cap+1) + chi_r) * 2 + fp32], 0 = the default rule
+    // autotuned rows per block of the FP64 Jacobi pass: [chi_l * (cap+1) + chi_r], 0 = the default rule
     std::vector<int> jb_table;
     int* d_jb_table = nullptr;
     // descriptors of the Gram-matrix GEMM sweeps (global.cu), grown on demand
@@ -176,9 +176,9 @@ struct ProfScope {
 void prof_collect(mpdo_ctx* c, int k, double flops, int kernels);
 
 // Jacobi rows per block of a (chi_l, chi_r) class: the autotuned value, else dflt.
-inline int tuned_block_rows(const mpdo_ctx* c, int cl, int cr, bool fp32, int dflt) {
+inline int tuned_block_rows(const mpdo_ctx* c, int cl, int cr, int dflt) {
     if (c->jb_table.empty() || cl > c->cap || cr > c->cap) return dflt;
-    const int v = c->jb_table[((size_t)cl * (c->cap + 1) + cr) * 2 + (fp32 ? 1 : 0)];
+    const int v = c->jb_table[(size_t)cl * (c->cap + 1) + cr];
     return v > 0 ? v : dflt;
 }
 
@@ -220,6 +220,10 @@ inline double fp64_jacobi_tol(const mpdo_ctx* c) {
 constexpr int kRefineMinSweeps = 16;
 inline bool refine_on(const mpdo_ctx* c) { return c->precond && c->cfg.jacobi_max_sweeps >= kRefineMinSweeps; }
 
+// From the FP32-orthogonal U32: Q, orthogonal to FP64 accuracy, and W = Q W0; with
+// first = OZ_FIRST from the QR's Q^T: W0 = Q theta~.
+cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st);
+int orthogonalise_kernels(const mpdo_ctx* c);
 // The stages between the FP32 preconditioning pass and the FP64 Jacobi pass:
 // Q, the orthogonalised U32, W = Q W0, and the refinement of W's rows.
 cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st);

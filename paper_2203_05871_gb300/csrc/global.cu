@@ -243,7 +243,6 @@ int run_svd(mpdo_ctx* c, double* W, const std::vector<int>& slots, const std::ve
         d.sweeps_out = c->d_sweeps + s;
         d.full_svd = 1;
         d.jb = jacobi_block_rows(n, n, 8);
-        d.jb32 = 1;
         c->h_desc[k] = d;
     }
     CU(cudaMemcpyAsync(c->d_desc, c->h_desc, sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));

@@ -28,15 +28,17 @@ namespace mpdo {
 namespace {
 
 // Shares R co-resident CTAs among the ops of a chunk in proportion to their
-// work, each op between 1 and cap_s CTAs (the host plan's rule).  out: [R] op
+// work, each op between 1 and cap_s CTAs (the host plan's rule; none for cap_s = 0).  out: [R] op
 // of each CTA (-1: unused, the CTA returns at once), [R] rank within the op,
 // [nops] CTAs per op.  Returns 0, or 1 if R < nops.
 __device__ int plan_ctas(const double* work, const int* cap, int nops, int R, int* out) {
     int* G = out + 2 * R;
     double wsum = 0.0;
-    for (int s = 0; s < nops; ++s) wsum += work[s];
+    for (int s = 0; s < nops; ++s) wsum += cap[s] > 0 ? work[s] : 0.0;
     int total = 0;
     for (int s = 0; s < nops; ++s) {
+        G[s] = 0;
+        if (cap[s] == 0) continue;
         int g = (int)floor((double)R * work[s] / fmax(wsum, 1.0));
         g = max(1, min(cap[s], g));
         const int passes = (cap[s] + g - 1) / g;
@@ -68,7 +70,7 @@ __device__ int plan_ctas(const double* work, const int* cap, int nops, int R, in
 constexpr int kMaxChunk = 1024;
 
 __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops, const int* dims, int N, int Rj,
-                                                         int Rq, int* cta64, int* cta32, int* ctaqr, int precond,
+                                                         int Rq, int* cta64, int* cta32, int* ctaqr, int* ctaq32, int Rq32, int precond, int blocked,
                                                          const int* jb_table, int chi_cap, int* error) {
     __shared__ double work[kMaxChunk];
     __shared__ int cap[kMaxChunk];
@@ -83,11 +85,9 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
         d.c = min(d.m, d.n);
         d.L = d.n;
         d.jb = jacobi_block_rows(d.L, d.c, 8);
-        d.jb32 = jacobi_block_rows_f32(d.L, d.c);
         if (jb_table) {   // autotuned rows per block of this (chi_l, chi_r) class
-            const int* t = jb_table + ((size_t)d.cl * (chi_cap + 1) + d.cr) * 2;
-            if (t[0] > 0) d.jb = t[0];
-            if (t[1] > 0) d.jb32 = t[1];
+            const int t = jb_table[(size_t)d.cl * (chi_cap + 1) + d.cr];
+            if (t > 0) d.jb = t;
         }
     }
     __syncthreads();
@@ -100,15 +100,19 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
     }
     bad |= plan_ctas(work, cap, nops, Rj, cta64);
     if (precond) {
-        for (int s = 0; s < nops; ++s) cap[s] = jacobi_pairs_per_round(descs[s].c, descs[s].jb32);
+        for (int s = 0; s < nops; ++s) cap[s] = jacobi_pairs_per_round(descs[s].c, kJacobiB32);
         bad |= plan_ctas(work, cap, nops, Rj, cta32);
     }
     for (int s = 0; s < nops; ++s) {
         const OpDesc& d = descs[s];
         work[s] = (double)d.m * d.n * d.c;
-        cap[s] = max(1, (d.n + kQrWarps - 1) / kQrWarps);
+        cap[s] = precond && qr32_takes(d.m, d.n) ? 0 : max(1, (d.n + kQrWarps - 1) / kQrWarps);
     }
-    bad |= plan_ctas(work, cap, nops, Rq, ctaqr);
+    if (!blocked) bad |= plan_ctas(work, cap, nops, Rq, ctaqr);
+    if (precond && !blocked) {
+        for (int s = 0; s < nops; ++s) cap[s] = cap[s] == 0 ? qr32_max_ctas(descs[s].m) : 0;
+        bad |= plan_ctas(work, cap, nops, Rq32, ctaq32);
+    }
     if (bad) *error = 1;
 }
 
@@ -123,7 +127,7 @@ __global__ void klog_kernel(const OpDesc* descs, int nops, int n_ops, int* klog)
 struct Chunk {
     int nops = 0;
     OpDesc* d_desc = nullptr;
-    int *d_cta64 = nullptr, *d_cta32 = nullptr, *d_ctaqr = nullptr;
+    int *d_cta64 = nullptr, *d_cta32 = nullptr, *d_ctaqr = nullptr, *d_ctaq32 = nullptr;
 };
 
 }  // namespace
@@ -136,7 +140,7 @@ struct GraphState {
     std::vector<std::vector<Chunk>> chunks;   // per layer
     int* d_klog = nullptr;                    // [B][n_ops] ranks of the last replayed step
     int* d_error = nullptr;
-    int Rj = 0, Rq = 0;
+    int Rj = 0, Rq = 0, Rq32 = 0;
 };
 
 namespace {
@@ -148,7 +152,7 @@ void release(GraphState* g) {
     g->graph = nullptr;
     for (auto& L : g->chunks)
         for (auto& ch : L) {
-            void* ptrs[] = {ch.d_desc, ch.d_cta64, ch.d_cta32, ch.d_ctaqr};
+            void* ptrs[] = {ch.d_desc, ch.d_cta64, ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32};
             for (void* p : ptrs)
                 if (p) cudaFree(p);
         }
@@ -164,11 +168,12 @@ void release(GraphState* g) {
 int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
     const int cap = c->cap, ld = c->ld;
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
+    const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap);
     for (auto& L : g->chunks)
         for (auto& ch : L) {
             const int nops = ch.nops;
             plan_chunk_kernel<<<1, 256, 0, st>>>(ch.d_desc, nops, c->d_dims, c->N, g->Rj, g->Rq, ch.d_cta64,
-                                                 ch.d_cta32, ch.d_ctaqr, c->precond ? 1 : 0, c->d_jb_table, cap,
+                                                 ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, g->Rq32, c->precond ? 1 : 0, blocked ? 1 : 0, c->d_jb_table, cap,
                                                  g->d_error);
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
@@ -180,11 +185,18 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             }
             const size_t sync_bytes = sizeof(unsigned) * jacobi_sync_words(nops);
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
-            if (c->mixed && c->cfg.qr_blocked && qrb_fits(cap))
+            if (blocked) {
                 CU(launch_qr_blocked(ch.d_desc, nops, cap, c->d_oz, c->oz_bf16, timeout_ns, st, 0));
-            else
+            } else {
                 CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
                              timeout_ns, ld, st));
+                if (c->precond) {
+                    CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
+                    CU(launch_qr32(ch.d_desc, ch.d_ctaq32, ch.d_ctaq32 + g->Rq32, ch.d_ctaq32 + 2 * g->Rq32,
+                                   c->d_sync, g->Rq32, timeout_ns, ld, st));
+                    CU(launch_orthogonalise(c, ch.d_desc, nops, OZ_FIRST, st));
+                }
+            }
             if (c->precond) {
                 CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
                 CU(launch_jacobi(ch.d_desc, nops, ch.d_cta32, ch.d_cta32 + g->Rj, ch.d_cta32 + 2 * g->Rj, c->d_sync,
@@ -212,6 +224,7 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
     if (!g->cap_st) CU(cudaStreamCreateWithFlags(&g->cap_st, cudaStreamNonBlocking));
     g->Rj = c->jacobi_resident;
     g->Rq = c->qr_resident;
+    g->Rq32 = c->qr32_resident;
     CU(dalloc(&g->d_klog, (size_t)c->B * c->n_ops));
     CU(dalloc(&g->d_error, 1));
     CU(cudaMemsetAsync(g->d_error, 0, sizeof(int), c->st));
@@ -221,7 +234,7 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
         const size_t cs = (size_t)chunk_ops(c);
         for (size_t s0 = 0; s0 < items.size(); s0 += cs) {
             const int nops = (int)std::min(cs, items.size() - s0);
-            if (nops > kMaxChunk || nops > std::min(g->Rj, g->Rq))
+            if (nops > kMaxChunk || nops > std::min(g->Rj, std::min(g->Rq, g->Rq32)))
                 return fail(MPDO_ECAPACITY, "graph step: more ops in one chunk than co-resident CTAs");
             Chunk ch;
             ch.nops = nops;
@@ -231,6 +244,7 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
             CU(dalloc(&ch.d_cta64, (size_t)2 * g->Rj + nops));
             CU(dalloc(&ch.d_ctaqr, (size_t)2 * g->Rq + nops));
             if (c->precond) CU(dalloc(&ch.d_cta32, (size_t)2 * g->Rj + nops));
+            if (c->precond) CU(dalloc(&ch.d_ctaq32, (size_t)2 * g->Rq32 + nops));
             CU(cudaMemcpyAsync(ch.d_desc, h.data(), sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
             CU(cudaStreamSynchronize(c->st));
             g->chunks[li].push_back(ch);

@@ -46,7 +46,6 @@ struct OpDesc {
     int transposed;    // 1: Jacobi rows carry a c x c accumulator Z (unused since the QR step)
     int c, L;          // Jacobi problem: c rows of length L
     int jb;            // Jacobi block size (rows per shared-memory block), FP64 pass
-    int jb32;          // same for the FP32 preconditioning pass
     int chi_max;
     double cutoff;
     const double* G;   // 16x16 gate, row-major G[(s1' s2'), (s1 s2)]
@@ -63,6 +62,7 @@ struct OpDesc {
     const double* Zinit;  // initial Z (nullptr => identity)
     float* W32;        // mixed path: FP32 rows of the preconditioning Jacobi (c x L)
     float* U32;        // mixed path: FP32 accumulated rotations (c x c)
+    float* D32;        // FP32 pass: Gram matrix of every row block [block][32][32]
     double* E;         // mixed path: U32 U32^T - I (c x c)
     double* Q;         // mixed path: orthogonalised U32 (c x c)
     double* Yk;        // k x n right singular vectors (rows), ld
@@ -126,23 +126,10 @@ __host__ __device__ inline int jacobi_block_rows(int rowlen, int c, int elem_byt
     while (b > 1 && b >= c) b >>= 1;
     return b;
 }
-// FP32 preconditioning pass: rows of at most kJacobiRegL elements take the
-// register path (one block of b <= kJacobiMaxB rows in shared memory, the
-// other in registers), longer rows the shared-memory path above; in both the
-// U32 rows are turned once per block pair by its accumulated rotation, so only
-// the L-long W rows are staged.
-constexpr int kJacobiRegL = 1024;
-__host__ __device__ inline bool jacobi_f32_reg(int L) { return L <= kJacobiRegL; }
-__host__ __device__ inline int jacobi_block_rows_f32(int L, int c) {
-    if (!jacobi_f32_reg(L)) return jacobi_block_rows(L, c, 4);
-    int b = kJacobiMaxB;
-    while (b > 1 && b >= c) b >>= 1;
-    return b;
-}
-// whether b rows per block fit the FP32 pass for rows of length L
-__host__ __device__ inline bool jacobi_f32_fits(int b, int L, int c) {
-    (void)c;
-    return jacobi_f32_reg(L) ? b <= kJacobiMaxB : (size_t)2 * b * L * 4 <= (size_t)kJacobiRowBytes;
+constexpr int kJacobiB32 = 32;   // rows per block of the FP32 preconditioning pass (jacobi32.cu)
+// floats of OpDesc::D32 for up to c rows
+inline size_t jacobi32_diag_floats(int c) {
+    return (size_t)((c + kJacobiB32 - 1) / kJacobiB32) * kJacobiB32 * kJacobiB32;
 }
 // block pairs per tournament round
 __host__ __device__ inline int jacobi_pairs_per_round(int c, int b) {
@@ -159,6 +146,11 @@ cudaError_t launch_jacobi(const OpDesc* d_desc, int nops, const int* d_cta_op, c
                           const int* d_group, unsigned* d_sync, int grid, int max_sweeps, double tol,
                           unsigned long long timeout_ns, int ld, bool fp32, cudaStream_t st,
                           double pre_rho = 1e-3);   // FP32 pass: stop once no rotation exceeds pre_rho
+// the FP32 pass (jacobi32.cu): its CTAs per SM, and its launch
+cudaError_t jacobi32_max_resident(int* per_sm);
+cudaError_t launch_jacobi32(const OpDesc* d_desc, const int* d_cta_op, const int* d_cta_rank, const int* d_group,
+                            unsigned* d_sync, int grid, int max_sweeps, unsigned long long timeout_ns, int ld,
+                            cudaStream_t st, double pre_rho);
 size_t jacobi_sync_words_per_op();
 // sync words of a Jacobi launch over nops ops (theirs and the grid barrier's)
 size_t jacobi_sync_words(int nops);
@@ -224,7 +216,9 @@ cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int m
 // OZ_Q Q = U - E U / 2, OZ_W W = Q W0; OZ_T T = U - 3 E U / 4 then OZ_Q3
 // Q = U - E T / 2 (third-order orthogonalisation); OZ_G G = W W^T and OZ_R3,
 // OZ_R2, OZ_R1 the refinement's rotation (refine.cu).  probs: scratch for nops problems.
-enum { OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T = 5, OZ_Q3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
+// OZ_FIRST + OZ_E, OZ_Q, OZ_T, OZ_Q3, OZ_W: the same on the QR's Q^T (ops of qr32_takes
+// only), OZ_W then being W0 = Q theta~.
+enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T = 5, OZ_Q3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
        OZ_R1 = 10 };
 cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16, int S,
                           unsigned long long timeout_ns, cudaStream_t st);
@@ -270,6 +264,15 @@ cudaError_t qrb_prepare();
 // r_max: the largest min(m, n) of the chunk's ops (<= 0: the capacity 4 chi_cap)
 cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs, bool bf16,
                               unsigned long long timeout_ns, cudaStream_t st, int r_max);
+
+// FP32 Householder QR (qr32.cu) of the preconditioned SVD's ops with m <= n: Q^T into
+// U32 (m x m), the row order of W0 = Q^T theta~ graded.  Wider panels than one CTA
+// per 16 rows would leave CTAs without a tile to update.
+__host__ __device__ inline bool qr32_takes(int m, int n) { return m <= n; }
+__host__ __device__ inline int qr32_max_ctas(int m) { return (m + 15) / 16; }
+cudaError_t qr32_max_resident(int* blocks);
+cudaError_t launch_qr32(const OpDesc* d_desc, const int* d_cta_op, const int* d_cta_rank, const int* d_group,
+                        unsigned* d_sync, int grid, unsigned long long timeout_ns, int ld, cudaStream_t st);
 
 int qr_threads();
 cudaError_t qr_max_resident(int* blocks);

@@ -617,6 +617,9 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
     const OpDesc& d = descs[s];
     const int ld = 4 * cap;
     OzProblem P{};
+    const bool first = (kind & OZ_FIRST) != 0;
+    kind &= OZ_FIRST - 1;
+    if (first && !qr32_takes(d.m, d.n)) kind = -1;
     auto rowmajor = [](const void* base, int f32, long long ld_) {   // (r, k) at r * ld + k
         return OzOperand{base, f32, ld_, 1, 0, 1, 1, nullptr, nullptr, 0};
     };
@@ -699,14 +702,16 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
             P.beta = kind == OZ_R3 ? 0.5 : 1.0;
             break;
         }
-        default:         // OZ_W: W = Q W0
+        case OZ_W:       // W = Q W0 (first: W0 = Q theta~, theta~ column-major)
             P.M = d.c;
             P.N = d.L;
             P.K = d.c;
             P.A = rowmajor(d.Q, 0, ld);
-            P.B = colmajor(d.W0, 0, ld);
-            P.C = d.W;
+            P.B = first ? rowmajor(d.Acm, 0, ld) : colmajor(d.W0, 0, ld);
+            P.C = first ? d.W0 : d.W;
             P.ldc = ld;
+            break;
+        default:         // an op that takes no part
             break;
     }
     if (kind == OZ_MERGE || kind == OZ_RECON || kind == OZ_E || kind == OZ_W) P.alpha = 1.0;

@@ -1,16 +1,15 @@
 // Autotuner of the Jacobi SVD's rows per block, per (chi_l, chi_r) class
 // (mpdo_autotune).
 //
-// The one-sided Jacobi stages two blocks of b rows per block pair (jacobi.cu:
-// both in shared memory, or for the FP32 pass on rows of at most 1024
-// elements one in shared memory and one in registers).  Larger blocks mean fewer rounds and barriers per sweep and
+// The FP64 one-sided Jacobi stages two blocks of b rows per block pair in shared
+// memory (jacobi.cu).  Larger blocks mean fewer rounds per sweep and
 // more work per shared-memory load; smaller ones more block pairs per round,
 // i.e. more CTAs per op.  The best b depends on the row length, the number of
 // rows and how many ops share the GPU, so it is measured: for every class the
 // tuner fills as many workspace slots as a layer has ops in flight with a
 // seeded graded matrix of the class's shape (rows scaled like the rows of a
-// pivoted R; at most 16 slots), and times the Jacobi launch for every b that fits (FP64 pass,
-// and the FP32 pass of the mixed path), keeping the fastest.  The winners go
+// pivoted R; at most 16 slots), and times the FP64 Jacobi launch for every b that
+// fits, keeping the fastest.  The FP32 pass has a fixed block of 32 rows.  The winners go
 // to a (chi_l, chi_r) table that both the host-planned and the graph step
 // read.  Different b change the order of the rotations, so results change at
 // rounding level only.
@@ -30,22 +29,18 @@ namespace mpdo {
 
 namespace {
 
-int time_jacobi(mpdo_ctx* c, std::vector<OpDesc>& h, bool fp32, int b, double* ms_out) {
+int time_jacobi(mpdo_ctx* c, std::vector<OpDesc>& h, int b, double* ms_out) {
     const int nops = (int)h.size();
     const int ld = c->ld;
-    for (auto& d : h) (fp32 ? d.jb32 : d.jb) = b;
-    // pristine rows back into W0 (and W) from Theta' (holding the synthetic input)
-    for (const auto& d : h) {
-        CU(cudaMemcpy2DAsync(d.W0, sizeof(double) * ld, d.thetap, sizeof(double) * ld, sizeof(double) * d.L, d.c,
+    for (auto& d : h) d.jb = b;
+    // pristine rows back into W from Theta' (holding the synthetic input)
+    for (const auto& d : h)
+        CU(cudaMemcpy2DAsync(d.W, sizeof(double) * ld, d.thetap, sizeof(double) * ld, sizeof(double) * d.L, d.c,
                              cudaMemcpyDeviceToDevice, c->st));
-        if (d.W != d.W0)
-            CU(cudaMemcpy2DAsync(d.W, sizeof(double) * ld, d.thetap, sizeof(double) * ld, sizeof(double) * d.L, d.c,
-                                 cudaMemcpyDeviceToDevice, c->st));
-    }
     CU(cudaMemcpyAsync(c->d_desc, h.data(), sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
     int total = 0;
     const int gcap = std::max(std::max(c->jacobi_resident, c->qr_resident), c->slots);
-    int rc = plan_jacobi(c, h.data(), nops, fp32, c->h_cta, total);
+    int rc = plan_jacobi(c, h.data(), nops, false, c->h_cta, total);
     if (rc) return rc;
     CU(cudaMemcpyAsync(c->d_cta, c->h_cta, sizeof(int) * (2 * total + nops), cudaMemcpyHostToDevice, c->st));
     (void)gcap;
@@ -56,8 +51,7 @@ int time_jacobi(mpdo_ctx* c, std::vector<OpDesc>& h, bool fp32, int b, double* m
     CU(cudaMemsetAsync(c->d_sync, 0, sizeof(unsigned) * jacobi_sync_words(nops), c->st));
     CU(cudaEventRecord(e0, c->st));
     CU(launch_jacobi(c->d_desc, nops, c->d_cta, c->d_cta + total, c->d_cta + 2 * total, c->d_sync, total,
-                     fp32 ? kMaxSweepsCap / 2 : c->cfg.jacobi_max_sweeps, fp32 ? 0.0 : fp64_jacobi_tol(c), timeout_ns, ld,
-                     fp32, c->st, precond_rho(c)));
+                     c->cfg.jacobi_max_sweeps, fp64_jacobi_tol(c), timeout_ns, ld, false, c->st));
     CU(cudaEventRecord(e1, c->st));
     CU(cudaEventSynchronize(e1));
     float ms = 0.0f;
@@ -81,7 +75,7 @@ extern "C" int mpdo_autotune(mpdo_ctx* c, const int* classes, int n_classes, int
     for (int i = 0; i < n_classes; ++i)
         if (classes[2 * i] < 1 || classes[2 * i] > cap || classes[2 * i + 1] < 1 || classes[2 * i + 1] > cap)
             return fail(MPDO_EINVAL, "class chi values must be in [1, chi_cap]");
-    if (c->jb_table.empty()) c->jb_table.assign((size_t)(cap + 1) * (cap + 1) * 2, 0);
+    if (c->jb_table.empty()) c->jb_table.assign((size_t)(cap + 1) * (cap + 1), 0);
     // ops in flight while timing: a layer's worth, at most 16 (enough to share
     // the GPU the way a layer does, and keeps tuning to seconds)
     const int nops = std::max(1, std::min(std::min(c->slots, c->B * c->max_layer), 16));
@@ -113,46 +107,37 @@ extern "C" int mpdo_autotune(mpdo_ctx* c, const int* classes, int n_classes, int
             const size_t mat = (size_t)ld * ld;
             d.thetap = c->d_thetap + (size_t)s * mat;
             d.W = c->d_W + (size_t)s * mat;
-            d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
-            d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
-            d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
             d.snorm = c->d_snorm + (size_t)s * 2 * ld;
             d.status = d_status;
             d.sweeps_out = c->d_sweeps + s;
             h[s] = d;
             CU(cudaMemcpyAsync(d.thetap, rows.data(), sizeof(double) * rows.size(), cudaMemcpyHostToDevice, c->st));
         }
-        for (int pass = 0; pass < (c->mixed ? 2 : 1); ++pass) {
-            const bool fp32 = pass == 1;
-            const int rowlen = n;
-            const int eb = 8;
-            double best = 1e300;
-            int best_b = fp32 ? jacobi_block_rows_f32(n, cc) : jacobi_block_rows(rowlen, cc, eb);
-            for (int b = 1; b <= kJacobiMaxB; b *= 2) {
-                if (fp32 ? !jacobi_f32_fits(b, n, cc) : (size_t)2 * b * rowlen * eb > (size_t)kJacobiRowBytes) break;
-                if (b > 1 && b >= cc) break;
-                if (fp32) {   // the FP32 pass starts from the FP64 rows of W0
-                    for (auto& d : h) d.jb = jacobi_block_rows(n, cc, 8);
+        double best = 1e300;
+        int best_b = jacobi_block_rows(n, cc, 8);
+        for (int b = 1; b <= kJacobiMaxB; b *= 2) {
+            if ((size_t)2 * b * n * 8 > (size_t)kJacobiRowBytes) break;
+            if (b > 1 && b >= cc) break;
+            double t = 1e300;
+            for (int rep = 0; rep < 2; ++rep) {
+                double ms = 0.0;
+                int rc = time_jacobi(c, h, b, &ms);
+                if (rc) {
+                    cudaFree(d_status);
+                    return rc;
                 }
-                double t = 1e300;
-                for (int rep = 0; rep < 2; ++rep) {
-                    double ms = 0.0;
-                    int rc = time_jacobi(c, h, fp32, b, &ms);
-                    if (rc) {
-                        cudaFree(d_status);
-                        return rc;
-                    }
-                    t = std::min(t, ms);
-                }
-                if (t < best) {
-                    best = t;
-                    best_b = b;
-                }
+                t = std::min(t, ms);
             }
-            c->jb_table[((size_t)cl * (cap + 1) + cr) * 2 + pass] = best_b;
-            if (chosen) chosen[2 * i + pass] = best_b;
+            if (t < best) {
+                best = t;
+                best_b = b;
+            }
         }
-        if (!c->mixed && chosen) chosen[2 * i + 1] = 0;
+        c->jb_table[(size_t)cl * (cap + 1) + cr] = best_b;
+        if (chosen) {
+            chosen[2 * i] = best_b;
+            chosen[2 * i + 1] = c->mixed ? kJacobiB32 : 0;   // the FP32 pass has one block size
+        }
     }
     cudaFree(d_status);
     if (!c->d_jb_table) CU(dalloc(&c->d_jb_table, c->jb_table.size()));
