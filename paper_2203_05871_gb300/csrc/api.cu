@@ -287,6 +287,11 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
 }
 
+// The SVD's own products take bf16 slices on every path: the slices are 8-bit
+// integers, exact in bf16 and tf32 alike, so the results are the same bit for bit,
+// at half the bytes and twice the MMA rate.  (The contractions keep the context's kind.)
+constexpr bool kSvdBf16 = true;
+
 cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     // E = U U^T - I (~1e-6), then one orthogonalisation step: second order
@@ -296,13 +301,13 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
     if (!c->mixed) kinds = {OZ_E, OZ_T, OZ_Q3, OZ_W};
     for (int kind : kinds) {
         const cudaError_t e =
-            launch_oz_ops(d_desc, nops, first + kind, c->d_oz, c->cap, c->oz_bf16, c->oz_s, timeout_ns, st);
+            launch_oz_ops(d_desc, nops, first + kind, c->cap, kSvdBf16, c->oz_s, timeout_ns, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-int orthogonalise_kernels(const mpdo_ctx* c) { return c->mixed ? 9 : 12; }
+int orthogonalise_kernels(const mpdo_ctx* c) { return (c->mixed ? 3 : 4) * kOzKernels; }
 
 cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
@@ -312,7 +317,7 @@ cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cud
     // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
     const double tol = fp64_jacobi_tol(c);
     const bool can = c->oz_s == 7 || tol >= 1e-12;
-    return launch_refine(d_desc, nops, c->d_oz, c->cap, c->oz_bf16, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
+    return launch_refine(d_desc, nops, c->cap, kSvdBf16, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
 }
 
 int svd_products_kernels(const mpdo_ctx* c) {
@@ -369,7 +374,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     ProfScope p_merge(c, K_MERGE);
     if (c->mixed) {
-        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, c->d_oz, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
         CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
     } else {
         CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
@@ -517,7 +522,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     p_tr.stop();
     ProfScope p_rec(c, K_RECON);
     if (c->mixed)
-        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, c->d_oz, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
     else
         CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
     p_rec.stop();
@@ -544,9 +549,9 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         const OpDesc& d = c->h_desc[s];
         fl_rec += 32.0 * d.cl * d.cr * c->h_dims[(size_t)d.b * (N + 1) + c->layers[items[s].layer][items[s].idx].p + 1];
     }
-    // kernels per stage: a tensor-core product is three (operand set-up,
-    // slicing, slice products), the merge adds the gate/weight kernel
-    prof_collect(c, K_MERGE, fl_merge, c->mixed ? 4 : 1);
+    // kernels per stage: a tensor-core product is two (slicing, slice
+    // products), the merge adds the gate/weight kernel
+    prof_collect(c, K_MERGE, fl_merge, c->mixed ? kOzKernels + 1 : 1);
     prof_collect(c, K_QR, qr_flops_chunk, qr_kernels_chunk);
     prof_collect(c, K_JACOBI, fl_svd, 1);
     if (c->precond) {
@@ -554,7 +559,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         prof_collect(c, K_GEMM, fl_gemm, svd_products_kernels(c));
     }
     prof_collect(c, K_TRUNC, 0.0, 1);
-    prof_collect(c, K_RECON, fl_rec, c->mixed ? 3 : 1);
+    prof_collect(c, K_RECON, fl_rec, c->mixed ? kOzKernels : 1);
     for (int s = 0; s < nops && log_ranks; ++s) {
         const Item& it = items[s];
         const Op& op = c->layers[it.layer][it.idx];

@@ -185,6 +185,7 @@ struct OzProblem {
     double alpha, beta;
     const void* D;
     int ldd, d_f32, sub_identity;
+    int levels;          // slice pairs (t, u) with t + u < levels are formed (0: all S levels)
     int sym;             // C (f64, no gather) is symmetric: tiles below the diagonal are mirrored, not computed
     void *as, *bs;       // slice blocks of A and B
     int *ea, *eb;        // row / column exponents
@@ -197,6 +198,12 @@ __host__ __device__ inline void oz_set_tiles(OzProblem& p, bool bf16) {
     p.Mt = (p.M + 127) / 128;
     p.Nt = (p.N + 63) / 64;
     p.Kt = (p.K + KT - 1) / KT;
+}
+// levels that a product needs whose left operand is below 2^e of its result's other
+// part: 8 bits each, at least two
+__host__ __device__ inline int oz_levels(int S, int e) {
+    const int drop = e < 0 ? -e / 8 : 0;
+    return S - drop > 2 ? S - drop : 2;
 }
 size_t oz_slice_bytes(int rows, int K, bool bf16, int S);   // slice blocks of an operand of rows x K
 size_t oz_exp_ints(int rows);                          // its exponent array (rows rounded up to a tile)
@@ -215,13 +222,14 @@ cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int m
 // gate and the left weights), OZ_RECON B_p' = Theta' Yk^T, OZ_E E = U U^T - I,
 // OZ_Q Q = U - E U / 2, OZ_W W = Q W0; OZ_T T = U - 3 E U / 4 then OZ_Q3
 // Q = U - E T / 2 (third-order orthogonalisation); OZ_G G = W W^T and OZ_R3,
-// OZ_R2, OZ_R1 the refinement's rotation (refine.cu).  probs: scratch for nops problems.
+// OZ_R2, OZ_R1 the refinement's rotation (refine.cu).
 // OZ_FIRST + OZ_E, OZ_Q, OZ_T, OZ_Q3, OZ_W: the same on the QR's Q^T (ops of qr32_takes
 // only), OZ_W then being W0 = Q theta~.
 enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T = 5, OZ_Q3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
        OZ_R1 = 10 };
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16, int S,
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, bool bf16, int S,
                           unsigned long long timeout_ns, cudaStream_t st);
+constexpr int kOzKernels = 2;   // kernels of one launch_oz_ops
 // ---------------------------------------------------------------------------
 // Refinement of nearly orthogonal rows through their Gram matrix (refine.cu)
 // ---------------------------------------------------------------------------
@@ -232,6 +240,7 @@ struct RefineOp {
     int order;        // terms of this iteration's rotation (0: none)
     unsigned rho2;    // largest g^2 / (a b) of a needed pair (float bits)
     int far;          // a needed pair's angle is beyond the expansion
+    unsigned blocks;  // CTAs of the X kernel that are done
     unsigned row1;    // largest absolute row sum of X (float bits)
     double thr;       // pairs of rows whose squared norms are both below it are not needed
     double floor2;    // squared norm of a numerically zero row
@@ -240,11 +249,10 @@ struct RefineOp {
 // rotated until every needed pair is orthogonal to tol (state kRefineDone) or the
 // op is left to the Jacobi pass.  Scratch: d.E (G), d.Q (X), d.W0, d.snorm.
 // tol_in as for launch_jacobi; can_finish = false: never kRefineDone.
-cudaError_t launch_refine(const OpDesc* d_desc, int nops, OzProblem* probs, int chi_cap, bool bf16, int S,
-                          double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, bool bf16, int S, double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
 constexpr int kRefineIters = 3;
 // kernels of one launch_refine
-constexpr int kRefineKernels = 1 + kRefineIters * (3 + 3 * 4);
+constexpr int kRefineKernels = kRefineIters * (2 + 4 * kOzKernels);
 
 // Theta' = G Theta in place in thetap and theta~ = lambda_l Theta' (column-major, Acm)
 cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st);

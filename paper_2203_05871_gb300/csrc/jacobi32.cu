@@ -445,6 +445,10 @@ __global__ void __launch_bounds__(NT, 1) jacobi32_kernel(const OpDesc* descs, co
 
     if (rank == 0 && threadIdx.x == 0) {   // set again only on success
         if (d.pre_ok) *d.pre_ok = 0;
+        if (d.rf) {
+            d.rf->state = kRefineLeft;
+            d.rf->order = 0;
+        }
     }
     for (int e = threadIdx.x; e < kSteps * NB; e += NT) {
         const int t = e / NB, i = e % NB;
@@ -670,6 +674,11 @@ __global__ void __launch_bounds__(NT, 1) jacobi32_kernel(const OpDesc* descs, co
         }
         if (rank == 0 && threadIdx.x == 0) {
             if (d.sweeps_out) *d.sweeps_out += used << 16;   // FP32 sweeps in the high half
+            if (d.rf) {   // the refinement starts (refine.cu)
+                d.rf->state = c > 1 ? kRefineActive : kRefineLeft;
+                d.rf->order = 0;
+                d.rf->thr = 0.0;
+            }
             if (d.pre_ok)
                 *d.pre_ok = used > 0 && __uint_as_float(ld_acquire(&sw[8 + kMaxSweepsCap + used - 1])) <= pre_rho2;
         }

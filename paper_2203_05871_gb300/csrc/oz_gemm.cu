@@ -28,7 +28,8 @@
 //    into one int64 (their exact integer parts) and adds it in FP64.  (Folding levels 3-5 into one
 //    accumulator was measured at 2e-12 on the GPU: the accumulator then holds
 //    level-3 magnitudes and drops the low bits of every level-5 product at
-//    every MMA.)
+//    every MMA.)  A product whose result is a small correction (the refinement's
+//    X W beside W) forms only the levels that reach the sum (levels).
 // 3. Epilogue: C_ij = alpha 2^(e_i + f_j - 14) sum_d L_d + beta D_ij.
 // Error: about 2^-46 |A_i|_max |B_j|_max per term of the sum (a numpy model of
 // the scheme with per-MMA rounding: 3e-14 of |A_i| |B_j| sqrt(K)), against
@@ -291,330 +292,18 @@ __device__ __forceinline__ void slice_group(const long long* X, bool nan, uint4*
     }
 }
 
-// Strided views (a transposed operand, the right site of a merge): a block
-// takes 32 consecutive rows, lane = row and warp = a slice of the K range, so
-// that the 32 lanes of a load read 32 neighbouring rows at one k (coalesced).
+// Where a launch finds its problems: an array, or one product kind of the ops of a
+// chunk, built from the op's descriptor by each CTA (a kernel of its own for that
+// would cost a launch per product).
+struct OzSource {
+    const OzProblem* probs;
+    const OpDesc* descs;
+    int kind, cap;
+};
+
+// The problem of one kind for an op.
 template <bool kBf16, int kS>
-__device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int Kt, unsigned char* out, int* ex,
-                                 int tile, int Rt) {
-    constexpr int esize = kBf16 ? 2 : 4;
-    constexpr int G = 16 / esize;
-    constexpr int KT = kt_elems(esize);
-    __shared__ unsigned long long s_mx[8][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool f32 = X.f32 != 0;
-    const int r = r0 + lane;
-    const bool live = r < R;
-    unsigned long long mx = 0;
-    if (live)
-        for (int k = warp; k < K; k += 8) {
-            const unsigned long long key = abs_key(oz_bits(X, r, k), f32);
-            mx = key > mx ? key : mx;
-        }
-    s_mx[warp][lane] = mx;
-    __syncthreads();
-    for (int w = 0; w < 8; ++w) mx = s_mx[w][lane] > mx ? s_mx[w][lane] : mx;
-    const bool bad = key_nonfinite(mx, f32);   // the largest key of a row with a NaN or an inf is one
-    const int e = bad ? 0 : key_exponent(mx, f32);
-    if (warp == 0) ex[r] = e;
-    const int rt = r / tile, rr = r % tile;
-    const size_t block = (size_t)tile * 64;
-    const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
-    for (int g0 = warp * G; g0 < Kt * KT; g0 += 8 * G) {
-        long long x[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int k = g0 + g;
-            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
-        }
-        uint4 sl[kS];
-        slice_group<G, kBf16, kS>(x, bad && live, sl);
-        const int kt = g0 / KT, kk = g0 % KT;
-#pragma unroll
-        for (int t = 0; t < kS; ++t) {
-            unsigned char* blk = out + (((size_t)t * Rt + rt) * Kt + kt) * block;
-            *reinterpret_cast<uint4*>(blk + within + (size_t)(kk / G) * LBO) = sl[t];
-        }
-    }
-}
-
-// grid (row groups of 8, 2 = A | B, problems).  Views whose rows are
-// contiguous (ks == 1) take one warp per row, lanes along k; the others 32 rows
-// per block (slice_rows_tiled), the blocks past rows / 32 returning at once.
-template <bool kBf16, int kS>
-__global__ void __launch_bounds__(256) oz_slice_kernel(const OzProblem* probs) {
-    constexpr int esize = kBf16 ? 2 : 4;
-    constexpr int G = 16 / esize;          // values per 16-byte store
-    constexpr int KT = kt_elems(esize);
-    const OzProblem& P = probs[blockIdx.z];
-    const bool isB = blockIdx.y == 1;
-    const OzOperand& X = isB ? P.B : P.A;
-    const int N = P.Ndyn ? *P.Ndyn : P.N;
-    const int R = isB ? N : P.M;
-    const int tile = isB ? kTileN : kTileM;         // rows per block
-    const int Rt = isB ? P.Nt : P.Mt;
-    const int K = P.K, Kt = P.Kt;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned char* out = static_cast<unsigned char*>(isB ? P.bs : P.as);
-    int* ex = isB ? P.eb : P.ea;
-    if (!(X.mode == 0 && X.ks == 1)) {
-        const int r0 = blockIdx.x * 32;
-        if (r0 >= Rt * tile) return;   // uniform over the block (Rt * tile is a multiple of 32)
-        slice_rows_tiled<kBf16, kS>(X, r0, R, K, Kt, out, ex, tile, Rt);
-        return;
-    }
-    const int r = blockIdx.x * 8 + warp;
-    if (r >= Rt * tile) return;
-    const bool live = r < R;
-    const bool f32 = X.f32 != 0;
-    unsigned long long mx = 0;
-    if (live)
-        for (int k = lane; k < K; k += 32) {
-            const unsigned long long key = abs_key(oz_bits(X, r, k), f32);
-            mx = key > mx ? key : mx;
-        }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-        mx = y > mx ? y : mx;
-    }
-    const bool bad = key_nonfinite(mx, f32);
-    const int e = bad ? 0 : key_exponent(mx, f32);
-    if (lane == 0) ex[r] = e;
-    const int rt = r / tile, rr = r % tile;
-    const size_t block = (size_t)tile * 64;
-    const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
-    for (int g0 = lane * G; g0 < Kt * KT; g0 += 32 * G) {
-        long long x[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int k = g0 + g;
-            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
-        }
-        uint4 sl[kS];
-        slice_group<G, kBf16, kS>(x, bad && live, sl);
-        const int kt = g0 / KT, kk = g0 % KT;
-#pragma unroll
-        for (int t = 0; t < kS; ++t) {
-            unsigned char* blk = out + (((size_t)t * Rt + rt) * Kt + kt) * block;
-            *reinterpret_cast<uint4*>(blk + within + (size_t)(kk / G) * LBO) = sl[t];
-        }
-    }
-}
-
-template <bool kBf16, int kS>
-__global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const OzProblem* probs,
-                                                               unsigned long long timeout_ns) {
-    constexpr int esize = kBf16 ? 2 : 4;
-    constexpr int KT = kt_elems(esize);
-    constexpr int kRangeTiles = kRangeK / KT;
-    constexpr int kLevels = kS, kStages = stages_of(kS), kStageBytes = stage_bytes(kS);
-    // barriers: full[kStages], empty[kStages], accumulators full, accumulators drained, final
-    constexpr int kBarFull = 0, kBarEmpty = kStages, kBarAccFull = 2 * kStages, kBarAccEmpty = 2 * kStages + 1,
-                  kBarFinal = 2 * kStages + 2;
-    extern __shared__ __align__(1024) unsigned char smem[];
-    const OzProblem& P = probs[blockIdx.z];
-    const int N = P.Ndyn ? *P.Ndyn : P.N;
-    const int mt = blockIdx.y, nt = blockIdx.x;
-    if (mt * kTileM >= P.M || nt * kTileN >= N) return;
-    if (P.sym && (nt + 1) * kTileN <= mt * kTileM) return;   // mirrored from above the diagonal
-    const int Kt = P.Kt;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kStages * kStageBytes + 128);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kStages * kStageBytes + 144);
-    if (threadIdx.x == 0) {
-        *abort_flag = 0;
-        for (int s = 0; s < kStages; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarFull + s)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarEmpty + s)));
-        }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarAccFull)));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(smem_u32(bar + kBarAccEmpty)));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarFinal)));
-        asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(512));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tmem = *tslot;
-    const int nrange = (Kt + kRangeTiles - 1) / kRangeTiles;
-
-    if (warp == 0) {
-        // producer: bulk copies of the slice blocks of k tile kt into stage kt % kStages
-        if (lane == 0) {
-            const unsigned char* as = static_cast<const unsigned char*>(P.as);
-            const unsigned char* bs = static_cast<const unsigned char*>(P.bs);
-            int issued = 0;
-            for (int kt = 0; kt < Kt; ++kt) {
-                const int s = kt % kStages;
-                if (kt >= kStages &&
-                    !mbar_wait(smem_u32(bar + kBarEmpty + s), ((kt / kStages) - 1) & 1, abort_flag, timeout_ns))
-                    break;
-                const uint32_t full = smem_u32(bar + kBarFull + s);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full), "r"(kStageBytes)
-                             : "memory");
-                unsigned char* st = smem + (size_t)s * kStageBytes;
-                for (int t = 0; t < kS; ++t) {
-                    const unsigned char* srcA = as + (((size_t)t * P.Mt + mt) * Kt + kt) * kBlockA;
-                    const unsigned char* srcB = bs + (((size_t)t * P.Nt + nt) * Kt + kt) * kBlockB;
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            smem_u32(st + t * kBlockA)),
-                        "l"(srcA), "r"(kBlockA), "r"(full)
-                        : "memory");
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            smem_u32(st + kS * kBlockA + t * kBlockB)),
-                        "l"(srcB), "r"(kBlockB), "r"(full)
-                        : "memory");
-                }
-                issued = kt + 1;
-            }
-            // copies still in flight complete on their full barrier before the CTA leaves
-            for (int kt = (issued > kStages ? issued - kStages : 0); kt < issued; ++kt)
-                mbar_wait(smem_u32(bar + kBarFull + kt % kStages), (kt / kStages) & 1, abort_flag, timeout_ns);
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t id = idesc(kBf16, kTileM, kTileN);
-            int r = 0;
-            bool first[kLevels];
-#pragma unroll
-            for (int l = 0; l < kLevels; ++l) first[l] = true;
-            for (int kt = 0; kt < Kt; ++kt) {
-                const int s = kt % kStages;
-                if (kt % kRangeTiles == 0 && kt > 0) {
-                    // accumulators of the previous range must be drained first
-                    if (!mbar_wait(smem_u32(bar + kBarAccEmpty), (r - 1) & 1, abort_flag, timeout_ns)) break;
-#pragma unroll
-                    for (int l = 0; l < kLevels; ++l) first[l] = true;
-                }
-                if (!mbar_wait(smem_u32(bar + kBarFull + s), (kt / kStages) & 1, abort_flag, timeout_ns)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t st = smem_u32(smem + (size_t)s * kStageBytes);
-#pragma unroll
-                for (int lvl = 0; lvl < kLevels; ++lvl) {
-                    const uint32_t d = tmem + (uint32_t)(lvl * kTileN);
-#pragma unroll
-                    for (int t = 0; t <= lvl; ++t) {
-                        const int u = lvl - t;
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const uint32_t off = q * 2 * LBO;
-                            mma(kBf16, d, smem_desc(st + t * kBlockA + off),
-                                smem_desc(st + kS * kBlockA + u * kBlockB + off), id, first[lvl] ? 0u : 1u);
-                            first[lvl] = false;
-                        }
-                    }
-                }
-                commit(smem_u32(bar + kBarEmpty + s));   // frees the stage once these MMAs have read it
-                if (kt % kRangeTiles == kRangeTiles - 1 || kt == Kt - 1) {
-                    commit(smem_u32(bar + kBarAccFull));   // accumulators of range r complete
-                    ++r;
-                }
-            }
-            commit(smem_u32(bar + kBarFinal));
-            mbar_wait(smem_u32(bar + kBarFinal), 0, abort_flag, timeout_ns);   // every MMA issued has completed
-        }
-    } else {
-        // epilogue warps 2..9: rows 32 (warp % 4) + lane, columns half * 32 .. + 31
-        const int ew = warp - 2;
-        const int lane_base = 32 * (warp & 3);
-        const int half = ew >> 2;
-        const uint32_t taddr = tmem + ((uint32_t)lane_base << 16) + (uint32_t)(half * 32);
-        double acc[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0.0;
-        bool ok = true;
-        for (int r = 0; r < nrange; ++r) {
-            if (!mbar_wait(smem_u32(bar + kBarAccFull), r & 1, abort_flag, timeout_ns)) {
-                ok = false;
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            // level d holds n_d 2^-8d with n_d an integer (exact for d <= 3;
-            // higher levels are rounded to the nearest 2^-8d): the range's
-            // sum is S 2^-40 with the integer S = sum_d n_d 2^(8 (5 - d)),
-            // |S| < 2^63 (level 6 rounded to that unit), formed in int64 and
-            // converted once (integer arithmetic instead of twelve FP64
-            // operations per element).  A NaN slice reaches level 0.
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                long long S[16];
-                unsigned nan = 0;
-#pragma unroll
-                for (int lvl = 0; lvl < kLevels; ++lvl) {
-                    float v[16];
-                    tmem_ld16(taddr + (uint32_t)(lvl * kTileN + c * 16), v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const float scale = __int_as_float((127 + 8 * lvl) << 23);   // 2^8d
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int n = __float2int_rn(v[i] * scale);
-                        if (lvl == 0) {
-                            S[i] = n;
-                            nan |= (v[i] != v[i]) ? 1u << i : 0u;
-                        } else if (lvl < 6) {
-                            S[i] = S[i] * 256 + n;
-                        } else {
-                            S[i] += (n + 128) >> 8;   // level 6 in units of 2^-40
-                        }
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    acc[c * 16 + i] += ((nan >> i) & 1u) ? __longlong_as_double(0x7ff8000000000000ll) : (double)S[i];
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncwarp();
-            if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + kBarAccEmpty)) : "memory");
-        }
-        if (ok && !*abort_flag) {
-            const int i = mt * kTileM + lane_base + lane;
-            if (i < P.M) {
-                const int ei = P.ea[i];
-#pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    const int j = nt * kTileN + half * 32 + jj;
-                    if (j >= N) continue;
-                    double v = P.alpha * ldexp(acc[jj], ei + P.eb[j] - 54);   // acc in units of 2^-40
-                    const size_t row = P.c_gather ? (size_t)P.c_gather[i] : (size_t)i;
-                    if (P.D) {
-                        const size_t di = row * P.ldd + j;
-                        v += P.beta * (P.d_f32 ? (double)static_cast<const float*>(P.D)[di]
-                                               : static_cast<const double*>(P.D)[di]);
-                    }
-                    if (P.sub_identity && i == j) v -= 1.0;
-                    const size_t ci = row * P.ldc + j;
-                    if (P.c_f32)
-                        static_cast<float*>(P.C)[ci] = (float)v;
-                    else
-                        static_cast<double*>(P.C)[ci] = v;
-                    if (P.sym && j > i) static_cast<double*>(P.C)[(size_t)j * P.ldc + i] = v;
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
-    if (threadIdx.x == 0 && *abort_flag && P.status) atomicOr(P.status, (int)MPDO_ST_TIMEOUT);
-}
-
-// The problems of one kind for every op of a chunk, from the op descriptors.
-__global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProblem* out, int cap, int bf16) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nops) return;
-    const OpDesc& d = descs[s];
+__device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
     const int ld = 4 * cap;
     OzProblem P{};
     const bool first = (kind & OZ_FIRST) != 0;
@@ -698,6 +387,9 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
             P.ldc = ld;
             P.D = d.W;
             P.ldd = ld;
+            // what X W adds to a row of W is below 2^e of it, e from the largest angle
+            // and the largest off-orthogonality: that many digits fewer are needed
+            P.levels = oz_levels(kS, max((int)(d.rf->row1 >> 23) - 126, ((int)(d.rf->rho2 >> 23) - 126) / 2 + 1));
             P.alpha = kind == OZ_R3 ? 0.125 : (kind == OZ_R2 && order == 2 ? 0.5 : 1.0);
             P.beta = kind == OZ_R3 ? 0.5 : 1.0;
             break;
@@ -720,8 +412,349 @@ __global__ void oz_prep_kernel(const OpDesc* descs, int nops, int kind, OzProble
     P.ea = d.oz_ea;
     P.eb = d.oz_eb;
     P.status = d.status;
-    oz_set_tiles(P, bf16 != 0);
-    out[s] = P;
+    oz_set_tiles(P, kBf16);
+    return P;
+}
+
+// the CTA's problem, through shared memory
+template <bool kBf16, int kS>
+__device__ __forceinline__ void fetch_problem(const OzSource& src, OzProblem& P) {
+    if (threadIdx.x == 0)
+        P = src.probs ? src.probs[blockIdx.z] : op_problem<kBf16, kS>(src.descs[blockIdx.z], src.kind, src.cap);
+    __syncthreads();
+}
+
+
+// Strided views (a transposed operand, the right site of a merge): a block
+// takes 32 consecutive rows, lane = row and warp = a slice of the K range, so
+// that the 32 lanes of a load read 32 neighbouring rows at one k (coalesced).
+template <bool kBf16, int kS>
+__device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int Kt, int lv, unsigned char* out, int* ex,
+                                 int tile, int Rt) {
+    constexpr int esize = kBf16 ? 2 : 4;
+    constexpr int G = 16 / esize;
+    constexpr int KT = kt_elems(esize);
+    __shared__ unsigned long long s_mx[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool f32 = X.f32 != 0;
+    const int r = r0 + lane;
+    const bool live = r < R;
+    unsigned long long mx = 0;
+    if (live)
+        for (int k = warp; k < K; k += 8) {
+            const unsigned long long key = abs_key(oz_bits(X, r, k), f32);
+            mx = key > mx ? key : mx;
+        }
+    s_mx[warp][lane] = mx;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w) mx = s_mx[w][lane] > mx ? s_mx[w][lane] : mx;
+    const bool bad = key_nonfinite(mx, f32);   // the largest key of a row with a NaN or an inf is one
+    const int e = bad ? 0 : key_exponent(mx, f32);
+    if (warp == 0) ex[r] = e;
+    const int rt = r / tile, rr = r % tile;
+    const size_t block = (size_t)tile * 64;
+    const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
+    for (int g0 = warp * G; g0 < Kt * KT; g0 += 8 * G) {
+        long long x[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int k = g0 + g;
+            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
+        }
+        uint4 sl[kS];
+        slice_group<G, kBf16, kS>(x, bad && live, sl);
+        const int kt = g0 / KT, kk = g0 % KT;
+#pragma unroll
+        for (int t = 0; t < kS; ++t) {
+            if (t >= lv) break;
+            unsigned char* blk = out + (((size_t)t * Rt + rt) * Kt + kt) * block;
+            *reinterpret_cast<uint4*>(blk + within + (size_t)(kk / G) * LBO) = sl[t];
+        }
+    }
+}
+
+// grid (row groups of 8, 2 = A | B, problems).  Views whose rows are
+// contiguous (ks == 1) take one warp per row, lanes along k; the others 32 rows
+// per block (slice_rows_tiled), the blocks past rows / 32 returning at once.
+template <bool kBf16, int kS>
+__global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
+    constexpr int esize = kBf16 ? 2 : 4;
+    constexpr int G = 16 / esize;          // values per 16-byte store
+    constexpr int KT = kt_elems(esize);
+    __shared__ OzProblem P;
+    fetch_problem<kBf16, kS>(src, P);
+    const bool isB = blockIdx.y == 1;
+    const OzOperand& X = isB ? P.B : P.A;
+    const int N = P.Ndyn ? *P.Ndyn : P.N;
+    const int R = isB ? N : P.M;
+    const int tile = isB ? kTileN : kTileM;         // rows per block
+    const int Rt = isB ? P.Nt : P.Mt;
+    const int K = P.K, Kt = P.Kt;
+    const int lv = P.levels > 0 ? P.levels : kS;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char* out = static_cast<unsigned char*>(isB ? P.bs : P.as);
+    int* ex = isB ? P.eb : P.ea;
+    if (!(X.mode == 0 && X.ks == 1)) {
+        const int r0 = blockIdx.x * 32;
+        if (r0 >= Rt * tile) return;   // uniform over the block (Rt * tile is a multiple of 32)
+        slice_rows_tiled<kBf16, kS>(X, r0, R, K, Kt, lv, out, ex, tile, Rt);
+        return;
+    }
+    const int r = blockIdx.x * 8 + warp;
+    if (r >= Rt * tile) return;
+    const bool live = r < R;
+    const bool f32 = X.f32 != 0;
+    unsigned long long mx = 0;
+    if (live)
+        for (int k = lane; k < K; k += 32) {
+            const unsigned long long key = abs_key(oz_bits(X, r, k), f32);
+            mx = key > mx ? key : mx;
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = y > mx ? y : mx;
+    }
+    const bool bad = key_nonfinite(mx, f32);
+    const int e = bad ? 0 : key_exponent(mx, f32);
+    if (lane == 0) ex[r] = e;
+    const int rt = r / tile, rr = r % tile;
+    const size_t block = (size_t)tile * 64;
+    const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
+    for (int g0 = lane * G; g0 < Kt * KT; g0 += 32 * G) {
+        long long x[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int k = g0 + g;
+            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
+        }
+        uint4 sl[kS];
+        slice_group<G, kBf16, kS>(x, bad && live, sl);
+        const int kt = g0 / KT, kk = g0 % KT;
+#pragma unroll
+        for (int t = 0; t < kS; ++t) {
+            if (t >= lv) break;
+            unsigned char* blk = out + (((size_t)t * Rt + rt) * Kt + kt) * block;
+            *reinterpret_cast<uint4*>(blk + within + (size_t)(kk / G) * LBO) = sl[t];
+        }
+    }
+}
+
+template <bool kBf16, int kS>
+__global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
+                                                               unsigned long long timeout_ns) {
+    constexpr int esize = kBf16 ? 2 : 4;
+    constexpr int KT = kt_elems(esize);
+    constexpr int kRangeTiles = kRangeK / KT;
+    constexpr int kLevels = kS, kStages = stages_of(kS), kStageBytes = stage_bytes(kS);
+    // barriers: full[kStages], empty[kStages], accumulators full, accumulators drained, final
+    constexpr int kBarFull = 0, kBarEmpty = kStages, kBarAccFull = 2 * kStages, kBarAccEmpty = 2 * kStages + 1,
+                  kBarFinal = 2 * kStages + 2;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ OzProblem P;
+    fetch_problem<kBf16, kS>(src, P);
+    const int N = P.Ndyn ? *P.Ndyn : P.N;
+    const int mt = blockIdx.y, nt = blockIdx.x;
+    if (mt * kTileM >= P.M || nt * kTileN >= N) return;
+    if (P.sym && (nt + 1) * kTileN <= mt * kTileM) return;   // mirrored from above the diagonal
+    const int Kt = P.Kt;
+    const int lv = P.levels > 0 ? P.levels : kS;   // slice pairs t + u < lv
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kStages * kStageBytes + 128);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kStages * kStageBytes + 144);
+    if (threadIdx.x == 0) {
+        *abort_flag = 0;
+        for (int s = 0; s < kStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarFull + s)));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarEmpty + s)));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarAccFull)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" ::"r"(smem_u32(bar + kBarAccEmpty)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + kBarFinal)));
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = *tslot;
+    const int nrange = (Kt + kRangeTiles - 1) / kRangeTiles;
+
+    if (warp == 0) {
+        // producer: bulk copies of the slice blocks of k tile kt into stage kt % kStages
+        if (lane == 0) {
+            const unsigned char* as = static_cast<const unsigned char*>(P.as);
+            const unsigned char* bs = static_cast<const unsigned char*>(P.bs);
+            int issued = 0;
+            for (int kt = 0; kt < Kt; ++kt) {
+                const int s = kt % kStages;
+                if (kt >= kStages &&
+                    !mbar_wait(smem_u32(bar + kBarEmpty + s), ((kt / kStages) - 1) & 1, abort_flag, timeout_ns))
+                    break;
+                const uint32_t full = smem_u32(bar + kBarFull + s);
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full), "r"(lv * (kBlockA + kBlockB))
+                             : "memory");
+                unsigned char* st = smem + (size_t)s * kStageBytes;
+                for (int t = 0; t < lv; ++t) {
+                    const unsigned char* srcA = as + (((size_t)t * P.Mt + mt) * Kt + kt) * kBlockA;
+                    const unsigned char* srcB = bs + (((size_t)t * P.Nt + nt) * Kt + kt) * kBlockB;
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            smem_u32(st + t * kBlockA)),
+                        "l"(srcA), "r"(kBlockA), "r"(full)
+                        : "memory");
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            smem_u32(st + kS * kBlockA + t * kBlockB)),
+                        "l"(srcB), "r"(kBlockB), "r"(full)
+                        : "memory");
+                }
+                issued = kt + 1;
+            }
+            // copies still in flight complete on their full barrier before the CTA leaves
+            for (int kt = (issued > kStages ? issued - kStages : 0); kt < issued; ++kt)
+                mbar_wait(smem_u32(bar + kBarFull + kt % kStages), (kt / kStages) & 1, abort_flag, timeout_ns);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t id = idesc(kBf16, kTileM, kTileN);
+            int r = 0;
+            bool first[kLevels];
+#pragma unroll
+            for (int l = 0; l < kLevels; ++l) first[l] = true;
+            for (int kt = 0; kt < Kt; ++kt) {
+                const int s = kt % kStages;
+                if (kt % kRangeTiles == 0 && kt > 0) {
+                    // accumulators of the previous range must be drained first
+                    if (!mbar_wait(smem_u32(bar + kBarAccEmpty), (r - 1) & 1, abort_flag, timeout_ns)) break;
+#pragma unroll
+                    for (int l = 0; l < kLevels; ++l) first[l] = true;
+                }
+                if (!mbar_wait(smem_u32(bar + kBarFull + s), (kt / kStages) & 1, abort_flag, timeout_ns)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t st = smem_u32(smem + (size_t)s * kStageBytes);
+#pragma unroll
+                for (int lvl = 0; lvl < kLevels; ++lvl) {
+                    if (lvl >= lv) break;
+                    const uint32_t d = tmem + (uint32_t)(lvl * kTileN);
+#pragma unroll
+                    for (int t = 0; t <= lvl; ++t) {
+                        const int u = lvl - t;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const uint32_t off = q * 2 * LBO;
+                            mma(kBf16, d, smem_desc(st + t * kBlockA + off),
+                                smem_desc(st + kS * kBlockA + u * kBlockB + off), id, first[lvl] ? 0u : 1u);
+                            first[lvl] = false;
+                        }
+                    }
+                }
+                commit(smem_u32(bar + kBarEmpty + s));   // frees the stage once these MMAs have read it
+                if (kt % kRangeTiles == kRangeTiles - 1 || kt == Kt - 1) {
+                    commit(smem_u32(bar + kBarAccFull));   // accumulators of range r complete
+                    ++r;
+                }
+            }
+            commit(smem_u32(bar + kBarFinal));
+            mbar_wait(smem_u32(bar + kBarFinal), 0, abort_flag, timeout_ns);   // every MMA issued has completed
+        }
+    } else {
+        // epilogue warps 2..9: rows 32 (warp % 4) + lane, columns half * 32 .. + 31
+        const int ew = warp - 2;
+        const int lane_base = 32 * (warp & 3);
+        const int half = ew >> 2;
+        const uint32_t taddr = tmem + ((uint32_t)lane_base << 16) + (uint32_t)(half * 32);
+        double acc[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] = 0.0;
+        bool ok = true;
+        for (int r = 0; r < nrange; ++r) {
+            if (!mbar_wait(smem_u32(bar + kBarAccFull), r & 1, abort_flag, timeout_ns)) {
+                ok = false;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            // level d holds n_d 2^-8d with n_d an integer (exact for d <= 3;
+            // higher levels are rounded to the nearest 2^-8d): the range's
+            // sum is S 2^-40 with the integer S = sum_d n_d 2^(8 (5 - d)),
+            // |S| < 2^63 (level 6 rounded to that unit), formed in int64 and
+            // converted once (integer arithmetic instead of twelve FP64
+            // operations per element).  A NaN slice reaches level 0.
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                long long S[16];
+                unsigned nan = 0;
+#pragma unroll
+                for (int lvl = 0; lvl < kLevels; ++lvl) {
+                    if (lvl >= lv) {   // uniform: not formed
+                        if (lvl < 6)
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) S[i] *= 256;
+                        continue;
+                    }
+                    float v[16];
+                    tmem_ld16(taddr + (uint32_t)(lvl * kTileN + c * 16), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const float scale = __int_as_float((127 + 8 * lvl) << 23);   // 2^8d
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const int n = __float2int_rn(v[i] * scale);
+                        if (lvl == 0) {
+                            S[i] = n;
+                            nan |= (v[i] != v[i]) ? 1u << i : 0u;
+                        } else if (lvl < 6) {
+                            S[i] = S[i] * 256 + n;
+                        } else {
+                            S[i] += (n + 128) >> 8;   // level 6 in units of 2^-40
+                        }
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    acc[c * 16 + i] += ((nan >> i) & 1u) ? __longlong_as_double(0x7ff8000000000000ll) : (double)S[i];
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + kBarAccEmpty)) : "memory");
+        }
+        if (ok && !*abort_flag) {
+            const int i = mt * kTileM + lane_base + lane;
+            if (i < P.M) {
+                const int ei = P.ea[i];
+#pragma unroll
+                for (int jj = 0; jj < 32; ++jj) {
+                    const int j = nt * kTileN + half * 32 + jj;
+                    if (j >= N) continue;
+                    double v = P.alpha * ldexp(acc[jj], ei + P.eb[j] - 54);   // acc in units of 2^-40
+                    const size_t row = P.c_gather ? (size_t)P.c_gather[i] : (size_t)i;
+                    if (P.D) {
+                        const size_t di = row * P.ldd + j;
+                        v += P.beta * (P.d_f32 ? (double)static_cast<const float*>(P.D)[di]
+                                               : static_cast<const double*>(P.D)[di]);
+                    }
+                    if (P.sub_identity && i == j) v -= 1.0;
+                    const size_t ci = row * P.ldc + j;
+                    if (P.c_f32)
+                        static_cast<float*>(P.C)[ci] = (float)v;
+                    else
+                        static_cast<double*>(P.C)[ci] = v;
+                    if (P.sym && j > i) static_cast<double*>(P.C)[(size_t)j * P.ldc + i] = v;
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    if (threadIdx.x == 0 && *abort_flag && P.status) atomicOr(P.status, (int)MPDO_ST_TIMEOUT);
 }
 
 // Theta' = G Theta in place (rows (l, s1), columns s2 cr + r) and theta~ =
@@ -752,16 +785,6 @@ __global__ void __launch_bounds__(256) gate_weight_kernel(const OpDesc* descs, i
 
 }  // namespace
 
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, OzProblem* probs, int chi_cap, bool bf16, int S,
-                          unsigned long long timeout_ns, cudaStream_t st) {
-    if (nops <= 0) return cudaSuccess;
-    oz_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, kind, probs, chi_cap, bf16 ? 1 : 0);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int big = 4 * chi_cap;
-    return launch_oz_gemm(probs, nops, big, big, big, bf16, S, timeout_ns, st);
-}
-
 cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st) {
     if (nops <= 0) return cudaSuccess;
     dim3 g((chi_cap * chi_cap + 255) / 256, nops);
@@ -791,26 +814,38 @@ cudaError_t oz_prepare() {
 namespace {
 
 template <bool kBf16, int S>
-cudaError_t launch_oz(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced,
+cudaError_t launch_oz(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced,
                       unsigned long long timeout_ns, cudaStream_t st) {
     const int mt = (max_m + kTileM - 1) / kTileM, nt = (max_n + kTileN - 1) / kTileN;
     const int rows = ((max_rows_sliced + kTileM - 1) / kTileM) * kTileM;
-    oz_slice_kernel<kBf16, S><<<dim3((rows + 7) / 8, 2, count), 256, 0, st>>>(d_probs);
+    oz_slice_kernel<kBf16, S><<<dim3((rows + 7) / 8, 2, count), 256, 0, st>>>(src);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    oz_gemm_kernel<kBf16, S><<<dim3(nt, mt, count), kThreads, smem_of(S), st>>>(d_probs, timeout_ns);
+    oz_gemm_kernel<kBf16, S><<<dim3(nt, mt, count), kThreads, smem_of(S), st>>>(src, timeout_ns);
     return cudaGetLastError();
+}
+
+cudaError_t launch_oz_source(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
+                             int S, unsigned long long timeout_ns, cudaStream_t st) {
+    if (count <= 0) return cudaSuccess;
+    if (S == 7)   // bf16 slices only
+        return launch_oz<true, 7>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
+    return bf16 ? launch_oz<true, 6>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st)
+                : launch_oz<false, 6>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
 }
 
 }  // namespace
 
 cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
                            int S, unsigned long long timeout_ns, cudaStream_t st) {
-    if (count <= 0) return cudaSuccess;
-    if (S == 7)   // bf16 slices only
-        return launch_oz<true, 7>(d_probs, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
-    return bf16 ? launch_oz<true, 6>(d_probs, count, max_m, max_n, max_rows_sliced, timeout_ns, st)
-                : launch_oz<false, 6>(d_probs, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
+    return launch_oz_source(OzSource{d_probs, nullptr, 0, 0}, count, max_m, max_n, max_rows_sliced, bf16, S,
+                            timeout_ns, st);
+}
+
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, bool bf16, int S,
+                          unsigned long long timeout_ns, cudaStream_t st) {
+    const int big = 4 * chi_cap;
+    return launch_oz_source(OzSource{nullptr, d_desc, kind, chi_cap}, nops, big, big, big, bf16, S, timeout_ns, st);
 }
 
 namespace {

@@ -38,25 +38,15 @@ namespace {
 
 constexpr int NT = 256;
 
-__global__ void refine_init_kernel(const OpDesc* descs, int nops) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nops) return;
-    RefineOp& r = *descs[s].rf;
-    r.state = descs[s].c > 1 ? kRefineActive : kRefineLeft;
-    r.order = 0;
-    r.rho2 = 0u;
-    r.row1 = 0u;
-    r.far = 0;
-    r.thr = 0.0;
-    r.floor2 = 0.0;
-}
-
 // squared row norms and their inverse roots from G's diagonal, the zero floor
 // (rows at or under it are set to zero) and the discard threshold, fixed once open
 __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, int ld) {
     const OpDesc& d = descs[blockIdx.x];
     RefineOp& r = *d.rf;
-    if (r.state != kRefineActive) return;
+    if (r.state != kRefineActive) {
+        if (threadIdx.x == 0) r.order = 0;   // no rotation in this iteration
+        return;
+    }
     const int c = d.c;
     double* a = d.snorm;
     double* inv = d.snorm + ld;
@@ -92,72 +82,16 @@ __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, in
         r.rho2 = 0u;
         r.row1 = 0u;
         r.far = 0;
+        r.blocks = 0u;
     }
 }
 
-// X from G, one warp per row; the largest g^2 / (a b) of a needed pair, the
-// largest absolute row sum of X (a bound of its norm), and whether an angle
-// was too large for the expansion
-__global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int ld, double tol_in, float tcap) {
-    const OpDesc& d = descs[blockIdx.y];
-    RefineOp& r = *d.rf;
-    const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (i >= d.c || r.state != kRefineActive) return;
-    const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
-    const double* a = d.snorm;
-    const double* inv = d.snorm + ld;
-    const double ai = a[i], vi = inv[i], thr = r.thr;
-    const bool dead = vi == 0.0, low = ai < thr;
-    float rho = 0.0f, sum = 0.0f;
-    int far = 0;
-    for (int j = lane; j < d.c; j += 32) {
-        const double aj = a[j], vj = inv[j];
-        double x = 0.0;
-        if (j != i && !dead && vj != 0.0 && !(low && aj < thr)) {
-            const double v = vi * vj;
-            const float q = (float)(d.E[(size_t)i * ld + j] * v);   // g / (|w_i| |w_j|)
-            rho = !(fabsf(q) <= rho) ? fabsf(q) : rho;              // a NaN stays
-            if (fabsf(q) > tol) {
-                const float zeta = (float)((aj - ai) * v) / (2.0f * q);
-                const float t = fabsf(zeta) > 1e18f   // a row far below the other (zeta^2 leaves FP32's range)
-                                    ? 0.5f / zeta
-                                    : copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
-                if (fabsf(t) <= tcap) {
-                    const float th = t * fmaf(-t * t, 1.0f / 3.0f, 1.0f);   // atan t
-                    x = -(double)th;
-                    sum += fabsf(th);
-                } else {
-                    far = 1;
-                }
-            }
-        }
-        d.Q[(size_t)i * ld + j] = x;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float v = __shfl_xor_sync(0xffffffffu, rho, o);
-        rho = !(v <= rho) ? v : rho;
-    }
-    sum = warp_sum(sum);
-    far = __any_sync(0xffffffffu, far);
-    if (lane == 0) {
-        atomicMax(&r.rho2, __float_as_uint(fabsf(rho * rho)));
-        atomicMax(&r.row1, __float_as_uint(sum));
-        if (far) atomicOr(&r.far, 1);
-    }
-}
-
-__global__ void refine_decide_kernel(const OpDesc* descs, int nops, double tol_in, int can_finish, float defect,
-                                     int last) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nops) return;
-    const OpDesc& d = descs[s];
-    RefineOp& r = *d.rf;
+// The op's state and the order of this iteration's rotation.
+__device__ void decide(const OpDesc& d, RefineOp& r, double tol_in, int can_finish, float defect, int last) {
     r.order = 0;
-    if (r.state != kRefineActive) return;
     if (d.sweeps_out) *d.sweeps_out += 1;
     const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
-    const float rho = sqrtf(__uint_as_float(r.rho2)), x = __uint_as_float(r.row1);
+    const float rho = sqrtf(__uint_as_float(__ldcg(&r.rho2))), x = __uint_as_float(__ldcg(&r.row1));
     if (rho <= tol) {
         r.state = can_finish ? kRefineDone : kRefineLeft;
         return;
@@ -173,33 +107,92 @@ __global__ void refine_decide_kernel(const OpDesc* descs, int nops, double tol_i
         r.state = kRefineLeft;   // beyond the expansion (or not finite)
         return;
     }
-    if (!r.far && 2.0f * rho * x <= 0.1f * tol)
+    if (!__ldcg(&r.far) && 2.0f * rho * x <= 0.1f * tol)
         r.state = can_finish ? kRefineDone : kRefineLeft;   // after this rotation
     else if (last)
         r.state = kRefineLeft;
 }
 
+// X from G, one warp per row; the largest g^2 / (a b) of a needed pair, the
+// largest absolute row sum of X (a bound of its norm), and whether an angle
+// was too large for the expansion.  The op's last CTA to finish decides.
+__global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int ld, double tol_in, float tcap,
+                                                      int can_finish, float defect, int last) {
+    const OpDesc& d = descs[blockIdx.y];
+    RefineOp& r = *d.rf;
+    const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int blocks = (d.c + NT / 32 - 1) / (NT / 32);
+    if ((int)blockIdx.x >= blocks || __ldcg(&r.state) != kRefineActive) return;
+    if (i < d.c) {
+        const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
+        const double* a = d.snorm;
+        const double* inv = d.snorm + ld;
+        const double ai = a[i], vi = inv[i], thr = r.thr;
+        const bool dead = vi == 0.0, low = ai < thr;
+        float rho = 0.0f, sum = 0.0f;
+        int far = 0;
+        for (int j = lane; j < d.c; j += 32) {
+            const double aj = a[j], vj = inv[j];
+            double x = 0.0;
+            if (j != i && !dead && vj != 0.0 && !(low && aj < thr)) {
+                const double v = vi * vj;
+                const float q = (float)(d.E[(size_t)i * ld + j] * v);   // g / (|w_i| |w_j|)
+                rho = !(fabsf(q) <= rho) ? fabsf(q) : rho;              // a NaN stays
+                if (fabsf(q) > tol) {
+                    const float zeta = (float)((aj - ai) * v) / (2.0f * q);
+                    const float t = fabsf(zeta) > 1e18f   // a row far below the other (zeta^2 leaves FP32's range)
+                                        ? 0.5f / zeta
+                                        : copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
+                    if (fabsf(t) <= tcap) {
+                        const float th = t * fmaf(-t * t, 1.0f / 3.0f, 1.0f);   // atan t
+                        x = -(double)th;
+                        sum += fabsf(th);
+                    } else {
+                        far = 1;
+                    }
+                }
+            }
+            d.Q[(size_t)i * ld + j] = x;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float v = __shfl_xor_sync(0xffffffffu, rho, o);
+            rho = !(v <= rho) ? v : rho;
+        }
+        sum = warp_sum(sum);
+        far = __any_sync(0xffffffffu, far);
+        if (lane == 0) {
+            atomicMax(&r.rho2, __float_as_uint(fabsf(rho * rho)));
+            atomicMax(&r.row1, __float_as_uint(sum));
+            if (far) atomicOr(&r.far, 1);
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&r.blocks, 1u) == (unsigned)blocks - 1u) {
+        __threadfence();
+        decide(d, r, tol_in, can_finish, defect, last);
+    }
+}
+
 }  // namespace
 
-cudaError_t launch_refine(const OpDesc* d_desc, int nops, OzProblem* probs, int chi_cap, bool bf16, int S,
-                          double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st) {
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, bool bf16, int S, double tol_in,
+                          bool can_finish, unsigned long long timeout_ns, cudaStream_t st) {
     if (nops <= 0) return cudaSuccess;
-    const int ld = 4 * chi_cap, g = (nops + 127) / 128;
+    const int ld = 4 * chi_cap;
     // defect of the rotation's orthogonality: FP64 rounding with 7 slices, the
     // level of 6 slices' products otherwise; the largest single angle follows
     const float defect = S == 7 ? 1e-17f : 1e-13f, tcap = S == 7 ? 2e-3f : 1e-2f;
-    refine_init_kernel<<<g, 128, 0, st>>>(d_desc, nops);
     for (int it = 0; it < kRefineIters; ++it) {
-        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, probs, chi_cap, bf16, S, timeout_ns, st);
+        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, chi_cap, bf16, S, timeout_ns, st);
         if (e != cudaSuccess) return e;
         refine_diag_kernel<<<nops, NT, 0, st>>>(d_desc, ld);
-        refine_x_kernel<<<dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st>>>(d_desc, ld, tol_in, tcap);
-        refine_decide_kernel<<<g, 128, 0, st>>>(d_desc, nops, tol_in, can_finish ? 1 : 0, defect,
-                                                it == kRefineIters - 1);
+        refine_x_kernel<<<dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st>>>(
+            d_desc, ld, tol_in, tcap, can_finish ? 1 : 0, defect, it == kRefineIters - 1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         for (int kind : {OZ_R3, OZ_R2, OZ_R1})
-            if ((e = launch_oz_ops(d_desc, nops, kind, probs, chi_cap, bf16, S, timeout_ns, st)) != cudaSuccess)
-                return e;
+            if ((e = launch_oz_ops(d_desc, nops, kind, chi_cap, bf16, S, timeout_ns, st)) != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }
