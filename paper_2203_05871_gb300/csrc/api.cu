@@ -50,8 +50,7 @@ void free_all(mpdo_ctx* c) {
     release_slots(c);
     void* ptrs[] = {c->d_sites, c->d_lam,  c->d_dims,  c->d_status, c->d_maxdisc, c->d_trace, c->d_params,
                     c->d_gates, c->d_specs, c->d_envL,  c->d_envR,   c->d_full,    c->d_one_a, c->d_one_b,
-                    c->d_out,   c->d_q,     c->d_pairs, c->d_need,   c->d_jb_table, c->d_gq,
-                    c->d_wstack, c->d_part};
+                    c->d_out,   c->d_q,     c->d_pairs, c->d_jb_table, c->d_gq,   c->d_wstack};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (auto& e : c->ev)
@@ -703,13 +702,11 @@ int mpdo_init(mpdo_ctx** out, const mpdo_config* cfg, void* cuda_stream) {
         (e = dalloc(&c->d_envR, (size_t)B * (N + 1) * c->cap)) != cudaSuccess ||
         (e = dalloc(&c->d_full, (size_t)B * N * N)) != cudaSuccess ||
         (e = dalloc(&c->d_wstack, two_stack_doubles(N, B, c->cap))) != cudaSuccess ||
-        (e = dalloc(&c->d_part, two_part_doubles(N, B, c->cap))) != cudaSuccess ||
         (e = dalloc(&c->d_one_a, (size_t)B * N * 4)) != cudaSuccess ||
         (e = dalloc(&c->d_one_b, (size_t)B * N)) != cudaSuccess ||
         (e = dalloc(&c->d_out, (size_t)B * N * N)) != cudaSuccess ||
         (e = dalloc(&c->d_q, (size_t)N)) != cudaSuccess ||
-        (e = dalloc(&c->d_pairs, (size_t)3 * N * N)) != cudaSuccess ||
-        (e = dalloc(&c->d_need, (size_t)N)) != cudaSuccess) {
+        (e = dalloc(&c->d_pairs, (size_t)3 * N * N + 2 * N)) != cudaSuccess) {
         fail(e == cudaErrorMemoryAllocation ? MPDO_ENOMEM : MPDO_ECUDA,
              std::string("device allocation: ") + cudaGetErrorString(e));
         return bail(e == cudaErrorMemoryAllocation ? MPDO_ENOMEM : MPDO_ECUDA);
@@ -1017,37 +1014,40 @@ int mpdo_measure_2q(mpdo_ctx* c, const int* pairs, int np, const char comp[2], i
         if (i < 0 || j < 0 || i >= N || j >= N || i == j) return fail(MPDO_EINVAL, "pair indices out of range or i == j");
     }
     CU(launch_environments(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, c->st));
-    std::vector<int> allq(N);
-    for (int q = 0; q < N; ++q) allq[q] = q;
-    CU(cudaMemcpyAsync(c->d_q, allq.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->st));
-    CU(launch_measure_1q(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, c->d_q, N, ca,
-                         c->d_one_a, c->st));
-    CU(launch_measure_1q(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, c->d_q, N, cb,
-                         c->d_one_b, c->st));
     double* dst = out_on_device ? out : c->d_out;
+    const double *one_a = c->d_one_a, *one_b = ca == cb ? c->d_one_a : c->d_one_b;
+    if (connected) {
+        CU(launch_measure_1q(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, nullptr, N, ca,
+                             c->d_one_a, c->st));
+        if (ca != cb)
+            CU(launch_measure_1q(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, nullptr, N,
+                                 cb, c->d_one_b, c->st));
+    }
     for (int pass = 0; pass < 2; ++pass) {
         // pass 0: pairs with i < j; pass 1: pairs with i > j, evaluated as (j, i) with swapped components
-        std::vector<int> trip;
-        std::vector<unsigned char> need(N, 0);
+        std::vector<int> up;   // (i, j, k) of every pair, then the rows and the columns asked for
+        up.reserve((size_t)3 * np + 2 * N);
+        std::vector<int> need(2 * N, 0);
         for (int k = 0; k < np; ++k) {
             int i = pairs[2 * k], j = pairs[2 * k + 1];
             if ((pass == 0) != (i < j)) continue;
             if (pass == 1) std::swap(i, j);
-            trip.push_back(i);
-            trip.push_back(j);
-            trip.push_back(k);
+            up.push_back(i);
+            up.push_back(j);
+            up.push_back(k);
             need[i] = 1;
+            need[N + j] = 1;
         }
-        if (trip.empty()) continue;
+        if (up.empty()) continue;
+        const int cnt = (int)up.size() / 3;
+        up.insert(up.end(), need.begin(), need.end());
         const int x = pass == 0 ? ca : cb, y = pass == 0 ? cb : ca;
-        CU(cudaMemcpyAsync(c->d_need, need.data(), N, cudaMemcpyHostToDevice, c->st));
-        CU(launch_measure_2q(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, x, y, c->d_need,
-                             c->d_wstack, c->d_part, c->d_full, c->st));
-        CU(cudaMemcpyAsync(c->d_pairs, trip.data(), sizeof(int) * trip.size(), cudaMemcpyHostToDevice, c->st));
-        const double* oa = pass == 0 ? c->d_one_a : c->d_one_b;
-        const double* ob = pass == 0 ? c->d_one_b : c->d_one_a;
-        CU(launch_gather_2q(c->d_full, oa, ob, c->d_pairs, (int)trip.size() / 3, np, N, B, connected, dst, c->st));
-        CU(cudaStreamSynchronize(c->st));   // host vectors above are reused by the next pass
+        CU(cudaMemcpyAsync(c->d_pairs, up.data(), sizeof(int) * up.size(), cudaMemcpyHostToDevice, c->st));
+        CU(launch_measure_2q(c->d_sites, sites_f32(c), c->d_dims, N, B, c->cap, c->d_envL, c->d_envR, x, y,
+                             c->d_pairs + 3 * cnt, c->d_wstack, c->d_full, c->st));
+        CU(launch_gather_2q(c->d_full, pass == 0 ? one_a : one_b, pass == 0 ? one_b : one_a, c->d_pairs, cnt, np, N,
+                            B, connected, dst, c->st));
+        CU(cudaStreamSynchronize(c->st));   // `up` is reused by the next pass
     }
     if (!out_on_device) {
         CU(cudaMemcpyAsync(out, dst, sizeof(double) * (size_t)np * B, cudaMemcpyDeviceToHost, c->st));

@@ -111,11 +111,10 @@ struct mpdo_ctx {
     int jacobi_resident = 0;
     int qr_resident = 0, qr32_resident = 0;
     // measurement
-    double *d_wstack = nullptr, *d_part = nullptr;   // all-pairs propagation scratch
+    double* d_wstack = nullptr;   // all-pairs propagation scratch
     double *d_envL = nullptr, *d_envR = nullptr, *d_full = nullptr, *d_one_a = nullptr, *d_one_b = nullptr,
            *d_out = nullptr;
     int *d_q = nullptr, *d_pairs = nullptr;
-    unsigned char* d_need = nullptr;
     // host mirrors
     std::vector<int> h_dims;
     std::vector<int> rank_log;    // [B][steps*n_ops] of the last trotter_step call

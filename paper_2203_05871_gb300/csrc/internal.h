@@ -324,19 +324,17 @@ cudaError_t launch_trace_normalize(void* sites, int sites_f32, const int* dims, 
                                    int force, double* trace_out, int* status, cudaStream_t st);
 cudaError_t launch_environments(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
                                 double* envL, double* envR, cudaStream_t st);
-// E(comp at q) for the listed qubits: out[b][k] = <sigma^c_q> (divided by E0)
+// E(comp at q) for the listed qubits (d_q null: all in order): out[b][k] = <sigma^c_q> (divided by E0)
 cudaError_t launch_measure_1q(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
                               const double* envL, const double* envR, const int* d_q, int nq,
                               int comp, double* out, cudaStream_t st);
-// all-pairs propagation: E(ca at i, cb at j) / E0 for every i with need[i] and
-// every j > i into full[b][i][j]; unused entries untouched.  Scratch: wstack
-// (two_stack_doubles) and part (two_part_doubles), device.
+// all-pairs propagation: E(ca at i, cb at j) / E0 into full[b][i][j] for every i < j
+// with need[i] and need[n + j]; unused entries untouched.  Scratch: wstack
+// (two_stack_doubles), device.
 size_t two_stack_doubles(int n, int B, int chi_cap);
-size_t two_part_doubles(int n, int B, int chi_cap);
 cudaError_t launch_measure_2q(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
-                              const double* envL, const double* envR, int ca, int cb,
-                              const unsigned char* d_need_i, double* wstack, double* part, double* full,
-                              cudaStream_t st);
+                              const double* envL, const double* envR, int ca, int cb, const int* d_need,
+                              double* wstack, double* full, cudaStream_t st);
 // d_trip[m][3] = (i, j, k): out[b][k] = full[b][i][j] (- one_a[b][i] one_b[b][j] if connected)
 cudaError_t launch_gather_2q(const double* full, const double* one_a, const double* one_b,
                              const int* d_trip, int m, int np, int n, int B, int connected,

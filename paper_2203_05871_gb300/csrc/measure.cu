@@ -7,6 +7,7 @@
 //   <sigma^a_i> = E(a at i)/E(I..I),  <sigma^a_i sigma^b_j> = E(a at i, b at j)/E(I..I).
 // Left environments L_p = E-prefix over sites < p (row vectors), right
 // environments R_p = suffix over sites >= p (column vectors), all with I.
+#include <cooperative_groups.h>
 #include <mpdo.h>
 
 #include "internal.h"
@@ -14,8 +15,6 @@
 namespace mpdo {
 
 namespace {
-
-constexpr int MT = 512;
 
 // one site tensor, read as double whatever the storage (f64 or f32)
 struct SiteRef {
@@ -31,42 +30,192 @@ __device__ __forceinline__ SiteRef site_ptr(const void* sites, int f32, int b, i
                    f32};
 }
 
-// v_out[r] = sum_l v_in[l] S[l][a][r]   (row vector times one Pauli slice)
-__device__ void vec_slice(SiteRef S, int a, int cl, int cr, int cap, const double* vin, double* vout) {
-    for (int r = threadIdx.x; r < cr; r += blockDim.x) {
-        double acc = 0.0;
-        for (int l = 0; l < cl; ++l) acc = fma(vin[l], S[((size_t)l * 4 + a) * cap + r], acc);
-        vout[r] = acc;
+// ---------------------------------------------------------------------------
+// Products of a vector with one Pauli slice, a CTA's share of the output.  A slice
+// is read once and its rows are contiguous, so the lanes run along r in both.  What
+// bounds them is the FP64 pipe, two FMAs per SM and clock: an instruction of a warp
+// takes it 16 clocks whether one lane or all are active, so lanes without a column
+// take other rows and the sums over lanes fold four rows at once.
+constexpr int CW = 8;                 // warps per CTA
+constexpr int kColTile = 64;          // columns per CTA of a row product at most
+
+// out(c) = sum_l v[l] S[l][comp][r0 + c], c < w <= kColTile; red: CW * kColTile doubles
+template <class F>
+__device__ __forceinline__ void row_product(SiteRef S, int comp, int cl, int cap, const double* v, int r0, int w,
+                                            double* red, F out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int U = 8;   // rows in flight
+    if (w > 32) {
+        double a0 = 0.0, a1 = 0.0;
+        const bool two = lane + 32 < w;
+        for (int l = warp; l < cl; l += U * CW) {
+            double x[U], y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const size_t at = ((size_t)(l + u * CW) * 4 + comp) * cap + r0 + lane;
+                x[u] = l + u * CW < cl ? S[at] : 0.0;
+                y[u] = l + u * CW < cl && two ? S[at + 32] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (l + u * CW < cl) {
+                    a0 = fma(v[l + u * CW], x[u], a0);
+                    a1 = fma(v[l + u * CW], y[u], a1);
+                }
+        }
+        red[warp * kColTile + lane] = a0;
+        red[warp * kColTile + 32 + lane] = a1;
+    } else if (w > 0) {
+        int cb = 1;
+        while (cb < w) cb <<= 1;   // lanes per row
+        const int rows = 32 / cb, g = lane / cb, c = lane % cb, step = CW * rows;
+        double a0 = 0.0;
+        for (int l0 = warp * rows; l0 < cl; l0 += U * step) {
+            double x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int l = l0 + u * step + g;
+                x[u] = l < cl && c < w ? S[((size_t)l * 4 + comp) * cap + r0 + c] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (l0 + u * step < cl) {
+                    const int l = l0 + u * step + g;
+                    a0 = fma(l < cl ? v[l] : 0.0, x[u], a0);
+                }
+        }
+        for (int o = cb; o < 32; o <<= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+        if (g == 0) red[warp * kColTile + c] = a0;
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < w; c += CW * 32) {
+        double sum = 0.0;
+#pragma unroll
+        for (int u = 0; u < CW; ++u) sum += red[u * kColTile + c];
+        out(c, sum);
+    }
+    __syncthreads();
+}
+
+// out(l) = sum_r S[l][comp][r] v[r] for l0 <= l < l1 (called by one lane of a warp),
+// four rows per warp at a time
+template <class F>
+__device__ __forceinline__ void column_product(SiteRef S, int comp, int cr, int cap, const double* v, int l0, int l1,
+                                               F out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int U = 4;   // loads in flight per row
+    for (int lb = l0 + 4 * warp; lb < l1; lb += 4 * CW) {
+        double a[4] = {};
+        for (int rb = 0; rb < cr; rb += 32 * U) {
+            double x[4][U];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int r = rb + 32 * u + lane;
+                    x[i][u] = lb + i < l1 && r < cr ? S[((size_t)(lb + i) * 4 + comp) * cap + r] : 0.0;
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (rb + 32 * u < cr) {
+                    const int r = rb + 32 * u + lane;
+                    const double vr = r < cr ? v[r] : 0.0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (lb + i < l1) a[i] = fma(x[i][u], vr, a[i]);
+                }
+        }
+        // lanes 0, 8, 16, 24 end with rows 0 .. 3
+        const bool h = lane & 16, q = lane & 8;
+        const double k0 = (h ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h ? a[0] : a[2], 16);
+        const double k1 = (h ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h ? a[1] : a[3], 16);
+        double k = (q ? k1 : k0) + __shfl_xor_sync(0xffffffffu, q ? k0 : k1, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+        const int l = lb + (h ? 2 : 0) + (q ? 1 : 0);
+        if ((lane & 7) == 0 && l < l1) out(l, k);
     }
 }
 
-__global__ void __launch_bounds__(MT) trace_kernel(void* sites, int f32, const int* dims, int n, int cap, int force,
-                                                   double* trace_out, int* status) {
-    const int b = blockIdx.x;
-    const int* dm = dims + (size_t)b * (n + 1);
-    __shared__ double v0[kMaxChi], v1[kMaxChi];
-    if (threadIdx.x == 0) v0[0] = 1.0;
-    __syncthreads();
-    double* vin = v0;
-    double* vout = v1;
-    for (int p = 0; p < n; ++p) {
-        vec_slice(site_ptr(sites, f32, b, p, n, cap), 0, dm[p], dm[p + 1], cap, vin, vout);
-        __syncthreads();
-        double* t = vin;
-        vin = vout;
-        vout = t;
-    }
-    const double tr = exp2(0.5 * n) * vin[0];
-    __shared__ double s_tr;
+// A cluster of 1 to 16 CTAs carries a vector through the chain, from the left
+// (v <- v B_p[I], p = 0 ..) or from the right (v <- B_p[I] v, p = n - 1 ..).  The
+// sites are serial, so what counts is a site's latency: every CTA takes its share
+// of the output, writes it into all copies of the vector through distributed
+// shared memory, and the cluster's barrier ends the site.  With a launch per site and
+// the pairs below carried through the whole chain, <X>, <Y>, <Z> and all <ZZ> of 40
+// sites at chi 512 took 3.97 ms, of four chains of 8 at chi 32 383 us; now 2.07 ms
+// and 263 us.  E, if not null, receives the vector at every bond.  Returns the first entry of the last vector.
+__device__ double chain(bool left, const void* sites, int f32, const int* dm, int b, int n, int cap, double* E) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), EC = (int)cluster.num_blocks();
+    __shared__ double v[2][kMaxChi];
+    __shared__ double red[CW * kColTile];
     if (threadIdx.x == 0) {
-        s_tr = tr;
+        v[0][0] = 1.0;
+        if (E && rank == 0) E[left ? 0 : (size_t)n * cap] = 1.0;
+    }
+    cluster.sync();   // every CTA runs before its shared memory is written
+    int cur = 0;
+    for (int t = 0; t < n; ++t) {
+        const int p = left ? t : n - 1 - t, cl = dm[p], cr = dm[p + 1];
+        const SiteRef S = site_ptr(sites, f32, b, p, n, cap);
+        const int len = left ? cr : cl, w = (len + EC - 1) / EC;
+        const int o0 = min(rank * w, len), o1 = min(o0 + w, len);
+        double* row = E ? E + (size_t)(left ? p + 1 : p) * cap : nullptr;
+        double* next = v[cur ^ 1];
+        auto put = [&](int o, double x) {
+            if (row) row[o] = x;
+            for (int k = 0; k < EC; ++k) cluster.map_shared_rank(next, k)[o] = x;
+        };
+        if (left)
+            row_product(S, 0, cl, cap, v[cur], o0, o1 - o0, red, [&](int c, double x) { put(o0 + c, x); });
+        else
+            column_product(S, 0, cr, cap, v[cur], o0, o1, put);
+        cur ^= 1;
+        cluster.sync();
+    }
+    return v[cur][0];
+}
+
+// CTAs per cluster: chi^2 / 2 clocks of the FP64 pipe per site are shared among them,
+// a cluster barrier is about 700.
+constexpr int kBigCluster = 16;   // beyond the portable 8
+int chain_ctas(int chi_cap) { return chi_cap <= 32 ? 1 : chi_cap <= 64 ? 4 : chi_cap <= 128 ? 8 : kBigCluster; }
+static_assert(kMaxChi <= 8 * kColTile && 32 <= kColTile && 64 <= 4 * kColTile, "a CTA's share of a row product");
+
+template <class... P, class... A>
+cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int ctas, cudaStream_t st, A... args) {
+    cudaError_t e = cudaSuccess;
+    if (ctas > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(CW * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Tr rho of every instance; force: site 0 over it
+__global__ void __launch_bounds__(CW * 32)
+    trace_kernel(void* sites, int f32, const int* dims, int n, int cap, int force, double* trace_out, int* status) {
+    const int EC = (int)cooperative_groups::this_cluster().num_blocks(), b = blockIdx.x / EC;
+    const int* dm = dims + (size_t)b * (n + 1);
+    const double tr = exp2(0.5 * n) * chain(true, sites, f32, dm, b, n, cap, nullptr);
+    if (blockIdx.x % EC) return;
+    if (threadIdx.x == 0) {
         trace_out[b] = tr;
         if (!isfinite(tr) || tr == 0.0) atomicOr(status + b, (int)MPDO_ST_NONFINITE);
     }
-    __syncthreads();
-    if (force && isfinite(s_tr) && s_tr != 0.0) {
+    if (force && isfinite(tr) && tr != 0.0) {
         void* S = const_cast<void*>(site_ptr(sites, f32, b, 0, n, cap).p);
-        const double inv = 1.0 / s_tr;
+        const double inv = 1.0 / tr;
         const int cr = dm[1];
         for (int e = threadIdx.x; e < 4 * cr; e += blockDim.x) {
             const size_t i = (size_t)(e / cr) * cap + (e % cr);
@@ -75,188 +224,184 @@ __global__ void __launch_bounds__(MT) trace_kernel(void* sites, int f32, const i
     }
 }
 
-// One step t of both environments, spread over CTAs (a single CTA per
-// environment would leave all but two SMs idle and run at one SM's FP64 rate):
-//   blockIdx.y == 0: L_{t+1} = L_t B_t[I], EW columns of L_{t+1} per CTA;
-//   blockIdx.y == 1: R_p = B_p[I] R_{p+1} with p = n - 1 - t, EW entries per CTA.
-// Step 0 uses L_0 = R_n = (1) and also stores them for the readers.
-constexpr int EW = 16;
-__global__ void __launch_bounds__(256) env_step_kernel(const void* sites, int f32, const int* dims, int n, int cap,
-                                                       int t, double* envL, double* envR) {
+// Both environments in one launch, blockIdx.y 0 from the left (L_{p+1} = L_p B_p[I]),
+// 1 from the right (R_p = B_p[I] R_{p+1}).
+__global__ void __launch_bounds__(CW * 32)
+    env_chain_kernel(const void* sites, int f32, const int* dims, int n, int cap, double* envL, double* envR) {
     const int b = blockIdx.z;
-    const int* dm = dims + (size_t)b * (n + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (blockIdx.y == 0) {
-        const int p = t, cl = dm[p], cr = dm[p + 1];
-        const int r0 = blockIdx.x * EW;
-        double* E = envL + (size_t)b * (n + 1) * cap;
-        if (p == 0 && blockIdx.x == 0 && threadIdx.x == 0) E[0] = 1.0;
-        if (r0 >= cr) return;
-        const SiteRef S = site_ptr(sites, f32, b, p, n, cap);
-        const double* vin = E + (size_t)p * cap;
-        const int c = threadIdx.x % EW, g = threadIdx.x / EW;   // column, row group (16 groups)
-        const int r = r0 + c;
-        double acc = 0.0;
-        if (r < cr)
-            for (int l = g; l < cl; l += 256 / EW) acc = fma(p == 0 ? 1.0 : vin[l], S[((size_t)l * 4) * cap + r], acc);
-        __shared__ double red[256];
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        if (g == 0 && r < cr) {
-            double sum = 0.0;
-            for (int k = 0; k < 256 / EW; ++k) sum += red[k * EW + c];
-            E[(size_t)(p + 1) * cap + r] = sum;
-        }
-    } else {
-        const int p = n - 1 - t, cl = dm[p], cr = dm[p + 1];
-        const int l0 = blockIdx.x * EW;
-        double* E = envR + (size_t)b * (n + 1) * cap;
-        if (p == n - 1 && blockIdx.x == 0 && threadIdx.x == 0) E[(size_t)n * cap] = 1.0;
-        if (l0 >= cl) return;
-        const SiteRef S = site_ptr(sites, f32, b, p, n, cap);
-        const double* rin = E + (size_t)(p + 1) * cap;
-        const int lend = min(l0 + EW, cl);
-        for (int l = l0 + warp; l < lend; l += 8) {
-            double acc = 0.0;
-            for (int r = lane; r < cr; r += 32) acc = fma(S[((size_t)l * 4) * cap + r], p == n - 1 ? 1.0 : rin[r], acc);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) E[(size_t)p * cap + l] = acc;
-        }
-    }
+    const bool left = blockIdx.y == 0;
+    chain(left, sites, f32, dims + (size_t)b * (n + 1), b, n, cap,
+          (left ? envL : envR) + (size_t)b * (n + 1) * cap);
 }
 
-__device__ double block_sum(double v) {
-    __shared__ double red[MT / 32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    return t;   // valid in thread 0
-}
-
-// out[b*nq + k] = E(comp at q_k) / E0
-__global__ void __launch_bounds__(MT) one_kernel(const void* sites, int f32, const int* dims, int n, int cap,
-                                                 const double* envL, const double* envR, const int* qs, int nq,
-                                                 int comp, double* out) {
-    const int k = blockIdx.x, b = blockIdx.y;
-    const int q = qs[k];
+// out[b*nq + k] = E(comp at q_k) / E0 (qs null: q_k = k), the rows of the site shared
+// by a cluster of CTAs
+__global__ void __launch_bounds__(CW * 32)
+    one_kernel(const void* sites, int f32, const int* dims, int n, int cap, const double* envL, const double* envR,
+               const int* qs, int nq, int comp, double* out) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), EC = (int)cluster.num_blocks();
+    const int k = blockIdx.x / EC, b = blockIdx.y;
+    const int q = qs ? qs[k] : k;
     const int* dm = dims + (size_t)b * (n + 1);
     const double* Lq = envL + ((size_t)b * (n + 1) + q) * cap;
     const double* Rq = envR + ((size_t)b * (n + 1) + q + 1) * cap;
-    const double E0 = envL[((size_t)b * (n + 1) + n) * cap];
     const SiteRef S = site_ptr(sites, f32, b, q, n, cap);
     const int cl = dm[q], cr = dm[q + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double sums[kBigCluster], red[CW];
+    const int w = (cl + EC - 1) / EC, l0 = min(rank * w, cl), l1 = min(l0 + w, cl);
     double part = 0.0;
-    for (int r = threadIdx.x; r < cr; r += blockDim.x) {
-        double acc = 0.0;
-        for (int l = 0; l < cl; ++l) acc = fma(Lq[l], S[((size_t)l * 4 + comp) * cap + r], acc);
-        part = fma(acc, Rq[r], part);
+    cluster.sync();   // every CTA runs before its shared memory is written
+    column_product(S, comp, cr, cap, Rq, l0, l1, [&](int l, double x) { part = fma(Lq[l], x, part); });
+#pragma unroll
+    for (int o = 16; o >= 8; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);   // lanes 0, 8, 16, 24
+    if (lane == 0) red[warp] = part;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int u = 0; u < CW; ++u) s += red[u];
+        cluster.map_shared_rank(sums, 0)[rank] = s;
     }
-    const double tot = block_sum(part);
-    if (threadIdx.x == 0) out[(size_t)b * nq + k] = tot / E0;
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        double s = 0.0;
+        for (int u = 0; u < EC; ++u) s += sums[u];
+        out[(size_t)b * nq + k] = s / envL[((size_t)b * (n + 1) + n) * cap];
+    }
 }
 
-// All-pairs two-point values as one stacked propagation over j (the rows
-// w_i for every i < j advance together, so site j's slices are read once per
-// j instead of once per (i, j)).  Step j, per instance b and per tile of TW
-// columns r of bond j+1:
-//   for i < j with need[i]:  x = w_i B_j[cb],  part[b][j][tile][i] = x . R_{j+1}
-//                            (over the tile's columns),  w_i <- w_i B_j[I]
-//   if need[j] (j < n-1):    w_j = L_j B_j[ca]   (the row starts here)
-// w lives in win (read) and wout (written), [b][n][cap] each, swapped per
-// step.  The tile's three slices are staged in shared memory ([l][TW] each);
-// a warp takes one row i at a time, its lanes split l.  The sum over tiles
-// (two_reduce_kernel) keeps the result independent of the launch shape.
+// ---------------------------------------------------------------------------
+// All-pairs two-point values.  With s_i = L_i B_i[ca] (at bond i + 1) and
+// u_j = B_j[cb] R_{j+1} (at bond j), E(ca at i, cb at j) is s_i carried through the
+// sites between them, dotted with u_j.  The chain is cut in the middle, at bond
+// m = n / 2: the s_i of the left half are carried right to it, the u_j of the right
+// half left to it, each step taking one site of either half:
+//   left, site t:  E(i, t) = w_i . u_t, then w_i <- w_i B_t[I], for i < t;
+//   right, site p: E(p, j) = s_p . u_j, then u_j <- B_p[I] u_j, for j > p;
+// and the pairs across the middle are dot products at bond m.  Against carrying
+// every s_i through all later sites with both slices, that is half the steps, an
+// eighth of the FP64 work and one slice per site instead of three (the propagation
+// is bound by the FP64 pipe at chi 512, by the serial steps below).
+//
+// Scratch (doubles): seeds s [b][n][cap], u [b][n][cap], then two buffers
+// [b][n][cap] of carried rows (i < m: w_i, j >= m: u_j).
+struct Pairs {
+    const void* sites;
+    int f32;
+    const int* dims;
+    int n, cap, B;
+    const double *envL, *envR;
+    const int* need;      // [n] rows i, then [n] columns j, that some pair asks for
+    double *s, *u, *buf;  // scratch
+    double* full;         // [b][i][j]
+    __device__ double* row(int which, int b, int i) const {
+        return buf + (((size_t)which * B + b) * n + i) * cap;
+    }
+    __device__ void put(int b, int i, int j, double e) const {
+        full[((size_t)b * n + i) * n + j] = e / envL[((size_t)b * (n + 1) + n) * cap];
+    }
+};
+
+__device__ __forceinline__ double warp_dot(const double* x, const double* y, int len, int lane) {
+    double a = 0.0;
+    for (int k = lane; k < len; k += 32) a = fma(x[k], y[k], a);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+// the seeds: grid (tiles of kColTile x 2, site, instance)
+__global__ void __launch_bounds__(CW * 32) pair_seed_kernel(Pairs P, int ca, int cb) {
+    const int p = blockIdx.y, b = blockIdx.z;
+    const bool left = (blockIdx.x & 1) == 0;
+    if (!P.need[left ? p : P.n + p]) return;
+    const int* dm = P.dims + (size_t)b * (P.n + 1);
+    const int cl = dm[p], cr = dm[p + 1], o0 = (blockIdx.x >> 1) * kColTile, len = left ? cr : cl;
+    if (o0 >= len) return;
+    const SiteRef S = site_ptr(P.sites, P.f32, b, p, P.n, P.cap);
+    __shared__ double red[CW * kColTile];
+    const size_t at = ((size_t)b * P.n + p) * P.cap, env = ((size_t)b * (P.n + 1) + p) * P.cap;
+    if (left)
+        row_product(S, ca, cl, P.cap, P.envL + env, o0, min(kColTile, len - o0), red,
+                    [&](int c, double x) { P.s[at + o0 + c] = x; });
+    else
+        column_product(S, cb, cr, P.cap, P.envR + env + P.cap, o0, min(o0 + kColTile, len),
+                       [&](int l, double x) { P.u[at + l] = x; });
+}
+
+// Step s: site s of the left half (blockIdx.y 0), site n - 1 - s of the right half
+// (1).  A CTA takes TW outputs of every carried row, the slice's part for them in
+// shared memory, a warp one row at a time; the rows' dot products are spread over
+// the CTAs.
 constexpr int TW = 4;
-__global__ void __launch_bounds__(256) two_stack_kernel(const void* sites, int f32, const int* dims, int n, int cap,
-                                                        const double* envL, const double* envR, int ca, int cb,
-                                                        const unsigned char* need, int j, const double* win,
-                                                        double* wout, double* part, int ntiles) {
-    const int b = blockIdx.y, tile = blockIdx.x;
-    const int* dm = dims + (size_t)b * (n + 1);
-    const int cl = dm[j], cr = dm[j + 1];
-    const int r0 = tile * TW;
-    if (r0 >= cr) return;
-    extern __shared__ double sm[];
-    double* sI = sm;                     // [cap][TW]: slice I of site j, the tile's columns
-    double* sB = sm + (size_t)cap * TW;  // slice cb
-    double* sA = sB + (size_t)cap * TW;  // slice ca
-    const SiteRef S = site_ptr(sites, f32, b, j, n, cap);
-    for (int e = threadIdx.x; e < cl * TW; e += blockDim.x) {
-        const int l = e / TW, c = e % TW, r = r0 + c;
-        const bool in = r < cr;
-        const size_t base = (size_t)l * 4 * cap + r;
-        sI[e] = in ? S[base] : 0.0;
-        sB[e] = in ? S[base + (size_t)cb * cap] : 0.0;
-        sA[e] = in ? S[base + (size_t)ca * cap] : 0.0;
+__global__ void __launch_bounds__(CW * 32) pair_step_kernel(Pairs P, int s, int m) {
+    const bool left = blockIdx.y == 0;
+    const int p = left ? s : P.n - 1 - s, b = blockIdx.z, n = P.n, cap = P.cap;
+    if (left ? p >= m : p < m) return;
+    const int* dm = P.dims + (size_t)b * (n + 1);
+    const int cl = dm[p], cr = dm[p + 1];
+    const int len = left ? cr : cl, in = left ? cl : cr;   // outputs, inputs
+    const int ntiles = (len + TW - 1) / TW, o0 = blockIdx.x * TW;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r0 = left ? 0 : p + 1, r1 = left ? p : n;     // carried rows
+    const int* need = left ? P.need : P.need + n;
+    auto source = [&](int r) -> const double* {   // a row enters from its seed
+        if (left ? r == p - 1 : r == p + 1) return (left ? P.s : P.u) + ((size_t)b * n + r) * cap;
+        return P.row((s - 1) & 1, b, r);
+    };
+    // dot products with the site's own seed, one row per warp of the launch
+    if (P.need[left ? n + p : p]) {
+        const double* own = (left ? P.u : P.s) + ((size_t)b * n + p) * cap;
+        for (int r = r0 + blockIdx.x * CW + warp; r < r1; r += gridDim.x * CW) {
+            if (!need[r]) continue;
+            const double e = warp_dot(source(r), own, in, lane);
+            if (lane == 0) P.put(b, left ? r : p, left ? p : r, e);
+        }
+    }
+    if ((int)blockIdx.x >= ntiles) return;
+    extern __shared__ double sI[];   // [in][TW]: slice I, the tile's outputs
+    const SiteRef S = site_ptr(P.sites, P.f32, b, p, n, cap);
+    for (int e = threadIdx.x; e < in * TW; e += CW * 32) {
+        const int x = left ? e / TW : e % in, o = left ? e % TW : e / in;   // along r in both
+        const int l = left ? x : o0 + o, r = left ? o0 + o : x;
+        sI[x * TW + o] = o0 + o < len ? S[(size_t)l * 4 * cap + r] : 0.0;
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double* Lj = envL + ((size_t)b * (n + 1) + j) * cap;
-    const double* Rn = envR + ((size_t)b * (n + 1) + j + 1) * cap;
-    const double* W = win + (size_t)b * n * cap;
-    double* Wn = wout + (size_t)b * n * cap;
-    for (int i = warp; i <= j; i += 8) {
-        if (!need[i] || (i == j && j >= n - 1)) continue;
-        const bool seed = i == j;
-        const double* w = seed ? Lj : W + (size_t)i * cap;
-        const double* s1 = seed ? sA : sI;
-        double a[TW] = {}, v[TW] = {};
-        for (int l = lane; l < cl; l += 32) {
-            const double wl = w[l];
-            const double2 p0 = *reinterpret_cast<const double2*>(s1 + l * TW);
-            const double2 p1 = *reinterpret_cast<const double2*>(s1 + l * TW + 2);
-            a[0] = fma(wl, p0.x, a[0]);
-            a[1] = fma(wl, p0.y, a[1]);
-            a[2] = fma(wl, p1.x, a[2]);
-            a[3] = fma(wl, p1.y, a[3]);
-            if (!seed) {
-                const double2 q0 = *reinterpret_cast<const double2*>(sB + l * TW);
-                const double2 q1 = *reinterpret_cast<const double2*>(sB + l * TW + 2);
-                v[0] = fma(wl, q0.x, v[0]);
-                v[1] = fma(wl, q0.y, v[1]);
-                v[2] = fma(wl, q1.x, v[2]);
-                v[3] = fma(wl, q1.y, v[3]);
-            }
+    for (int r = r0 + warp; r < r1; r += CW) {
+        if (!need[r]) continue;
+        const double* w = source(r);
+        double a[TW] = {};
+        for (int x = lane; x < in; x += 32) {
+            const double wx = w[x];
+            const double2 q0 = *reinterpret_cast<const double2*>(sI + x * TW);
+            const double2 q1 = *reinterpret_cast<const double2*>(sI + x * TW + 2);
+            a[0] = fma(wx, q0.x, a[0]);
+            a[1] = fma(wx, q0.y, a[1]);
+            a[2] = fma(wx, q1.x, a[2]);
+            a[3] = fma(wx, q1.y, a[3]);
         }
 #pragma unroll
         for (int c = 0; c < TW; ++c)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                a[c] += __shfl_xor_sync(0xffffffffu, a[c], o);
-                v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-            }
-        if (lane == 0) {
-            double dot = 0.0;
-#pragma unroll
-            for (int c = 0; c < TW; ++c)
-                if (r0 + c < cr) {
-                    Wn[(size_t)i * cap + r0 + c] = a[c];
-                    dot = fma(v[c], Rn[r0 + c], dot);
-                }
-            if (!seed) part[(((size_t)b * n + j) * ntiles + tile) * n + i] = dot;
-        }
+            for (int o = 16; o > 0; o >>= 1) a[c] += __shfl_xor_sync(0xffffffffu, a[c], o);
+        if (lane < TW && o0 + lane < len)
+            P.row(s & 1, b, r)[o0 + lane] = lane == 0 ? a[0] : lane == 1 ? a[1] : lane == 2 ? a[2] : a[3];
     }
 }
 
-// full[b][i][j] = sum over the tiles of step j of part[b][j][tile][i], / E0
-__global__ void two_reduce_kernel(const double* part, const int* dims, const double* envL,
-                                  const unsigned char* need, int n, int cap, int B, int ntiles, double* full) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)B * n * n) return;
-    const int b = (int)(t / ((long long)n * n)), i = (int)((t / n) % n), j = (int)(t % n);
-    if (j <= i || !need[i]) return;
-    const int cr = dims[(size_t)b * (n + 1) + j + 1];
-    const int nt = (cr + TW - 1) / TW;
-    double sum = 0.0;
-    for (int k = 0; k < nt; ++k) sum += part[(((size_t)b * n + j) * ntiles + k) * n + i];
-    full[((size_t)b * n + i) * n + j] = sum / envL[((size_t)b * (n + 1) + n) * cap];
+// pairs i < m <= j at bond m, one per warp
+__global__ void __launch_bounds__(CW * 32) pair_cross_kernel(Pairs P, int m) {
+    const int b = blockIdx.y, n = P.n, lane = threadIdx.x & 31;
+    const int e = blockIdx.x * CW + (threadIdx.x >> 5);
+    if (e >= m * (n - m)) return;
+    const int i = e / (n - m), j = m + e % (n - m);
+    if (!P.need[i] || !P.need[n + j]) return;
+    const double* w = i == m - 1 ? P.s + ((size_t)b * n + i) * P.cap : P.row((m - 1) & 1, b, i);
+    const double* u = j == m ? P.u + ((size_t)b * n + j) * P.cap : P.row((n - 1 - m) & 1, b, j);
+    const double v = warp_dot(w, u, P.dims[(size_t)b * (n + 1) + m], lane);
+    if (lane == 0) P.put(b, i, j, v);
 }
 
 // trip[t] = (i, j, k): out[b][k] = full[b][i][j] (minus one_a[b][i] one_b[b][j] if connected)
@@ -275,48 +420,44 @@ __global__ void gather_kernel(const double* full, const double* one_a, const dou
 
 cudaError_t launch_trace_normalize(void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap, int force,
                                    double* trace_out, int* status, cudaStream_t st) {
-    trace_kernel<<<B, MT, 0, st>>>(sites, sites_f32, dims, n, chi_cap, force, trace_out, status);
-    return cudaGetLastError();
+    const int ctas = chain_ctas(chi_cap);
+    return launch_cluster(trace_kernel, dim3(ctas * B), ctas, st, sites, sites_f32, dims, n, chi_cap, force, trace_out,
+                          status);
 }
 
 cudaError_t launch_environments(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
                                 double* envL, double* envR, cudaStream_t st) {
-    const dim3 grid((chi_cap + EW - 1) / EW, 2, B);
-    for (int t = 0; t < n; ++t) {
-        env_step_kernel<<<grid, 256, 0, st>>>(sites, sites_f32, dims, n, chi_cap, t, envL, envR);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const int ctas = chain_ctas(chi_cap);
+    return launch_cluster(env_chain_kernel, dim3(ctas, 2, B), ctas, st, sites, sites_f32, dims, n, chi_cap, envL, envR);
 }
 
 cudaError_t launch_measure_1q(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
                               const double* envL, const double* envR, const int* d_q, int nq, int comp, double* out,
                               cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
-    one_kernel<<<dim3(nq, B), MT, 0, st>>>(sites, sites_f32, dims, n, chi_cap, envL, envR, d_q, nq, comp, out);
-    return cudaGetLastError();
+    const int ctas = chi_cap <= 64 ? 1 : chi_cap <= 128 ? 4 : 8;
+    return launch_cluster(one_kernel, dim3(ctas * nq, B), ctas, st, sites, sites_f32, dims, n, chi_cap, envL, envR, d_q,
+                          nq, comp, out);
 }
 
-size_t two_stack_doubles(int n, int B, int chi_cap) { return (size_t)2 * B * n * chi_cap; }
-size_t two_part_doubles(int n, int B, int chi_cap) { return (size_t)B * n * n * ((chi_cap + TW - 1) / TW); }
+size_t two_stack_doubles(int n, int B, int chi_cap) { return (size_t)4 * B * n * chi_cap; }
 
 cudaError_t launch_measure_2q(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
-                              const double* envL, const double* envR, int ca, int cb, const unsigned char* d_need_i,
-                              double* wstack, double* part, double* full, cudaStream_t st) {
-    const int ntiles = (chi_cap + TW - 1) / TW;
-    const size_t smem = (size_t)3 * chi_cap * TW * sizeof(double);
-    static_assert((size_t)3 * kMaxChi * TW * sizeof(double) <= 48 * 1024, "within the default shared memory");
-    double* w[2] = {wstack, wstack + (size_t)B * n * chi_cap};
-    for (int j = 0; j < n; ++j) {
-        two_stack_kernel<<<dim3(ntiles, B), 256, smem, st>>>(sites, sites_f32, dims, n, chi_cap, envL, envR, ca, cb,
-                                                            d_need_i, j, w[j & 1], w[(j + 1) & 1], part, ntiles);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+                              const double* envL, const double* envR, int ca, int cb, const int* d_need,
+                              double* wstack, double* full, cudaStream_t st) {
+    const size_t rows = (size_t)B * n * chi_cap;
+    const Pairs P{sites, sites_f32, dims, n, chi_cap, B, envL, envR, d_need, wstack, wstack + rows, wstack + 2 * rows, full};
+    const int m = n / 2, steps = n - 1 - m > m - 1 ? n - 1 - m : m - 1;
+    pair_seed_kernel<<<dim3(2 * ((chi_cap + kColTile - 1) / kColTile), n, B), CW * 32, 0, st>>>(P, ca, cb);
+    cudaError_t e = cudaGetLastError();
+    const size_t smem = (size_t)chi_cap * TW * sizeof(double);
+    static_assert((size_t)kMaxChi * TW * sizeof(double) <= 48 * 1024, "within the default shared memory");
+    for (int s = 1; s <= steps && e == cudaSuccess; ++s) {
+        pair_step_kernel<<<dim3((chi_cap + TW - 1) / TW, 2, B), CW * 32, smem, st>>>(P, s, m);
+        e = cudaGetLastError();
     }
-    const long long tot = (long long)B * n * n;
-    two_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(part, dims, envL, d_need_i, n, chi_cap, B,
-                                                                      ntiles, full);
+    if (e != cudaSuccess) return e;
+    pair_cross_kernel<<<dim3((m * (n - m) + CW - 1) / CW, B), CW * 32, 0, st>>>(P, m);
     return cudaGetLastError();
 }
 
