@@ -104,7 +104,7 @@ int alloc_slots(mpdo_ctx* c, int want) {
     const size_t mat = (size_t)c->ld * c->ld;
     size_t per_slot_bytes = (3 * mat + (size_t)c->cap * c->ld + 2 * c->ld) * sizeof(double);
     if (c->precond) {
-        c->oz_slot_bytes = oz_slice_bytes(c->ld, c->ld, c->oz_bf16, c->oz_s);
+        c->oz_slot_bytes = oz_slice_bytes(c->ld, c->ld, c->oz_s);
         per_slot_bytes += 3 * mat * sizeof(double) + 2 * mat * sizeof(float) + 2 * c->oz_slot_bytes +
                           2 * oz_exp_ints(c->ld) * sizeof(int);
     }
@@ -286,11 +286,6 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
 }
 
-// The SVD's own products take bf16 slices on every path: the slices are 8-bit
-// integers, exact in bf16 and tf32 alike, so the results are the same bit for bit,
-// at half the bytes and twice the MMA rate.  (The contractions keep the context's kind.)
-constexpr bool kSvdBf16 = true;
-
 cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     // E = U U^T - I (~1e-6), then one orthogonalisation step: second order
@@ -300,7 +295,7 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
     if (!c->mixed) kinds = {OZ_E, OZ_T, OZ_Q3, OZ_W};
     for (int kind : kinds) {
         const cudaError_t e =
-            launch_oz_ops(d_desc, nops, first + kind, c->cap, kSvdBf16, c->oz_s, timeout_ns, st);
+            launch_oz_ops(d_desc, nops, first + kind, c->cap, c->oz_s, timeout_ns, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -316,7 +311,7 @@ cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cud
     // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
     const double tol = fp64_jacobi_tol(c);
     const bool can = c->oz_s == 7 || tol >= 1e-12;
-    return launch_refine(d_desc, nops, c->cap, kSvdBf16, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
+    return launch_refine(d_desc, nops, c->cap, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
 }
 
 int svd_products_kernels(const mpdo_ctx* c) {
@@ -373,7 +368,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     ProfScope p_merge(c, K_MERGE);
     if (c->mixed) {
-        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, c->st));
         CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
     } else {
         CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
@@ -475,7 +470,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
             int r_max = 1;
             for (int s = 0; s < nops; ++s) r_max = std::max(r_max, c->h_desc[s].c);
             ProfScope p_qr(c, K_QR);
-            CU(launch_qr_blocked(c->d_desc, nops, cap, c->d_oz, c->oz_bf16, timeout_ns, c->st, r_max));
+            CU(launch_qr_blocked(c->d_desc, nops, cap, c->d_oz, timeout_ns, c->st, r_max));
             p_qr.stop();
             qr_kernels_chunk = qrb_kernels(cap, r_max);
         } else {
@@ -521,7 +516,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     p_tr.stop();
     ProfScope p_rec(c, K_RECON);
     if (c->mixed)
-        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_bf16, c->oz_s, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_s, timeout_ns, c->st));
     else
         CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
     p_rec.stop();
@@ -676,7 +671,6 @@ int mpdo_init(mpdo_ctx** out, const mpdo_config* cfg, void* cuda_stream) {
     if (!c) return fail(MPDO_ENOMEM, "host allocation failed");
     c->dev = dev;
     c->mixed = cfg->precision != MPDO_FP64;
-    c->oz_bf16 = cfg->precision != MPDO_MIXED_TF32;
     c->oz_s = c->mixed ? 6 : 7;
     c->precond = c->mixed || cfg->jacobi_max_sweeps >= kRefineMinSweeps;
     c->cfg = *cfg;

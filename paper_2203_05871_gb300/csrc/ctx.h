@@ -88,7 +88,6 @@ struct mpdo_ctx {
     int* d_pre_ok = nullptr;      // [slots] mixed path: the FP32 pass ended by its off-orthogonality rule
     bool mixed = false;           // mixed-precision SVD (FP32 preconditioning + FP64 finish)
     bool precond = false;         // SVD with FP32 preconditioning and Gram-matrix refinement (mixed and FP64 paths)
-    bool oz_bf16 = false;         // tensor-core slices in bf16 (MPDO_MIXED_BF16X3, FP64 path), else tf32
     int oz_s = 6;                 // slices per operand of the SVD's products: 6 (mixed path), 7 (FP64 path)
     mpdo::RefineOp* d_refine = nullptr;   // [slots]
     unsigned char *d_oz_as = nullptr, *d_oz_bs = nullptr;   // [slots] slice blocks of the tensor-core products

@@ -223,7 +223,7 @@ int alloc_backward(mpdo_ctx* c, GradState* g) {
     // backward slots: as many ops in flight as a layer has, within half the free memory
     g->ws_slot = (size_t)12 * ld * cap + (size_t)2 * ld * ld + (size_t)kGateBwdParts * 256;
     // mixed path: slices of both operands of one product per slot, every dimension <= ld
-    const size_t oz_bytes = (size_t)256 * ((oz_slice_bytes(ld, ld, c->oz_bf16, 6) + 255) / 256);
+    const size_t oz_bytes = (size_t)256 * ((oz_slice_bytes(ld, ld, 6) + 255) / 256);
     const size_t oz_ints = oz_exp_ints(ld);
     const size_t oz_slot = c->mixed ? 2 * oz_bytes + 2 * oz_ints * sizeof(int) + sizeof(OzProblem) : 0;
     size_t free_b = 0, total_b = 0;
@@ -369,7 +369,7 @@ int run_bwd_chunk(mpdo_ctx* c, GradState* g, const std::vector<const TapeRec*>& 
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     auto gemm = [&](int q) {
         const bool tc = c->mixed && (q == 4 || q >= 6);
-        return tc ? launch_gemm_tc(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], mx[q][2], g->oz, c->oz_bf16,
+        return tc ? launch_gemm_tc(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], mx[q][2], g->oz,
                                    timeout_ns, c->st)
                   : launch_gemm(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], false, c->st);
     };

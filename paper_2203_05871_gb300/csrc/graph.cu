@@ -178,7 +178,7 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
             if (c->mixed) {
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, cap, c->oz_bf16, c->oz_s, timeout_ns, st));
+                CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, st));
                 CU(launch_gate_weight(ch.d_desc, nops, cap, st));
             } else {
                 CU(launch_merge_gate(ch.d_desc, nops, cap, st));
@@ -186,7 +186,7 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             const size_t sync_bytes = sizeof(unsigned) * jacobi_sync_words(nops);
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
             if (blocked) {
-                CU(launch_qr_blocked(ch.d_desc, nops, cap, c->d_oz, c->oz_bf16, timeout_ns, st, 0));
+                CU(launch_qr_blocked(ch.d_desc, nops, cap, c->d_oz, timeout_ns, st, 0));
             } else {
                 CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
                              timeout_ns, ld, st));
@@ -208,7 +208,7 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
                              c->cfg.jacobi_max_sweeps, fp64_jacobi_tol(c), timeout_ns, ld, false, st, precond_rho(c)));
             CU(launch_truncate(ch.d_desc, nops, cap, st));
             if (c->mixed)
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, cap, c->oz_bf16, c->oz_s, timeout_ns, st));
+                CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, cap, c->oz_s, timeout_ns, st));
             else
                 CU(launch_reconstruct(ch.d_desc, nops, cap, st));
             klog_kernel<<<(nops + 127) / 128, 128, 0, st>>>(ch.d_desc, nops, c->n_ops, g->d_klog);

@@ -192,9 +192,9 @@ struct OzProblem {
     int Mt, Nt, Kt;      // tiles (128 rows, 64 columns, 64 bytes of K)
     int* status;         // MPDO_ST_TIMEOUT when a wait gives up (or nullptr)
 };
-// tiles of a problem: 128 rows of A, 64 columns of B, 64 bytes of K (32 bf16 or 16 tf32 values)
-__host__ __device__ inline void oz_set_tiles(OzProblem& p, bool bf16) {
-    const int KT = bf16 ? 32 : 16;
+// tiles of a problem: 128 rows of A, 64 columns of B, 64 bytes of K (32 values)
+__host__ __device__ inline void oz_set_tiles(OzProblem& p) {
+    constexpr int KT = 32;
     p.Mt = (p.M + 127) / 128;
     p.Nt = (p.N + 63) / 64;
     p.Kt = (p.K + KT - 1) / KT;
@@ -205,15 +205,14 @@ __host__ __device__ inline int oz_levels(int S, int e) {
     const int drop = e < 0 ? -e / 8 : 0;
     return S - drop > 2 ? S - drop : 2;
 }
-size_t oz_slice_bytes(int rows, int K, bool bf16, int S);   // slice blocks of an operand of rows x K
+size_t oz_slice_bytes(int rows, int K, int S);   // slice blocks of an operand of rows x K
 size_t oz_exp_ints(int rows);                          // its exponent array (rows rounded up to a tile)
-void oz_tiles(OzProblem& p, bool bf16);
 cudaError_t oz_prepare();
 // slices both operands of count problems, then multiplies; max_m / max_n /
 // max_rows_sliced bound the grids (CTAs outside a problem's tiles return)
 // S slices per operand: 6 (error 2^-46 of the row and column maxima per term) or
-// 7 (2^-54, an FP64 product's level; bf16 slices only)
-cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
+// 7 (2^-54, an FP64 product's level)
+cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced,
                            int S, unsigned long long timeout_ns, cudaStream_t st);
 
 // The mixed path's tensor-core products of a chunk of ops, built on the
@@ -227,7 +226,7 @@ cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int m
 // only), OZ_W then being W0 = Q theta~.
 enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T = 5, OZ_Q3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
        OZ_R1 = 10 };
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, bool bf16, int S,
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S,
                           unsigned long long timeout_ns, cudaStream_t st);
 constexpr int kOzKernels = 2;   // kernels of one launch_oz_ops
 // ---------------------------------------------------------------------------
@@ -249,7 +248,7 @@ struct RefineOp {
 // rotated until every needed pair is orthogonal to tol (state kRefineDone) or the
 // op is left to the Jacobi pass.  Scratch: d.E (G), d.Q (X), d.W0, d.snorm.
 // tol_in as for launch_jacobi; can_finish = false: never kRefineDone.
-cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, bool bf16, int S, double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
 constexpr int kRefineIters = 3;
 // kernels of one launch_refine
 constexpr int kRefineKernels = kRefineIters * (2 + 4 * kOzKernels);
@@ -270,7 +269,7 @@ int qrb_kernels(int chi_cap, int r_max);
 inline bool qrb_fits(int chi_cap) { return 4 * chi_cap >= 128; }
 cudaError_t qrb_prepare();
 // r_max: the largest min(m, n) of the chunk's ops (<= 0: the capacity 4 chi_cap)
-cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs, bool bf16,
+cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs,
                               unsigned long long timeout_ns, cudaStream_t st, int r_max);
 
 // FP32 Householder QR (qr32.cu) of the preconditioned SVD's ops with m <= n: Q^T into
@@ -318,7 +317,7 @@ struct OzScratch {
     size_t slot_bytes, exp_ints;
 };
 cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max_n, int max_k, const OzScratch& scr,
-                           bool bf16, unsigned long long timeout_ns, cudaStream_t st);
+                           unsigned long long timeout_ns, cudaStream_t st);
 
 cudaError_t launch_trace_normalize(void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
                                    int force, double* trace_out, int* status, cudaStream_t st);

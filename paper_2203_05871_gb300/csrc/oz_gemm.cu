@@ -11,10 +11,12 @@
 //    binary exponent of its largest |A_ik| (so |a| < 1), rounded to the
 //    integer X = round(2^47 a) and cut into S = 6 balanced base-256 digits,
 //    a ~ 2^-7 sum_t sigma_t 2^-8t with integers |sigma_t| <= 128; a slice
-//    keeps 8 significant bits, so it is exact in bf16 (MPDO_MIXED_BF16X3) and
-//    in tf32 (MPDO_MIXED_TF32), and it is stored as sigma_t 2^-8t.  B is cut
-//    the same way per column j (exponent f_j).  The rounding error is at most
-//    2^-48 of the row's largest entry.
+//    keeps 8 significant bits, so it is exact in bf16, and it is stored as
+//    sigma_t 2^-8t.  B is cut the same way per column j (exponent f_j).  The
+//    rounding error is at most 2^-48 of the row's largest entry.  S = 7 (2^55 a)
+//    serves the FP64 path, 2^-56.  (tf32 holds the same digits and gives the same
+//    products; it takes twice the bytes and half the MMA rate.  Both tensor
+//    precisions are formed from bf16 slices.)
 // 2. Products (oz_gemm_kernel).  Every slice pair (t, u) with t + u <= 5 is
 //    multiplied on the tensor core: a product sigma_t sigma_u has at most 16
 //    bits, so it is exact in FP32, and the sums stay exact while they fit 24
@@ -36,8 +38,8 @@
 // FP64's 2^-53 |A_ik B_kj|: FP64-class accuracy at tensor-core speed.
 //
 // Data layout.  The slices are written in the tcgen05 canonical K-major,
-// no-swizzle layout, pre-tiled: a block of R rows x 64 bytes of K (32 bf16 or
-// 16 tf32 values; R = 128 for A, 64 for B) is R x 64 bytes, element (row, k) at
+// no-swizzle layout, pre-tiled: a block of R rows x 64 bytes of K (32 bf16
+// values; R = 128 for A, 64 for B) is R x 64 bytes, element (row, k) at
 // (row/8)*512 + (k/g)*128 + (row%8)*16 + (k%g)*esize, g = 16/esize (core
 // matrices of 8 rows x 16 bytes, LBO = 128 B along K, SBO = 512 B along rows),
 // so one cp.async.bulk moves a block into shared memory as it is.  Blocks are
@@ -45,8 +47,8 @@
 //
 // Kernel.  One CTA per 128 x 64 tile of C, 320 threads: warp 0 issues the
 // bulk copies of the 6 + 6 slice blocks of each k tile into a 3-stage ring
-// (72 KB per stage), warp 1 issues the 42 MMAs of a k tile (21 pairs x 2
-// instructions of K = 16 bf16 / 8 tf32; M = 128, N = 64) and commits, warps
+// (72 KB per stage; 7 + 7 blocks: two stages of 84 KB), warp 1 issues the 42 MMAs of a k tile (21 pairs x 2
+// instructions of K = 16; M = 128, N = 64) and commits, warps
 // 2-9 drain the six accumulators (384 TMEM columns; warp w reads lanes
 // 32 (w % 4) .. +31, its half of the 64 columns).  Every wait is bounded by timeout_ns; a wait that
 // gives up records MPDO_ST_TIMEOUT in the problem's status word, the other roles
@@ -79,7 +81,8 @@ static_assert(smem_of(6) <= 227 * 1024 && smem_of(7) <= 227 * 1024, "the ring ex
 static_assert(kTileM == 128 && kTileN == 64, "oz_set_tiles (internal.h) assumes 128 x 64 tiles");
 constexpr int LBO = 128, SBO = 512;
 
-__host__ __device__ constexpr int kt_elems(int esize) { return 64 / esize; }
+constexpr int G = 8;                   // bf16 values per 16-byte store
+constexpr int KT = 32;                 // K values of a block
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -89,11 +92,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
            (1ull << 46);
 }
 
-// D = F32 (bits 4-5 = 1); A, B = BF16 (1) or TF32 (2) at bits 7-9, 10-12; K-major;
+// D = F32 (bits 4-5 = 1); A, B = BF16 (1) at bits 7-9, 10-12; K-major;
 // N >> 3 at bits 17-22; M >> 4 at bits 24-28
-__host__ __device__ constexpr uint32_t idesc(bool bf16, int M, int N) {
-    const uint32_t ab = bf16 ? 1u : 2u;
-    return (1u << 4) | (ab << 7) | (ab << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+__host__ __device__ constexpr uint32_t idesc(int M, int N) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ unsigned long long gtimer() {
@@ -129,18 +131,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volati
     }
 }
 
-__device__ __forceinline__ void mma(bool bf16, uint32_t dtmem, uint64_t a, uint64_t b, uint32_t id,
-                                    uint32_t accumulate) {
-    if (bf16)
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-            "l"(a), "l"(b), "r"(id), "r"(accumulate));
-    else
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-            "l"(a), "l"(b), "r"(id), "r"(accumulate));
+__device__ __forceinline__ void mma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t id, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(id), "r"(accumulate));
 }
 
 __device__ __forceinline__ void commit(uint32_t mbar) {
@@ -257,7 +252,7 @@ __device__ __forceinline__ long long fixed_of(unsigned long long bits, bool f32,
 // balanced base-256 digits X = sum_t sigma_t 2^(8(S - 1 - t)), |sigma_t| <= 128,
 // from the lowest digit up; stored as sigma_t 2^-8t, 16 bytes per slice.
 // nan: the row has a non-finite entry, every slice is NaN.
-template <int G, bool kBf16, int kS>
+template <int kS>
 __device__ __forceinline__ void slice_group(const long long* X, bool nan, uint4* out /* [kS] */) {
     int sig[kS][G];
 #pragma unroll
@@ -277,32 +272,28 @@ __device__ __forceinline__ void slice_group(const long long* X, bool nan, uint4*
         float sl[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) sl[g] = nan ? __int_as_float(0x7fc00000) : (float)sig[t][g] * scale;
-        if constexpr (kBf16) {
-            uint32_t w[4];
+        uint32_t w[4];
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const __nv_bfloat162 p = __floats2bfloat162_rn(sl[2 * h], sl[2 * h + 1]);
-                w[h] = *reinterpret_cast<const uint32_t*>(&p);
-            }
-            out[t] = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-            out[t] = make_uint4(__float_as_uint(sl[0]), __float_as_uint(sl[1]), __float_as_uint(sl[2]),
-                                __float_as_uint(sl[3]));
+        for (int h = 0; h < 4; ++h) {
+            const __nv_bfloat162 p = __floats2bfloat162_rn(sl[2 * h], sl[2 * h + 1]);
+            w[h] = *reinterpret_cast<const uint32_t*>(&p);
         }
+        out[t] = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
-// Where a launch finds its problems: an array, or one product kind of the ops of a
+// Where a launch finds its problems: an array, one product kind of the ops of a
 // chunk, built from the op's descriptor by each CTA (a kernel of its own for that
-// would cost a launch per product).
+// would cost a launch per product), or the launch's own argument.
 struct OzSource {
     const OzProblem* probs;
     const OpDesc* descs;
     int kind, cap;
+    OzProblem one;   // neither: this one problem
 };
 
 // The problem of one kind for an op.
-template <bool kBf16, int kS>
+template <int kS>
 __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
     const int ld = 4 * cap;
     OzProblem P{};
@@ -412,15 +403,17 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
     P.ea = d.oz_ea;
     P.eb = d.oz_eb;
     P.status = d.status;
-    oz_set_tiles(P, kBf16);
+    oz_set_tiles(P);
     return P;
 }
 
 // the CTA's problem, through shared memory
-template <bool kBf16, int kS>
+template <int kS>
 __device__ __forceinline__ void fetch_problem(const OzSource& src, OzProblem& P) {
     if (threadIdx.x == 0)
-        P = src.probs ? src.probs[blockIdx.z] : op_problem<kBf16, kS>(src.descs[blockIdx.z], src.kind, src.cap);
+        P = src.probs   ? src.probs[blockIdx.z]
+            : src.descs ? op_problem<kS>(src.descs[blockIdx.z], src.kind, src.cap)
+                        : src.one;
     __syncthreads();
 }
 
@@ -428,12 +421,9 @@ __device__ __forceinline__ void fetch_problem(const OzSource& src, OzProblem& P)
 // Strided views (a transposed operand, the right site of a merge): a block
 // takes 32 consecutive rows, lane = row and warp = a slice of the K range, so
 // that the 32 lanes of a load read 32 neighbouring rows at one k (coalesced).
-template <bool kBf16, int kS>
+template <int kS>
 __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int Kt, int lv, unsigned char* out, int* ex,
                                  int tile, int Rt) {
-    constexpr int esize = kBf16 ? 2 : 4;
-    constexpr int G = 16 / esize;
-    constexpr int KT = kt_elems(esize);
     __shared__ unsigned long long s_mx[8][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool f32 = X.f32 != 0;
@@ -462,7 +452,7 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int K
             x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
         }
         uint4 sl[kS];
-        slice_group<G, kBf16, kS>(x, bad && live, sl);
+        slice_group<kS>(x, bad && live, sl);
         const int kt = g0 / KT, kk = g0 % KT;
 #pragma unroll
         for (int t = 0; t < kS; ++t) {
@@ -476,13 +466,10 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int K
 // grid (row groups of 8, 2 = A | B, problems).  Views whose rows are
 // contiguous (ks == 1) take one warp per row, lanes along k; the others 32 rows
 // per block (slice_rows_tiled), the blocks past rows / 32 returning at once.
-template <bool kBf16, int kS>
+template <int kS>
 __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
-    constexpr int esize = kBf16 ? 2 : 4;
-    constexpr int G = 16 / esize;          // values per 16-byte store
-    constexpr int KT = kt_elems(esize);
     __shared__ OzProblem P;
-    fetch_problem<kBf16, kS>(src, P);
+    fetch_problem<kS>(src, P);
     const bool isB = blockIdx.y == 1;
     const OzOperand& X = isB ? P.B : P.A;
     const int N = P.Ndyn ? *P.Ndyn : P.N;
@@ -497,7 +484,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     if (!(X.mode == 0 && X.ks == 1)) {
         const int r0 = blockIdx.x * 32;
         if (r0 >= Rt * tile) return;   // uniform over the block (Rt * tile is a multiple of 32)
-        slice_rows_tiled<kBf16, kS>(X, r0, R, K, Kt, lv, out, ex, tile, Rt);
+        slice_rows_tiled<kS>(X, r0, R, K, Kt, lv, out, ex, tile, Rt);
         return;
     }
     const int r = blockIdx.x * 8 + warp;
@@ -529,7 +516,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
             x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
         }
         uint4 sl[kS];
-        slice_group<G, kBf16, kS>(x, bad && live, sl);
+        slice_group<kS>(x, bad && live, sl);
         const int kt = g0 / KT, kk = g0 % KT;
 #pragma unroll
         for (int t = 0; t < kS; ++t) {
@@ -540,11 +527,9 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     }
 }
 
-template <bool kBf16, int kS>
+template <int kS>
 __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                                                                unsigned long long timeout_ns) {
-    constexpr int esize = kBf16 ? 2 : 4;
-    constexpr int KT = kt_elems(esize);
     constexpr int kRangeTiles = kRangeK / KT;
     constexpr int kLevels = kS, kStages = stages_of(kS), kStageBytes = stage_bytes(kS);
     // barriers: full[kStages], empty[kStages], accumulators full, accumulators drained, final
@@ -552,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                   kBarFinal = 2 * kStages + 2;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ OzProblem P;
-    fetch_problem<kBf16, kS>(src, P);
+    fetch_problem<kS>(src, P);
     const int N = P.Ndyn ? *P.Ndyn : P.N;
     const int mt = blockIdx.y, nt = blockIdx.x;
     if (mt * kTileM >= P.M || nt * kTileN >= N) return;
@@ -623,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t id = idesc(kBf16, kTileM, kTileN);
+            const uint32_t id = idesc(kTileM, kTileN);
             int r = 0;
             bool first[kLevels];
 #pragma unroll
@@ -649,7 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
 #pragma unroll
                         for (int q = 0; q < 2; ++q) {
                             const uint32_t off = q * 2 * LBO;
-                            mma(kBf16, d, smem_desc(st + t * kBlockA + off),
+                            mma(d, smem_desc(st + t * kBlockA + off),
                                 smem_desc(st + kS * kBlockA + u * kBlockB + off), id, first[lvl] ? 0u : 1u);
                             first[lvl] = false;
                         }
@@ -792,66 +777,60 @@ cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cuda
     return cudaGetLastError();
 }
 
-size_t oz_slice_bytes(int rows, int K, bool bf16, int S) {
+size_t oz_slice_bytes(int rows, int K, int S) {
     // room for either operand: ceil(rows / 128) tiles of 8 KB cover ceil(rows / 64) of 4 KB
-    const int KT = kt_elems(bf16 ? 2 : 4);
     const size_t Rt = (rows + kTileM - 1) / kTileM, Kt = (K + KT - 1) / KT;
     return (size_t)S * Rt * Kt * kBlockA;
 }
 
 size_t oz_exp_ints(int rows) { return (size_t)((rows + kTileM - 1) / kTileM) * kTileM; }
 
-void oz_tiles(OzProblem& p, bool bf16) { oz_set_tiles(p, bf16); }
-
 cudaError_t oz_prepare() {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<true, 6>, a, smem_of(6));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<false, 6>, a, smem_of(6));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<true, 7>, a, smem_of(7));
+    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<6>, a, smem_of(6));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<7>, a, smem_of(7));
     return e;
 }
 
 namespace {
 
-template <bool kBf16, int S>
+template <int S>
 cudaError_t launch_oz(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced,
                       unsigned long long timeout_ns, cudaStream_t st) {
     const int mt = (max_m + kTileM - 1) / kTileM, nt = (max_n + kTileN - 1) / kTileN;
     const int rows = ((max_rows_sliced + kTileM - 1) / kTileM) * kTileM;
-    oz_slice_kernel<kBf16, S><<<dim3((rows + 7) / 8, 2, count), 256, 0, st>>>(src);
+    oz_slice_kernel<S><<<dim3((rows + 7) / 8, 2, count), 256, 0, st>>>(src);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    oz_gemm_kernel<kBf16, S><<<dim3(nt, mt, count), kThreads, smem_of(S), st>>>(src, timeout_ns);
+    oz_gemm_kernel<S><<<dim3(nt, mt, count), kThreads, smem_of(S), st>>>(src, timeout_ns);
     return cudaGetLastError();
 }
 
-cudaError_t launch_oz_source(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
-                             int S, unsigned long long timeout_ns, cudaStream_t st) {
+cudaError_t launch_oz_source(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced, int S,
+                             unsigned long long timeout_ns, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    if (S == 7)   // bf16 slices only
-        return launch_oz<true, 7>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
-    return bf16 ? launch_oz<true, 6>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st)
-                : launch_oz<false, 6>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
+    return S == 7 ? launch_oz<7>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st)
+                  : launch_oz<6>(src, count, max_m, max_n, max_rows_sliced, timeout_ns, st);
 }
 
 }  // namespace
 
-cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, bool bf16,
-                           int S, unsigned long long timeout_ns, cudaStream_t st) {
-    return launch_oz_source(OzSource{d_probs, nullptr, 0, 0}, count, max_m, max_n, max_rows_sliced, bf16, S,
+cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, int S,
+                           unsigned long long timeout_ns, cudaStream_t st) {
+    return launch_oz_source(OzSource{d_probs, nullptr, 0, 0, {}}, count, max_m, max_n, max_rows_sliced, S,
                             timeout_ns, st);
 }
 
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, bool bf16, int S,
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S,
                           unsigned long long timeout_ns, cudaStream_t st) {
     const int big = 4 * chi_cap;
-    return launch_oz_source(OzSource{nullptr, d_desc, kind, chi_cap}, nops, big, big, big, bf16, S, timeout_ns, st);
+    return launch_oz_source(OzSource{nullptr, d_desc, kind, chi_cap, {}}, nops, big, big, big, S, timeout_ns, st);
 }
 
 namespace {
 
 // problem s of a GemmDesc batch as an OzProblem (one thread per problem)
-__global__ void gemm_desc_oz_kernel(const GemmDesc* descs, int count, OzScratch scr, int bf16) {
+__global__ void gemm_desc_oz_kernel(const GemmDesc* descs, int count, OzScratch scr) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= count) return;
     const GemmDesc& d = descs[s];
@@ -878,23 +857,23 @@ __global__ void gemm_desc_oz_kernel(const GemmDesc* descs, int count, OzScratch 
     P.ea = scr.ea + (size_t)s * scr.exp_ints;
     P.eb = scr.eb + (size_t)s * scr.exp_ints;
     P.status = d.status;
-    oz_set_tiles(P, bf16 != 0);
+    oz_set_tiles(P);
     scr.probs[s] = P;
 }
 
 }  // namespace
 
 cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max_n, int max_k, const OzScratch& scr,
-                           bool bf16, unsigned long long timeout_ns, cudaStream_t st) {
+                           unsigned long long timeout_ns, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     // every operand must fit its slot
     const int big = max_m > max_n ? max_m : max_n;
-    if (oz_slice_bytes(big, max_k, bf16, 6) > scr.slot_bytes || oz_exp_ints(big) > scr.exp_ints)
+    if (oz_slice_bytes(big, max_k, 6) > scr.slot_bytes || oz_exp_ints(big) > scr.exp_ints)
         return cudaErrorInvalidValue;
-    gemm_desc_oz_kernel<<<(count + 127) / 128, 128, 0, st>>>(d_desc, count, scr, bf16 ? 1 : 0);
+    gemm_desc_oz_kernel<<<(count + 127) / 128, 128, 0, st>>>(d_desc, count, scr);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_oz_gemm(scr.probs, count, max_m, max_n, big, bf16, 6, timeout_ns, st);
+    return launch_oz_gemm(scr.probs, count, max_m, max_n, big, 6, timeout_ns, st);
 }
 
 }  // namespace mpdo
@@ -902,7 +881,50 @@ cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max
 // ---------------------------------------------------------------------------
 // mpdo_gemm_tc: the same product on caller matrices (include/mpdo.h)
 // ---------------------------------------------------------------------------
+#include <mutex>
 #include <string>
+
+namespace mpdo {
+namespace {
+
+// The scratch of mpdo_gemm_tc comes from a pool of its own per device, which keeps
+// up to 256 MB between calls (the slices of a 4096 x 4096 x 2048 product) and
+// returns the rest when a call's stream is synchronised; the driver also takes
+// it back when another allocation runs out.  Allocation is in stream order, so calls
+// on several streams and threads do not share a buffer.
+constexpr unsigned long long kGemmPoolKeep = 256ull << 20;
+constexpr int kMaxPools = 64;
+
+cudaError_t gemm_pool(cudaMemPool_t* out) {
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxPools] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxPools) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+        if ((e = oz_prepare()) != cudaSuccess) return e;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+        unsigned long long keep = kGemmPoolKeep;
+        if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+            cudaMemPoolDestroy(p);
+            return e;
+        }
+        pools[dev] = p;
+    }
+    *out = pools[dev];
+    return cudaSuccess;
+}
+
+}  // namespace
+}  // namespace mpdo
 
 extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,
                             int ldc, int kind, void* cuda_stream) {
@@ -915,7 +937,6 @@ extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const
         set_last_error("mpdo_gemm_tc: kind must be MPDO_MIXED_TF32 or MPDO_MIXED_BF16X3");
         return MPDO_EINVAL;
     }
-    const bool bf16 = kind == MPDO_MIXED_BF16X3;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     OzProblem P{};
     P.M = M;
@@ -926,13 +947,16 @@ extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const
     P.C = C;
     P.ldc = ldc;
     P.alpha = 1.0;
-    oz_tiles(P, bf16);
-    const size_t sa = oz_slice_bytes(M, K, bf16, 6), sb = oz_slice_bytes(N, K, bf16, 6);
-    unsigned char* buf = nullptr;
+    oz_set_tiles(P);
+    const size_t sa = oz_slice_bytes(M, K, 6), sb = oz_slice_bytes(N, K, 6);
     const size_t ia = oz_exp_ints(M), ib = oz_exp_ints(N);
-    const size_t bytes = sa + sb + sizeof(int) * (ia + ib) + sizeof(OzProblem) + 256;
-    cudaError_t e = cudaMalloc((void**)&buf, bytes);
+    const size_t bytes = sa + sb + sizeof(int) * (ia + ib);
+    unsigned char* buf = nullptr;
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = gemm_pool(&pool);
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&buf, bytes, pool, st);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         set_last_error(std::string("mpdo_gemm_tc: ") + cudaGetErrorString(e));
         return MPDO_ENOMEM;
     }
@@ -940,13 +964,12 @@ extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const
     P.bs = buf + sa;
     P.ea = reinterpret_cast<int*>(buf + sa + sb);
     P.eb = P.ea + ia;
-    OzProblem* d_p = reinterpret_cast<OzProblem*>(
-        (reinterpret_cast<uintptr_t>(P.eb + ib) + 255) & ~static_cast<uintptr_t>(255));
-    e = oz_prepare();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_p, &P, sizeof(P), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_oz_gemm(d_p, 1, M, N, M > N ? M : N, bf16, 6, 4000000000ull, st);
+    OzSource src{};
+    src.one = P;
+    e = launch_oz_source(src, 1, M, N, M > N ? M : N, 6, 4000000000ull, st);
+    const cudaError_t ef = cudaFreeAsync(buf, st);
+    if (e == cudaSuccess) e = ef;
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(buf);
     if (e != cudaSuccess) {
         set_last_error(std::string("mpdo_gemm_tc: ") + cudaGetErrorString(e));
         return MPDO_ECUDA;

@@ -288,8 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) qrb_panel_kernel(const OpDesc* de
 
 // The two products of the trailing update of panel k0, built per op:
 // which = 0: Wt = A_t^T V^T (n' x jb); which = 1: A_t^T <- A_t^T - W2t V.
-__global__ void qrb_prep_kernel(const OpDesc* descs, int nops, int k0, int nb, int which, OzProblem* out, int ld,
-                                int bf16) {
+__global__ void qrb_prep_kernel(const OpDesc* descs, int nops, int k0, int nb, int which, OzProblem* out, int ld) {
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= nops) return;
     const OpDesc& d = descs[o];
@@ -328,7 +327,7 @@ __global__ void qrb_prep_kernel(const OpDesc* descs, int nops, int k0, int nb, i
     P.ea = d.oz_ea;
     P.eb = d.oz_eb;
     P.status = d.status;
-    oz_set_tiles(P, bf16 != 0);
+    oz_set_tiles(P);
     out[o] = P;
 }
 
@@ -408,7 +407,7 @@ int qrb_kernels(int chi_cap, int r_max) {
     return 2 + ((r_max + nb - 1) / nb) * 9;
 }
 
-cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs, bool bf16,
+cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs,
                               unsigned long long timeout_ns, cudaStream_t st, int r_max) {
     if (nops <= 0) return cudaSuccess;
     const int ld = 4 * chi_cap, nb = qrb_panel_width(chi_cap);
@@ -419,14 +418,14 @@ cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzPro
     for (int k0 = 0; k0 < r_max && e == cudaSuccess; k0 += nb) {
         qrb_panel_kernel<<<nops, kThreads, smem, st>>>(d_desc, k0, nb, ld);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        qrb_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, k0, nb, 0, probs, ld, bf16 ? 1 : 0);
+        qrb_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, k0, nb, 0, probs, ld);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        if ((e = launch_oz_gemm(probs, nops, ld, nb, ld, bf16, 6, timeout_ns, st)) != cudaSuccess) break;
+        if ((e = launch_oz_gemm(probs, nops, ld, nb, ld, 6, timeout_ns, st)) != cudaSuccess) break;
         qrb_wt_kernel<<<dim3((ld * kMaxNb + 255) / 256, nops), 256, 0, st>>>(d_desc, k0, nb, ld);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        qrb_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, k0, nb, 1, probs, ld, bf16 ? 1 : 0);
+        qrb_prep_kernel<<<(nops + 127) / 128, 128, 0, st>>>(d_desc, nops, k0, nb, 1, probs, ld);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        if ((e = launch_oz_gemm(probs, nops, ld, ld, ld, bf16, 6, timeout_ns, st)) != cudaSuccess) break;
+        if ((e = launch_oz_gemm(probs, nops, ld, ld, ld, 6, timeout_ns, st)) != cudaSuccess) break;
         qrb_norms_kernel<<<dim3((ld + 63) / 64, nops), 256, 0, st>>>(d_desc, k0, nb, ld);
         e = cudaGetLastError();
     }

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
 
 }  // namespace
 
-cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, bool bf16, int S, double tol_in,
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, double tol_in,
                           bool can_finish, unsigned long long timeout_ns, cudaStream_t st) {
     if (nops <= 0) return cudaSuccess;
     const int ld = 4 * chi_cap;
@@ -185,14 +185,14 @@ cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, bool bf16
     // level of 6 slices' products otherwise; the largest single angle follows
     const float defect = S == 7 ? 1e-17f : 1e-13f, tcap = S == 7 ? 2e-3f : 1e-2f;
     for (int it = 0; it < kRefineIters; ++it) {
-        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, chi_cap, bf16, S, timeout_ns, st);
+        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, chi_cap, S, timeout_ns, st);
         if (e != cudaSuccess) return e;
         refine_diag_kernel<<<nops, NT, 0, st>>>(d_desc, ld);
         refine_x_kernel<<<dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st>>>(
             d_desc, ld, tol_in, tcap, can_finish ? 1 : 0, defect, it == kRefineIters - 1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         for (int kind : {OZ_R3, OZ_R2, OZ_R1})
-            if ((e = launch_oz_ops(d_desc, nops, kind, chi_cap, bf16, S, timeout_ns, st)) != cudaSuccess) return e;
+            if ((e = launch_oz_ops(d_desc, nops, kind, chi_cap, S, timeout_ns, st)) != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }
