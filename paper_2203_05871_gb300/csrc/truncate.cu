@@ -4,11 +4,12 @@
 // row order.  k_cut = smallest k >= 1 whose discarded weight
 // sum_{i>=k} s_i^2 is <= cutoff * sum_i s_i^2 (the tail is summed from the
 // smallest value up); k = min(chi_max, k_cut).  Writes lambda_p = s[:k],
-// Yk[j] = v_j^T (rows of W normalised, or rows of Z), the new site p+1
+// Yk[j] = v_j^T (rows of W normalised), the new site p+1
 // B'[j][s2][r] = Yk[j][s2*cr + r] and the new bond dimension.  A forced rank
 // (replay of a recorded run) replaces k_cut, still capped by chi_max and c.
 // When the adjoint records a tape, all c sorted singular values and
 // normalised rows are written as well.
+#include <cooperative_groups.h>
 #include <mpdo.h>
 
 #include "internal.h"
@@ -17,8 +18,7 @@ namespace mpdo {
 
 namespace {
 
-constexpr int TT = 1024;
-constexpr int kMaxRows = 4 * kMaxChi;
+constexpr int TT = 512;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -26,16 +26,28 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__global__ void __launch_bounds__(TT) truncate_kernel(const OpDesc* descs, int chi_cap) {
-    const OpDesc& d = descs[blockIdx.x];
+// A cluster of 8 CTAs per op: the rows' norms, the normalised rows and the new site
+// are an eighth each (one CTA read and wrote 16 MB through one SM at chi = 256,
+// 1.3 ms); every CTA ranks all norms and sums the tails itself.
+constexpr int TC = 8;
+__global__ void __cluster_dims__(TC, 1, 1) __launch_bounds__(TT, 1) truncate_kernel(const OpDesc* descs, int chi_cap) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const OpDesc& d = descs[blockIdx.x / TC];
     const int c = d.c, L = d.L, ld = 4 * chi_cap;
-    __shared__ double s[kMaxRows];
-    __shared__ int perm[kMaxRows];
+    extern __shared__ double smem[];
+    double* s = smem;                        // [c] norms
+    double* tail = smem + ld;                // [c + 1] sum_{i >= k} s_perm(i)^2; first the sorted norms
+    int* perm = reinterpret_cast<int*>(smem + 2 * ld + 1);
     __shared__ int s_k, s_bad;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) s_bad = 0;
-    __syncthreads();
-    for (int j = warp; j < c; j += TT / 32) {
+    if (threadIdx.x == 0) {
+        s_bad = 0;
+        s_k = c;
+    }
+    cluster.sync();   // every CTA runs before its shared memory is written
+    for (int j = rank + TC * warp; j < c; j += TC * (TT / 32)) {
         const double* w = d.W + (size_t)j * ld;
         double a = 0.0;
         for (int i = lane; i < L; i += 32) {
@@ -43,12 +55,12 @@ __global__ void __launch_bounds__(TT) truncate_kernel(const OpDesc* descs, int c
             a = fma(x, x, a);
         }
         a = warp_sum(a);
-        if (lane == 0) {
-            const double v = sqrt(a);
-            if (!isfinite(v)) s_bad = 1;
-            s[j] = v;
-        }
+        const double v = sqrt(a);
+        if (lane < TC) cluster.map_shared_rank(s, lane)[j] = v;
     }
+    cluster.sync();
+    for (int j = threadIdx.x; j < c; j += TT)
+        if (!isfinite(s[j])) s_bad = 1;
     __syncthreads();
     const int bad = s_bad;
     for (int j = threadIdx.x; j < c; j += TT) {
@@ -63,59 +75,43 @@ __global__ void __launch_bounds__(TT) truncate_kernel(const OpDesc* descs, int c
             r += (si > sj) || (si == sj && i < j);
         }
         perm[r] = j;
+        tail[r] = sj;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int k = 1;
-        double disc = 0.0;
-        if (!bad) {
-            // tail[k] = sum_{i>=k} s_perm(i)^2, accumulated from the smallest
-            double tail = 0.0;
-            double total = 0.0;
-            for (int i = c - 1; i >= 0; --i) {
-                const double v = s[perm[i]];
-                total += v * v;
-            }
-            // find the smallest k with tail(k) <= cutoff*total by walking up from the end
-            // (tail(k) is non-increasing in k, so scan k = c, c-1, ... while it holds)
-            const double thr = d.cutoff * total;
-            int kcut = c;
-            tail = 0.0;
-            for (int kk = c; kk >= 1; --kk) {
-                // tail currently = sum_{i>=kk} w_i
-                if (tail <= thr)
-                    kcut = kk;
-                else
-                    break;
-                const double v = s[perm[kk - 1]];
-                tail += v * v;
-            }
-            k = kcut;
-            if (k > d.chi_max) k = d.chi_max;
-            if (d.forced_k > 0) k = d.forced_k < d.chi_max ? d.forced_k : d.chi_max;
-            if (k > c) k = c;
-            if (k < 1) k = 1;
-            double dsum = 0.0;
-            for (int i = c - 1; i >= k; --i) {
-                const double v = s[perm[i]];
-                dsum += v * v;
-            }
-            disc = total > 0.0 ? dsum / total : 0.0;
-        } else {
-            atomicOr(d.status, (int)MPDO_ST_NONFINITE);
+    if (threadIdx.x == 0 && !bad) {
+        // the tails, accumulated from the smallest value up
+        double t = 0.0;
+        tail[c] = 0.0;
+        for (int i = c - 1; i >= 0; --i) {
+            const double v = tail[i];
+            t = fma(v, v, t);
+            tail[i] = t;
         }
-        s_k = k;
+    }
+    __syncthreads();
+    // the smallest k >= 1 whose tail is within the cutoff (the tails do not increase with k)
+    if (!bad)
+        for (int k = 1 + threadIdx.x; k < c; k += TT)
+            if (tail[k] <= d.cutoff * tail[0]) atomicMin(&s_k, k);
+    __syncthreads();
+    int k = s_k;
+    if (k > d.chi_max) k = d.chi_max;
+    if (d.forced_k > 0) k = d.forced_k < d.chi_max ? d.forced_k : d.chi_max;
+    if (k > c) k = c;
+    if (k < 1 || bad) k = 1;
+    if (rank == 0 && threadIdx.x == 0) {
+        if (bad) atomicOr(d.status, (int)MPDO_ST_NONFINITE);
         *d.k_out = k;
         if (d.rank_log) *d.rank_log = k;
+        const double disc = !bad && tail[0] > 0.0 ? tail[k] / tail[0] : 0.0;
         atomicMax((unsigned long long*)d.max_disc, (unsigned long long)__double_as_longlong(disc));
     }
-    __syncthreads();
-    const int k = s_k;
-    for (int j = threadIdx.x; j < k; j += TT) d.lam_out[j] = bad ? 0.0 : s[perm[j]];
+    const int t0 = rank * TT + threadIdx.x, w0 = rank + TC * warp;
+    for (int j = t0; j < k; j += TC * TT) d.lam_out[j] = bad ? 0.0 : s[perm[j]];
     if (d.tape_V) {
         // every sorted right singular vector (zero rows stay zero) for the adjoint
-        for (int j = threadIdx.x; j < c; j += TT) d.tape_s[j] = bad ? 0.0 : s[perm[j]];
-        for (int j = warp; j < c; j += TT / 32) {
+        for (int j = t0; j < c; j += TC * TT) d.tape_s[j] = bad ? 0.0 : s[perm[j]];
+        for (int j = w0; j < c; j += TC * (TT / 32)) {
             const int src = perm[j];
             const double sv = s[src];
             const double inv = (sv > 0.0 && !bad) ? 1.0 / sv : 0.0;
@@ -124,36 +120,32 @@ __global__ void __launch_bounds__(TT) truncate_kernel(const OpDesc* descs, int c
             for (int i = lane; i < d.n; i += 32) v[i] = wr[i] * inv;
         }
     }
-    const int n = d.n, cr = d.cr;
-    for (int j = warp; j < k; j += TT / 32) {
+    const int cr = d.cr;
+    for (int j = w0; j < k; j += TC * (TT / 32)) {
         const int src = perm[j];
         double* y = d.Yk + (size_t)j * ld;
         const size_t bnew = (size_t)j * 4 * chi_cap;   // row j of the new site p+1
-        if (d.transposed) {
-            const double* zr = d.Z + (size_t)src * ld;
-            for (int i = lane; i < n; i += 32) {
-                const double v = zr[i];
-                y[i] = v;
-                site_st(d.B, bnew + (i / cr) * chi_cap + (i % cr), v, d.site_f32);
-            }
-        } else {
-            const double* wr = d.W + (size_t)src * ld;
-            const double sv = s[src];
-            const double inv = (sv > 0.0 && !bad) ? 1.0 / sv : 0.0;
-            for (int i = lane; i < n; i += 32) {
+        const double* wr = d.W + (size_t)src * ld;
+        const double sv = s[src];
+        const double inv = (sv > 0.0 && !bad) ? 1.0 / sv : 0.0;
+        for (int s2 = 0; s2 < 4; ++s2)
+            for (int r = lane; r < cr; r += 32) {
+                const int i = s2 * cr + r;
                 const double v = wr[i] * inv;
                 y[i] = v;
-                site_st(d.B, bnew + (i / cr) * chi_cap + (i % cr), v, d.site_f32);
+                site_st(d.B, bnew + (size_t)s2 * chi_cap + r, v, d.site_f32);
             }
-        }
     }
 }
+
+static_assert((2 * 4 * kMaxChi + 1) * 8 + 4 * kMaxChi * 4 <= 48 * 1024, "within the default shared memory");
 
 }  // namespace
 
 cudaError_t launch_truncate(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st) {
     if (nops <= 0) return cudaSuccess;
-    truncate_kernel<<<nops, TT, 0, st>>>(d_desc, chi_cap);
+    const size_t ld = 4 * (size_t)chi_cap;
+    truncate_kernel<<<TC * nops, TT, (2 * ld + 1) * sizeof(double) + ld * sizeof(int), st>>>(d_desc, chi_cap);
     return cudaGetLastError();
 }
 
