@@ -229,6 +229,25 @@ int chunk_ops(mpdo_ctx* c) {
     return std::max(1, std::min(c->slots, std::max(16, c->jacobi_resident / 4)));
 }
 
+// slot s's buffers of the SVD stages
+void svd_buffers(mpdo_ctx* c, int s, OpDesc& d) {
+    const int ld = c->ld;
+    const size_t mat = (size_t)ld * ld;
+    d.W = c->d_W + (size_t)s * mat;
+    d.pre_ok = c->precond ? c->d_pre_ok + s : nullptr;
+    d.rf = refine_on(c) ? c->d_refine + s : nullptr;
+    d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
+    d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
+    d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
+    d.D32 = c->precond ? c->d_D32 + (size_t)s * jacobi32_diag_floats(ld) : nullptr;
+    d.E = c->precond ? c->d_E + (size_t)s * mat : nullptr;
+    d.Q = c->precond ? c->d_Q + (size_t)s * mat : nullptr;
+    d.oz_as = c->precond ? c->d_oz_as + (size_t)s * c->oz_slot_bytes : nullptr;
+    d.oz_bs = c->precond ? c->d_oz_bs + (size_t)s * c->oz_slot_bytes : nullptr;
+    d.oz_ea = c->precond ? c->d_oz_ea + (size_t)s * oz_exp_ints(ld) : nullptr;
+    d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
+}
+
 void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     const int N = c->N, cap = c->cap, ld = c->ld;
     const size_t mat = (size_t)ld * ld;
@@ -256,7 +275,6 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.lam_left = p > 0 ? c->d_lam + ((size_t)b * N + (p - 1)) * cap : nullptr;
     d.lam_out = c->d_lam + ((size_t)b * N + p) * cap;
     d.thetap = c->d_thetap + (size_t)s * mat;
-    d.W = c->d_W + (size_t)s * mat;
     d.Z = nullptr;
     d.Acm = c->d_Z + (size_t)s * mat;
     d.Yk = c->d_Yk + (size_t)s * cap * ld;
@@ -267,23 +285,12 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.rank_log = nullptr;
     d.jb = tuned_block_rows(c, d.cl, d.cr, jacobi_block_rows(d.L, d.c, 8));
     d.sweeps_out = c->d_sweeps + s;
-    d.pre_ok = c->precond ? c->d_pre_ok + s : nullptr;
-    d.rf = refine_on(c) ? c->d_refine + s : nullptr;
     d.forced_k = 0;
     d.full_svd = c->full_svd ? 1 : 0;
     d.tape_V = nullptr;
     d.tape_s = nullptr;
-    d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
-    d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
-    d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
-    d.D32 = c->precond ? c->d_D32 + (size_t)s * jacobi32_diag_floats(ld) : nullptr;
-    d.E = c->precond ? c->d_E + (size_t)s * mat : nullptr;
-    d.Q = c->precond ? c->d_Q + (size_t)s * mat : nullptr;
+    svd_buffers(c, s, d);
     d.Zinit = nullptr;
-    d.oz_as = c->precond ? c->d_oz_as + (size_t)s * c->oz_slot_bytes : nullptr;
-    d.oz_bs = c->precond ? c->d_oz_bs + (size_t)s * c->oz_slot_bytes : nullptr;
-    d.oz_ea = c->precond ? c->d_oz_ea + (size_t)s * oz_exp_ints(ld) : nullptr;
-    d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
 }
 
 cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st) {
@@ -292,7 +299,7 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
     // (Q = U - E U / 2, defect 3 E^2 / 4) on the mixed path, third order (defect
     // 5 E^3 / 8, below FP64 rounding) on the FP64 path
     std::vector<int> kinds = {OZ_E, OZ_Q, OZ_W};
-    if (!c->mixed) kinds = {OZ_E, OZ_T, OZ_Q3, OZ_W};
+    if (!c->mixed) kinds = {OZ_E, OZ_T4, OZ_T3, OZ_T2, OZ_W};
     for (int kind : kinds) {
         const cudaError_t e =
             launch_oz_ops(d_desc, nops, first + kind, c->cap, c->oz_s, timeout_ns, st);
@@ -301,15 +308,14 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
     return cudaSuccess;
 }
 
-int orthogonalise_kernels(const mpdo_ctx* c) { return (c->mixed ? 3 : 4) * kOzKernels; }
+int orthogonalise_kernels(const mpdo_ctx* c) { return (c->mixed ? 3 : 5) * kOzKernels; }
 
-cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st) {
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     const cudaError_t e = launch_orthogonalise(c, d_desc, nops, 0, st);
     if (e != cudaSuccess) return e;
     if (!refine_on(c)) return cudaSuccess;
     // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
-    const double tol = fp64_jacobi_tol(c);
     const bool can = c->oz_s == 7 || tol >= 1e-12;
     return launch_refine(d_desc, nops, c->cap, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
 }
@@ -318,75 +324,17 @@ int svd_products_kernels(const mpdo_ctx* c) {
     return orthogonalise_kernels(c) + (refine_on(c) ? kRefineKernels : 0);
 }
 
-int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* forced, const TapeSlot* tape,
-              bool log_ranks) {
-    const int nops = (int)items.size();
-    const int N = c->N, cap = c->cap, ld = c->ld;
-    std::vector<double> work(nops), qwork(nops);
-    for (int s = 0; s < nops; ++s) {
-        const Item& it = items[s];
-        OpDesc& d = c->h_desc[s];
-        fill_desc(c, it, s, d);
-        int fk = forced ? forced[s] : 0;
-        if (!forced && step < c->forced_steps)
-            fk = c->forced[((size_t)d.b * c->forced_steps + step) * c->n_ops + d.op];
-        d.forced_k = fk;
-        d.tape_V = tape ? tape[s].V : nullptr;
-        if (tape) d.full_svd = 1;
-        d.tape_s = tape ? tape[s].s : nullptr;
-        work[s] = (double)d.c * d.c * (double)d.L;
-        qwork[s] = (double)d.m * d.n * d.c;
-    }
-    CU(cudaMemcpyAsync(c->d_desc, c->h_desc, sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
-    if (tape) {
-        // inputs of every op (sites p, p+1, lambda_{p-1}) before the merge
-        // overwrites them, and Theta' after it
-        Copy2D* hc = c->h_copy;
-        int nc = 0, max_rows = 1;
-        for (int s = 0; s < nops; ++s) {
-            const OpDesc& d = c->h_desc[s];
-            // (the gradient runs on FP64 site storage only)
-            hc[nc++] = Copy2D{static_cast<const double*>(d.A), tape[s].A, 4 * d.cl, d.cm, cap, d.cm, 1.0};
-            hc[nc++] = Copy2D{static_cast<const double*>(d.B), tape[s].B, 4 * d.cm, d.cr, cap, d.cr, 1.0};
-            if (d.lam_left) hc[nc++] = Copy2D{d.lam_left, tape[s].lam, 1, d.cl, cap, d.cl, 1.0};
-            max_rows = std::max(max_rows, 4 * std::max(d.cl, d.cm));
-        }
-        for (int s = 0; s < nops; ++s) {
-            const OpDesc& d = c->h_desc[s];
-            hc[nc + s] = Copy2D{d.thetap, tape[s].thetap, d.m, d.n, ld, d.n, 1.0};
-        }
-        CU(cudaMemcpyAsync(c->d_copy, hc, sizeof(Copy2D) * (nc + nops), cudaMemcpyHostToDevice, c->st));
-        CU(launch_copy2d(c->d_copy, nc, max_rows, c->st));
-    }
-    double fl_merge = 0.0, fl_svd = 0.0;
+// The SVDs of the nops ops whose descriptors are in h_desc and d_desc: theta~ (Acm)
+// to rows W, orthogonal to tol (0: sqrt(L) eps).
+int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
+    const int cap = c->cap, ld = c->ld;
+    const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
+    std::vector<double> qwork(nops);
     for (int s = 0; s < nops; ++s) {
         const OpDesc& d = c->h_desc[s];
-        fl_merge += 32.0 * d.cl * d.cm * d.cr + 512.0 * d.cl * d.cr;
-        const double nn = 4.0 * std::max(d.cl, d.cr);
-        fl_svd += 21.0 * nn * nn * nn;
+        qwork[s] = (double)d.m * d.n * d.c;
     }
-    const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
-    ProfScope p_merge(c, K_MERGE);
-    if (c->mixed) {
-        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, c->st));
-        CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
-    } else {
-        CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
-    }
-    p_merge.stop();
-    if (tape) {
-        int nc = 0, max_rows = 1;
-        for (int s = 0; s < nops; ++s) {
-            const OpDesc& d = c->h_desc[s];
-            nc += 2 + (d.lam_left ? 1 : 0);
-            max_rows = std::max(max_rows, d.m);
-        }
-        CU(launch_copy2d(c->d_copy + nc, nops, max_rows, c->st));
-    }
-
     const int gcap = std::max(std::max(c->jacobi_resident, c->qr_resident), c->slots);
-    double qr_flops_chunk = 0.0;
-    int qr_kernels_chunk = 1;
     // Jacobi launch plan: share the co-resident CTAs among the ops in
     // proportion to their work; h_cta/d_cta hold [op of each CTA | rank | CTAs per op]
     auto plan = [&](bool fp32, int* hbase, int& total) -> int {
@@ -401,7 +349,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         CU(cudaMemcpyAsync(dbase, hbase, sizeof(int) * (2 * total + nops), cudaMemcpyHostToDevice, c->st));
         CU(cudaMemsetAsync(c->d_sync, 0, sizeof(unsigned) * jacobi_sync_words(nops), c->st));
         CU(launch_jacobi(c->d_desc, nops, dbase, dbase + total, dbase + 2 * total, c->d_sync, total,
-                         fp32 ? kMaxSweepsCap / 2 : c->cfg.jacobi_max_sweeps, fp32 ? 0.0 : fp64_jacobi_tol(c),
+                         fp32 ? kMaxSweepsCap / 2 : c->cfg.jacobi_max_sweeps, fp32 ? 0.0 : tol,
                          timeout_ns, ld, fp32, c->st, precond_rho(c)));
         return MPDO_OK;
     };
@@ -464,7 +412,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
             const OpDesc& d = c->h_desc[s];
             fl_qr += 4.0 * d.m * d.n * d.c - 2.0 * (d.m + d.n) * d.c * d.c + 4.0 / 3.0 * d.c * d.c * d.c;
         }
-        qr_flops_chunk = fl_qr;
+        out.qr_flops = fl_qr;
         if (blocked) {
             // mixed path: blocked QR, trailing updates on the tensor cores
             int r_max = 1;
@@ -472,24 +420,23 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
             ProfScope p_qr(c, K_QR);
             CU(launch_qr_blocked(c->d_desc, nops, cap, c->d_oz, timeout_ns, c->st, r_max));
             p_qr.stop();
-            qr_kernels_chunk = qrb_kernels(cap, r_max);
+            out.qr_kernels = qrb_kernels(cap, r_max);
         } else {
             ProfScope p_qr(c, K_QR);
             int total = 0, *db = nullptr;
             int rc = plan_qr(false, 2, total, db);
             if (rc) return rc;
-            qr_kernels_chunk = total > 0;
+            out.qr_kernels = total > 0;
             CU(launch_qr(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
             if ((rc = plan_qr(true, 3, total, db))) return rc;
             if (total > 0) {
                 CU(launch_qr32(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
                 CU(launch_orthogonalise(c, c->d_desc, nops, OZ_FIRST, c->st));
-                qr_kernels_chunk += 1 + orthogonalise_kernels(c);
+                out.qr_kernels += 1 + orthogonalise_kernels(c);
             }
             p_qr.stop();
         }
     }
-    double fl_gemm = 0.0;
     if (c->precond) {
         // FP32 preconditioning Jacobi on (W32 | U32)
         ProfScope p_j32(c, K_JACOBI32);
@@ -499,10 +446,10 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         // Q from U32, W = Q W0 and the rows' refinement: FP64-accurate tensor-core products
         for (int s = 0; s < nops; ++s) {
             const OpDesc& d = c->h_desc[s];
-            fl_gemm += 2.0 * d.c * d.c * d.c * 2 + 2.0 * d.c * d.c * d.L;
+            out.gemm_flops += 2.0 * d.c * d.c * d.c * 2 + 2.0 * d.c * d.c * d.L;
         }
         ProfScope p_gemm(c, K_GEMM);
-        CU(launch_svd_products(c, c->d_desc, nops, c->st));
+        CU(launch_svd_products(c, c->d_desc, nops, tol, c->st));
         p_gemm.stop();
     }
     ProfScope p_jac(c, K_JACOBI);
@@ -511,11 +458,80 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         if (rc) return rc;
     }
     p_jac.stop();
+    return MPDO_OK;
+}
+
+int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* forced, const TapeSlot* tape,
+              bool log_ranks) {
+    const int nops = (int)items.size();
+    const int N = c->N, cap = c->cap, ld = c->ld;
+    for (int s = 0; s < nops; ++s) {
+        const Item& it = items[s];
+        OpDesc& d = c->h_desc[s];
+        fill_desc(c, it, s, d);
+        int fk = forced ? forced[s] : 0;
+        if (!forced && step < c->forced_steps)
+            fk = c->forced[((size_t)d.b * c->forced_steps + step) * c->n_ops + d.op];
+        d.forced_k = fk;
+        d.tape_V = tape ? tape[s].V : nullptr;
+        if (tape) d.full_svd = 1;
+        d.tape_s = tape ? tape[s].s : nullptr;
+    }
+    CU(cudaMemcpyAsync(c->d_desc, c->h_desc, sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
+    if (tape) {
+        // inputs of every op (sites p, p+1, lambda_{p-1}) before the merge
+        // overwrites them, and Theta' after it
+        Copy2D* hc = c->h_copy;
+        int nc = 0, max_rows = 1;
+        for (int s = 0; s < nops; ++s) {
+            const OpDesc& d = c->h_desc[s];
+            // (the gradient runs on FP64 site storage only)
+            hc[nc++] = Copy2D{static_cast<const double*>(d.A), tape[s].A, 4 * d.cl, d.cm, cap, d.cm, 1.0};
+            hc[nc++] = Copy2D{static_cast<const double*>(d.B), tape[s].B, 4 * d.cm, d.cr, cap, d.cr, 1.0};
+            if (d.lam_left) hc[nc++] = Copy2D{d.lam_left, tape[s].lam, 1, d.cl, cap, d.cl, 1.0};
+            max_rows = std::max(max_rows, 4 * std::max(d.cl, d.cm));
+        }
+        for (int s = 0; s < nops; ++s) {
+            const OpDesc& d = c->h_desc[s];
+            hc[nc + s] = Copy2D{d.thetap, tape[s].thetap, d.m, d.n, ld, d.n, 1.0};
+        }
+        CU(cudaMemcpyAsync(c->d_copy, hc, sizeof(Copy2D) * (nc + nops), cudaMemcpyHostToDevice, c->st));
+        CU(launch_copy2d(c->d_copy, nc, max_rows, c->st));
+    }
+    double fl_merge = 0.0, fl_svd = 0.0;
+    for (int s = 0; s < nops; ++s) {
+        const OpDesc& d = c->h_desc[s];
+        fl_merge += 32.0 * d.cl * d.cm * d.cr + 512.0 * d.cl * d.cr;
+        const double nn = 4.0 * std::max(d.cl, d.cr);
+        fl_svd += 21.0 * nn * nn * nn;
+    }
+    const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
+    ProfScope p_merge(c, K_MERGE);
+    if (c->precond) {
+        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, c->st));
+        CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
+    } else {
+        CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
+    }
+    p_merge.stop();
+    if (tape) {
+        int nc = 0, max_rows = 1;
+        for (int s = 0; s < nops; ++s) {
+            const OpDesc& d = c->h_desc[s];
+            nc += 2 + (d.lam_left ? 1 : 0);
+            max_rows = std::max(max_rows, d.m);
+        }
+        CU(launch_copy2d(c->d_copy + nc, nops, max_rows, c->st));
+    }
+
+    SvdWork svd;
+    int rc = run_svd(c, nops, fp64_jacobi_tol(c), svd);
+    if (rc) return rc;
     ProfScope p_tr(c, K_TRUNC);
     CU(launch_truncate(c->d_desc, nops, cap, c->st));
     p_tr.stop();
     ProfScope p_rec(c, K_RECON);
-    if (c->mixed)
+    if (c->precond)
         CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_s, timeout_ns, c->st));
     else
         CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
@@ -545,15 +561,15 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     }
     // kernels per stage: a tensor-core product is two (slicing, slice
     // products), the merge adds the gate/weight kernel
-    prof_collect(c, K_MERGE, fl_merge, c->mixed ? kOzKernels + 1 : 1);
-    prof_collect(c, K_QR, qr_flops_chunk, qr_kernels_chunk);
+    prof_collect(c, K_MERGE, fl_merge, c->precond ? kOzKernels + 1 : 1);
+    prof_collect(c, K_QR, svd.qr_flops, svd.qr_kernels);
     prof_collect(c, K_JACOBI, fl_svd, 1);
     if (c->precond) {
         prof_collect(c, K_JACOBI32, 0.0, 1);
-        prof_collect(c, K_GEMM, fl_gemm, svd_products_kernels(c));
+        prof_collect(c, K_GEMM, svd.gemm_flops, svd_products_kernels(c));
     }
     prof_collect(c, K_TRUNC, 0.0, 1);
-    prof_collect(c, K_RECON, fl_rec, c->mixed ? kOzKernels : 1);
+    prof_collect(c, K_RECON, fl_rec, c->precond ? kOzKernels : 1);
     for (int s = 0; s < nops && log_ranks; ++s) {
         const Item& it = items[s];
         const Op& op = c->layers[it.layer][it.idx];

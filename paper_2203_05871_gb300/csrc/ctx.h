@@ -193,6 +193,7 @@ int chunk_ops(mpdo_ctx* c);
 
 // Descriptor of item `it` in workspace slot s, with the bond dimensions of
 // c->h_dims (forced rank and tape cleared).
+void svd_buffers(mpdo_ctx* c, int s, OpDesc& d);   // slot s's buffers of the SVD stages
 void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d);
 
 // One chunk of (instance, op) items of a layer: merge + gate, QR, Jacobi SVD,
@@ -224,7 +225,13 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
 int orthogonalise_kernels(const mpdo_ctx* c);
 // The stages between the FP32 preconditioning pass and the FP64 Jacobi pass:
 // Q, the orthogonalised U32, W = Q W0, and the refinement of W's rows.
-cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, cudaStream_t st);
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, cudaStream_t st);
+// A chunk's SVDs, with the work of the stages whose flop counts depend on the route.
+struct SvdWork {
+    double qr_flops = 0.0, gemm_flops = 0.0;
+    int qr_kernels = 1;
+};
+int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out);
 // kernels one launch_svd_products issues
 int svd_products_kernels(const mpdo_ctx* c);
 

@@ -37,7 +37,7 @@ namespace mpdo {
 
 namespace {
 
-// X and Y of instance i of a chunk: W slots 2i and 2i+1; [0][0] = 1
+// X and Y of instance i of a chunk: slots 2i and 2i+1; [0][0] = 1
 __global__ void gram_unit_kernel(double* W, size_t mat, int m) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 2 * m) return;
@@ -59,13 +59,14 @@ __global__ void row_norms_kernel(const double* W, size_t mat, int ld, const int*
     }
 }
 
-// C_i[j][k] /= sqrt(|x_j| |y_k|) (0 where either norm is 0): C = F_X F_Y^T
-__global__ void scale_kernel(double* C, size_t mat, int ld, const int* chi, const double* norms) {
-    const int i = blockIdx.y;
-    const int n = chi[2 * i];
-    const double* nx = norms + (size_t)(2 * i) * 2 * ld;
-    const double* ny = norms + (size_t)(2 * i + 1) * 2 * ld;
-    double* M = C + (size_t)(2 * i) * mat;
+// slot s of C: [j][k] /= sqrt(|x_j| |y_k|) (0 where either norm is 0), x the rows of slot
+// s and y those of its partner: F_X F_Y^T (even slots) or its transpose (odd ones)
+__global__ void scale_kernel(double* C, size_t mat, int ld, const int* chi, const double* norms, int step) {
+    const int s = blockIdx.y * step;
+    const int n = chi[s];
+    const double* nx = norms + (size_t)s * 2 * ld;
+    const double* ny = norms + (size_t)(s ^ 1) * 2 * ld;
+    double* M = C + (size_t)s * mat;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * n; e += gridDim.x * blockDim.x) {
         const int j = e / n, k = e % n;
         const double d = nx[j] * ny[k];
@@ -153,7 +154,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
             const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
-            double* X = c->d_W + (size_t)(2 * i) * mat;
+            double* X = c->d_Z + (size_t)(2 * i) * mat;
             double* T = c->d_thetap + (size_t)(2 * i) * mat;
             // T[l][(s, r)] = sum_l' X[l][l'] B[l'][s][r]
             P.add(GemmDesc{l, 3 * cap + r, l, X, ld, 0, site_v(c, b, q), 4 * cap, f32, 0, T, 4 * cap, 1.0, 0.0,
@@ -163,7 +164,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
             const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
-            double* X = c->d_W + (size_t)(2 * i) * mat;
+            double* X = c->d_Z + (size_t)(2 * i) * mat;
             double* T = c->d_thetap + (size_t)(2 * i) * mat;
             // X'[r][r'] = sum_{(l, s)} B[(l, s)][r] T[(l, s)][r']  (both (4 l) x r with row stride cap)
             P.add(GemmDesc{r, r, 4 * l, site_v(c, b, q), cap, f32, T, cap, 0, 0, X, ld, 1.0, 0.0, nullptr, 0, 0, 0, 1,
@@ -182,7 +183,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
             const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
-            double* Y = c->d_W + (size_t)(2 * i + 1) * mat;
+            double* Y = c->d_Z + (size_t)(2 * i + 1) * mat;
             double* U = c->d_thetap + (size_t)(2 * i + 1) * mat;
             // U[(l, s)][r'] = sum_r B[(l, s)][r] Y[r][r']
             P.add(GemmDesc{4 * l, r, r, site_v(c, b, q), cap, f32, Y, ld, 0, 0, U, cap, 1.0, 0.0, nullptr, 0, 0, 0, 0,
@@ -193,7 +194,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
             for (int i = 0; i < m; ++i) {
                 const int b = b0 + i;
                 const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
-                double* Y = c->d_W + (size_t)(2 * i + 1) * mat;
+                double* Y = c->d_Z + (size_t)(2 * i + 1) * mat;
                 double* U = c->d_thetap + (size_t)(2 * i + 1) * mat;
                 const void* Bs = static_cast<const char*>(site_v(c, b, q)) + (size_t)s * cap * site_esize(c);
                 // Y'[l][l'] (+)= sum_r U[(l, s)][r] B[(l', s)][r]
@@ -220,24 +221,46 @@ int run_plan(mpdo_ctx* c, GqPlan& P) {
     return MPDO_OK;
 }
 
-// FP64 Jacobi SVD (strict tolerance, every pair) of the chi x chi matrices in
-// W + slot * mat for the listed slots (rows j < chi of length chi).
-int run_svd(mpdo_ctx* c, double* W, const std::vector<int>& slots, const std::vector<int>& chis,
-            const std::vector<int>& inst) {
+// Whether SVDs of n x n matrices, n >= min_chi, take the stages of a step's SVDs
+// (FP32 QR and Jacobi, tensor-core refinement, FP64 Jacobi) in place of the FP64
+// Jacobi alone.  FP64 contexts only: a mixed one's products resolve 2^-48.  Below
+// 32 rows a matrix is a single block pair of one CTA and the stages' launches cost
+// more than its sweeps.
+bool staged_svd(const mpdo_ctx* c, int min_chi) { return refine_on(c) && c->oz_s == 7 && min_chi >= 32; }
+
+// zero rows and columns from chi up to the next multiple of 4 (the stages' row groups)
+__global__ void pad_kernel(double* M, size_t mat, int ld, const int* chi) {
+    const int s = blockIdx.x, n = chi[s], n4 = (n + 3) & ~3;
+    double* X = M + (size_t)s * mat;
+    for (int e = threadIdx.x; e < n4; e += blockDim.x)
+        for (int k = n; k < n4; ++k) X[(size_t)e * ld + k] = X[(size_t)k * ld + e] = 0.0;
+}
+
+// SVD (strict tolerance, every pair) of the chi x chi matrices in M + slot * mat for
+// the listed slots (rows j < chi of length chi), in place; staged: into W + slot * mat,
+// the transposed matrices being in MT + slot * mat.
+int run_svds(mpdo_ctx* c, double* M, double* MT, bool staged, const std::vector<int>& slots, const std::vector<int>& chis,
+             const std::vector<int>& inst) {
     const int ld = c->ld;
     const size_t mat = (size_t)ld * ld;
     const int nops = (int)slots.size();
     for (int k = 0; k < nops; ++k) {
         OpDesc d{};
-        const int s = slots[k], n = chis[k];
+        const int s = slots[k], n = staged ? (chis[k] + 3) & ~3 : chis[k];
         d.b = inst[k];
         d.c = n;
         d.L = n;
         d.m = n;
         d.n = n;
         d.chi_max = n;
-        d.W = W + (size_t)s * mat;
-        d.W0 = d.W;
+        if (staged) {
+            d.thetap = M + (size_t)s * mat;   // row-major
+            d.Acm = MT + (size_t)s * mat;     // column-major
+            svd_buffers(c, s, d);
+        } else {
+            d.W = M + (size_t)s * mat;
+            d.W0 = d.W;
+        }
         d.snorm = c->d_snorm + (size_t)s * 2 * ld;
         d.status = c->d_status + inst[k];
         d.sweeps_out = c->d_sweeps + s;
@@ -246,6 +269,16 @@ int run_svd(mpdo_ctx* c, double* W, const std::vector<int>& slots, const std::ve
         c->h_desc[k] = d;
     }
     CU(cudaMemcpyAsync(c->d_desc, c->h_desc, sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
+    if (staged) {
+        const bool prof = c->prof;   // the stage counters are those of the steps
+        c->prof = false;
+        SvdWork w;
+        const int rc = run_svd(c, nops, 0.0, w);
+        c->prof = prof;
+        if (rc) return rc;
+        CU(cudaStreamSynchronize(c->st));   // h_desc / h_cta are reused by the next call
+        return MPDO_OK;
+    }
     int total = 0;
     int rc = plan_jacobi(c, c->h_desc, nops, false, c->h_cta, total);
     if (rc) return rc;
@@ -290,13 +323,13 @@ extern "C" int mpdo_renyi2(mpdo_ctx* c, double* out, int out_on_device) {
     const int per = std::max(1, c->slots / 2);
     for (int b0 = 0; b0 < B; b0 += per) {
         const int m = std::min(per, B - b0);
-        gram_unit_kernel<<<(2 * m + 127) / 128, 128, 0, c->st>>>(c->d_W, mat, m);
+        gram_unit_kernel<<<(2 * m + 127) / 128, 128, 0, c->st>>>(c->d_Z, mat, m);
         CU(cudaGetLastError());
         GqPlan P;
         plan_left(c, b0, m, N - 1, P);
         rc = run_plan(c, P);
         if (rc) return rc;
-        renyi2_kernel<<<(m + 127) / 128, 128, 0, c->st>>>(c->d_W, mat, c->d_envL, N, c->cap, b0, m, dst);
+        renyi2_kernel<<<(m + 127) / 128, 128, 0, c->st>>>(c->d_Z, mat, c->d_envL, N, c->cap, b0, m, dst);
         CU(cudaGetLastError());
     }
     return finish(c, out, out_on_device);
@@ -314,7 +347,7 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
     const int per_chi = std::max(1, N / 2);
     for (int b0 = 0; b0 < B; b0 += std::min(per, per_chi)) {
         const int m = std::min(std::min(per, per_chi), B - b0);
-        gram_unit_kernel<<<(2 * m + 127) / 128, 128, 0, c->st>>>(c->d_W, mat, m);
+        gram_unit_kernel<<<(2 * m + 127) / 128, 128, 0, c->st>>>(c->d_Z, mat, m);
         CU(cudaGetLastError());
         GqPlan P;
         plan_left(c, b0, m, bond, P);
@@ -333,23 +366,29 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
             }
         }
         CU(cudaMemcpyAsync(d_chi, chi2.data(), sizeof(int) * 2 * m, cudaMemcpyHostToDevice, c->st));
-        rc = run_svd(c, c->d_W, slots, chis, inst);   // X and Y factored
+        const auto mm = std::minmax_element(chis.begin(), chis.end());
+        const int maxchi = *mm.second;
+        const bool staged = staged_svd(c, *mm.first);
+        double* F = staged ? c->d_W : c->d_Z;   // the rows of X and Y
+        if (staged) {
+            pad_kernel<<<2 * m, 256, 0, c->st>>>(c->d_Z, mat, ld, d_chi);
+            CU(cudaGetLastError());
+        }
+        rc = run_svds(c, c->d_Z, c->d_Z, staged, slots, chis, inst);   // X and Y factored
         if (rc) return rc;
-        int maxchi = 1;
-        for (int v : chis) maxchi = std::max(maxchi, v);
-        row_norms_kernel<<<dim3((maxchi + 7) / 8, 2 * m), 256, 0, c->st>>>(c->d_W, mat, ld, d_chi, c->d_snorm);
+        row_norms_kernel<<<dim3((maxchi + 7) / 8, 2 * m), 256, 0, c->st>>>(F, mat, ld, d_chi, c->d_snorm);
         CU(cudaGetLastError());
         // C_i = (rows of X) (rows of Y)^T into thetap slot 2i, then scaled to F_X F_Y^T
+        // (staged: its transpose into slot 2i + 1)
         GqPlan Pc;
         Pc.begin();
-        for (int i = 0; i < m; ++i) {
-            const int n = chi2[2 * i];
-            Pc.add(GemmDesc{n, n, n, c->d_W + (size_t)(2 * i) * mat, ld, 0, c->d_W + (size_t)(2 * i + 1) * mat, ld, 0,
-                            1, c->d_thetap + (size_t)(2 * i) * mat, ld, 1.0, 0.0, nullptr, 0, 0, 0, 0, 0});
-        }
+        const int step = staged ? 1 : 2;
+        for (int s = 0; s < 2 * m; s += step)
+            Pc.add(GemmDesc{chi2[s], chi2[s], chi2[s], F + (size_t)s * mat, ld, 0, F + (size_t)(s ^ 1) * mat, ld, 0,
+                            1, c->d_thetap + (size_t)s * mat, ld, 1.0, 0.0, nullptr, 0, 0, 0, 0, 0});
         rc = run_plan(c, Pc);
         if (rc) return rc;
-        scale_kernel<<<dim3(64, m), 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, c->d_snorm);
+        scale_kernel<<<dim3(64, staged ? 2 * m : m), 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, c->d_snorm, step);
         CU(cudaGetLastError());
         std::vector<int> s1, c1, i1;
         for (int i = 0; i < m; ++i) {
@@ -357,9 +396,13 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
             c1.push_back(chi2[2 * i]);
             i1.push_back(b0 + i);
         }
-        rc = run_svd(c, c->d_thetap, s1, c1, i1);
+        if (staged) {
+            pad_kernel<<<2 * m, 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi);
+            CU(cudaGetLastError());
+        }
+        rc = run_svds(c, c->d_thetap, c->d_thetap + mat, staged, s1, c1, i1);
         if (rc) return rc;
-        osee_kernel<<<m, 512, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, b0, dst);
+        osee_kernel<<<m, 512, 0, c->st>>>(staged ? c->d_W : c->d_thetap, mat, ld, d_chi, b0, dst);
         CU(cudaGetLastError());
     }
     return finish(c, out, out_on_device);

@@ -177,7 +177,7 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
                                                  g->d_error);
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
-            if (c->mixed) {
+            if (c->precond) {
                 CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, st));
                 CU(launch_gate_weight(ch.d_desc, nops, cap, st));
             } else {
@@ -201,13 +201,13 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
                 CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
                 CU(launch_jacobi(ch.d_desc, nops, ch.d_cta32, ch.d_cta32 + g->Rj, ch.d_cta32 + 2 * g->Rj, c->d_sync,
                                  g->Rj, kMaxSweepsCap / 2, 0.0, timeout_ns, ld, true, st, precond_rho(c)));
-                CU(launch_svd_products(c, ch.d_desc, nops, st));
+                CU(launch_svd_products(c, ch.d_desc, nops, fp64_jacobi_tol(c), st));
             }
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
             CU(launch_jacobi(ch.d_desc, nops, ch.d_cta64, ch.d_cta64 + g->Rj, ch.d_cta64 + 2 * g->Rj, c->d_sync, g->Rj,
                              c->cfg.jacobi_max_sweeps, fp64_jacobi_tol(c), timeout_ns, ld, false, st, precond_rho(c)));
             CU(launch_truncate(ch.d_desc, nops, cap, st));
-            if (c->mixed)
+            if (c->precond)
                 CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, cap, c->oz_s, timeout_ns, st));
             else
                 CU(launch_reconstruct(ch.d_desc, nops, cap, st));

@@ -56,15 +56,16 @@ struct OpDesc {
     double* lam_out;   // lambda_p
     double* thetap;    // Theta'  m x n (ld)
     double* Acm;       // theta~ column-major (column k at Acm + k*ld), input of the QR
-    double* W0;        // rows of R from the QR (== W in the FP64 path)
+    double* W0;        // rows from the QR (== W without the preconditioning stages)
     double* W;         // Jacobi rows: theta~ (m x n) or theta~^T (n x m)
     double* Z;         // c x c rotation accumulator when transposed
     const double* Zinit;  // initial Z (nullptr => identity)
-    float* W32;        // mixed path: FP32 rows of the preconditioning Jacobi (c x L)
-    float* U32;        // mixed path: FP32 accumulated rotations (c x c)
+    // the preconditioning stages (mixed contexts, FP64 ones with a sweep limit >= 16):
+    float* W32;        // FP32 rows of the preconditioning Jacobi (c x L)
+    float* U32;        // FP32 accumulated rotations (c x c), first the FP32 QR's Q^T
     float* D32;        // FP32 pass: Gram matrix of every row block [block][32][32]
-    double* E;         // mixed path: U32 U32^T - I (c x c)
-    double* Q;         // mixed path: orthogonalised U32 (c x c)
+    double* E;         // U32 U32^T - I (c x c), later W W^T
+    double* Q;         // orthogonalised U32 (c x c), later the refinement's X
     double* Yk;        // k x n right singular vectors (rows), ld
     double* snorm;     // 2*ld doubles of scratch: row norms (Jacobi), R diagonal and column norms (QR)
     int* k_out;        // new chi_p
@@ -72,7 +73,7 @@ struct OpDesc {
     double* max_disc;  // per-instance max discarded weight
     int* rank_log;     // &log[b][step*n_ops + op] or nullptr
     int* sweeps_out;   // Jacobi sweeps used (or nullptr)
-    int* pre_ok;       // mixed path: 1 when the FP32 pass ended with every pair orthogonal to ~1e-6
+    int* pre_ok;       // 1 when the FP32 pass ended with every pair orthogonal to ~1e-6
                        // (its last sweep rotated by at most 1e-3); written by that pass, read by
                        // the FP64 pass (or nullptr)
     RefineOp* rf;      // state of the Gram-matrix refinement (refine.cu), or nullptr without it
@@ -80,9 +81,32 @@ struct OpDesc {
     int full_svd;      // 1: orthogonalise every pair of rows (the adjoint needs all singular vectors)
     double* tape_V;    // adjoint recompute: all c sorted right singular vectors (c x n), or nullptr
     double* tape_s;    // adjoint recompute: all c sorted singular values
-    void *oz_as, *oz_bs;   // mixed path: slice blocks of the tensor-core products (oz_gemm.cu)
+    void *oz_as, *oz_bs;   // slice blocks of the tensor-core products (oz_gemm.cu)
     int *oz_ea, *oz_eb;    // and their row / column exponents
 };
+
+// Launch of a kernel that begins with grid_begin(): its CTAs may be scheduled while the
+// stream's previous kernel runs out, and wait there for all of that kernel's results.
+template <class... P, class... A>
+inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
 
 // Site tensor element i as double (storage f64 or f32), and the store back.
 __device__ __forceinline__ double site_ld(const void* p, size_t i, int f32) {
@@ -186,6 +210,7 @@ struct OzProblem {
     const void* D;
     int ldd, d_f32, sub_identity;
     int levels;          // slice pairs (t, u) with t + u < levels are formed (0: all S levels)
+    int unit_d;          // D's rows are of unit norm: levels follow from the operands' exponents
     int sym;             // C (f64, no gather) is symmetric: tiles below the diagonal are mirrored, not computed
     void *as, *bs;       // slice blocks of A and B
     int *ea, *eb;        // row / column exponents
@@ -224,8 +249,8 @@ cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int m
 // OZ_R2, OZ_R1 the refinement's rotation (refine.cu).
 // OZ_FIRST + OZ_E, OZ_Q, OZ_T, OZ_Q3, OZ_W: the same on the QR's Q^T (ops of qr32_takes
 // only), OZ_W then being W0 = Q theta~.
-enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T = 5, OZ_Q3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
-       OZ_R1 = 10 };
+enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T4 = 5, OZ_T3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
+       OZ_R1 = 10, OZ_T2 = 11 };
 cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S,
                           unsigned long long timeout_ns, cudaStream_t st);
 constexpr int kOzKernels = 2;   // kernels of one launch_oz_ops

@@ -30,24 +30,20 @@
 // kept rows are normalised into singular vectors, so they must be orthogonal
 // relative to their own norms.
 //
-// The same kernel, instantiated for float, is the preconditioning pass of the
-// mixed-precision SVD: it orthogonalises an FP32 copy of the rows (scaled to
-// unit mean square norm) and accumulates its rotations in U32; the FP64 pass
-// then starts from Q W with Q the FP64-orthogonalised U32 (see api.cu).
-// A row whose norm is at most eps * ||W||_F (FP64 eps, in both passes) is
-// numerically zero: it is set to zero and never rotated (its direction is
-// rounding noise).
+// After the FP32 pass (jacobi32.cu) and the refinement through the Gram matrix
+// (refine.cu) most ops arrive finished and their CTAs return at once; what is
+// left is what those stages do not cover, and every SVD of contexts whose sweep
+// limit leaves them out.  A row whose norm is at most eps * ||W||_F (FP64 eps, in
+// every stage) is numerically zero: it is set to zero and never rotated (its
+// direction is rounding noise).
 //
 // Further pieces, each described where it is implemented:
-//  - FP32 pass on rows of at most 1024 elements: the register path (16 warps,
-//    one block of each pair in registers, U32 turned by the block pair's
-//    accumulated rotation);
-//  - FP64 pass: scaled (fast) rotations, one FMA per element (scaled_rotate);
-//  - FP64 pass: pairs of two rows the truncation discards are skipped once the
-//    ranking is settled (kth_largest and the sweep-start gate);
-//  - convergence: the FP32 pass stops at <= c/4 rotations or a largest rotated
-//    off-orthogonality of 1e-3, the FP64 pass at no rotation or a largest
-//    rotated rho with rho^2 <= 1e-6 tol.
+//  - scaled (fast) rotations, one FMA per element (scaled_rotate);
+//  - pairs of two rows the truncation discards are skipped once the ranking is
+//    settled (kth_largest and the sweep-start gate);
+//  - convergence: no rotation or a largest rotated rho with rho^2 <= 1e-6 tol
+//    (the FP32 pass: <= c/4 rotations or a largest rotated off-orthogonality of
+//    1e-3).
 #include <float.h>
 #include <mpdo.h>
 

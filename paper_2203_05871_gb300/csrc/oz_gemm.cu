@@ -68,17 +68,21 @@ namespace {
 // t + u < S, one accumulator per level t + u
 
 constexpr int kTileM = 128;            // rows of A (and of C) per tile
-constexpr int kTileN = 64;             // columns of B (and of C) per tile
+constexpr int kTileN = 64;             // columns of B per slice block
 constexpr int kBlockA = kTileM * 64;   // bytes of one slice block of A (8 KB)
 constexpr int kBlockB = kTileN * 64;   // of B (4 KB)
-__host__ __device__ constexpr int stage_bytes(int S) { return S * (kBlockA + kBlockB); }   // A and B slices of one k tile
-__host__ __device__ constexpr int stages_of(int S) { return S == 6 ? 3 : 2; }               // 216 KB / 168 KB of shared memory
+// bytes of one k tile of a CTA with TN columns, its stages (up to 210 KB), and shared memory
+__host__ __device__ constexpr int stage_bytes(int S, int TN) { return S * (kBlockA + TN * 64); }
+__host__ __device__ constexpr int stages_of(int S, int TN) { return 216 * 1024 / stage_bytes(S, TN); }
 constexpr int kRangeK = 256;           // K values between accumulator drains
 constexpr int kThreads = 320;
-__host__ __device__ constexpr int smem_of(int S) { return stages_of(S) * stage_bytes(S) + 1024; }
+__host__ __device__ constexpr int smem_of(int S, int TN) { return stages_of(S, TN) * stage_bytes(S, TN) + 1024; }
+__host__ __device__ constexpr int tmem_cols(int S, int TN) {   // a power of two
+    return S * TN <= 128 ? 128 : S * TN <= 256 ? 256 : 512;
+}
 static_assert(7 * kTileN <= 512, "accumulators exceed tensor memory");
-static_assert(smem_of(6) <= 227 * 1024 && smem_of(7) <= 227 * 1024, "the ring exceeds shared memory");
-static_assert(kTileM == 128 && kTileN == 64, "oz_set_tiles (internal.h) assumes 128 x 64 tiles");
+static_assert(smem_of(6, 64) <= 227 * 1024 && stages_of(7, 64) >= 2, "the ring in shared memory");
+static_assert(kTileM == 128 && kTileN == 64, "oz_set_tiles (internal.h) assumes blocks of 128 and 64 rows");
 constexpr int LBO = 128, SBO = 512;
 
 constexpr int G = 8;                   // bf16 values per 16-byte store
@@ -143,15 +147,48 @@ __device__ __forceinline__ void commit(uint32_t mbar) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+// 8 accumulator columns of this warp's 32 lanes
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// (hi 2^24 + lo) 2^e, |hi| < 2^62, |lo| < 2^62, rounded to nearest even: the double is
+// put together with integer instructions (GB300 issues about 60 of them in the time
+// of one FP64 instruction), unless it leaves the normal range.
+__device__ __forceinline__ double scaled(long long hi, long long lo, int e) {
+    hi += lo >> 24;
+    unsigned long long w = ((unsigned long long)lo & 0xffffffull) << 40;   // the fraction below hi
+    const bool neg = hi < 0;
+    unsigned long long u = (unsigned long long)hi;
+    if (neg) {
+        u = ~u + (w == 0);
+        w = 0 - w;
+    }
+    e += 24;
+    if (u == 0) {
+        u = w;
+        w = 0;
+        e -= 64;
+    }
+    if (u == 0) return 0.0;
+    const int nz = __clzll((long long)u);
+    const unsigned long long v = nz ? (u << nz) | (w >> (64 - nz)) : u;
+    const bool sticky = (w << nz) != 0;
+    unsigned long long m = v >> 11;
+    const unsigned low = (unsigned)v & 0x7ffu;
+    m += low > 0x400u || (low == 0x400u && (sticky || (m & 1)));
+    const int E = 63 - nz + e + 1023;
+    if (E >= 1 && E < 2046) {
+        const long long bits = (long long)(((unsigned long long)(E - 1) << 52) + m);
+        return __longlong_as_double(neg ? bits | (1ll << 63) : bits);
+    }
+    const double x = ldexp((double)m, E - 1023 - 52);
+    return neg ? -x : x;
 }
 
 // index of element (r, k) of an operand view
@@ -337,15 +374,17 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
             P.sym = 1;
             break;
         case OZ_Q:       // Q = U - E U / 2
-        case OZ_T:       // T = U - 3 E U / 4 (in W, free until OZ_W)
-        case OZ_Q3:      // Q = U - E T / 2
+        case OZ_T4:      // T = U - 5 E U / 6 (in W, free until OZ_W)
+        case OZ_T3:      // T = U - 3 E T / 4
+        case OZ_T2:      // Q = U - E T / 2
             P.M = P.N = P.K = d.c;
             P.A = rowmajor(d.E, 0, ld);
-            P.B = kind == OZ_Q3 ? colmajor(d.W, 0, ld) : colmajor(d.U32, 1, ld);
-            P.C = kind == OZ_T ? d.W : d.Q;
+            P.B = kind == OZ_T3 || kind == OZ_T2 ? colmajor(d.W, 0, ld) : colmajor(d.U32, 1, ld);
+            P.C = kind == OZ_T4 || kind == OZ_T3 ? d.W : d.Q;
             P.ldc = ld;
-            P.alpha = kind == OZ_T ? -0.75 : -0.5;
+            P.alpha = kind == OZ_T4 ? -5.0 / 6.0 : kind == OZ_T3 ? -0.75 : -0.5;
             P.beta = 1.0;
+            P.unit_d = 1;
             P.D = d.U32;
             P.ldd = ld;
             P.d_f32 = 1;
@@ -407,16 +446,23 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
     return P;
 }
 
-// the CTA's problem, through shared memory
+// the CTA's problem, through shared memory (the op's descriptor read by all threads at
+// once: one thread's chain of loads from it cost 1 to 2 us)
 template <int kS>
 __device__ __forceinline__ void fetch_problem(const OzSource& src, OzProblem& P) {
-    if (threadIdx.x == 0)
-        P = src.probs   ? src.probs[blockIdx.z]
-            : src.descs ? op_problem<kS>(src.descs[blockIdx.z], src.kind, src.cap)
-                        : src.one;
+    if (src.descs) {
+        __shared__ __align__(16) int sd[sizeof(OpDesc) / 4];
+        const int* g = reinterpret_cast<const int*>(src.descs + blockIdx.z);
+        for (int i = threadIdx.x; i < (int)(sizeof(OpDesc) / 4); i += blockDim.x) sd[i] = g[i];
+        __syncthreads();
+        if (threadIdx.x == 0) P = op_problem<kS>(*reinterpret_cast<const OpDesc*>(sd), src.kind, src.cap);
+    } else if (threadIdx.x == 0) {
+        P = src.probs ? src.probs[blockIdx.z] : src.one;
+    }
     __syncthreads();
 }
 
+static_assert(sizeof(OpDesc) % 4 == 0, "copied as words");
 
 // Strided views (a transposed operand, the right site of a merge): a block
 // takes 32 consecutive rows, lane = row and warp = a slice of the K range, so
@@ -469,6 +515,7 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int K
 template <int kS>
 __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     __shared__ OzProblem P;
+    grid_begin();
     fetch_problem<kS>(src, P);
     const bool isB = blockIdx.y == 1;
     const OzOperand& X = isB ? P.B : P.A;
@@ -527,24 +574,27 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     }
 }
 
-template <int kS>
+template <int kS, int TN>
 __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                                                                unsigned long long timeout_ns) {
     constexpr int kRangeTiles = kRangeK / KT;
-    constexpr int kLevels = kS, kStages = stages_of(kS), kStageBytes = stage_bytes(kS);
+    constexpr int kLevels = kS, kStages = stages_of(kS, TN), kStageBytes = stage_bytes(kS, TN);
+    constexpr int kBytesB = TN * 64;   // of one slice block of B
     // barriers: full[kStages], empty[kStages], accumulators full, accumulators drained, final
     constexpr int kBarFull = 0, kBarEmpty = kStages, kBarAccFull = 2 * kStages, kBarAccEmpty = 2 * kStages + 1,
                   kBarFinal = 2 * kStages + 2;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ OzProblem P;
+    grid_begin();
     fetch_problem<kS>(src, P);
     const int N = P.Ndyn ? *P.Ndyn : P.N;
     const int mt = blockIdx.y, nt = blockIdx.x;
-    if (mt * kTileM >= P.M || nt * kTileN >= N) return;
-    if (P.sym && (nt + 1) * kTileN <= mt * kTileM) return;   // mirrored from above the diagonal
+    if (mt * kTileM >= P.M || nt * TN >= N) return;
+    if (P.sym && (nt + 1) * TN <= mt * kTileM) return;   // mirrored from above the diagonal
     const int Kt = P.Kt;
-    const int lv = P.levels > 0 ? P.levels : kS;   // slice pairs t + u < lv
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ int s_ea, s_eb;
+    if (threadIdx.x == 0) s_ea = s_eb = -(1 << 20);
 
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kStages * kStageBytes + 128);
@@ -562,13 +612,25 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(512));
+                     "r"(tmem_cols(kS, TN)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tslot;
+    int lv = P.levels > 0 ? P.levels : kS;   // slice pairs t + u < lv
+    if (P.unit_d) {   // what A B adds to entries of a unit row of D is below 2^(e_i + f_j)
+        if (threadIdx.x < kTileM) {
+            const int i = mt * kTileM + threadIdx.x;
+            if (i < P.M) atomicMax(&s_ea, P.ea[i]);
+        } else if (threadIdx.x < kTileM + TN) {
+            const int j = nt * TN + threadIdx.x - kTileM;
+            if (j < N) atomicMax(&s_eb, P.eb[j]);
+        }
+        __syncthreads();
+        lv = oz_levels(kS, s_ea + s_eb);
+    }
     const int nrange = (Kt + kRangeTiles - 1) / kRangeTiles;
 
     if (warp == 0) {
@@ -583,12 +645,13 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                     !mbar_wait(smem_u32(bar + kBarEmpty + s), ((kt / kStages) - 1) & 1, abort_flag, timeout_ns))
                     break;
                 const uint32_t full = smem_u32(bar + kBarFull + s);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full), "r"(lv * (kBlockA + kBlockB))
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full), "r"(lv * (kBlockA + kBytesB))
                              : "memory");
                 unsigned char* st = smem + (size_t)s * kStageBytes;
                 for (int t = 0; t < lv; ++t) {
                     const unsigned char* srcA = as + (((size_t)t * P.Mt + mt) * Kt + kt) * kBlockA;
-                    const unsigned char* srcB = bs + (((size_t)t * P.Nt + nt) * Kt + kt) * kBlockB;
+                    const unsigned char* srcB = bs + (((size_t)t * P.Nt + nt * TN / kTileN) * Kt + kt) * kBlockB +
+                                                (nt * TN % kTileN) * 64;   // 8 rows are 512 consecutive bytes
                     asm volatile(
                         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                             smem_u32(st + t * kBlockA)),
@@ -596,8 +659,8 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                         : "memory");
                     asm volatile(
                         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            smem_u32(st + kS * kBlockA + t * kBlockB)),
-                        "l"(srcB), "r"(kBlockB), "r"(full)
+                            smem_u32(st + kS * kBlockA + t * kBytesB)),
+                        "l"(srcB), "r"(kBytesB), "r"(full)
                         : "memory");
                 }
                 issued = kt + 1;
@@ -608,7 +671,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t id = idesc(kTileM, kTileN);
+            const uint32_t id = idesc(kTileM, TN);
             int r = 0;
             bool first[kLevels];
 #pragma unroll
@@ -627,7 +690,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
 #pragma unroll
                 for (int lvl = 0; lvl < kLevels; ++lvl) {
                     if (lvl >= lv) break;
-                    const uint32_t d = tmem + (uint32_t)(lvl * kTileN);
+                    const uint32_t d = tmem + (uint32_t)(lvl * TN);
 #pragma unroll
                     for (int t = 0; t <= lvl; ++t) {
                         const int u = lvl - t;
@@ -635,7 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                         for (int q = 0; q < 2; ++q) {
                             const uint32_t off = q * 2 * LBO;
                             mma(d, smem_desc(st + t * kBlockA + off),
-                                smem_desc(st + kS * kBlockA + u * kBlockB + off), id, first[lvl] ? 0u : 1u);
+                                smem_desc(st + kS * kBlockA + u * kBytesB + off), id, first[lvl] ? 0u : 1u);
                             first[lvl] = false;
                         }
                     }
@@ -650,14 +713,21 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
             mbar_wait(smem_u32(bar + kBarFinal), 0, abort_flag, timeout_ns);   // every MMA issued has completed
         }
     } else {
-        // epilogue warps 2..9: rows 32 (warp % 4) + lane, columns half * 32 .. + 31
+        // epilogue warps 2..9: rows 32 (warp % 4) + lane, columns half * CP .. + CP - 1
+        constexpr int CP = TN / 2;
         const int ew = warp - 2;
         const int lane_base = 32 * (warp & 3);
         const int half = ew >> 2;
-        const uint32_t taddr = tmem + ((uint32_t)lane_base << 16) + (uint32_t)(half * 32);
-        double acc[32];
+        const uint32_t taddr = tmem + ((uint32_t)lane_base << 16) + (uint32_t)(half * CP);
+        // Level d holds n_d 2^-8d with n_d an integer (exact for d <= 3; higher levels are
+        // rounded to the nearest 2^-8d).  The sum over the ranges is kept exactly:
+        // hi 2^24 + lo in units of 2^-40, hi = n_0 2^16 + n_1 2^8 + n_2 (|.| < 2^39 per
+        // range), lo = n_3 2^16 + n_4 2^8 + n_5 + n_6 / 2^8 rounded (|.| < 2^41).  A NaN
+        // slice reaches level 0.
+        long long hi[CP], lo[CP];
+        unsigned nan = 0;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0.0;
+        for (int j = 0; j < CP; ++j) hi[j] = lo[j] = 0;
         bool ok = true;
         for (int r = 0; r < nrange; ++r) {
             if (!mbar_wait(smem_u32(bar + kBarAccFull), r & 1, abort_flag, timeout_ns)) {
@@ -665,80 +735,71 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;");
-            // level d holds n_d 2^-8d with n_d an integer (exact for d <= 3;
-            // higher levels are rounded to the nearest 2^-8d): the range's
-            // sum is S 2^-40 with the integer S = sum_d n_d 2^(8 (5 - d)),
-            // |S| < 2^63 (level 6 rounded to that unit), formed in int64 and
-            // converted once (integer arithmetic instead of twelve FP64
-            // operations per element).  A NaN slice reaches level 0.
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                long long S[16];
-                unsigned nan = 0;
+            for (int lvl = 0; lvl < kLevels; ++lvl) {
+                if (lvl >= lv) break;   // uniform: not formed
+                const float scale = __int_as_float((127 + 8 * lvl) << 23);   // 2^8d
 #pragma unroll
-                for (int lvl = 0; lvl < kLevels; ++lvl) {
-                    if (lvl >= lv) {   // uniform: not formed
-                        if (lvl < 6)
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) S[i] *= 256;
-                        continue;
-                    }
-                    float v[16];
-                    tmem_ld16(taddr + (uint32_t)(lvl * kTileN + c * 16), v);
+                for (int c = 0; c < CP; c += 8) {
+                    float v[8];
+                    tmem_ld8(taddr + (uint32_t)(lvl * TN + c), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const float scale = __int_as_float((127 + 8 * lvl) << 23);   // 2^8d
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
+                    for (int i = 0; i < 8; ++i) {
                         const int n = __float2int_rn(v[i] * scale);
-                        if (lvl == 0) {
-                            S[i] = n;
-                            nan |= (v[i] != v[i]) ? 1u << i : 0u;
-                        } else if (lvl < 6) {
-                            S[i] = S[i] * 256 + n;
-                        } else {
-                            S[i] += (n + 128) >> 8;   // level 6 in units of 2^-40
-                        }
+                        if (lvl == 0) nan |= (v[i] != v[i]) ? 1u << (c + i) : 0u;
+                        if (lvl < 3)
+                            hi[c + i] += (long long)n * (1 << (16 - 8 * lvl));
+                        else if (lvl < 6)
+                            lo[c + i] += (long long)n * (1 << (40 - 8 * lvl));
+                        else
+                            lo[c + i] += (n + 128) >> 8;
                     }
                 }
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    acc[c * 16 + i] += ((nan >> i) & 1u) ? __longlong_as_double(0x7ff8000000000000ll) : (double)S[i];
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
             if (lane == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar + kBarAccEmpty)) : "memory");
         }
-        if (ok && !*abort_flag) {
-            const int i = mt * kTileM + lane_base + lane;
-            if (i < P.M) {
-                const int ei = P.ea[i];
+        const int i = mt * kTileM + lane_base + lane;
+        if (ok && !*abort_flag && i < P.M) {
+            // alpha a power of two: into the exponent
+            const long long ab = __double_as_longlong(P.alpha);
+            const int aE = (int)((ab >> 52) & 0x7ff);
+            const bool pow2 = (ab & 0xfffffffffffffll) == 0 && aE > 0 && aE < 0x7ff;
+            const int ei = P.ea[i] + (pow2 ? aE - 1023 : 0) - 54;   // the sum is in units of 2^-40
+            const size_t row = P.c_gather ? (size_t)P.c_gather[i] : (size_t)i;
+            const int j0 = nt * TN + half * CP;
 #pragma unroll
-                for (int jj = 0; jj < 32; ++jj) {
-                    const int j = nt * kTileN + half * 32 + jj;
-                    if (j >= N) continue;
-                    double v = P.alpha * ldexp(acc[jj], ei + P.eb[j] - 54);   // acc in units of 2^-40
-                    const size_t row = P.c_gather ? (size_t)P.c_gather[i] : (size_t)i;
-                    if (P.D) {
-                        const size_t di = row * P.ldd + j;
-                        v += P.beta * (P.d_f32 ? (double)static_cast<const float*>(P.D)[di]
-                                               : static_cast<const double*>(P.D)[di]);
-                    }
-                    if (P.sub_identity && i == j) v -= 1.0;
-                    const size_t ci = row * P.ldc + j;
-                    if (P.c_f32)
-                        static_cast<float*>(P.C)[ci] = (float)v;
-                    else
-                        static_cast<double*>(P.C)[ci] = v;
-                    if (P.sym && j > i) static_cast<double*>(P.C)[(size_t)j * P.ldc + i] = v;
+            for (int jj = 0; jj < CP; ++jj) {
+                const int j = j0 + jj;
+                if (j >= N) continue;
+                double v = scaled(hi[jj], lo[jj], ei + P.eb[j]);
+                if (pow2)
+                    v = __longlong_as_double(__double_as_longlong(v) ^ (ab & (1ll << 63)));
+                else
+                    v *= P.alpha;
+                if ((nan >> jj) & 1u) v = __longlong_as_double(0x7ff8000000000000ll);
+                if (P.D) {
+                    const size_t di = row * P.ldd + j;
+                    v += P.beta * (P.d_f32 ? (double)static_cast<const float*>(P.D)[di]
+                                           : static_cast<const double*>(P.D)[di]);
                 }
+                if (P.sub_identity && i == j) v -= 1.0;
+                const size_t ci = row * P.ldc + j;
+                if (P.c_f32)
+                    static_cast<float*>(P.C)[ci] = (float)v;
+                else
+                    static_cast<double*>(P.C)[ci] = v;
+                if (P.sym && j > i) static_cast<double*>(P.C)[(size_t)j * P.ldc + i] = v;
             }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols(kS, TN)));
     if (threadIdx.x == 0 && *abort_flag && P.status) atomicOr(P.status, (int)MPDO_ST_TIMEOUT);
 }
 
@@ -785,25 +846,47 @@ size_t oz_slice_bytes(int rows, int K, int S) {
 
 size_t oz_exp_ints(int rows) { return (size_t)((rows + kTileM - 1) / kTileM) * kTileM; }
 
+namespace {
+
+template <int S, int TN>
+cudaError_t prepare_one() {
+    return cudaFuncSetAttribute(oz_gemm_kernel<S, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of(S, TN));
+}
+
+}  // namespace
+
 cudaError_t oz_prepare() {
-    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<6>, a, smem_of(6));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<7>, a, smem_of(7));
-    return e;
+    for (cudaError_t e : {prepare_one<6, 16>(), prepare_one<6, 32>(), prepare_one<6, 64>(), prepare_one<7, 16>(),
+                          prepare_one<7, 32>(), prepare_one<7, 64>()})
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 namespace {
 
+template <int S, int TN>
+cudaError_t launch_tiles(const OzSource& src, int count, int max_m, int max_n, unsigned long long timeout_ns,
+                         cudaStream_t st) {
+    const dim3 grid((max_n + TN - 1) / TN, (max_m + kTileM - 1) / kTileM, count);
+    return launch_early(oz_gemm_kernel<S, TN>, grid, kThreads, smem_of(S, TN), st, src, timeout_ns);
+}
+
+// Columns per CTA: 64, the most that the accumulators leave room for, unless the
+// launch would not fill the chip; an MMA takes 2/3 of the time with 16 columns
+// (A's 4 KB per MMA through shared memory is what bounds it) and the epilogue a
+// quarter, so that narrower tiles win as long as each still has an SM.
+constexpr int kFill = 152;
+
 template <int S>
 cudaError_t launch_oz(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced,
                       unsigned long long timeout_ns, cudaStream_t st) {
-    const int mt = (max_m + kTileM - 1) / kTileM, nt = (max_n + kTileN - 1) / kTileN;
     const int rows = ((max_rows_sliced + kTileM - 1) / kTileM) * kTileM;
-    oz_slice_kernel<S><<<dim3((rows + 7) / 8, 2, count), 256, 0, st>>>(src);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_early(oz_slice_kernel<S>, dim3((rows + 7) / 8, 2, count), 256, 0, st, src);
     if (e != cudaSuccess) return e;
-    oz_gemm_kernel<S><<<dim3(nt, mt, count), kThreads, smem_of(S), st>>>(src, timeout_ns);
-    return cudaGetLastError();
+    const long long tiles = (long long)((max_m + kTileM - 1) / kTileM) * ((max_n + kTileN - 1) / kTileN) * count;
+    if (tiles * 4 <= kFill) return launch_tiles<S, 16>(src, count, max_m, max_n, timeout_ns, st);
+    if (tiles * 2 <= kFill) return launch_tiles<S, 32>(src, count, max_m, max_n, timeout_ns, st);
+    return launch_tiles<S, 64>(src, count, max_m, max_n, timeout_ns, st);
 }
 
 cudaError_t launch_oz_source(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced, int S,

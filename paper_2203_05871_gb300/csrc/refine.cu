@@ -41,6 +41,7 @@ constexpr int NT = 256;
 // squared row norms and their inverse roots from G's diagonal, the zero floor
 // (rows at or under it are set to zero) and the discard threshold, fixed once open
 __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, int ld) {
+    grid_begin();
     const OpDesc& d = descs[blockIdx.x];
     RefineOp& r = *d.rf;
     if (r.state != kRefineActive) {
@@ -118,6 +119,7 @@ __device__ void decide(const OpDesc& d, RefineOp& r, double tol_in, int can_fini
 // was too large for the expansion.  The op's last CTA to finish decides.
 __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int ld, double tol_in, float tcap,
                                                       int can_finish, float defect, int last) {
+    grid_begin();
     const OpDesc& d = descs[blockIdx.y];
     RefineOp& r = *d.rf;
     const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -125,6 +127,11 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
     if ((int)blockIdx.x >= blocks || __ldcg(&r.state) != kRefineActive) return;
     if (i < d.c) {
         const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
+        // pairs within a tolerance well above the Gram matrix's own error are turned too,
+        // down to 1/100 of it, where that takes an angle of the tolerance's size (1000 of
+        // them add 4e-14 to the rotation's defect): it costs nothing and leaves the rows'
+        // errors far below the tolerance (a chi 256 step's: 3e-10 without, 1e-11 with it)
+        const float turn = tol >= 1e-11f ? 0.01f * tol : tol;
         const double* a = d.snorm;
         const double* inv = d.snorm + ld;
         const double ai = a[i], vi = inv[i], thr = r.thr;
@@ -138,16 +145,17 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
                 const double v = vi * vj;
                 const float q = (float)(d.E[(size_t)i * ld + j] * v);   // g / (|w_i| |w_j|)
                 rho = !(fabsf(q) <= rho) ? fabsf(q) : rho;              // a NaN stays
-                if (fabsf(q) > tol) {
+                if (fabsf(q) > turn) {
                     const float zeta = (float)((aj - ai) * v) / (2.0f * q);
                     const float t = fabsf(zeta) > 1e18f   // a row far below the other (zeta^2 leaves FP32's range)
                                         ? 0.5f / zeta
                                         : copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)));
-                    if (fabsf(t) <= tcap) {
+                    const bool small = fabsf(q) <= tol;
+                    if (fabsf(t) <= (small ? 2.0f * tol : tcap)) {
                         const float th = t * fmaf(-t * t, 1.0f / 3.0f, 1.0f);   // atan t
                         x = -(double)th;
-                        sum += fabsf(th);
-                    } else {
+                        if (!small) sum += fabsf(th);
+                    } else if (!small) {
                         far = 1;
                     }
                 }
@@ -187,10 +195,10 @@ cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, do
     for (int it = 0; it < kRefineIters; ++it) {
         cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, chi_cap, S, timeout_ns, st);
         if (e != cudaSuccess) return e;
-        refine_diag_kernel<<<nops, NT, 0, st>>>(d_desc, ld);
-        refine_x_kernel<<<dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st>>>(
-            d_desc, ld, tol_in, tcap, can_finish ? 1 : 0, defect, it == kRefineIters - 1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_early(refine_diag_kernel, nops, NT, 0, st, d_desc, ld)) != cudaSuccess) return e;
+        e = launch_early(refine_x_kernel, dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st, d_desc, ld, tol_in,
+                         tcap, can_finish ? 1 : 0, defect, it == kRefineIters - 1);
+        if (e != cudaSuccess) return e;
         for (int kind : {OZ_R3, OZ_R2, OZ_R1})
             if ((e = launch_oz_ops(d_desc, nops, kind, chi_cap, S, timeout_ns, st)) != cudaSuccess) return e;
     }
