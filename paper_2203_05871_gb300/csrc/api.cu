@@ -65,11 +65,12 @@ int release_slots(mpdo_ctx* c) {
     void* ptrs[] = {c->d_thetap, c->d_W,    c->d_Z,     c->d_Yk,    c->d_snorm, c->d_desc,  c->d_cta,
                     c->d_sync,   c->d_sweeps, c->d_pre_ok, c->d_W0,  c->d_E,     c->d_Q,     c->d_W32,
                     c->d_U32,    c->d_gemm,  c->d_copy,  c->d_oz_as, c->d_oz_bs, c->d_oz_ea, c->d_oz_eb,
-                    c->d_oz,     c->d_refine, c->d_D32};
+                    c->d_oz,     c->d_refine, c->d_D32,   c->d_Zrot};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     c->d_refine = nullptr;
     c->d_D32 = nullptr;
+    c->d_Zrot = nullptr;
     c->d_thetap = c->d_W = c->d_Z = c->d_Yk = c->d_snorm = nullptr;
     c->d_W0 = c->d_E = c->d_Q = nullptr;
     c->d_W32 = c->d_U32 = nullptr;
@@ -105,8 +106,9 @@ int alloc_slots(mpdo_ctx* c, int want) {
     size_t per_slot_bytes = (3 * mat + (size_t)c->cap * c->ld + 2 * c->ld) * sizeof(double);
     if (c->precond) {
         c->oz_slot_bytes = oz_slice_bytes(c->ld, c->ld, c->oz_s);
-        per_slot_bytes += 3 * mat * sizeof(double) + 2 * mat * sizeof(float) + 2 * c->oz_slot_bytes +
-                          2 * oz_exp_ints(c->ld) * sizeof(int);
+        per_slot_bytes += 4 * mat * sizeof(double) + 2 * mat * sizeof(float) +
+                          jacobi32_diag_floats(c->ld) * sizeof(float) + 4 * c->oz_slot_bytes +
+                          4 * oz_exp_ints(c->ld) * sizeof(int);
     }
     size_t free_b = 0, total_b = 0;
     CU(cudaMemGetInfo(&free_b, &total_b));
@@ -138,12 +140,13 @@ int alloc_slots(mpdo_ctx* c, int want) {
         CU(dalloc(&c->d_W0, (size_t)s * mat));
         CU(dalloc(&c->d_E, (size_t)s * mat));
         CU(dalloc(&c->d_Q, (size_t)s * mat));
+        CU(dalloc(&c->d_Zrot, (size_t)s * mat));
         CU(dalloc(&c->d_W32, (size_t)s * mat));
         CU(dalloc(&c->d_U32, (size_t)s * mat));
-        CU(dalloc(&c->d_oz_as, (size_t)s * c->oz_slot_bytes));
-        CU(dalloc(&c->d_oz_bs, (size_t)s * c->oz_slot_bytes));
-        CU(dalloc(&c->d_oz_ea, (size_t)s * oz_exp_ints(c->ld)));
-        CU(dalloc(&c->d_oz_eb, (size_t)s * oz_exp_ints(c->ld)));
+        CU(dalloc(&c->d_oz_as, (size_t)2 * s * c->oz_slot_bytes));
+        CU(dalloc(&c->d_oz_bs, (size_t)2 * s * c->oz_slot_bytes));
+        CU(dalloc(&c->d_oz_ea, (size_t)2 * s * oz_exp_ints(c->ld)));
+        CU(dalloc(&c->d_oz_eb, (size_t)2 * s * oz_exp_ints(c->ld)));
         CU(dalloc(&c->d_oz, (size_t)s));
     }
     return MPDO_OK;
@@ -246,6 +249,12 @@ void svd_buffers(mpdo_ctx* c, int s, OpDesc& d) {
     d.oz_bs = c->precond ? c->d_oz_bs + (size_t)s * c->oz_slot_bytes : nullptr;
     d.oz_ea = c->precond ? c->d_oz_ea + (size_t)s * oz_exp_ints(ld) : nullptr;
     d.oz_eb = c->precond ? c->d_oz_eb + (size_t)s * oz_exp_ints(ld) : nullptr;
+    const size_t z = (size_t)(c->slots + s);   // the second half serves Z
+    d.Z = c->precond ? c->d_Zrot + (size_t)s * mat : nullptr;
+    d.oz_as_z = c->precond ? c->d_oz_as + z * c->oz_slot_bytes : nullptr;
+    d.oz_bs_z = c->precond ? c->d_oz_bs + z * c->oz_slot_bytes : nullptr;
+    d.oz_ea_z = c->precond ? c->d_oz_ea + z * oz_exp_ints(ld) : nullptr;
+    d.oz_eb_z = c->precond ? c->d_oz_eb + z * oz_exp_ints(ld) : nullptr;
 }
 
 void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
@@ -263,9 +272,9 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.cr = dm[p + 2];
     d.m = 4 * d.cl;
     d.n = 4 * d.cr;
-    d.transposed = 0;                 // the QR step leaves min(m, n) rows of length n
+    d.transposed = use_qr32(c) && d.m > d.n;
     d.c = std::min(d.m, d.n);
-    d.L = d.n;
+    d.L = d.transposed ? d.m : d.n;   // rows of theta~^T, of Q^T theta~ or of R
     d.chi_max = c->chi_max[b];
     d.cutoff = c->cutoff[b];
     d.G = c->d_gates + ((size_t)b * c->n_ops + d.op) * 256;
@@ -275,7 +284,6 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.lam_left = p > 0 ? c->d_lam + ((size_t)b * N + (p - 1)) * cap : nullptr;
     d.lam_out = c->d_lam + ((size_t)b * N + p) * cap;
     d.thetap = c->d_thetap + (size_t)s * mat;
-    d.Z = nullptr;
     d.Acm = c->d_Z + (size_t)s * mat;
     d.Yk = c->d_Yk + (size_t)s * cap * ld;
     d.snorm = c->d_snorm + (size_t)s * 2 * ld;
@@ -283,26 +291,27 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.status = c->d_status + b;
     d.max_disc = c->d_maxdisc + b;
     d.rank_log = nullptr;
-    d.jb = tuned_block_rows(c, d.cl, d.cr, jacobi_block_rows(d.L, d.c, 8));
+    d.jb = d.transposed ? jacobi_block_rows(d.L + d.c, d.c, 8)
+                        : tuned_block_rows(c, d.cl, d.cr, jacobi_block_rows(d.L, d.c, 8));
     d.sweeps_out = c->d_sweeps + s;
     d.forced_k = 0;
     d.full_svd = c->full_svd ? 1 : 0;
     d.tape_V = nullptr;
     d.tape_s = nullptr;
     svd_buffers(c, s, d);
-    d.Zinit = nullptr;
 }
 
-cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st) {
+cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, bool with_z, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     // E = U U^T - I (~1e-6), then one orthogonalisation step: second order
-    // (Q = U - E U / 2, defect 3 E^2 / 4) on the mixed path, third order (defect
-    // 5 E^3 / 8, below FP64 rounding) on the FP64 path
+    // (Q = U - E U / 2, defect 3 E^2 / 4) on the mixed path, fourth order (defect
+    // 35 E^4 / 64, below FP64 rounding; the third order's 5 E^3 / 8 showed as 2e-13 in
+    // the entropies at chi 256) on the FP64 path
     std::vector<int> kinds = {OZ_E, OZ_Q, OZ_W};
     if (!c->mixed) kinds = {OZ_E, OZ_T4, OZ_T3, OZ_T2, OZ_W};
     for (int kind : kinds) {
         const cudaError_t e =
-            launch_oz_ops(d_desc, nops, first + kind, c->cap, c->oz_s, timeout_ns, st);
+            launch_oz_ops(d_desc, nops, first + kind, c->cap, c->oz_s, with_z && !first && kind == OZ_W, timeout_ns, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -310,14 +319,14 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
 
 int orthogonalise_kernels(const mpdo_ctx* c) { return (c->mixed ? 3 : 5) * kOzKernels; }
 
-cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, cudaStream_t st) {
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, bool with_z, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
-    const cudaError_t e = launch_orthogonalise(c, d_desc, nops, 0, st);
+    const cudaError_t e = launch_orthogonalise(c, d_desc, nops, 0, with_z, st);
     if (e != cudaSuccess) return e;
     if (!refine_on(c)) return cudaSuccess;
     // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
     const bool can = c->oz_s == 7 || tol >= 1e-12;
-    return launch_refine(d_desc, nops, c->cap, c->oz_s, can ? tol : 1e-12, can, timeout_ns, st);
+    return launch_refine(d_desc, nops, c->cap, c->oz_s, with_z, can ? tol : 1e-12, can, timeout_ns, st);
 }
 
 int svd_products_kernels(const mpdo_ctx* c) {
@@ -357,20 +366,17 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
     // QR of every theta~: its rows turned and graded go to W0
     {
         const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap);
-        // ops of the FP32 QR (q32) or of the FP64 column QR, each launch with all
-        // co-resident CTAs shared in proportion to the work
-        auto plan_qr = [&](bool q32, int slot, int& total, int*& dbase) -> int {
+        // FP32 QR (q32) or FP64 column QR: all co-resident CTAs shared in proportion to the work
+        const bool q32 = use_qr32(c);
+        auto plan_qr = [&](int slot, int& total, int*& dbase) -> int {
             std::vector<int> G(nops, 0);
             double wsum = 0.0;
-            auto takes = [&](int s) { return (c->precond && qr32_takes(c->h_desc[s].m, c->h_desc[s].n)) == q32; };
-            for (int s = 0; s < nops; ++s)
-                if (takes(s)) wsum += qwork[s];
+            for (int s = 0; s < nops; ++s) wsum += qwork[s];
             const int R = q32 ? c->qr32_resident : c->qr_resident, QW = qr_threads() / 32;
             total = 0;
             for (int s = 0; s < nops; ++s) {
-                if (!takes(s)) continue;
                 const OpDesc& d = c->h_desc[s];
-                const int need = q32 ? qr32_max_ctas(d.m) : std::max(1, (d.n + QW - 1) / QW);
+                const int need = q32 ? qr32_max_ctas(d.c) : std::max(1, (d.n + QW - 1) / QW);
                 const int g = (int)std::floor((double)R * qwork[s] / std::max(wsum, 1.0));
                 G[s] = std::max(1, std::min(need, g));
                 total += G[s];
@@ -424,15 +430,14 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
         } else {
             ProfScope p_qr(c, K_QR);
             int total = 0, *db = nullptr;
-            int rc = plan_qr(false, 2, total, db);
+            const int rc = plan_qr(2, total, db);
             if (rc) return rc;
-            out.qr_kernels = total > 0;
-            CU(launch_qr(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
-            if ((rc = plan_qr(true, 3, total, db))) return rc;
-            if (total > 0) {
+            if (q32) {
                 CU(launch_qr32(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
-                CU(launch_orthogonalise(c, c->d_desc, nops, OZ_FIRST, c->st));
-                out.qr_kernels += 1 + orthogonalise_kernels(c);
+                CU(launch_orthogonalise(c, c->d_desc, nops, OZ_FIRST, false, c->st));
+                out.qr_kernels = 1 + orthogonalise_kernels(c);
+            } else {
+                CU(launch_qr(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
             }
             p_qr.stop();
         }
@@ -449,7 +454,9 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
             out.gemm_flops += 2.0 * d.c * d.c * d.c * 2 + 2.0 * d.c * d.c * d.L;
         }
         ProfScope p_gemm(c, K_GEMM);
-        CU(launch_svd_products(c, c->d_desc, nops, tol, c->st));
+        bool with_z = false;
+        for (int s = 0; s < nops; ++s) with_z = with_z || c->h_desc[s].transposed;
+        CU(launch_svd_products(c, c->d_desc, nops, tol, with_z, c->st));
         p_gemm.stop();
     }
     ProfScope p_jac(c, K_JACOBI);
@@ -508,7 +515,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     ProfScope p_merge(c, K_MERGE);
     if (c->precond) {
-        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_s, false, timeout_ns, c->st));
         CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
     } else {
         CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
@@ -532,7 +539,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     p_tr.stop();
     ProfScope p_rec(c, K_RECON);
     if (c->precond)
-        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_s, timeout_ns, c->st));
+        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_s, false, timeout_ns, c->st));
     else
         CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
     p_rec.stop();

@@ -153,4 +153,15 @@ __device__ float kth_largest_f(F val, int c, int kk) {
     return __uint_as_float(x);
 }
 
+// Squared norm under which two rows need not be made orthogonal to one another, whatever
+// the margin below chi_max: the rows under it hold less than a thousandth of the weight
+// that the cutoff discards, and rotations among them leave that sum as it is, so the
+// rank and the kept rows do not depend on them (0: every row may be needed).  total is
+// the sum of all squared norms.  Bonds with a handful of kept rows out of tens are where
+// it counts: their tails, down to rounding level, kept the FP32 pass at 8 to 15 sweeps
+// and left one op in five of a grid's evolution to the FP64 pass.
+__device__ __forceinline__ double cutoff_floor(const OpDesc& d, double total) {
+    return d.full_svd || d.forced_k > 0 ? 0.0 : 1e-3 * fmin(fmax(d.cutoff, 0.0), 1.0) * total / d.c;
+}
+
 }  // namespace mpdo

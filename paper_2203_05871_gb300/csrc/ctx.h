@@ -94,7 +94,7 @@ struct mpdo_ctx {
     int *d_oz_ea = nullptr, *d_oz_eb = nullptr;             // [slots][4 chi_cap] their exponents
     mpdo::OzProblem* d_oz = nullptr;                        // [slots] problems of one launch
     size_t oz_slot_bytes = 0;
-    double *d_W0 = nullptr, *d_E = nullptr, *d_Q = nullptr;
+    double *d_W0 = nullptr, *d_E = nullptr, *d_Q = nullptr, *d_Zrot = nullptr;
     float *d_W32 = nullptr, *d_U32 = nullptr, *d_D32 = nullptr;
     mpdo::GemmDesc* d_gemm = nullptr;
     mpdo::GemmDesc* h_gemm = nullptr;   // pinned, [3][slots]
@@ -217,15 +217,17 @@ inline double fp64_jacobi_tol(const mpdo_ctx* c) {
 // path: the FP64 pass alone), whose sweeps the limit counts; the other stages
 // take the place of a handful of them.
 constexpr int kRefineMinSweeps = 16;
+// The FP32 QR serves every preconditioned SVD but those of the blocked-QR option.
+inline bool use_qr32(const mpdo_ctx* c) { return c->precond && !(c->mixed && c->cfg.qr_blocked && qrb_fits(c->cap)); }
 inline bool refine_on(const mpdo_ctx* c) { return c->precond && c->cfg.jacobi_max_sweeps >= kRefineMinSweeps; }
 
 // From the FP32-orthogonal U32: Q, orthogonal to FP64 accuracy, and W = Q W0; with
 // first = OZ_FIRST from the QR's Q^T: W0 = Q theta~.
-cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, cudaStream_t st);
+cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, bool with_z, cudaStream_t st);
 int orthogonalise_kernels(const mpdo_ctx* c);
 // The stages between the FP32 preconditioning pass and the FP64 Jacobi pass:
 // Q, the orthogonalised U32, W = Q W0, and the refinement of W's rows.
-cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, cudaStream_t st);
+cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, bool with_z, cudaStream_t st);
 // A chunk's SVDs, with the work of the stages whose flop counts depend on the route.
 struct SvdWork {
     double qr_flops = 0.0, gemm_flops = 0.0;

@@ -17,8 +17,11 @@
 // w_j / sqrt(x_j) with F_X^T F_X = X, and likewise F_Y; then eig(X Y) =
 // sv(F_X F_Y^T)^2, so a third Jacobi SVD, of C = F_X F_Y^T, gives the Schmidt
 // values s_k and OSEE = -sum_k p_k ln p_k with p_k = s_k^2 / sum s^2.
-// FP64 throughout: the Gram sweeps are batched FP64 GEMMs (gemm.cu), the SVDs
-// the FP64 pass of jacobi.cu at its strict tolerance sqrt(L) eps.  Squaring
+// FP64 throughout.  The Gram sweeps are batched products: on FP64 contexts exact
+// slice products on the tensor cores (oz_gemm.cu, seven slices), else FP64 GEMMs
+// (gemm.cu: 0.68 ms for X' at chi 256, where 16 CTAs share it, against 0.07 ms).
+// The SVDs end at the strict tolerance sqrt(L) eps, through a step's stages where
+// staged_svd says so, else in the FP64 pass of jacobi.cu alone.  Squaring
 // the bond matrix into X and Y costs accuracy only on the smallest p_k, at the
 // 1e-16 level of the largest, which moves the entropy by ~1e-14.
 #include <mpdo.h>
@@ -134,7 +137,8 @@ struct GqPlan {
     };
     std::vector<Launch> launches;
     void begin() { launches.push_back(Launch{g.size(), 0, 1, 1}); }
-    void add(const GemmDesc& d) {
+    void add(GemmDesc d, int* status) {
+        d.status = status;
         g.push_back(d);
         Launch& L = launches.back();
         ++L.count;
@@ -158,7 +162,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
             double* T = c->d_thetap + (size_t)(2 * i) * mat;
             // T[l][(s, r)] = sum_l' X[l][l'] B[l'][s][r]
             P.add(GemmDesc{l, 3 * cap + r, l, X, ld, 0, site_v(c, b, q), 4 * cap, f32, 0, T, 4 * cap, 1.0, 0.0,
-                           nullptr, 0, 0, 0, 0, 0});
+                           nullptr, 0, 0, 0, 0, 0}, c->d_status + b);
         }
         P.begin();
         for (int i = 0; i < m; ++i) {
@@ -168,7 +172,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
             double* T = c->d_thetap + (size_t)(2 * i) * mat;
             // X'[r][r'] = sum_{(l, s)} B[(l, s)][r] T[(l, s)][r']  (both (4 l) x r with row stride cap)
             P.add(GemmDesc{r, r, 4 * l, site_v(c, b, q), cap, f32, T, cap, 0, 0, X, ld, 1.0, 0.0, nullptr, 0, 0, 0, 1,
-                           1});
+                           1}, c->d_status + b);
         }
     }
 }
@@ -187,7 +191,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
             double* U = c->d_thetap + (size_t)(2 * i + 1) * mat;
             // U[(l, s)][r'] = sum_r B[(l, s)][r] Y[r][r']
             P.add(GemmDesc{4 * l, r, r, site_v(c, b, q), cap, f32, Y, ld, 0, 0, U, cap, 1.0, 0.0, nullptr, 0, 0, 0, 0,
-                           0});
+                           0}, c->d_status + b);
         }
         for (int s = 0; s < 4; ++s) {
             P.begin();
@@ -199,7 +203,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
                 const void* Bs = static_cast<const char*>(site_v(c, b, q)) + (size_t)s * cap * site_esize(c);
                 // Y'[l][l'] (+)= sum_r U[(l, s)][r] B[(l', s)][r]
                 P.add(GemmDesc{l, l, r, U + (size_t)s * cap, 4 * cap, 0, Bs, 4 * cap, f32, 1, Y, ld, 1.0,
-                               s > 0 ? 1.0 : 0.0, s > 0 ? Y : nullptr, ld, 0, 0, 0, 0});
+                               s > 0 ? 1.0 : 0.0, s > 0 ? Y : nullptr, ld, 0, 0, 0, 0}, c->d_status + b);
             }
         }
     }
@@ -215,8 +219,17 @@ int run_plan(mpdo_ctx* c, GqPlan& P) {
         c->gq_cap = P.g.size();
     }
     CU(cudaMemcpyAsync(c->d_gq, P.g.data(), sizeof(GemmDesc) * P.g.size(), cudaMemcpyHostToDevice, c->st));
-    for (const auto& L : P.launches)
-        if (L.count > 0) CU(launch_gemm(c->d_gq + L.first, L.count, L.max_m, L.max_n, false, c->st));
+    const bool tc = c->precond && c->oz_s == 7;
+    const OzScratch scr{static_cast<unsigned char*>(c->d_oz_as), static_cast<unsigned char*>(c->d_oz_bs), c->d_oz_ea,
+                        c->d_oz_eb, c->d_oz, c->oz_slot_bytes, oz_exp_ints(c->ld)};
+    const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
+    for (const auto& L : P.launches) {
+        if (L.count == 0) continue;
+        if (tc)
+            CU(launch_gemm_tc(c->d_gq + L.first, L.count, L.max_m, L.max_n, c->ld, scr, 7, timeout_ns, c->st));
+        else
+            CU(launch_gemm(c->d_gq + L.first, L.count, L.max_m, L.max_n, false, c->st));
+    }
     CU(cudaStreamSynchronize(c->st));   // the host descriptors are rebuilt by the next plan
     return MPDO_OK;
 }
@@ -385,7 +398,8 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
         const int step = staged ? 1 : 2;
         for (int s = 0; s < 2 * m; s += step)
             Pc.add(GemmDesc{chi2[s], chi2[s], chi2[s], F + (size_t)s * mat, ld, 0, F + (size_t)(s ^ 1) * mat, ld, 0,
-                            1, c->d_thetap + (size_t)s * mat, ld, 1.0, 0.0, nullptr, 0, 0, 0, 0, 0});
+                            1, c->d_thetap + (size_t)s * mat, ld, 1.0, 0.0, nullptr, 0, 0, 0, 0, 0},
+                   c->d_status + b0 + s / 2);
         rc = run_plan(c, Pc);
         if (rc) return rc;
         scale_kernel<<<dim3(64, staged ? 2 * m : m), 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, c->d_snorm, step);

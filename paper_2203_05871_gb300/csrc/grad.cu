@@ -370,7 +370,7 @@ int run_bwd_chunk(mpdo_ctx* c, GradState* g, const std::vector<const TapeRec*>& 
     auto gemm = [&](int q) {
         const bool tc = c->mixed && (q == 4 || q >= 6);
         return tc ? launch_gemm_tc(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], mx[q][2], g->oz,
-                                   timeout_ns, c->st)
+                                   6, timeout_ns, c->st)
                   : launch_gemm(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], false, c->st);
     };
     CU(launch_copy2d(g->d_bc, 2 * nops, max_pack, c->st));

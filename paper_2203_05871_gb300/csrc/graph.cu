@@ -70,7 +70,8 @@ __device__ int plan_ctas(const double* work, const int* cap, int nops, int R, in
 constexpr int kMaxChunk = 1024;
 
 __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops, const int* dims, int N, int Rj,
-                                                         int Rq, int* cta64, int* cta32, int* ctaqr, int* ctaq32, int Rq32, int precond, int blocked,
+                                                         int Rq, int* cta64, int* cta32, int* ctaqr, int* ctaq32, int Rq32, int precond, int q32,
+                                                         int blocked,
                                                          const int* jb_table, int chi_cap, int* error) {
     __shared__ double work[kMaxChunk];
     __shared__ int cap[kMaxChunk];
@@ -82,10 +83,11 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
         d.cr = dm[d.p + 2];
         d.m = 4 * d.cl;
         d.n = 4 * d.cr;
+        d.transposed = q32 && d.m > d.n;
         d.c = min(d.m, d.n);
-        d.L = d.n;
-        d.jb = jacobi_block_rows(d.L, d.c, 8);
-        if (jb_table) {   // autotuned rows per block of this (chi_l, chi_r) class
+        d.L = d.transposed ? d.m : d.n;
+        d.jb = jacobi_block_rows(d.transposed ? d.L + d.c : d.L, d.c, 8);
+        if (jb_table && !d.transposed) {   // autotuned rows per block of this (chi_l, chi_r) class
             const int t = jb_table[(size_t)d.cl * (chi_cap + 1) + d.cr];
             if (t > 0) d.jb = t;
         }
@@ -106,13 +108,9 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
     for (int s = 0; s < nops; ++s) {
         const OpDesc& d = descs[s];
         work[s] = (double)d.m * d.n * d.c;
-        cap[s] = precond && qr32_takes(d.m, d.n) ? 0 : max(1, (d.n + kQrWarps - 1) / kQrWarps);
+        cap[s] = q32 ? qr32_max_ctas(d.c) : max(1, (d.n + kQrWarps - 1) / kQrWarps);
     }
-    if (!blocked) bad |= plan_ctas(work, cap, nops, Rq, ctaqr);
-    if (precond && !blocked) {
-        for (int s = 0; s < nops; ++s) cap[s] = cap[s] == 0 ? qr32_max_ctas(descs[s].m) : 0;
-        bad |= plan_ctas(work, cap, nops, Rq32, ctaq32);
-    }
+    if (!blocked) bad |= plan_ctas(work, cap, nops, q32 ? Rq32 : Rq, q32 ? ctaq32 : ctaqr);
     if (bad) *error = 1;
 }
 
@@ -168,17 +166,18 @@ void release(GraphState* g) {
 int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
     const int cap = c->cap, ld = c->ld;
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
-    const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap);
+    const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap), q32 = use_qr32(c);
     for (auto& L : g->chunks)
         for (auto& ch : L) {
             const int nops = ch.nops;
             plan_chunk_kernel<<<1, 256, 0, st>>>(ch.d_desc, nops, c->d_dims, c->N, g->Rj, g->Rq, ch.d_cta64,
-                                                 ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, g->Rq32, c->precond ? 1 : 0, blocked ? 1 : 0, c->d_jb_table, cap,
+                                                 ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, g->Rq32,
+                                                 c->precond ? 1 : 0, q32 ? 1 : 0, blocked ? 1 : 0, c->d_jb_table, cap,
                                                  g->d_error);
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
             if (c->precond) {
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, cap, c->oz_s, timeout_ns, st));
+                CU(launch_oz_ops(ch.d_desc, nops, OZ_MERGE, cap, c->oz_s, false, timeout_ns, st));
                 CU(launch_gate_weight(ch.d_desc, nops, cap, st));
             } else {
                 CU(launch_merge_gate(ch.d_desc, nops, cap, st));
@@ -187,28 +186,26 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
             if (blocked) {
                 CU(launch_qr_blocked(ch.d_desc, nops, cap, c->d_oz, timeout_ns, st, 0));
+            } else if (q32) {
+                CU(launch_qr32(ch.d_desc, ch.d_ctaq32, ch.d_ctaq32 + g->Rq32, ch.d_ctaq32 + 2 * g->Rq32, c->d_sync,
+                               g->Rq32, timeout_ns, ld, st));
+                CU(launch_orthogonalise(c, ch.d_desc, nops, OZ_FIRST, false, st));
             } else {
                 CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
                              timeout_ns, ld, st));
-                if (c->precond) {
-                    CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
-                    CU(launch_qr32(ch.d_desc, ch.d_ctaq32, ch.d_ctaq32 + g->Rq32, ch.d_ctaq32 + 2 * g->Rq32,
-                                   c->d_sync, g->Rq32, timeout_ns, ld, st));
-                    CU(launch_orthogonalise(c, ch.d_desc, nops, OZ_FIRST, st));
-                }
             }
             if (c->precond) {
                 CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
                 CU(launch_jacobi(ch.d_desc, nops, ch.d_cta32, ch.d_cta32 + g->Rj, ch.d_cta32 + 2 * g->Rj, c->d_sync,
                                  g->Rj, kMaxSweepsCap / 2, 0.0, timeout_ns, ld, true, st, precond_rho(c)));
-                CU(launch_svd_products(c, ch.d_desc, nops, fp64_jacobi_tol(c), st));
+                CU(launch_svd_products(c, ch.d_desc, nops, fp64_jacobi_tol(c), q32, st));
             }
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
             CU(launch_jacobi(ch.d_desc, nops, ch.d_cta64, ch.d_cta64 + g->Rj, ch.d_cta64 + 2 * g->Rj, c->d_sync, g->Rj,
                              c->cfg.jacobi_max_sweeps, fp64_jacobi_tol(c), timeout_ns, ld, false, st, precond_rho(c)));
             CU(launch_truncate(ch.d_desc, nops, cap, st));
             if (c->precond)
-                CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, cap, c->oz_s, timeout_ns, st));
+                CU(launch_oz_ops(ch.d_desc, nops, OZ_RECON, cap, c->oz_s, false, timeout_ns, st));
             else
                 CU(launch_reconstruct(ch.d_desc, nops, cap, st));
             klog_kernel<<<(nops + 127) / 128, 128, 0, st>>>(ch.d_desc, nops, c->n_ops, g->d_klog);

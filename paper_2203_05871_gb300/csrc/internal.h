@@ -43,7 +43,7 @@ struct OpDesc {
     int p;             // left path position
     int cl, cm, cr;    // bond dims chi_{p-1}, chi_p, chi_{p+1}
     int m, n;          // 4*cl, 4*cr
-    int transposed;    // 1: Jacobi rows carry a c x c accumulator Z (unused since the QR step)
+    int transposed;    // 1 (m > n, preconditioning stages): the SVD is that of theta~^T, and Z carries its rotations
     int c, L;          // Jacobi problem: c rows of length L
     int jb;            // Jacobi block size (rows per shared-memory block), FP64 pass
     int chi_max;
@@ -55,11 +55,10 @@ struct OpDesc {
     const double* lam_left;  // lambda_{p-1} (nullptr => 1)
     double* lam_out;   // lambda_p
     double* thetap;    // Theta'  m x n (ld)
-    double* Acm;       // theta~ column-major (column k at Acm + k*ld), input of the QR
+    double* Acm;       // theta~ (transposed: theta~^T) column-major (column k at Acm + k*ld), input of the QR
     double* W0;        // rows from the QR (== W without the preconditioning stages)
     double* W;         // Jacobi rows: theta~ (m x n) or theta~^T (n x m)
-    double* Z;         // c x c rotation accumulator when transposed
-    const double* Zinit;  // initial Z (nullptr => identity)
+    double* Z;         // transposed: c x c, all rotations so far; its rows become the right singular vectors
     // the preconditioning stages (mixed contexts, FP64 ones with a sweep limit >= 16):
     float* W32;        // FP32 rows of the preconditioning Jacobi (c x L)
     float* U32;        // FP32 accumulated rotations (c x c), first the FP32 QR's Q^T
@@ -83,6 +82,8 @@ struct OpDesc {
     double* tape_s;    // adjoint recompute: all c sorted singular values
     void *oz_as, *oz_bs;   // slice blocks of the tensor-core products (oz_gemm.cu)
     int *oz_ea, *oz_eb;    // and their row / column exponents
+    void *oz_as_z, *oz_bs_z;   // the same for the products on Z
+    int *oz_ea_z, *oz_eb_z;
 };
 
 // Launch of a kernel that begins with grid_begin(): its CTAs may be scheduled while the
@@ -244,14 +245,15 @@ cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int m
 // device from the op descriptors (so the host-planned and the graph step
 // share them): kind OZ_MERGE Theta = A B (then launch_gate_weight applies the
 // gate and the left weights), OZ_RECON B_p' = Theta' Yk^T, OZ_E E = U U^T - I,
-// OZ_Q Q = U - E U / 2, OZ_W W = Q W0; OZ_T T = U - 3 E U / 4 then OZ_Q3
-// Q = U - E T / 2 (third-order orthogonalisation); OZ_G G = W W^T and OZ_R3,
-// OZ_R2, OZ_R1 the refinement's rotation (refine.cu).
-// OZ_FIRST + OZ_E, OZ_Q, OZ_T, OZ_Q3, OZ_W: the same on the QR's Q^T (ops of qr32_takes
-// only), OZ_W then being W0 = Q theta~.
+// OZ_Q Q = U - E U / 2, OZ_W W = Q W0; OZ_T4 T = U - 5 E U / 6, OZ_T3 T = U - 3 E T / 4
+// and OZ_T2 Q = U - E T / 2 (fourth-order orthogonalisation); OZ_G G = W W^T and
+// OZ_R3, OZ_R2, OZ_R1 the refinement's rotation (refine.cu).
+// OZ_FIRST + OZ_E, OZ_Q, OZ_T4, OZ_T3, OZ_T2, OZ_W: the same on the QR's Q^T, OZ_W then
+// being W0 = Q theta~ (transposed ops: theta~^T, and Q is Z's first value).
+// with_z: the products that turn W (OZ_W, OZ_R*) also turn Z of the transposed ops.
 enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T4 = 5, OZ_T3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
        OZ_R1 = 10, OZ_T2 = 11 };
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S,
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S, bool with_z,
                           unsigned long long timeout_ns, cudaStream_t st);
 constexpr int kOzKernels = 2;   // kernels of one launch_oz_ops
 // ---------------------------------------------------------------------------
@@ -264,19 +266,21 @@ struct RefineOp {
     int order;        // terms of this iteration's rotation (0: none)
     unsigned rho2;    // largest g^2 / (a b) of a needed pair (float bits)
     int far;          // a needed pair's angle is beyond the expansion
+    int turn;         // some such pairs are turned exactly in this iteration
     unsigned blocks;  // CTAs of the X kernel that are done
     unsigned row1;    // largest absolute row sum of X (float bits)
-    double thr;       // pairs of rows whose squared norms are both below it are not needed
+    double thr;       // the (chi_max + margin)-th largest squared norm, once settled
+    double need;      // pairs of rows whose squared norms are both below it are not needed
     double floor2;    // squared norm of a numerically zero row
 };
 // The iterations of a chunk: W's rows, as orthogonal as the FP32 pass left them, are
 // rotated until every needed pair is orthogonal to tol (state kRefineDone) or the
 // op is left to the Jacobi pass.  Scratch: d.E (G), d.Q (X), d.W0, d.snorm.
 // tol_in as for launch_jacobi; can_finish = false: never kRefineDone.
-cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
-constexpr int kRefineIters = 3;
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, bool with_z, double tol_in, bool can_finish, unsigned long long timeout_ns, cudaStream_t st);
+constexpr int kRefineIters = 4;
 // kernels of one launch_refine
-constexpr int kRefineKernels = kRefineIters * (2 + 4 * kOzKernels);
+constexpr int kRefineKernels = kRefineIters * (3 + 4 * kOzKernels);
 
 // Theta' = G Theta in place in thetap and theta~ = lambda_l Theta' (column-major, Acm)
 cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st);
@@ -297,10 +301,9 @@ cudaError_t qrb_prepare();
 cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs,
                               unsigned long long timeout_ns, cudaStream_t st, int r_max);
 
-// FP32 Householder QR (qr32.cu) of the preconditioned SVD's ops with m <= n: Q^T into
-// U32 (m x m), the row order of W0 = Q^T theta~ graded.  Wider panels than one CTA
+// FP32 Householder QR (qr32.cu) of the preconditioned SVD: Q^T (c x c) into U32, the
+// row order of W0 = Q^T theta~ (or Q^T theta~^T) graded.  Wider panels than one CTA
 // per 16 rows would leave CTAs without a tile to update.
-__host__ __device__ inline bool qr32_takes(int m, int n) { return m <= n; }
 __host__ __device__ inline int qr32_max_ctas(int m) { return (m + 15) / 16; }
 cudaError_t qr32_max_resident(int* blocks);
 cudaError_t launch_qr32(const OpDesc* d_desc, const int* d_cta_op, const int* d_cta_rank, const int* d_group,
@@ -331,8 +334,7 @@ struct GemmDesc {
 };
 cudaError_t launch_gemm(const GemmDesc* d_desc, int count, int max_m, int max_n, bool fp32_compute,
                         cudaStream_t st);
-// The batched GemmDesc products (f64 operands, sym computed in full) on the
-// tensor cores: problem s takes slot s of the scratch (slices of slot_bytes per
+// The batched GemmDesc products (f64 operands; S slices) on the tensor cores: problem s takes slot s of the scratch (slices of slot_bytes per
 // operand, exponents of exp_ints per operand, oz_slice_bytes / oz_exp_ints of
 // the largest dimension) and probs[s]; max_m, max_n, max_k bound every product.
 struct OzScratch {
@@ -342,7 +344,7 @@ struct OzScratch {
     size_t slot_bytes, exp_ints;
 };
 cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max_n, int max_k, const OzScratch& scr,
-                           unsigned long long timeout_ns, cudaStream_t st);
+                           int S, unsigned long long timeout_ns, cudaStream_t st);
 
 cudaError_t launch_trace_normalize(void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap,
                                    int force, double* trace_out, int* status, cudaStream_t st);

@@ -1,9 +1,8 @@
 // FP64 one-sided (Hestenes) Jacobi SVD of the bond matrices of one layer.
 //
 // App. B compresses |rho>> bond by bond from its Schmidt spectrum.  Each op
-// hands this kernel c rows of length L (the rows of theta~ when m <= n, or
-// its columns when m > n, then with a c x c accumulator Z whose rows turn
-// alongside).  Plane rotations from the left make the rows mutually
+// hands this kernel c rows of length L (those of theta~ or of R, or of theta~^T when
+// m > n, then with the c x c rotations so far, Z, whose rows turn alongside).  Plane rotations from the left make the rows mutually
 // orthogonal; row j then equals s_j v_j^T (or Z row j = v_j^T), which the
 // truncation step reads.
 //
@@ -267,6 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
     double* dscale = d.snorm + ld;   // per-row scales (the QR's column norms are dead here)
     C.rho2 = &s_rho2;
     C.thr = 0.0;
+    double kth = 0.0;
     float rho2_stop;
     {
         const double tol = tol_in > 0.0 ? tol_in : sqrt((double)(L > 1 ? L : 1)) * DBL_EPSILON;
@@ -302,12 +302,6 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
         }
         __syncthreads();
     }
-    // initial Z (identity, or Zinit)
-    if (Z)
-        for (int row = g * kWarps + warp; row < c; row += G * kWarps)
-            for (int i = lane; i < c; i += 32)
-                __stcg(Z + (size_t)row * ld + i,
-                       d.Zinit ? __ldcg(d.Zinit + (size_t)row * ld + i) : (i == row ? 1.0 : 0.0));
     C.floor2 = s_floor2;
     if (!op_barrier(sw, G, gen, timeout_ns)) goto timeout;
     {
@@ -353,7 +347,8 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
             // the threshold is fixed when the gate first opens, so that a row
             // near it keeps its side (a row changing side later would bring its
             // unprocessed pairs back and cost another sweep)
-            if (s_conv && C.thr == 0.0) C.thr = kth_largest<kThreads, 4 * kMaxChi>(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
+            if (s_conv && kth == 0.0) kth = kth_largest<kThreads, 4 * kMaxChi>(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
+            C.thr = fmax(kth, cutoff_floor(d, s_floor2 / (DBL_EPSILON * DBL_EPSILON)));
             __syncthreads();
             // The block pairs of a sweep go to the op's CTAs through a shared
             // counter (position q: round q / npair, pair q % npair), and a round

@@ -525,6 +525,7 @@ __global__ void __launch_bounds__(NT, 1) jacobi32_kernel(const OpDesc* descs, co
                                      },
                                      c, kk);
             }
+            lm.lim = fmaxf(lm.lim, (float)cutoff_floor(d, (double)c));   // rows of unit mean square norm
             if (rank == 0 && threadIdx.x == 0) atomicExch(&sw[kSwQueue + ((sweep + 1) & 1)], 0u);
             int next = 0;
             for (;;) {

@@ -325,18 +325,18 @@ __device__ __forceinline__ void slice_group(const long long* X, bool nan, uint4*
 struct OzSource {
     const OzProblem* probs;
     const OpDesc* descs;
-    int kind, cap;
-    OzProblem one;   // neither: this one problem
+    int kind, cap, nops;   // problems nops .. 2 nops - 1: the same product on Z
+    OzProblem one;         // neither: this one problem
 };
 
-// The problem of one kind for an op.
+// The problem of one kind for an op (z: of the same product on Z).
 template <int kS>
-__device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
+__device__ OzProblem op_problem(const OpDesc& d, int kind, int cap, bool z) {
     const int ld = 4 * cap;
     OzProblem P{};
     const bool first = (kind & OZ_FIRST) != 0;
     kind &= OZ_FIRST - 1;
-    if (first && !qr32_takes(d.m, d.n)) kind = -1;
+    if (z && !d.transposed) kind = -1;
     auto rowmajor = [](const void* base, int f32, long long ld_) {   // (r, k) at r * ld + k
         return OzOperand{base, f32, ld_, 1, 0, 1, 1, nullptr, nullptr, 0};
     };
@@ -380,7 +380,7 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
             P.M = P.N = P.K = d.c;
             P.A = rowmajor(d.E, 0, ld);
             P.B = kind == OZ_T3 || kind == OZ_T2 ? colmajor(d.W, 0, ld) : colmajor(d.U32, 1, ld);
-            P.C = kind == OZ_T4 || kind == OZ_T3 ? d.W : d.Q;
+            P.C = kind == OZ_T4 || kind == OZ_T3 ? d.W : first && d.transposed ? d.Z : d.Q;
             P.ldc = ld;
             P.alpha = kind == OZ_T4 ? -5.0 / 6.0 : kind == OZ_T3 ? -0.75 : -0.5;
             P.beta = 1.0;
@@ -406,41 +406,46 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap) {
             const int order = d.rf->order;
             if (order < (kind == OZ_R3 ? 3 : kind == OZ_R2 ? 2 : 1)) break;
             P.M = P.K = d.c;
-            P.N = d.L;
+            P.N = z ? d.c : d.L;
             P.A = rowmajor(d.Q, 0, ld);
             const bool fromT = (kind == OZ_R2 && order == 3) || (kind == OZ_R1 && order >= 2);
-            P.B = colmajor(fromT ? d.W0 : d.W, 0, ld);
-            P.A.kn = P.B.kn = d.snorm;   // squared row norms of W: X_ik |w_k| times w_k / |w_k|
-            P.A.ksgn = 1;
-            P.B.ksgn = -1;
-            P.C = kind == OZ_R1 ? d.W : d.W0;
+            double *X = z ? d.Z : d.W, *T = z ? d.Acm : d.W0;   // Acm is free once W0 is formed
+            P.B = colmajor(fromT ? T : X, 0, ld);
+            P.C = kind == OZ_R1 ? X : T;
             P.ldc = ld;
-            P.D = d.W;
+            P.D = X;
             P.ldd = ld;
-            // what X W adds to a row of W is below 2^e of it, e from the largest angle
-            // and the largest off-orthogonality: that many digits fewer are needed
-            P.levels = oz_levels(kS, max((int)(d.rf->row1 >> 23) - 126, ((int)(d.rf->rho2 >> 23) - 126) / 2 + 1));
+            if (z) {
+                P.unit_d = 1;
+            } else {
+                P.A.kn = P.B.kn = d.snorm;   // squared row norms of W: X_ik |w_k| times w_k / |w_k|
+                P.A.ksgn = 1;
+                P.B.ksgn = -1;
+                // what X W adds to a row of W is below 2^e of it, e from the largest angle
+                // and the largest off-orthogonality: that many digits fewer are needed
+                P.levels = oz_levels(kS, max((int)(d.rf->row1 >> 23) - 126, ((int)(d.rf->rho2 >> 23) - 126) / 2 + 1));
+            }
             P.alpha = kind == OZ_R3 ? 0.125 : (kind == OZ_R2 && order == 2 ? 0.5 : 1.0);
             P.beta = kind == OZ_R3 ? 0.5 : 1.0;
             break;
         }
         case OZ_W:       // W = Q W0 (first: W0 = Q theta~, theta~ column-major)
             P.M = d.c;
-            P.N = d.L;
+            P.N = z ? d.c : d.L;
             P.K = d.c;
-            P.A = rowmajor(d.Q, 0, ld);
-            P.B = first ? rowmajor(d.Acm, 0, ld) : colmajor(d.W0, 0, ld);
-            P.C = first ? d.W0 : d.W;
+            P.A = rowmajor(first && d.transposed ? d.Z : d.Q, 0, ld);
+            P.B = first ? rowmajor(d.Acm, 0, ld) : colmajor(z ? d.Z : d.W0, 0, ld);
+            P.C = z ? d.Z : first ? d.W0 : d.W;
             P.ldc = ld;
             break;
         default:         // an op that takes no part
             break;
     }
     if (kind == OZ_MERGE || kind == OZ_RECON || kind == OZ_E || kind == OZ_W) P.alpha = 1.0;
-    P.as = d.oz_as;
-    P.bs = d.oz_bs;
-    P.ea = d.oz_ea;
-    P.eb = d.oz_eb;
+    P.as = z ? d.oz_as_z : d.oz_as;
+    P.bs = z ? d.oz_bs_z : d.oz_bs;
+    P.ea = z ? d.oz_ea_z : d.oz_ea;
+    P.eb = z ? d.oz_eb_z : d.oz_eb;
     P.status = d.status;
     oz_set_tiles(P);
     return P;
@@ -452,10 +457,11 @@ template <int kS>
 __device__ __forceinline__ void fetch_problem(const OzSource& src, OzProblem& P) {
     if (src.descs) {
         __shared__ __align__(16) int sd[sizeof(OpDesc) / 4];
-        const int* g = reinterpret_cast<const int*>(src.descs + blockIdx.z);
+        const bool z = (int)blockIdx.z >= src.nops;
+        const int* g = reinterpret_cast<const int*>(src.descs + (z ? blockIdx.z - src.nops : blockIdx.z));
         for (int i = threadIdx.x; i < (int)(sizeof(OpDesc) / 4); i += blockDim.x) sd[i] = g[i];
         __syncthreads();
-        if (threadIdx.x == 0) P = op_problem<kS>(*reinterpret_cast<const OpDesc*>(sd), src.kind, src.cap);
+        if (threadIdx.x == 0) P = op_problem<kS>(*reinterpret_cast<const OpDesc*>(sd), src.kind, src.cap, z);
     } else if (threadIdx.x == 0) {
         P = src.probs ? src.probs[blockIdx.z] : src.one;
     }
@@ -464,33 +470,47 @@ __device__ __forceinline__ void fetch_problem(const OzSource& src, OzProblem& P)
 
 static_assert(sizeof(OpDesc) % 4 == 0, "copied as words");
 
-// Strided views (a transposed operand, the right site of a merge): a block
-// takes 32 consecutive rows, lane = row and warp = a slice of the K range, so
-// that the 32 lanes of a load read 32 neighbouring rows at one k (coalesced).
+// the largest |x| key of elements k0, k0 + step, ... of row r, eight loads in flight
+__device__ __forceinline__ unsigned long long row_max(const OzOperand& X, int r, int k0, int step, int K) {
+    const bool f32 = X.f32 != 0;
+    unsigned long long mx = 0;
+    for (int k = k0; k < K; k += 8 * step) {
+        unsigned long long b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) b[u] = k + u * step < K ? oz_bits(X, r, k + u * step) : 0ull;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const unsigned long long key = abs_key(b[u], f32);
+            mx = key > mx ? key : mx;
+        }
+    }
+    return mx;
+}
+
+// Strided views (a transposed operand, the right site of a merge): four blocks
+// take 32 consecutive rows, lane = row and warp = a slice of the K range, so that
+// the 32 lanes of a load read 32 neighbouring rows at one k (coalesced).  Each block
+// scans all of K for the rows' exponents and cuts a quarter of it (one block per 32
+// rows left a product of 1000 x 1500 x 777 with 47 of them and 107 us of slicing).
 template <int kS>
-__device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int Kt, int lv, unsigned char* out, int* ex,
-                                 int tile, int Rt) {
+__device__ void slice_rows_tiled(const OzOperand& X, int r0, int quarter, int R, int K, int Kt, int lv,
+                                 unsigned char* out, int* ex, int tile, int Rt) {
     __shared__ unsigned long long s_mx[8][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool f32 = X.f32 != 0;
     const int r = r0 + lane;
     const bool live = r < R;
-    unsigned long long mx = 0;
-    if (live)
-        for (int k = warp; k < K; k += 8) {
-            const unsigned long long key = abs_key(oz_bits(X, r, k), f32);
-            mx = key > mx ? key : mx;
-        }
+    unsigned long long mx = live ? row_max(X, r, warp, 8, K) : 0;
     s_mx[warp][lane] = mx;
     __syncthreads();
     for (int w = 0; w < 8; ++w) mx = s_mx[w][lane] > mx ? s_mx[w][lane] : mx;
     const bool bad = key_nonfinite(mx, f32);   // the largest key of a row with a NaN or an inf is one
     const int e = bad ? 0 : key_exponent(mx, f32);
-    if (warp == 0) ex[r] = e;
+    if (warp == 0 && quarter == 0) ex[r] = e;
     const int rt = r / tile, rr = r % tile;
     const size_t block = (size_t)tile * 64;
     const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
-    for (int g0 = warp * G; g0 < Kt * KT; g0 += 8 * G) {
+    for (int g0 = (quarter * 8 + warp) * G; g0 < Kt * KT; g0 += 32 * G) {
         long long x[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -511,7 +531,7 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int R, int K, int K
 
 // grid (row groups of 8, 2 = A | B, problems).  Views whose rows are
 // contiguous (ks == 1) take one warp per row, lanes along k; the others 32 rows
-// per block (slice_rows_tiled), the blocks past rows / 32 returning at once.
+// per four blocks (slice_rows_tiled).
 template <int kS>
 __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     __shared__ OzProblem P;
@@ -529,21 +549,16 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     unsigned char* out = static_cast<unsigned char*>(isB ? P.bs : P.as);
     int* ex = isB ? P.eb : P.ea;
     if (!(X.mode == 0 && X.ks == 1)) {
-        const int r0 = blockIdx.x * 32;
+        const int r0 = (blockIdx.x >> 2) * 32;
         if (r0 >= Rt * tile) return;   // uniform over the block (Rt * tile is a multiple of 32)
-        slice_rows_tiled<kS>(X, r0, R, K, Kt, lv, out, ex, tile, Rt);
+        slice_rows_tiled<kS>(X, r0, blockIdx.x & 3, R, K, Kt, lv, out, ex, tile, Rt);
         return;
     }
     const int r = blockIdx.x * 8 + warp;
     if (r >= Rt * tile) return;
     const bool live = r < R;
     const bool f32 = X.f32 != 0;
-    unsigned long long mx = 0;
-    if (live)
-        for (int k = lane; k < K; k += 32) {
-            const unsigned long long key = abs_key(oz_bits(X, r, k), f32);
-            mx = key > mx ? key : mx;
-        }
+    unsigned long long mx = live ? row_max(X, r, lane, 32, K) : 0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -804,7 +819,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
 }
 
 // Theta' = G Theta in place (rows (l, s1), columns s2 cr + r) and theta~ =
-// lambda_{p-1}[l] Theta' column-major in Acm; one thread per (l, r).
+// lambda_{p-1}[l] Theta' (transposed: theta~^T) column-major in Acm; one thread per (l, r).
 __global__ void __launch_bounds__(256) gate_weight_kernel(const OpDesc* descs, int chi_cap) {
     const OpDesc& d = descs[blockIdx.y];
     __shared__ double Gs[256];
@@ -825,7 +840,7 @@ __global__ void __launch_bounds__(256) gate_weight_kernel(const OpDesc* descs, i
         for (int i = 0; i < 16; ++i) v = fma(Gs[o * 16 + i], th[i], v);
         const int row = l * 4 + (o >> 2), col = (o & 3) * d.cr + r;
         d.thetap[(size_t)row * ld + col] = v;
-        d.Acm[(size_t)col * ld + row] = lam * v;
+        d.Acm[d.transposed ? (size_t)row * ld + col : (size_t)col * ld + row] = lam * v;
     }
 }
 
@@ -900,14 +915,15 @@ cudaError_t launch_oz_source(const OzSource& src, int count, int max_m, int max_
 
 cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced, int S,
                            unsigned long long timeout_ns, cudaStream_t st) {
-    return launch_oz_source(OzSource{d_probs, nullptr, 0, 0, {}}, count, max_m, max_n, max_rows_sliced, S,
+    return launch_oz_source(OzSource{d_probs, nullptr, 0, 0, 0, {}}, count, max_m, max_n, max_rows_sliced, S,
                             timeout_ns, st);
 }
 
-cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S,
+cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S, bool with_z,
                           unsigned long long timeout_ns, cudaStream_t st) {
     const int big = 4 * chi_cap;
-    return launch_oz_source(OzSource{nullptr, d_desc, kind, chi_cap, {}}, nops, big, big, big, S, timeout_ns, st);
+    return launch_oz_source(OzSource{nullptr, d_desc, kind, chi_cap, nops, {}}, with_z ? 2 * nops : nops, big, big, big,
+                            S, timeout_ns, st);
 }
 
 namespace {
@@ -935,6 +951,7 @@ __global__ void gemm_desc_oz_kernel(const GemmDesc* descs, int count, OzScratch 
     P.ldd = d.ldd;
     P.d_f32 = d.d_f32;
     P.sub_identity = d.sub_identity;
+    P.sym = d.sym;
     P.as = scr.as + (size_t)s * scr.slot_bytes;
     P.bs = scr.bs + (size_t)s * scr.slot_bytes;
     P.ea = scr.ea + (size_t)s * scr.exp_ints;
@@ -947,16 +964,16 @@ __global__ void gemm_desc_oz_kernel(const GemmDesc* descs, int count, OzScratch 
 }  // namespace
 
 cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max_n, int max_k, const OzScratch& scr,
-                           unsigned long long timeout_ns, cudaStream_t st) {
+                           int S, unsigned long long timeout_ns, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     // every operand must fit its slot
     const int big = max_m > max_n ? max_m : max_n;
-    if (oz_slice_bytes(big, max_k, 6) > scr.slot_bytes || oz_exp_ints(big) > scr.exp_ints)
+    if (oz_slice_bytes(big, max_k, S) > scr.slot_bytes || oz_exp_ints(big) > scr.exp_ints)
         return cudaErrorInvalidValue;
     gemm_desc_oz_kernel<<<(count + 127) / 128, 128, 0, st>>>(d_desc, count, scr);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_oz_gemm(scr.probs, count, max_m, max_n, big, 6, timeout_ns, st);
+    return launch_oz_gemm(scr.probs, count, max_m, max_n, big, S, timeout_ns, st);
 }
 
 }  // namespace mpdo

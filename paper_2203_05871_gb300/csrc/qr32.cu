@@ -1,14 +1,18 @@
-// FP32 Householder QR of the weighted bond matrices with m <= n: the orthogonal
-// start of the SVD.
+// FP32 Householder QR of the weighted bond matrices: the orthogonal start of the
+// SVD.
 //
-// The SVD needs the rows of theta~ (m x n) turned by an orthogonal matrix that
-// grades them (qr.cu says why: Jacobi then converges in a third of the sweeps).
-// Any such matrix will do as long as it is orthogonal to FP64 accuracy when it is
-// applied, so it is found in FP32: A_1, the m columns of theta~ of largest norm in
-// that order, is factored A_1 = Q R by blocked Householder reflections, Q^T is
+// The SVD needs the rows of theta~ (m x n, m <= n; theta~^T otherwise) turned by an
+// orthogonal matrix that grades them (qr.cu says why: Jacobi then converges in a
+// third of the sweeps).  Any such matrix will do as long as it is orthogonal to
+// FP64 accuracy when it is applied, so it is found in FP32: A_1, the m columns of
+// largest norm in that order with the other n - m folded onto them (from the last
+// on; alone, the rows of theta~ of largest weight can leave out whole directions:
+// a third more Jacobi sweeps on some), is factored A_1 = Q R by blocked Householder
+// reflections, Q^T is
 // accumulated explicitly in U32, and the tensor-core products (api.cu) then
 // orthogonalise it (E = U U^T - I, one step) and form W0 = Q^T theta~ in FP64
-// accuracy.  W0's rows are graded like those of R down to FP32 rounding of the
+// accuracy.  (theta~^T is turned as it is, Z following along: R alone would need
+// the factorisation itself to be accurate to FP64.)  W0's rows are graded like those of R down to FP32 rounding of the
 // largest; below that they are resolved by the FP32 Jacobi pass that follows,
 // which sees them as they are.
 // Sorting the columns once by norm replaces pivoting at every column: on the
@@ -299,7 +303,7 @@ __global__ void __launch_bounds__(NT, 1) qr32_kernel(const OpDesc* descs, const 
     const int G = group[op];
     const OpDesc& d = descs[op];
     unsigned* sw = sync + (size_t)op * kSyncWords;
-    const int m = d.m, n = d.n;
+    const int m = d.c, n = d.L;   // of theta~, or of theta~^T
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned gen = 0;
     float* A = d.W32;
@@ -344,9 +348,16 @@ __global__ void __launch_bounds__(NT, 1) qr32_kernel(const OpDesc* descs, const 
         // A_1 and Q^T = I, row by row
         const double sc = S.scale;
         for (int i = rank * NWARP + warp; i < m; i += G * NWARP) {
-            const double lam = sc * (d.lam_left ? d.lam_left[i >> 2] : 1.0);
             for (int j = lane; j < m; j += 32) {
-                __stcg(A + (size_t)i * ld + j, (float)(lam * d.thetap[(size_t)i * ld + perm[j]]));
+                double a = 0.0;
+                for (int f = 0; f * m < n; ++f) {   // fold f, every other one backwards
+                    const int k = f * m + (f & 1 ? m - 1 - j : j);
+                    if (k >= n) continue;
+                    const int row = d.transposed ? perm[k] : i, col = d.transposed ? i : perm[k];
+                    const double lam = d.lam_left ? d.lam_left[row >> 2] : 1.0;
+                    a += lam * d.thetap[(size_t)row * ld + col];
+                }
+                __stcg(A + (size_t)i * ld + j, (float)(sc * a));
                 __stcg(U + (size_t)i * ld + j, i == j ? 1.0f : 0.0f);
             }
         }

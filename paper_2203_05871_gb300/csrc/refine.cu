@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, in
     const OpDesc& d = descs[blockIdx.x];
     RefineOp& r = *d.rf;
     if (r.state != kRefineActive) {
-        if (threadIdx.x == 0) r.order = 0;   // no rotation in this iteration
+        if (threadIdx.x == 0) r.order = r.turn = 0;   // no rotation in this iteration
         return;
     }
     const int c = d.c;
@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, in
     if (thr == 0.0 && settled && !d.full_svd && kk < c) thr = kth_largest<NT, 4 * kMaxChi>(a, c, kk);
     if (threadIdx.x == 0) {
         r.thr = thr;
+        r.need = fmax(thr, cutoff_floor(d, floor2 / (DBL_EPSILON * DBL_EPSILON)));
         r.floor2 = floor2;
         r.rho2 = 0u;
         r.row1 = 0u;
@@ -87,8 +88,13 @@ __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, in
     }
 }
 
+// scratch of the pairing, in the FP32 pass's Gram blocks: the row each row chose (-1: none)
+// and the tangent of its angle
+__device__ __forceinline__ int* partner_of(const OpDesc& d) { return reinterpret_cast<int*>(d.D32); }
+__device__ __forceinline__ float* angle_of(const OpDesc& d, int ld) { return d.D32 + ld; }
+
 // The op's state and the order of this iteration's rotation.
-__device__ void decide(const OpDesc& d, RefineOp& r, double tol_in, int can_finish, float defect, int last) {
+__device__ void decide(const OpDesc& d, RefineOp& r, double tol_in, int can_finish, float defect, int last, int turn) {
     r.order = 0;
     if (d.sweeps_out) *d.sweeps_out += 1;
     const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
@@ -105,7 +111,8 @@ __device__ void decide(const OpDesc& d, RefineOp& r, double tol_in, int can_fini
     else if (x2 * x2 * x2 <= 64.0f * defect)
         r.order = 3;
     else {
-        r.state = kRefineLeft;   // beyond the expansion (or not finite)
+        if (!turn) r.state = kRefineLeft;   // beyond the expansion (or not finite)
+        if (last) r.state = kRefineLeft;
         return;
     }
     if (!__ldcg(&r.far) && 2.0f * rho * x <= 0.1f * tol)
@@ -134,10 +141,11 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
         const float turn = tol >= 1e-11f ? 0.01f * tol : tol;
         const double* a = d.snorm;
         const double* inv = d.snorm + ld;
-        const double ai = a[i], vi = inv[i], thr = r.thr;
+        const double ai = a[i], vi = inv[i], thr = r.need;
         const bool dead = vi == 0.0, low = ai < thr;
-        float rho = 0.0f, sum = 0.0f;
+        float rho = 0.0f, sum = 0.0f, tfar = 0.0f;
         int far = 0;
+        unsigned long long best = 0;   // of the pairs beyond tcap: |t|, then the smallest pair of rows
         for (int j = lane; j < d.c; j += 32) {
             const double aj = a[j], vj = inv[j];
             double x = 0.0;
@@ -157,6 +165,13 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
                         if (!small) sum += fabsf(th);
                     } else if (!small) {
                         far = 1;
+                        const unsigned pair = ((unsigned)min(i, j) << 16) | (unsigned)max(i, j);
+                        const unsigned long long key =
+                            ((unsigned long long)__float_as_uint(fabsf(t)) << 32) | (0xffffffffu - pair);
+                        if (key > best) {
+                            best = key;
+                            tfar = t;
+                        }
                     }
                 }
             }
@@ -169,6 +184,21 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
         }
         sum = warp_sum(sum);
         far = __any_sync(0xffffffffu, far);
+        if (far) {
+            unsigned long long top = best;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long v = __shfl_xor_sync(0xffffffffu, top, o);
+                top = v > top ? v : top;
+            }
+            if (best == top) {   // pairs are unique: one lane
+                const unsigned pair = 0xffffffffu - (unsigned)top;
+                __stcg(partner_of(d) + i, (int)((pair >> 16) == (unsigned)i ? pair & 0xffffu : pair >> 16));
+                __stcg(angle_of(d, ld) + i, tfar);
+            }
+        } else if (lane == 0) {
+            __stcg(partner_of(d) + i, -1);
+        }
         if (lane == 0) {
             atomicMax(&r.rho2, __float_as_uint(fabsf(rho * rho)));
             atomicMax(&r.row1, __float_as_uint(sum));
@@ -177,15 +207,73 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&r.blocks, 1u) == (unsigned)blocks - 1u) {
-        __threadfence();
-        decide(d, r, tol_in, can_finish, defect, last);
+    __shared__ int s_last, s_turn;
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&r.blocks, 1u) == (unsigned)blocks - 1u;
+        s_turn = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // Rows that chose one another are turned by their exact rotation (refine_turn_kernel)
+    // and take no other part in this iteration.
+    __shared__ unsigned mate[4 * kMaxChi / 32];
+    const bool any = __ldcg(&r.far) != 0;
+    if (any) {
+        int* partner = partner_of(d);
+        for (int w = threadIdx.x; w < 4 * kMaxChi / 32; w += NT) mate[w] = 0;
+        __syncthreads();
+        for (int k = threadIdx.x; k < d.c; k += NT) {
+            const int j = __ldcg(partner + k);
+            if (j >= 0 && __ldcg(partner + j) == k) {
+                atomicOr(&mate[k >> 5], 1u << (k & 31));
+                s_turn = 1;
+            }
+        }
+        __syncthreads();
+        for (int k = threadIdx.x >> 5; k < d.c; k += NT / 32) {
+            if ((mate[k >> 5] >> (k & 31)) & 1u) {
+                for (int j = lane; j < d.c; j += 32) d.Q[(size_t)k * ld + j] = d.Q[(size_t)j * ld + k] = 0.0;
+            } else if (lane == 0) {
+                __stcg(partner + k, -1);
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        decide(d, r, tol_in, can_finish, defect, last, s_turn);
+        r.turn = s_turn && r.state == kRefineActive;
+    }
+}
+
+// The exact rotations of the rows that refine_x_kernel paired, one pair per warp: rows
+// of nearly equal norm that are not yet orthogonal, whose angle is beyond the
+// expansion.  Left to the FP64 Jacobi pass, a few of them cost an op whole sweeps over
+// all of its pairs (a quarter of the time of a 3 x 3 grid's evolution).
+__global__ void __launch_bounds__(NT) refine_turn_kernel(const OpDesc* descs, int ld) {
+    grid_begin();
+    const OpDesc& d = descs[blockIdx.y];
+    if (!d.rf->turn) return;
+    const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= d.c) return;
+    const int j = partner_of(d)[i];
+    if (j <= i) return;
+    const double t = (double)angle_of(d, ld)[i], cs = 1.0 / sqrt(fma(t, t, 1.0)), sn = cs * t;
+    for (int part = 0; part < (d.transposed ? 2 : 1); ++part) {
+        double* p = (part ? d.Z : d.W) + (size_t)i * ld;
+        double* q = (part ? d.Z : d.W) + (size_t)j * ld;
+        const int len = part ? d.c : d.L;
+        for (int k = lane; k < len; k += 32) {
+            const double x = p[k], y = q[k];
+            p[k] = cs * x - sn * y;
+            q[k] = sn * x + cs * y;
+        }
     }
 }
 
 }  // namespace
 
-cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, double tol_in,
+cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, bool with_z, double tol_in,
                           bool can_finish, unsigned long long timeout_ns, cudaStream_t st) {
     if (nops <= 0) return cudaSuccess;
     const int ld = 4 * chi_cap;
@@ -193,14 +281,16 @@ cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, do
     // level of 6 slices' products otherwise; the largest single angle follows
     const float defect = S == 7 ? 1e-17f : 1e-13f, tcap = S == 7 ? 2e-3f : 1e-2f;
     for (int it = 0; it < kRefineIters; ++it) {
-        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, chi_cap, S, timeout_ns, st);
+        cudaError_t e = launch_oz_ops(d_desc, nops, OZ_G, chi_cap, S, false, timeout_ns, st);
         if (e != cudaSuccess) return e;
         if ((e = launch_early(refine_diag_kernel, nops, NT, 0, st, d_desc, ld)) != cudaSuccess) return e;
         e = launch_early(refine_x_kernel, dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st, d_desc, ld, tol_in,
                          tcap, can_finish ? 1 : 0, defect, it == kRefineIters - 1);
         if (e != cudaSuccess) return e;
+        e = launch_early(refine_turn_kernel, dim3((ld + NT / 32 - 1) / (NT / 32), nops), NT, 0, st, d_desc, ld);
+        if (e != cudaSuccess) return e;
         for (int kind : {OZ_R3, OZ_R2, OZ_R1})
-            if ((e = launch_oz_ops(d_desc, nops, kind, chi_cap, S, timeout_ns, st)) != cudaSuccess) return e;
+            if ((e = launch_oz_ops(d_desc, nops, kind, chi_cap, S, with_z, timeout_ns, st)) != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }

@@ -4,7 +4,7 @@
 // row order.  k_cut = smallest k >= 1 whose discarded weight
 // sum_{i>=k} s_i^2 is <= cutoff * sum_i s_i^2 (the tail is summed from the
 // smallest value up); k = min(chi_max, k_cut).  Writes lambda_p = s[:k],
-// Yk[j] = v_j^T (rows of W normalised), the new site p+1
+// Yk[j] = v_j^T (rows of W normalised, or rows of Z), the new site p+1
 // B'[j][s2][r] = Yk[j][s2*cr + r] and the new bond dimension.  A forced rank
 // (replay of a recorded run) replaces k_cut, still capped by chi_max and c.
 // When the adjoint records a tape, all c sorted singular values and
@@ -68,14 +68,17 @@ __global__ void __cluster_dims__(TC, 1, 1) __launch_bounds__(TT, 1) truncate_ker
             perm[j] = j;
             continue;
         }
-        const double sj = s[j];
+        // by their bit patterns (norms are >= 0): c^2 FP64 comparisons would take the FP64
+        // pipe 0.5 ms at chi = 256
+        const long long sj = __double_as_longlong(s[j]);
         int r = 0;
+#pragma unroll 8
         for (int i = 0; i < c; ++i) {
-            const double si = s[i];
-            r += (si > sj) || (si == sj && i < j);
+            const long long si = __double_as_longlong(s[i]);
+            r += si > sj || (si == sj && i < j);
         }
         perm[r] = j;
-        tail[r] = sj;
+        tail[r] = s[j];
     }
     __syncthreads();
     if (threadIdx.x == 0 && !bad) {
@@ -108,14 +111,15 @@ __global__ void __cluster_dims__(TC, 1, 1) __launch_bounds__(TT, 1) truncate_ker
     }
     const int t0 = rank * TT + threadIdx.x, w0 = rank + TC * warp;
     for (int j = t0; j < k; j += TC * TT) d.lam_out[j] = bad ? 0.0 : s[perm[j]];
+    const double* rows = d.transposed ? d.Z : d.W;   // s_j v_j^T, or of unit norm
     if (d.tape_V) {
         // every sorted right singular vector (zero rows stay zero) for the adjoint
         for (int j = t0; j < c; j += TC * TT) d.tape_s[j] = bad ? 0.0 : s[perm[j]];
         for (int j = w0; j < c; j += TC * (TT / 32)) {
             const int src = perm[j];
             const double sv = s[src];
-            const double inv = (sv > 0.0 && !bad) ? 1.0 / sv : 0.0;
-            const double* wr = d.W + (size_t)src * ld;
+            const double inv = (sv > 0.0 && !bad) ? (d.transposed ? 1.0 : 1.0 / sv) : 0.0;
+            const double* wr = rows + (size_t)src * ld;
             double* v = d.tape_V + (size_t)j * d.n;
             for (int i = lane; i < d.n; i += 32) v[i] = wr[i] * inv;
         }
@@ -125,9 +129,9 @@ __global__ void __cluster_dims__(TC, 1, 1) __launch_bounds__(TT, 1) truncate_ker
         const int src = perm[j];
         double* y = d.Yk + (size_t)j * ld;
         const size_t bnew = (size_t)j * 4 * chi_cap;   // row j of the new site p+1
-        const double* wr = d.W + (size_t)src * ld;
+        const double* wr = rows + (size_t)src * ld;
         const double sv = s[src];
-        const double inv = (sv > 0.0 && !bad) ? 1.0 / sv : 0.0;
+        const double inv = (sv > 0.0 && !bad) ? (d.transposed ? 1.0 : 1.0 / sv) : 0.0;
         for (int s2 = 0; s2 < 4; ++s2)
             for (int r = lane; r < cr; r += 32) {
                 const int i = s2 * cr + r;
