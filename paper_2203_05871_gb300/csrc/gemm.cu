@@ -6,7 +6,7 @@
 // float or double (converted on load), accumulated in TC (double or float),
 // written as double.  One launch serves a list of problems of different
 // sizes (grid.z = problem); CTAs outside a problem's tiles return at once.
-// 64 x 64 tiles, k-step 16, 256 threads with a 4 x 4 register tile each.
+// 64 x 64 tiles (32 or 16 where few), k-step 16, 256 threads.
 // A symmetric product (sym: E = U U^T) computes the tiles on and above the
 // diagonal only and writes each strictly upper tile to both triangles; entry
 // (j, i) is then the same products summed in the same order as (i, j), so
@@ -17,7 +17,6 @@ namespace mpdo {
 
 namespace {
 
-constexpr int GT = 64;
 constexpr int GK = 16;
 
 template <typename TC>
@@ -25,8 +24,13 @@ __device__ __forceinline__ TC load_as(const void* p, int is_f32, size_t i) {
     return is_f32 ? (TC)(static_cast<const float*>(p)[i]) : (TC)(static_cast<const double*>(p)[i]);
 }
 
-template <typename TC>
+// GT x GT tiles, R x R outputs per thread; the next k tile is on its way into
+// registers while this one is used.  Every output is the same sum in the same order
+// whatever GT is.
+template <typename TC, int GT>
 __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* descs) {
+    constexpr int R = GT / 16;
+    static_assert(GT * GK == 256 * R, "R elements of each operand per thread");
     const GemmDesc& g = descs[blockIdx.z];
     const int i0 = blockIdx.y * GT, j0 = blockIdx.x * GT;
     if (i0 >= g.M || j0 >= g.N) return;
@@ -34,61 +38,70 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* descs) {
     __shared__ TC As[GK][GT + 1];
     __shared__ TC Bs[GK][GT + 1];
     const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-    TC acc[4][4];
+    TC acc[R][R], pa[R], pb[R];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < R; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = (TC)0;
-    for (int k0 = 0; k0 < g.K; k0 += GK) {
-        if (g.a_trans) {   // A stored K x M row-major
-            for (int e = t; e < GT * GK; e += 256) {
-                const int kk = e / GT, ii = e % GT;
-                const int gi = i0 + ii, gk = k0 + kk;
-                As[kk][ii] = (gi < g.M && gk < g.K) ? load_as<TC>(g.A, g.a_f32, (size_t)gk * g.lda + gi) : (TC)0;
-            }
-        } else {
-            for (int e = t; e < GT * GK; e += 256) {
-                const int ii = e / GK, kk = e % GK;
-                const int gi = i0 + ii, gk = k0 + kk;
-                As[kk][ii] = (gi < g.M && gk < g.K) ? load_as<TC>(g.A, g.a_f32, (size_t)gi * g.lda + gk) : (TC)0;
-            }
+        for (int v = 0; v < R; ++v) acc[u][v] = (TC)0;
+    // element e of a tile's operand: along the stored rows
+    auto at_a = [&](int e, int& kk, int& ii) {   // A stored M x K, or K x M when a_trans
+        kk = g.a_trans ? e / GT : e % GK;
+        ii = g.a_trans ? e % GT : e / GK;
+    };
+    auto at_b = [&](int e, int& kk, int& jj) {   // B stored K x N, or N x K when b_trans
+        kk = g.b_trans ? e % GK : e / GT;
+        jj = g.b_trans ? e / GK : e % GT;
+    };
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            int kk, x;
+            at_a(t + 256 * u, kk, x);
+            const int gi = i0 + x, ka = k0 + kk;
+            pa[u] = gi < g.M && ka < g.K
+                        ? load_as<TC>(g.A, g.a_f32, g.a_trans ? (size_t)ka * g.lda + gi : (size_t)gi * g.lda + ka)
+                        : (TC)0;
+            at_b(t + 256 * u, kk, x);
+            const int gj = j0 + x, kb = k0 + kk;
+            pb[u] = gj < g.N && kb < g.K
+                        ? load_as<TC>(g.B, g.b_f32, g.b_trans ? (size_t)gj * g.ldb + kb : (size_t)kb * g.ldb + gj)
+                        : (TC)0;
         }
-        if (g.b_trans) {
-            for (int e = t; e < GT * GK; e += 256) {
-                const int jj = e / GK, kk = e % GK;
-                const int gj = j0 + jj, gk = k0 + kk;
-                Bs[kk][jj] = (gj < g.N && gk < g.K) ? load_as<TC>(g.B, g.b_f32, (size_t)gj * g.ldb + gk) : (TC)0;
-            }
-        } else {
-            for (int e = t; e < GT * GK; e += 256) {
-                const int kk = e / GT, jj = e % GT;
-                const int gj = j0 + jj, gk = k0 + kk;
-                Bs[kk][jj] = (gj < g.N && gk < g.K) ? load_as<TC>(g.B, g.b_f32, (size_t)gk * g.ldb + gj) : (TC)0;
-            }
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < g.K; k0 += GK) {
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            int kk, x;
+            at_a(t + 256 * u, kk, x);
+            As[kk][x] = pa[u];
+            at_b(t + 256 * u, kk, x);
+            Bs[kk][x] = pb[u];
         }
         __syncthreads();
+        if (k0 + GK < g.K) fetch(k0 + GK);
 #pragma unroll 4
         for (int kk = 0; kk < GK; ++kk) {
-            TC a[4], b[4];
+            TC a[R], b[R];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = As[kk][ty * 4 + u];
-                b[u] = Bs[kk][tx * 4 + u];
+            for (int u = 0; u < R; ++u) {
+                a[u] = As[kk][ty * R + u];
+                b[u] = Bs[kk][tx * R + u];
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < R; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+                for (int v = 0; v < R; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int gi = i0 + ty * 4 + u;
+    for (int u = 0; u < R; ++u) {
+        const int gi = i0 + ty * R + u;
         if (gi >= g.M) continue;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int gj = j0 + tx * 4 + v;
+        for (int v = 0; v < R; ++v) {
+            const int gj = j0 + tx * R + v;
             if (gj >= g.N) continue;
             double r = g.alpha * (double)acc[u][v];
             if (g.D) r += g.beta * load_as<double>(g.D, g.d_f32, (size_t)gi * g.ldd + gj);
@@ -99,17 +112,28 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* descs) {
     }
 }
 
+template <int GT>
+cudaError_t launch_tiles(const GemmDesc* d_desc, int count, int max_m, int max_n, bool fp32_compute, cudaStream_t st) {
+    const dim3 grid((max_n + GT - 1) / GT, (max_m + GT - 1) / GT, count);
+    if (fp32_compute)
+        gemm_kernel<float, GT><<<grid, 256, 0, st>>>(d_desc);
+    else
+        gemm_kernel<double, GT><<<grid, 256, 0, st>>>(d_desc);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_gemm(const GemmDesc* d_desc, int count, int max_m, int max_n, bool fp32_compute,
                         cudaStream_t st) {
     if (count <= 0 || max_m <= 0 || max_n <= 0) return cudaSuccess;
-    dim3 grid((max_n + GT - 1) / GT, (max_m + GT - 1) / GT, count);
-    if (fp32_compute)
-        gemm_kernel<float><<<grid, 256, 0, st>>>(d_desc);
-    else
-        gemm_kernel<double><<<grid, 256, 0, st>>>(d_desc);
-    return cudaGetLastError();
+    // The FP64 pipe, two FMAs per SM and clock, bounds every tile: 64 x 64 outputs take
+    // it 2048 K clocks, so tiles shrink until the launch fills the chip (the adjoint's
+    // products of 128 x 64 x 64 ran on two SMs, 120 us each).
+    const long long tiles = (long long)((max_n + 63) / 64) * ((max_m + 63) / 64) * count;
+    if (tiles * 4 <= 152) return launch_tiles<16>(d_desc, count, max_m, max_n, fp32_compute, st);
+    if (tiles <= 152) return launch_tiles<32>(d_desc, count, max_m, max_n, fp32_compute, st);
+    return launch_tiles<64>(d_desc, count, max_m, max_n, fp32_compute, st);
 }
 
 }  // namespace mpdo

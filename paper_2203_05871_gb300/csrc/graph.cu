@@ -31,36 +31,53 @@ namespace {
 // work, each op between 1 and cap_s CTAs (the host plan's rule; none for cap_s = 0).  out: [R] op
 // of each CTA (-1: unused, the CTA returns at once), [R] rank within the op,
 // [nops] CTAs per op.  Returns 0, or 1 if R < nops.
-__device__ int plan_ctas(const double* work, const int* cap, int nops, int R, int* out) {
-    int* G = out + 2 * R;
-    double wsum = 0.0;
-    for (int s = 0; s < nops; ++s) wsum += cap[s] > 0 ? work[s] : 0.0;
-    int total = 0;
-    for (int s = 0; s < nops; ++s) {
-        G[s] = 0;
-        if (cap[s] == 0) continue;
-        int g = (int)floor((double)R * work[s] / fmax(wsum, 1.0));
-        g = max(1, min(cap[s], g));
-        const int passes = (cap[s] + g - 1) / g;
-        g = (cap[s] + passes - 1) / passes;
+// Called by a whole CTA; G: [nops] in shared memory.
+__device__ int plan_ctas(const double* work, const int* cap, int nops, int R, int* out, int* G) {
+    __shared__ double s_wsum;
+    __shared__ int s_total;
+    __syncthreads();   // work and cap are there, G is free
+    if (threadIdx.x == 0) {
+        double wsum = 0.0;
+        for (int s = 0; s < nops; ++s) wsum += cap[s] > 0 ? work[s] : 0.0;
+        s_wsum = fmax(wsum, 1.0);
+        s_total = 0;
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < nops; s += blockDim.x) {
+        int g = 0;
+        if (cap[s] > 0) {
+            g = (int)floor((double)R * work[s] / s_wsum);
+            g = max(1, min(cap[s], g));
+            const int passes = (cap[s] + g - 1) / g;
+            g = (cap[s] + passes - 1) / passes;
+        }
         G[s] = g;
-        total += g;
+        if (g > 0) atomicAdd(&s_total, g);
     }
-    while (total > R) {
-        int arg = 0;
-        for (int s = 1; s < nops; ++s)
-            if (G[s] > G[arg]) arg = s;
-        if (G[arg] <= 1) return 1;
-        G[arg]--;
-        total--;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        while (s_total > R) {
+            int arg = 0;
+            for (int s = 1; s < nops; ++s)
+                if (G[s] > G[arg]) arg = s;
+            if (G[arg] <= 1) break;
+            G[arg]--;
+            s_total--;
+        }
     }
-    int t = 0;
-    for (int s = 0; s < nops; ++s)
+    __syncthreads();
+    const int total = s_total;
+    if (total > R) return 1;
+    for (int s = threadIdx.x; s < nops; s += blockDim.x) {
+        int t = 0;
+        for (int u = 0; u < s; ++u) t += G[u];
+        out[2 * R + s] = G[s];
         for (int g = 0; g < G[s]; ++g, ++t) {
             out[t] = s;
             out[R + t] = g;
         }
-    for (; t < R; ++t) {
+    }
+    for (int t = total + threadIdx.x; t < R; t += blockDim.x) {
         out[t] = -1;
         out[R + t] = 0;
     }
@@ -92,25 +109,26 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
             if (t > 0) d.jb = t;
         }
     }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
+    __shared__ int G[kMaxChunk];
     int bad = 0;
-    for (int s = 0; s < nops; ++s) {
+    for (int s = threadIdx.x; s < nops; s += blockDim.x) {   // the thread's own descriptors
         const OpDesc& d = descs[s];
         work[s] = (double)d.c * d.c * (double)d.L;
         cap[s] = jacobi_pairs_per_round(d.c, d.jb);
     }
-    bad |= plan_ctas(work, cap, nops, Rj, cta64);
+    bad |= plan_ctas(work, cap, nops, Rj, cta64, G);
     if (precond) {
-        for (int s = 0; s < nops; ++s) cap[s] = jacobi_pairs_per_round(descs[s].c, kJacobiB32);
-        bad |= plan_ctas(work, cap, nops, Rj, cta32);
+        __syncthreads();
+        for (int s = threadIdx.x; s < nops; s += blockDim.x) cap[s] = jacobi_pairs_per_round(descs[s].c, kJacobiB32);
+        bad |= plan_ctas(work, cap, nops, Rj, cta32, G);
     }
-    for (int s = 0; s < nops; ++s) {
+    __syncthreads();
+    for (int s = threadIdx.x; s < nops; s += blockDim.x) {
         const OpDesc& d = descs[s];
         work[s] = (double)d.m * d.n * d.c;
         cap[s] = q32 ? qr32_max_ctas(d.c) : max(1, (d.n + kQrWarps - 1) / kQrWarps);
     }
-    if (!blocked) bad |= plan_ctas(work, cap, nops, q32 ? Rq32 : Rq, q32 ? ctaq32 : ctaqr);
+    if (!blocked) bad |= plan_ctas(work, cap, nops, q32 ? Rq32 : Rq, q32 ? ctaq32 : ctaqr, G);
     if (bad) *error = 1;
 }
 

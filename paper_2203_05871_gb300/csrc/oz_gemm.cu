@@ -500,12 +500,14 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int quarter, int R,
     const bool f32 = X.f32 != 0;
     const int r = r0 + lane;
     const bool live = r < R;
+    __syncthreads();   // the previous rows' maxima are read
     unsigned long long mx = live ? row_max(X, r, warp, 8, K) : 0;
     s_mx[warp][lane] = mx;
     __syncthreads();
     for (int w = 0; w < 8; ++w) mx = s_mx[w][lane] > mx ? s_mx[w][lane] : mx;
     const bool bad = key_nonfinite(mx, f32);   // the largest key of a row with a NaN or an inf is one
     const int e = bad ? 0 : key_exponent(mx, f32);
+    if (!live) return;
     if (warp == 0 && quarter == 0) ex[r] = e;
     const int rt = r / tile, rr = r % tile;
     const size_t block = (size_t)tile * 64;
@@ -515,10 +517,10 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int quarter, int R,
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const int k = g0 + g;
-            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
+            x[g] = (!bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
         }
         uint4 sl[kS];
-        slice_group<kS>(x, bad && live, sl);
+        slice_group<kS>(x, bad, sl);
         const int kt = g0 / KT, kk = g0 % KT;
 #pragma unroll
         for (int t = 0; t < kS; ++t) {
@@ -533,7 +535,7 @@ __device__ void slice_rows_tiled(const OzOperand& X, int r0, int quarter, int R,
 // contiguous (ks == 1) take one warp per row, lanes along k; the others 32 rows
 // per four blocks (slice_rows_tiled).
 template <int kS>
-__global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
+__global__ void __launch_bounds__(256, 3) oz_slice_kernel(OzSource src) {
     __shared__ OzProblem P;
     grid_begin();
     fetch_problem<kS>(src, P);
@@ -548,43 +550,46 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzSource src) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char* out = static_cast<unsigned char*>(isB ? P.bs : P.as);
     int* ex = isB ? P.eb : P.ea;
-    if (!(X.mode == 0 && X.ks == 1)) {
-        const int r0 = (blockIdx.x >> 2) * 32;
-        if (r0 >= Rt * tile) return;   // uniform over the block (Rt * tile is a multiple of 32)
-        slice_rows_tiled<kS>(X, r0, blockIdx.x & 3, R, K, Kt, lv, out, ex, tile, Rt);
-        return;
-    }
-    const int r = blockIdx.x * 8 + warp;
-    if (r >= Rt * tile) return;
-    const bool live = r < R;
-    const bool f32 = X.f32 != 0;
-    unsigned long long mx = live ? row_max(X, r, lane, 32, K) : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-        mx = y > mx ? y : mx;
-    }
-    const bool bad = key_nonfinite(mx, f32);
-    const int e = bad ? 0 : key_exponent(mx, f32);
-    if (lane == 0) ex[r] = e;
-    const int rt = r / tile, rr = r % tile;
-    const size_t block = (size_t)tile * 64;
-    const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
-    for (int g0 = lane * G; g0 < Kt * KT; g0 += 32 * G) {
-        long long x[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int k = g0 + g;
-            x[g] = (live && !bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
+    // Rows past R need no slices: a row of the result depends on its own rows alone.
+    // The groups of 8 rows go round the launch's blocks.
+    const bool strided = !(X.mode == 0 && X.ks == 1);
+    const int groups = strided ? 4 * ((R + 31) / 32) : (R + 7) / 8;
+    for (int rb = blockIdx.x; rb < groups; rb += gridDim.x) {
+        if (strided) {
+            slice_rows_tiled<kS>(X, (rb >> 2) * 32, rb & 3, R, K, Kt, lv, out, ex, tile, Rt);
+            continue;
         }
-        uint4 sl[kS];
-        slice_group<kS>(x, bad && live, sl);
-        const int kt = g0 / KT, kk = g0 % KT;
+        const int r = rb * 8 + warp;
+        if (r >= R) return;
+        const bool f32 = X.f32 != 0;
+        unsigned long long mx = row_max(X, r, lane, 32, K);
 #pragma unroll
-        for (int t = 0; t < kS; ++t) {
-            if (t >= lv) break;
-            unsigned char* blk = out + (((size_t)t * Rt + rt) * Kt + kt) * block;
-            *reinterpret_cast<uint4*>(blk + within + (size_t)(kk / G) * LBO) = sl[t];
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
+            mx = y > mx ? y : mx;
+        }
+        const bool bad = key_nonfinite(mx, f32);
+        const int e = bad ? 0 : key_exponent(mx, f32);
+        if (lane == 0) ex[r] = e;
+        const int rt = r / tile, rr = r % tile;
+        const size_t block = (size_t)tile * 64;
+        const size_t within = (size_t)(rr >> 3) * SBO + (size_t)(rr & 7) * 16;
+        for (int g0 = lane * G; g0 < Kt * KT; g0 += 32 * G) {
+            long long x[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const int k = g0 + g;
+                x[g] = (!bad && k < K) ? fixed_of<kS>(oz_bits(X, r, k), f32, e) : 0;
+            }
+            uint4 sl[kS];
+            slice_group<kS>(x, bad, sl);
+            const int kt = g0 / KT, kk = g0 % KT;
+#pragma unroll
+            for (int t = 0; t < kS; ++t) {
+                if (t >= lv) break;
+                unsigned char* blk = out + (((size_t)t * Rt + rt) * Kt + kt) * block;
+                *reinterpret_cast<uint4*>(blk + within + (size_t)(kk / G) * LBO) = sl[t];
+            }
         }
     }
 }
@@ -896,7 +901,14 @@ template <int S>
 cudaError_t launch_oz(const OzSource& src, int count, int max_m, int max_n, int max_rows_sliced,
                       unsigned long long timeout_ns, cudaStream_t st) {
     const int rows = ((max_rows_sliced + kTileM - 1) / kTileM) * kTileM;
-    const cudaError_t e = launch_early(oz_slice_kernel<S>, dim3((rows + 7) / 8, 2, count), 256, 0, st, src);
+    // Many short products (an ensemble of chains at chi 24: 160 of them): about 1200
+    // blocks that go round the rows, as each first builds its problem, 1 to 2 us of one
+    // thread (a replayed step 17.0 -> 15.5 ms).  Rows of more than 256 are worth a block
+    // per eight of them (with the limit, the products of a chi 256 step took a quarter
+    // longer).
+    const int all = (rows + 7) / 8, share = 1216 / (2 * count) > 0 ? 1216 / (2 * count) : 1;
+    const int blocks = rows <= 256 && share < all ? share : all;
+    const cudaError_t e = launch_early(oz_slice_kernel<S>, dim3(blocks, 2, count), 256, 0, st, src);
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)((max_m + kTileM - 1) / kTileM) * ((max_n + kTileN - 1) / kTileN) * count;
     if (tiles * 4 <= kFill) return launch_tiles<S, 16>(src, count, max_m, max_n, timeout_ns, st);
