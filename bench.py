@@ -439,16 +439,15 @@ def measured_peaks():
 SLICE_PRODUCTS = 21   # slice pairs (t, u), t + u <= 5, per useful multiply-add of the tensor-core products
 
 
-def contraction_roofline(prof, kind):
+def contraction_roofline(prof):
     """The tensor-core contractions (merge + reconstruct, oz_gemm_kernel with its
-    slicing kernels) against the tensor peak of their kind: executed flops = 21
-    slice products per useful flop (the hardware's work), with the useful rate
-    beside it."""
+    slicing kernels) against the bf16 tensor peak (both kinds are formed from bf16
+    slices): executed flops = 21 slice products per useful flop (the hardware's
+    work), with the useful rate beside it."""
     fl = prof["merge_gate"]["flops"] + prof["reconstruct"]["flops"]
     ms = prof["merge_gate"]["ms"] + prof["reconstruct"]["ms"]
     bf16 = measured_peaks().get("bf16_tflops")
-    base = bf16 if bf16 else 1900.0
-    peak = base if kind == "bf16" else base * 1.1 / 2.25
+    peak = bf16 if bf16 else 1900.0
     useful = fl / (ms / 1e3) / 1e12 if ms > 0 else None
     achieved = useful * SLICE_PRODUCTS if useful else None
     return {"kernel": "oz_gemm_kernel (merge + reconstruct, incl. slicing and the gate/weight kernel)",
@@ -456,14 +455,15 @@ def contraction_roofline(prof, kind):
             "frac": achieved / peak if achieved else None, "traffic": None, "useful_tflops": useful,
             "note": "achieved = 21 slice products x useful flops (32 cl cm cr + 512 cl cr merge, 32 cl cr k "
                     "reconstruct) / CUDA-event time of the merge and reconstruct stages; peak = measured bf16 burst"
-                    + (" x 1.1/2.25 (nominal TF32/BF16)" if kind != "bf16" else "") + ("" if bf16 else ", of fallback")}
+                    + ("" if bf16 else ", of fallback")}
 
 
 def qr_roofline(prof):
-    """Householder QR with column pivoting against the nominal FP64 peak."""
+    """The QR stage (FP32 Householder QR, its orthogonalisation and W0 = Q^T theta~ on
+    the tensor cores) against the nominal FP64 peak of a QR in FP64."""
     q = prof["qr"]
     achieved = q["flops"] / (q["ms"] / 1e3) / 1e12 if q["ms"] > 0 else None
-    return {"kernel": "qr_kernel (Householder, column pivoting)", "bound": "alu", "achieved": achieved,
+    return {"kernel": "qr32_kernel and its products", "bound": "alu", "achieved": achieved,
             "peak": FP64_PEAK_NOMINAL_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_NOMINAL_TFLOPS if achieved else None, "traffic": None,
             "note": "flops 4 m n r - 2 (m + n) r^2 + 4/3 r^3 per op (r = min(m, n)); peak = nominal FP64"}
@@ -516,11 +516,10 @@ def run_observables(args, local, reps=5):
     res["z_all"]["roofline"] = {"bound": "hbm", "algorithmic_bytes": b1,
                                 "achieved": b1 / (res["z_all"]["ms"] * 1e-3) / 1e9,
                                 "peak": hbm, "unit": "GB/s"}
-    # all pairs: the I and Z slices once each beyond the environments
-    # (the stacked form); FP64 flops of the stacked propagation, sum over j of
-    # (rows alive) x 2 slices x chi_j chi_j+1 FMA
+    # all pairs: the I and Z slices once each beyond the environments; FP64 flops of the seeds (one slice per site and side)
+    # and of carrying each half's rows to the middle bond, (rows alive) x chi_p chi_p+1 FMA
     b2 = 4.0 * slice_bytes
-    fl2 = sum(4.0 * j * d[j] * d[j + 1] for j in range(n))
+    fl2 = sum(2.0 * (2 + (p if p < n // 2 else n - 1 - p)) * d[p] * d[p + 1] for p in range(n))
     res["zz_connected_all_pairs"]["roofline"] = {
         "bound": "hbm", "algorithmic_bytes": b2, "achieved": b2 / (res["zz_connected_all_pairs"]["ms"] * 1e-3) / 1e9,
         "peak": hbm, "unit": "GB/s", "fp64_flops": fl2,
@@ -609,11 +608,11 @@ def truncation_roofline(prof, precision):
     """The truncation stage (QR + SVD, about 95% of the step) against the FP64
     peak, with the fixed algorithmic convention of 21 n^3 flops per n x n SVD."""
     jac = prof["jacobi_svd"]
-    parts = ["qr", "jacobi_svd"] + (["jacobi_fp32", "precond_gemm"] if precision == "mixed" else [])
+    parts = ["qr", "jacobi_svd"] + [k for k in ("jacobi_fp32", "precond_gemm") if prof[k]["launches"]]
     ms = sum(prof[k]["ms"] for k in parts)
     achieved = jac["flops"] / (ms / 1e3) / 1e12 if ms > 0 else None
-    names = {"qr": "qr_kernel", "jacobi_svd": "jacobi_kernel<double>", "jacobi_fp32": "jacobi_kernel<float>",
-             "precond_gemm": "oz_prep/slice/gemm kernels x3 (preconditioner products)"}
+    names = {"qr": "qr32_kernel and its products", "jacobi_svd": "jacobi_kernel", "jacobi_fp32": "jacobi32_kernel",
+             "precond_gemm": "oz_slice/oz_gemm/refine kernels (orthogonalisation and refinement)"}
     return {"kernel": "truncation stage: " + " + ".join(names[k] for k in parts),
             "bound": "alu", "achieved": achieved, "peak": FP64_PEAK_NOMINAL_TFLOPS, "unit": "TFLOP/s",
             "frac": (achieved / FP64_PEAK_NOMINAL_TFLOPS) if achieved else None,
@@ -621,9 +620,8 @@ def truncation_roofline(prof, precision):
             "note": "achieved = 21 n^3 flops per n x n SVD (n = 4 max(chi_l, chi_r)), the FP64 work of an ideal "
                     "Golub-Kahan SVD, over the summed CUDA-event time of the listed kernels (QR included); peak = "
                     "nominal FP64 of GB300 (2 DFMA/SM/clk x 152 SMs x 2.07 GHz; MEASURED_PEAKS.json has no "
-                    "FP64 figure), of nominal; traffic: null, the stage is several kernels whose rows stay in "
-                    "L2 (a jacobi_kernel<double> launch of the chain10_chi256 case read 2.8 MB of DRAM, "
-                    "profiles/kernels_chain10_chi256.md)"}
+                    "FP64 figure), of nominal (the kernels do little of it in FP64, so the fraction can pass 1); "
+                    "traffic: null, the stage is several kernels whose rows stay in L2"}
 
 
 def main():
@@ -658,7 +656,7 @@ def main():
     prof = head["prof"]
     launches = sum(v["launches"] for v in prof.values())      # kernels, as counted by the library
     dtype = (("mixed: tcgen05 %s slice products (six 8-bit slices, exact level sums, fp64 re-accumulated) for the "
-              "contractions and preconditioner GEMMs, fp32-preconditioned fp64 QR + Jacobi SVD" % args.mixed_kind)
+              "contractions and SVD products, fp32 QR and Jacobi refined to fp64 accuracy" % args.mixed_kind)
              if hp == "mixed" else "f64")
     line = {
         "metric": "gate_applications_per_sec", "value": hs["value"], "unit": "gate-applications/s",
@@ -669,7 +667,7 @@ def main():
         "config": {"workload": args.workload, "n_qubits": wl.n, "batch": wl.batch, "chi_max": cap,
                    "cutoff": float(wl.cutoff[0]),
                    "dt": wl.dt, "ops_per_step": n_ops, "swaps_per_step": head["n_swaps"], "precision": hp,
-                   "qr": "blocked" if (hp == "mixed" and args.qr_blocked) else "column",
+                   "qr": "blocked" if (hp == "mixed" and args.qr_blocked) else "fp32",
                    "parallelism": f"replicas{world}", "l2": "flushed (256 MB write) between timed steps",
                    "start": "seeded random MPO at chi_max, Schmidt grading exp(-%.3f r)" % (
                        DECAY if "flat" not in args.workload else 0.0)},
@@ -685,7 +683,7 @@ def main():
                                     prof["jacobi_svd"]["critical_sweeps_fp32"] / prof["jacobi_svd"]["chunks"]]
                                    if prof["jacobi_svd"].get("chunks") else None),
         "roofline": truncation_roofline(prof, hp),
-        "roofline_contraction": contraction_roofline(prof, args.mixed_kind) if hp == "mixed" else None,
+        "roofline_contraction": contraction_roofline(prof) if hp == "mixed" else None,
         "roofline_qr": qr_roofline(prof),
         "autotune": {"jacobi_rows_per_block": head["tuned"],
                      "note": "(chi_l x chi_r): [FP64 pass, FP32 pass], measured before the timed steps"},

@@ -76,7 +76,10 @@ typedef struct {
                                 S2(w1 dt) S2(w0 dt) S2(w1 dt), w1 = 1/(2 - 2^(1/3)), w0 = 1 - 2 w1
                                 (App. B uses order 4; odd orders are not built) */
     int force_trace;         /* 1: rho /= tr rho after every step (App. B b_force_rho_trace) */
-    int jacobi_max_sweeps;   /* sweep limit of the Jacobi SVD (default 100, at most 128) */
+    int jacobi_max_sweeps;   /* sweep limit of the Jacobi SVD (default 100, at most 128); under 16
+                                every SVD is left to the Jacobi passes alone (FP64: the FP64 pass
+                                on the rows of R), without the refinement through the Gram matrix
+                                and, for MPDO_FP64, without the FP32 stages before it */
     double jacobi_tol;       /* <= 0: sqrt(L) * DBL_EPSILON for rows of length L */
     unsigned barrier_timeout_ms;  /* limit of every device-side wait (default 4000) */
     int max_slots;           /* <= 0: automatic; else max two-site ops in flight */
@@ -175,8 +178,8 @@ int mpdo_renyi2(mpdo_ctx *ctx, double *out, int out_on_device);
  * normalised vectorised state |rho>> for the cut between path positions bond
  * and bond + 1 (bond in [0, N-2]; the paper's central bond is N/2 - 1), from
  * its exact Schmidt values s_k: Gram matrices X, Y of the two halves (batched
- * FP64 GEMM sweeps), X = F_X^T F_X and Y = F_Y^T F_Y from FP64 Jacobi SVDs, s_k
- * the singular values of F_X F_Y^T (a third Jacobi SVD).  Independent of the
+ * products of FP64 accuracy), X = F_X^T F_X and Y = F_Y^T F_Y from SVDs at the strict
+ * FP64 tolerance, s_k the singular values of F_X F_Y^T (a third SVD).  Independent of the
  * gauge of the stored tensors.  out as for mpdo_renyi2.  A Jacobi SVD that hits
  * cfg.jacobi_max_sweeps sets MPDO_ST_NOCONV for its instance (mpdo_status).
  * EINVAL (bond), ESTATE, ECUDA. */
@@ -218,8 +221,9 @@ int mpdo_force_ranks(mpdo_ctx *ctx, const int *k, int n_steps);
  * (chi_l, chi_r) in classes[n_classes][2] (each in [1, chi_cap]): for every
  * candidate block size that fits shared memory, the Jacobi launch is timed on
  * seeded graded matrices of the class's shape, one per op in flight (the
- * largest layer), and the fastest is kept (FP64 pass, and the FP32 pass of the
- * mixed path).  Later steps (plain and graph) use the table; classes not tuned
+ * largest layer), and the fastest is kept (FP64 pass; the FP32 pass has one block
+ * size; bonds with chi_l > chi_r whose SVD is that of the transposed matrix keep the
+ * default rule).  Later steps (plain and graph) use the table; classes not tuned
  * keep the default rule (largest block that fits).  chosen (host, may be NULL)
  * receives [n_classes][2] = (FP64 block, FP32 block or 0).  Uses the per-op
  * workspaces only (the state is untouched); synchronises.  EINVAL, ESTATE, ECUDA. */
@@ -252,7 +256,8 @@ int mpdo_inject_fault(mpdo_ctx *ctx, int kind);
  * of the step with CUDA events on the context stream and accumulates, per
  * kernel kind k (0 merge+gate, 1 Jacobi SVD (FP64), 2 truncate, 3 reconstruct,
  * 4 trace, 5 environments/measure, 6 gate build, 7 FP32 preconditioning
- * Jacobi, 8 preconditioner GEMMs, 9 Householder QR), the device time in ms,
+ * Jacobi, 8 the products and the refinement after it, 9 Householder QR with its
+ * products), the device time in ms,
  * the number of kernels launched and the algorithmic flops of the work launched
  * (merge 32 cl cm cr, gate 512 cl cr, SVD 21 n^3 with n = 4 max(cl, cr),
  * reconstruct 32 cl cr k; 0 for the other kinds).  mpdo_profile_read copies
@@ -304,7 +309,8 @@ int mpdo_measure_1q_noalloc(const double *sites, const int *dims, int n_qubits, 
  * uses for its contractions and SVD-preconditioner GEMMs, on caller matrices
  * (the paper has none; its contractions are FP64 ITensor/LAPACK calls).  Each
  * row of A and column of B is scaled by a power of two and cut into six 8-bit
- * slices, exact in tf32 (kind = MPDO_MIXED_TF32) or bf16 (MPDO_MIXED_BF16X3);
+ * slices, exact in tf32 and bf16 alike (kind = MPDO_MIXED_TF32 or
+ * MPDO_MIXED_BF16X3: both are formed from bf16 slices, with the same result);
  * the 21 slice products of the leading levels are formed by tcgen05 MMAs with
  * error-free FP32 accumulation per 256 values of K and summed in FP64, so the
  * error is about 2^-46 |A_i|max |B_j|max per term of the sum.

@@ -103,7 +103,8 @@ namespace {
 int alloc_slots(mpdo_ctx* c, int want) {
     release_slots(c);
     const size_t mat = (size_t)c->ld * c->ld;
-    size_t per_slot_bytes = (3 * mat + (size_t)c->cap * c->ld + 2 * c->ld) * sizeof(double);
+    const size_t plain_bytes = (3 * mat + (size_t)c->cap * c->ld + 2 * c->ld) * sizeof(double);
+    size_t per_slot_bytes = plain_bytes;
     if (c->precond) {
         c->oz_slot_bytes = oz_slice_bytes(c->ld, c->ld, c->oz_s);
         per_slot_bytes += 4 * mat * sizeof(double) + 2 * mat * sizeof(float) +
@@ -112,6 +113,10 @@ int alloc_slots(mpdo_ctx* c, int want) {
     }
     size_t free_b = 0, total_b = 0;
     CU(cudaMemGetInfo(&free_b, &total_b));
+    if (!c->mixed && 2 * per_slot_bytes > free_b) {   // an FP64 context can do without the stages' buffers
+        c->precond = false;
+        per_slot_bytes = plain_bytes;
+    }
     const size_t budget = free_b / 2;
     int s = std::max(1, std::min(want, (int)std::min<size_t>(budget / per_slot_bytes, 1 << 20)));
     if (c->cfg.max_slots > 0) s = std::min(s, c->cfg.max_slots);
