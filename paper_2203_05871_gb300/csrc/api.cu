@@ -244,7 +244,8 @@ void svd_buffers(mpdo_ctx* c, int s, OpDesc& d) {
     d.W = c->d_W + (size_t)s * mat;
     d.pre_ok = c->precond ? c->d_pre_ok + s : nullptr;
     d.rf = refine_on(c) ? c->d_refine + s : nullptr;
-    d.W0 = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
+    d.W0_staged = c->precond ? c->d_W0 + (size_t)s * mat : d.W;
+    d.W0 = d.plain ? d.W : d.W0_staged;
     d.W32 = c->precond ? c->d_W32 + (size_t)s * mat : nullptr;
     d.U32 = c->precond ? c->d_U32 + (size_t)s * mat : nullptr;
     d.D32 = c->precond ? c->d_D32 + (size_t)s * jacobi32_diag_floats(ld) : nullptr;
@@ -262,7 +263,7 @@ void svd_buffers(mpdo_ctx* c, int s, OpDesc& d) {
     d.oz_eb_z = c->precond ? c->d_oz_eb + z * oz_exp_ints(ld) : nullptr;
 }
 
-void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
+void fill_desc(mpdo_ctx* c, const Item& it, int s, bool plain, OpDesc& d) {
     const int N = c->N, cap = c->cap, ld = c->ld;
     const size_t mat = (size_t)ld * ld;
     const Op& op = c->layers[it.layer][it.idx];
@@ -277,8 +278,9 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d) {
     d.cr = dm[p + 2];
     d.m = 4 * d.cl;
     d.n = 4 * d.cr;
-    d.transposed = use_qr32(c) && d.m > d.n;
     d.c = std::min(d.m, d.n);
+    d.plain = plain;
+    d.transposed = use_qr32(c) && !d.plain && d.m > d.n;
     d.L = d.transposed ? d.m : d.n;   // rows of theta~^T, of Q^T theta~ or of R
     d.chi_max = c->chi_max[b];
     d.cutoff = c->cutoff[b];
@@ -372,14 +374,16 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
     {
         const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap);
         // FP32 QR (q32) or FP64 column QR: all co-resident CTAs shared in proportion to the work
-        const bool q32 = use_qr32(c);
-        auto plan_qr = [&](int slot, int& total, int*& dbase) -> int {
+        auto plan_qr = [&](bool q32, int slot, int& total, int*& dbase) -> int {
             std::vector<int> G(nops, 0);
             double wsum = 0.0;
-            for (int s = 0; s < nops; ++s) wsum += qwork[s];
+            auto takes = [&](int s) { return (use_qr32(c) && !c->h_desc[s].plain) == q32; };
+            for (int s = 0; s < nops; ++s)
+                if (takes(s)) wsum += qwork[s];
             const int R = q32 ? c->qr32_resident : c->qr_resident, QW = qr_threads() / 32;
             total = 0;
             for (int s = 0; s < nops; ++s) {
+                if (!takes(s)) continue;
                 const OpDesc& d = c->h_desc[s];
                 const int need = q32 ? qr32_max_ctas(d.c) : std::max(1, (d.n + QW - 1) / QW);
                 const int g = (int)std::floor((double)R * qwork[s] / std::max(wsum, 1.0));
@@ -435,19 +439,23 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
         } else {
             ProfScope p_qr(c, K_QR);
             int total = 0, *db = nullptr;
-            const int rc = plan_qr(2, total, db);
+            int rc = plan_qr(false, 2, total, db);
             if (rc) return rc;
-            if (q32) {
+            CU(launch_qr(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
+            out.qr_kernels = total > 0;
+            if ((rc = plan_qr(true, 3, total, db))) return rc;
+            if (total > 0) {
                 CU(launch_qr32(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
                 CU(launch_orthogonalise(c, c->d_desc, nops, OZ_FIRST, false, c->st));
-                out.qr_kernels = 1 + orthogonalise_kernels(c);
-            } else {
-                CU(launch_qr(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
+                out.qr_kernels += 1 + orthogonalise_kernels(c);
             }
             p_qr.stop();
         }
     }
-    if (c->precond) {
+    bool staged = false;
+    for (int s = 0; s < nops; ++s) staged = staged || (c->precond && !c->h_desc[s].plain);
+    out.staged = staged;
+    if (staged) {
         // FP32 preconditioning Jacobi on (W32 | U32)
         ProfScope p_j32(c, K_JACOBI32);
         int rc = run_jacobi(true, 1);
@@ -477,10 +485,15 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
               bool log_ranks) {
     const int nops = (int)items.size();
     const int N = c->N, cap = c->cap, ld = c->ld;
+    bool plain = use_qr32(c) && !c->mixed;
+    for (const Item& it : items) {
+        const int* dm = &c->h_dims[(size_t)it.b * (N + 1) + c->layers[it.layer][it.idx].p];
+        plain = plain && 4 * std::min(dm[0], dm[2]) <= kPlainRows;
+    }
     for (int s = 0; s < nops; ++s) {
         const Item& it = items[s];
         OpDesc& d = c->h_desc[s];
-        fill_desc(c, it, s, d);
+        fill_desc(c, it, s, plain, d);
         int fk = forced ? forced[s] : 0;
         if (!forced && step < c->forced_steps)
             fk = c->forced[((size_t)d.b * c->forced_steps + step) * c->n_ops + d.op];
@@ -576,7 +589,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     prof_collect(c, K_MERGE, fl_merge, c->precond ? kOzKernels + 1 : 1);
     prof_collect(c, K_QR, svd.qr_flops, svd.qr_kernels);
     prof_collect(c, K_JACOBI, fl_svd, 1);
-    if (c->precond) {
+    if (svd.staged) {
         prof_collect(c, K_JACOBI32, 0.0, 1);
         prof_collect(c, K_GEMM, svd.gemm_flops, svd_products_kernels(c));
     }

@@ -194,7 +194,7 @@ int chunk_ops(mpdo_ctx* c);
 // Descriptor of item `it` in workspace slot s, with the bond dimensions of
 // c->h_dims (forced rank and tape cleared).
 void svd_buffers(mpdo_ctx* c, int s, OpDesc& d);   // slot s's buffers of the SVD stages
-void fill_desc(mpdo_ctx* c, const Item& it, int s, OpDesc& d);
+void fill_desc(mpdo_ctx* c, const Item& it, int s, bool plain, OpDesc& d);
 
 // One chunk of (instance, op) items of a layer: merge + gate, QR, Jacobi SVD,
 // truncate, reconstruct.  forced (per item, or nullptr) imposes ranks; tape
@@ -232,6 +232,7 @@ cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, dou
 struct SvdWork {
     double qr_flops = 0.0, gemm_flops = 0.0;
     int qr_kernels = 1;
+    bool staged = false;   // some op took the preconditioning stages
 };
 int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out);
 // kernels one launch_svd_products issues

@@ -88,9 +88,12 @@ constexpr int kMaxChunk = 1024;
 
 __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops, const int* dims, int N, int Rj,
                                                          int Rq, int* cta64, int* cta32, int* ctaqr, int* ctaq32, int Rq32, int precond, int q32,
-                                                         int blocked,
+                                                         int mixed, int blocked,
                                                          const int* jb_table, int chi_cap, int* error) {
     __shared__ double work[kMaxChunk];
+    __shared__ int s_big;
+    if (threadIdx.x == 0) s_big = 0;
+    __syncthreads();
     __shared__ int cap[kMaxChunk];
     for (int s = threadIdx.x; s < nops; s += blockDim.x) {
         OpDesc& d = descs[s];
@@ -100,8 +103,15 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
         d.cr = dm[d.p + 2];
         d.m = 4 * d.cl;
         d.n = 4 * d.cr;
-        d.transposed = q32 && d.m > d.n;
         d.c = min(d.m, d.n);
+        if (d.c > kPlainRows) s_big = 1;
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < nops; s += blockDim.x) {
+        OpDesc& d = descs[s];
+        d.plain = q32 && !mixed && !s_big;
+        d.transposed = q32 && !d.plain && d.m > d.n;
+        d.W0 = d.plain ? d.W : d.W0_staged;
         d.L = d.transposed ? d.m : d.n;
         d.jb = jacobi_block_rows(d.transposed ? d.L + d.c : d.L, d.c, 8);
         if (jb_table && !d.transposed) {   // autotuned rows per block of this (chi_l, chi_r) class
@@ -126,9 +136,14 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
     for (int s = threadIdx.x; s < nops; s += blockDim.x) {
         const OpDesc& d = descs[s];
         work[s] = (double)d.m * d.n * d.c;
-        cap[s] = q32 ? qr32_max_ctas(d.c) : max(1, (d.n + kQrWarps - 1) / kQrWarps);
+        cap[s] = q32 && !d.plain ? 0 : max(1, (d.n + kQrWarps - 1) / kQrWarps);
     }
-    if (!blocked) bad |= plan_ctas(work, cap, nops, q32 ? Rq32 : Rq, q32 ? ctaq32 : ctaqr, G);
+    if (!blocked) bad |= plan_ctas(work, cap, nops, Rq, ctaqr, G);
+    if (q32) {
+        __syncthreads();
+        for (int s = threadIdx.x; s < nops; s += blockDim.x) cap[s] = descs[s].plain ? 0 : qr32_max_ctas(descs[s].c);
+        bad |= plan_ctas(work, cap, nops, Rq32, ctaq32, G);
+    }
     if (bad) *error = 1;
 }
 
@@ -190,7 +205,8 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             const int nops = ch.nops;
             plan_chunk_kernel<<<1, 256, 0, st>>>(ch.d_desc, nops, c->d_dims, c->N, g->Rj, g->Rq, ch.d_cta64,
                                                  ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, g->Rq32,
-                                                 c->precond ? 1 : 0, q32 ? 1 : 0, blocked ? 1 : 0, c->d_jb_table, cap,
+                                                 c->precond ? 1 : 0, q32 ? 1 : 0, c->mixed ? 1 : 0, blocked ? 1 : 0,
+                                                 c->d_jb_table, cap,
                                                  g->d_error);
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
@@ -204,13 +220,16 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
             if (blocked) {
                 CU(launch_qr_blocked(ch.d_desc, nops, cap, c->d_oz, timeout_ns, st, 0));
-            } else if (q32) {
-                CU(launch_qr32(ch.d_desc, ch.d_ctaq32, ch.d_ctaq32 + g->Rq32, ch.d_ctaq32 + 2 * g->Rq32, c->d_sync,
-                               g->Rq32, timeout_ns, ld, st));
-                CU(launch_orthogonalise(c, ch.d_desc, nops, OZ_FIRST, false, st));
             } else {
-                CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
-                             timeout_ns, ld, st));
+                if (!q32 || !c->mixed)   // mixed contexts have no plain ops
+                    CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
+                                 timeout_ns, ld, st));
+                if (q32) {
+                    CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
+                    CU(launch_qr32(ch.d_desc, ch.d_ctaq32, ch.d_ctaq32 + g->Rq32, ch.d_ctaq32 + 2 * g->Rq32, c->d_sync,
+                                   g->Rq32, timeout_ns, ld, st));
+                    CU(launch_orthogonalise(c, ch.d_desc, nops, OZ_FIRST, false, st));
+                }
             }
             if (c->precond) {
                 CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
@@ -254,7 +273,7 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
             Chunk ch;
             ch.nops = nops;
             std::vector<OpDesc> h(nops);
-            for (int s = 0; s < nops; ++s) fill_desc(c, items[s0 + s], s, h[s]);
+            for (int s = 0; s < nops; ++s) fill_desc(c, items[s0 + s], s, false, h[s]);
             CU(dalloc(&ch.d_desc, (size_t)nops));
             CU(dalloc(&ch.d_cta64, (size_t)2 * g->Rj + nops));
             CU(dalloc(&ch.d_ctaqr, (size_t)2 * g->Rq + nops));

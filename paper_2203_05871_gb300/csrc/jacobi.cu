@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
     const int g = cta_rank[blockIdx.x];
     const int G = group[op];
     const OpDesc& d = descs[op];
-    if (d.rf && d.rf->state == kRefineDone) return;   // finished by the refinement (refine.cu)
+    if (d.rf && !d.plain && d.rf->state == kRefineDone) return;   // finished by the refinement (refine.cu)
     unsigned* sw = sync + (size_t)op * kSyncWords;
     const int c = d.c, L = d.L;
     const int b = d.jb;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned gen = 0;
     __shared__ double s_floor2, s_red[kWarps];
-    __shared__ int s_conv;
+    __shared__ int s_conv, s_settled;
     __shared__ unsigned s_rho2;
     __shared__ int s_pair;
 
@@ -266,7 +266,8 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
     double* dscale = d.snorm + ld;   // per-row scales (the QR's column norms are dead here)
     C.rho2 = &s_rho2;
     C.thr = 0.0;
-    double kth = 0.0;
+    double kth = 0.0, cut = 0.0;   // cut: cutoff_floor, from the same sweep on (before, rows that are not
+                                   // yet orthogonal to one another would draw the rest along sweep by sweep)
     float rho2_stop;
     {
         const double tol = tol_in > 0.0 ? tol_in : sqrt((double)(L > 1 ? L : 1)) * DBL_EPSILON;
@@ -340,15 +341,17 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
                 const int kk = d.chi_max + max(16, d.chi_max / 8);
                 const bool settled = sweep > 0
                                          ? __uint_as_float(ld_acquire(&sw[8 + kMaxSweepsCap + sweep - 1])) <= 1e-8f
-                                         : (d.pre_ok && __ldcg(d.pre_ok) == 1);
+                                         : (d.pre_ok && !d.plain && __ldcg(d.pre_ok) == 1);
                 s_conv = settled && !d.full_svd && kk < c;
+                s_settled = settled;
             }
             __syncthreads();
             // the threshold is fixed when the gate first opens, so that a row
             // near it keeps its side (a row changing side later would bring its
             // unprocessed pairs back and cost another sweep)
             if (s_conv && kth == 0.0) kth = kth_largest<kThreads, 4 * kMaxChi>(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
-            C.thr = fmax(kth, cutoff_floor(d, s_floor2 / (DBL_EPSILON * DBL_EPSILON)));
+            if (s_settled) cut = cutoff_floor(d, s_floor2 / (DBL_EPSILON * DBL_EPSILON));
+            C.thr = fmax(kth, cut);
             __syncthreads();
             // The block pairs of a sweep go to the op's CTAs through a shared
             // counter (position q: round q / npair, pair q % npair), and a round

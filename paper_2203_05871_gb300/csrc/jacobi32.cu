@@ -434,6 +434,7 @@ __global__ void __launch_bounds__(NT, 1) jacobi32_kernel(const OpDesc* descs, co
     const int rank = cta_rank[blockIdx.x];
     const int G = group[op];
     const OpDesc& d = descs[op];
+    if (d.plain) return;
     unsigned* sw = sync + (size_t)op * kSyncWords;
     const int c = d.c, L = d.L;
     float* W = d.W32;

@@ -337,6 +337,7 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap, bool z) {
     const bool first = (kind & OZ_FIRST) != 0;
     kind &= OZ_FIRST - 1;
     if (z && !d.transposed) kind = -1;
+    if (d.plain && kind != OZ_MERGE && kind != OZ_RECON) kind = -1;
     auto rowmajor = [](const void* base, int f32, long long ld_) {   // (r, k) at r * ld + k
         return OzOperand{base, f32, ld_, 1, 0, 1, 1, nullptr, nullptr, 0};
     };
@@ -1001,7 +1002,7 @@ namespace {
 
 // The scratch of mpdo_gemm_tc comes from a pool of its own per device, which keeps
 // up to 256 MB between calls (the slices of a 4096 x 4096 x 2048 product) and
-// returns the rest when a call's stream is synchronised; the driver also takes
+// returns the rest when a call's stream is synchronised; CUDA also takes
 // it back when another allocation runs out.  Allocation is in stream order, so calls
 // on several streams and threads do not share a buffer.
 constexpr unsigned long long kGemmPoolKeep = 256ull << 20;

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(NT) refine_diag_kernel(const OpDesc* descs, in
     grid_begin();
     const OpDesc& d = descs[blockIdx.x];
     RefineOp& r = *d.rf;
+    if (d.plain) return;
     if (r.state != kRefineActive) {
         if (threadIdx.x == 0) r.order = r.turn = 0;   // no rotation in this iteration
         return;
@@ -131,7 +132,7 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
     RefineOp& r = *d.rf;
     const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int blocks = (d.c + NT / 32 - 1) / (NT / 32);
-    if ((int)blockIdx.x >= blocks || __ldcg(&r.state) != kRefineActive) return;
+    if ((int)blockIdx.x >= blocks || d.plain || __ldcg(&r.state) != kRefineActive) return;
     if (i < d.c) {
         const float tol = (float)(tol_in > 0.0 ? tol_in : sqrt((double)d.L) * DBL_EPSILON);
         // pairs within a tolerance well above the Gram matrix's own error are turned too,
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(NT) refine_x_kernel(const OpDesc* descs, int l
 __global__ void __launch_bounds__(NT) refine_turn_kernel(const OpDesc* descs, int ld) {
     grid_begin();
     const OpDesc& d = descs[blockIdx.y];
-    if (!d.rf->turn) return;
+    if (d.plain || !d.rf->turn) return;
     const int i = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= d.c) return;
     const int j = partner_of(d)[i];
