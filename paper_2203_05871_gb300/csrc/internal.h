@@ -214,7 +214,7 @@ struct OzProblem {
     int ldd, d_f32, sub_identity;
     int levels;          // slice pairs (t, u) with t + u < levels are formed (0: all S levels)
     int unit_d;          // D's rows are of unit norm: levels follow from the operands' exponents
-    int sym;             // C (f64, no gather) is symmetric: tiles below the diagonal are mirrored, not computed
+    int sym;             // C (f64, no gather) is symmetric: entries below the diagonal are mirrored, not computed
     void *as, *bs;       // slice blocks of A and B
     int *ea, *eb;        // row / column exponents
     int Mt, Nt, Kt;      // tiles (128 rows, 64 columns, 64 bytes of K)

@@ -795,7 +795,9 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
 #pragma unroll
             for (int jj = 0; jj < CP; ++jj) {
                 const int j = j0 + jj;
-                if (j >= N) continue;
+                // every entry of a symmetric result has one writer: below the diagonal the mirror
+                // of (j, i), whose value differs by rounding where the operands do
+                if (j >= N || (P.sym && j < i)) continue;
                 double v = scaled(hi[jj], lo[jj], ei + P.eb[j]);
                 if (pow2)
                     v = __longlong_as_double(__double_as_longlong(v) ^ (ab & (1ll << 63)));
