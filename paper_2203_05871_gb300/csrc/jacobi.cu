@@ -349,7 +349,11 @@ __global__ void __launch_bounds__(kThreads, 1) jacobi_kernel(const OpDesc* descs
             // the threshold is fixed when the gate first opens, so that a row
             // near it keeps its side (a row changing side later would bring its
             // unprocessed pairs back and cost another sweep)
-            if (s_conv && kth == 0.0) kth = kth_largest<kThreads, 4 * kMaxChi>(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
+            // (every CTA reads all norms, so a barrier before a pair of this sweep changes them)
+            if (s_conv && kth == 0.0) {
+                kth = kth_largest<kThreads, 4 * kMaxChi>(d.snorm, c, d.chi_max + max(16, d.chi_max / 8));
+                if (!op_barrier(sw, G, gen, timeout_ns)) goto timeout;
+            }
             if (s_settled) cut = cutoff_floor(d, s_floor2 / (DBL_EPSILON * DBL_EPSILON));
             C.thr = fmax(kth, cut);
             __syncthreads();

@@ -525,6 +525,9 @@ __global__ void __launch_bounds__(NT, 1) jacobi32_kernel(const OpDesc* descs, co
                                                            : __ldcg(diag + (size_t)(j / NB) * NB * NB + (j % NB) * (NB + 1));
                                      },
                                      c, kk);
+                // every CTA has read the norms before a pair of this sweep changes them, or
+                // their limits, and with them the sweep that ends the pass, could differ
+                if (sweep > 0 && !op_barrier(sw, G, gen, timeout_ns)) goto timeout;
             }
             lm.lim = fmaxf(lm.lim, (float)cutoff_floor(d, (double)c));   // rows of unit mean square norm
             if (rank == 0 && threadIdx.x == 0) atomicExch(&sw[kSwQueue + ((sweep + 1) & 1)], 0u);

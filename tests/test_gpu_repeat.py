@@ -35,3 +35,25 @@ def test_entropies_repeat_themselves(chi):
         first = got if first is None else first
         assert np.array_equal(got, first)
     s.close()
+
+
+@pytest.mark.parametrize("precision", ["FP64", "MIXED_TF32"])
+def test_step_repeats_itself(precision):
+    """A step from one state, several times, bit for bit: many CTAs work on a bond of 384
+    rows, most of them discarded, and every CTA has to find the same limit below which
+    rows do not count from norms that others are about to change."""
+    import paper_2203_05871_gb300 as M
+    n, chi = 10, 96
+    wl = W.random_model(n, W.chain_bonds(n), 63, chi_max=chi, cutoff=1e-12)
+    dims, tens = W.random_mpo_state(n, chi, seed=64, decay=0.05)
+    s = M.Solver(n, batch=1, chi_cap=chi, precision=getattr(M, precision))
+    s.build_gates(wl)
+    first = None
+    for _ in range(6):
+        s.set_state(0, dims, tens)
+        s.step(1)
+        got = s.get_state(0)
+        first = got if first is None else first
+        assert got[0] == first[0]
+        assert all(np.array_equal(a, b) for a, b in zip(got[1], first[1]))
+    s.close()
