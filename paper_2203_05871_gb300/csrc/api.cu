@@ -481,19 +481,25 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
     return MPDO_OK;
 }
 
+// Whether instance b's ops of a layer leave the SVD's stages out (kPlainRows).  The
+// bonds on either side of an op are not touched by the layer's other ops, so the
+// answer is the same for every chunk of the layer.
+static bool plain_layer(const mpdo_ctx* c, int b, int layer) {
+    if (!use_qr32(c) || c->mixed) return false;
+    const int* dm = &c->h_dims[(size_t)b * (c->N + 1)];
+    for (const Op& o : c->layers[layer])
+        if (4 * std::min(dm[o.p], dm[o.p + 2]) > kPlainRows) return false;
+    return true;
+}
+
 int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* forced, const TapeSlot* tape,
               bool log_ranks) {
     const int nops = (int)items.size();
     const int N = c->N, cap = c->cap, ld = c->ld;
-    bool plain = use_qr32(c) && !c->mixed;
-    for (const Item& it : items) {
-        const int* dm = &c->h_dims[(size_t)it.b * (N + 1) + c->layers[it.layer][it.idx].p];
-        plain = plain && 4 * std::min(dm[0], dm[2]) <= kPlainRows;
-    }
     for (int s = 0; s < nops; ++s) {
         const Item& it = items[s];
         OpDesc& d = c->h_desc[s];
-        fill_desc(c, it, s, plain, d);
+        fill_desc(c, it, s, plain_layer(c, it.b, it.layer), d);
         int fk = forced ? forced[s] : 0;
         if (!forced && step < c->forced_steps)
             fk = c->forced[((size_t)d.b * c->forced_steps + step) * c->n_ops + d.op];
@@ -740,7 +746,7 @@ int mpdo_init(mpdo_ctx** out, const mpdo_config* cfg, void* cuda_stream) {
         (e = dalloc(&c->d_one_a, (size_t)B * N * 4)) != cudaSuccess ||
         (e = dalloc(&c->d_one_b, (size_t)B * N)) != cudaSuccess ||
         (e = dalloc(&c->d_out, (size_t)B * N * N)) != cudaSuccess ||
-        (e = dalloc(&c->d_q, (size_t)N)) != cudaSuccess ||
+        (e = dalloc(&c->d_q, (size_t)2 * N)) != cudaSuccess ||
         (e = dalloc(&c->d_pairs, (size_t)3 * N * N + 2 * N)) != cudaSuccess) {
         fail(e == cudaErrorMemoryAllocation ? MPDO_ENOMEM : MPDO_ECUDA,
              std::string("device allocation: ") + cudaGetErrorString(e));

@@ -47,12 +47,13 @@ __global__ void gram_unit_kernel(double* W, size_t mat, int m) {
     W[(size_t)i * mat] = 1.0;
 }
 
-// norms[s * 2 ld + j] = |row j| of the matrix in slot s (rows j < chi[s])
-__global__ void row_norms_kernel(const double* W, size_t mat, int ld, const int* chi, double* norms) {
+// norms[s * 2 ld + j] = |row j| of the matrix in slot s (rows j < chi[s]), staged or not
+__global__ void row_norms_kernel(const double* W, const double* Ws, size_t mat, int ld, const int* chi,
+                                 const int* staged, double* norms) {
     const int s = blockIdx.y;
     const int n = chi[s];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double* M = W + (size_t)s * mat;
+    const double* M = (staged[s] ? Ws : W) + (size_t)s * mat;
     for (int j = blockIdx.x * 8 + warp; j < n; j += gridDim.x * 8) {
         double a = 0.0;
         for (int k = lane; k < n; k += 32) a = fma(M[(size_t)j * ld + k], M[(size_t)j * ld + k], a);
@@ -63,9 +64,10 @@ __global__ void row_norms_kernel(const double* W, size_t mat, int ld, const int*
 }
 
 // slot s of C: [j][k] /= sqrt(|x_j| |y_k|) (0 where either norm is 0), x the rows of slot
-// s and y those of its partner: F_X F_Y^T (even slots) or its transpose (odd ones)
-__global__ void scale_kernel(double* C, size_t mat, int ld, const int* chi, const double* norms, int step) {
-    const int s = blockIdx.y * step;
+// s and y those of its partner: F_X F_Y^T (even slots) or its transpose (odd ones, staged)
+__global__ void scale_kernel(double* C, size_t mat, int ld, const int* chi, const int* staged, const double* norms) {
+    const int s = blockIdx.y;
+    if ((s & 1) && !staged[s]) return;
     const int n = chi[s];
     const double* nx = norms + (size_t)s * 2 * ld;
     const double* ny = norms + (size_t)(s ^ 1) * 2 * ld;
@@ -78,10 +80,11 @@ __global__ void scale_kernel(double* C, size_t mat, int ld, const int* chi, cons
 }
 
 // out[b0 + i] = OSEE from the row norms s_k of C_i after its Jacobi SVD
-__global__ void osee_kernel(const double* C, size_t mat, int ld, const int* chi, int b0, double* out) {
+__global__ void osee_kernel(const double* C, const double* Cs, size_t mat, int ld, const int* chi, const int* staged,
+                            int b0, double* out) {
     const int i = blockIdx.x;
     const int n = chi[2 * i];
-    const double* M = C + (size_t)(2 * i) * mat;
+    const double* M = (staged[2 * i] ? Cs : C) + (size_t)(2 * i) * mat;
     __shared__ double s2[4 * kMaxChi];
     __shared__ double red[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -234,12 +237,12 @@ int run_plan(mpdo_ctx* c, GqPlan& P) {
     return MPDO_OK;
 }
 
-// Whether SVDs of n x n matrices, n >= min_chi, take the stages of a step's SVDs
+// Whether the SVDs of an instance's chi x chi matrices take the stages of a step's SVDs
 // (FP32 QR and Jacobi, tensor-core refinement, FP64 Jacobi) in place of the FP64
 // Jacobi alone.  FP64 contexts only: a mixed one's products resolve 2^-48.  Below
 // 32 rows a matrix is a single block pair of one CTA and the stages' launches cost
 // more than its sweeps.
-bool staged_svd(const mpdo_ctx* c, int min_chi) { return refine_on(c) && c->oz_s == 7 && min_chi >= 32; }
+bool staged_svd(const mpdo_ctx* c, int chi) { return refine_on(c) && c->oz_s == 7 && chi >= 32; }
 
 // zero rows and columns from chi up to the next multiple of 4 (the stages' row groups)
 __global__ void pad_kernel(double* M, size_t mat, int ld, const int* chi) {
@@ -257,6 +260,7 @@ int run_svds(mpdo_ctx* c, double* M, double* MT, bool staged, const std::vector<
     const int ld = c->ld;
     const size_t mat = (size_t)ld * ld;
     const int nops = (int)slots.size();
+    if (nops == 0) return MPDO_OK;
     for (int k = 0; k < nops; ++k) {
         OpDesc d{};
         const int s = slots[k], n = staged ? (chis[k] + 3) & ~3 : chis[k];
@@ -357,6 +361,7 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
     double* dst = out_on_device ? out : c->d_out;
     const int per = std::max(1, c->slots / 2);
     int* d_chi = c->d_q;   // [2 m] chi of each slot (ints; N >= 2 m is not guaranteed, so chunk by it too)
+    int* d_staged = c->d_q + N;   // [2 m] whether its SVD takes the stages
     const int per_chi = std::max(1, N / 2);
     for (int b0 = 0; b0 < B; b0 += std::min(per, per_chi)) {
         const int m = std::min(std::min(per, per_chi), B - b0);
@@ -367,56 +372,66 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
         plan_right(c, b0, m, bond + 1, P);
         rc = run_plan(c, P);
         if (rc) return rc;
-        std::vector<int> slots, chis, inst, chi2(2 * m);
+        // the instances of each route: [0] the FP64 Jacobi alone, [1] the stages
+        std::vector<int> slots[2], chis[2], inst[2], chi2(2 * m), route(2 * m);
+        int maxchi = 1;
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
             const int chi = c->h_dims[(size_t)b * (N + 1) + bond + 1];
+            const int st = staged_svd(c, chi) ? 1 : 0;
+            maxchi = std::max(maxchi, chi);
             for (int h = 0; h < 2; ++h) {
-                slots.push_back(2 * i + h);
-                chis.push_back(chi);
-                inst.push_back(b);
+                slots[st].push_back(2 * i + h);
+                chis[st].push_back(chi);
+                inst[st].push_back(b);
                 chi2[2 * i + h] = chi;
+                route[2 * i + h] = st;
             }
         }
         CU(cudaMemcpyAsync(d_chi, chi2.data(), sizeof(int) * 2 * m, cudaMemcpyHostToDevice, c->st));
-        const auto mm = std::minmax_element(chis.begin(), chis.end());
-        const int maxchi = *mm.second;
-        const bool staged = staged_svd(c, *mm.first);
-        double* F = staged ? c->d_W : c->d_Z;   // the rows of X and Y
-        if (staged) {
+        CU(cudaMemcpyAsync(d_staged, route.data(), sizeof(int) * 2 * m, cudaMemcpyHostToDevice, c->st));
+        const bool any = !slots[1].empty();
+        if (any) {
             pad_kernel<<<2 * m, 256, 0, c->st>>>(c->d_Z, mat, ld, d_chi);
             CU(cudaGetLastError());
         }
-        rc = run_svds(c, c->d_Z, c->d_Z, staged, slots, chis, inst);   // X and Y factored
-        if (rc) return rc;
-        row_norms_kernel<<<dim3((maxchi + 7) / 8, 2 * m), 256, 0, c->st>>>(F, mat, ld, d_chi, c->d_snorm);
+        for (int st = 0; st < 2; ++st) {   // X and Y factored: their rows in d_Z, staged in d_W
+            rc = run_svds(c, c->d_Z, c->d_Z, st == 1, slots[st], chis[st], inst[st]);
+            if (rc) return rc;
+        }
+        row_norms_kernel<<<dim3((maxchi + 7) / 8, 2 * m), 256, 0, c->st>>>(c->d_Z, c->d_W, mat, ld, d_chi, d_staged,
+                                                                           c->d_snorm);
         CU(cudaGetLastError());
         // C_i = (rows of X) (rows of Y)^T into thetap slot 2i, then scaled to F_X F_Y^T
         // (staged: its transpose into slot 2i + 1)
         GqPlan Pc;
         Pc.begin();
-        const int step = staged ? 1 : 2;
-        for (int s = 0; s < 2 * m; s += step)
+        for (int s = 0; s < 2 * m; ++s) {
+            if ((s & 1) && !route[s]) continue;
+            double* F = route[s] ? c->d_W : c->d_Z;
             Pc.add(GemmDesc{chi2[s], chi2[s], chi2[s], F + (size_t)s * mat, ld, 0, F + (size_t)(s ^ 1) * mat, ld, 0,
                             1, c->d_thetap + (size_t)s * mat, ld, 1.0, 0.0, nullptr, 0, 0, 0, 0, 0},
                    c->d_status + b0 + s / 2);
+        }
         rc = run_plan(c, Pc);
         if (rc) return rc;
-        scale_kernel<<<dim3(64, staged ? 2 * m : m), 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, c->d_snorm, step);
+        scale_kernel<<<dim3(64, 2 * m), 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, d_staged, c->d_snorm);
         CU(cudaGetLastError());
-        std::vector<int> s1, c1, i1;
-        for (int i = 0; i < m; ++i) {
-            s1.push_back(2 * i);
-            c1.push_back(chi2[2 * i]);
-            i1.push_back(b0 + i);
-        }
-        if (staged) {
+        if (any) {
             pad_kernel<<<2 * m, 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi);
             CU(cudaGetLastError());
         }
-        rc = run_svds(c, c->d_thetap, c->d_thetap + mat, staged, s1, c1, i1);
-        if (rc) return rc;
-        osee_kernel<<<m, 512, 0, c->st>>>(staged ? c->d_W : c->d_thetap, mat, ld, d_chi, b0, dst);
+        for (int st = 0; st < 2; ++st) {
+            std::vector<int> s1, c1, i1;
+            for (size_t k = 0; k < slots[st].size(); k += 2) {
+                s1.push_back(slots[st][k]);
+                c1.push_back(chis[st][k]);
+                i1.push_back(inst[st][k]);
+            }
+            rc = run_svds(c, c->d_thetap, c->d_thetap + mat, st == 1, s1, c1, i1);
+            if (rc) return rc;
+        }
+        osee_kernel<<<m, 512, 0, c->st>>>(c->d_thetap, c->d_W, mat, ld, d_chi, d_staged, b0, dst);
         CU(cudaGetLastError());
     }
     return finish(c, out, out_on_device);

@@ -89,11 +89,9 @@ constexpr int kMaxChunk = 1024;
 __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops, const int* dims, int N, int Rj,
                                                          int Rq, int* cta64, int* cta32, int* ctaqr, int* ctaq32, int Rq32, int precond, int q32,
                                                          int mixed, int blocked,
-                                                         const int* jb_table, int chi_cap, int* error) {
+                                                         const int* jb_table, int chi_cap, const int* lp, int n_lp,
+                                                         int* error) {
     __shared__ double work[kMaxChunk];
-    __shared__ int s_big;
-    if (threadIdx.x == 0) s_big = 0;
-    __syncthreads();
     __shared__ int cap[kMaxChunk];
     for (int s = threadIdx.x; s < nops; s += blockDim.x) {
         OpDesc& d = descs[s];
@@ -104,12 +102,8 @@ __global__ void __launch_bounds__(256) plan_chunk_kernel(OpDesc* descs, int nops
         d.m = 4 * d.cl;
         d.n = 4 * d.cr;
         d.c = min(d.m, d.n);
-        if (d.c > kPlainRows) s_big = 1;
-    }
-    __syncthreads();
-    for (int s = threadIdx.x; s < nops; s += blockDim.x) {
-        OpDesc& d = descs[s];
-        d.plain = q32 && !mixed && !s_big;
+        d.plain = q32 && !mixed;   // the rule of run_chunk: all bonds of the instance's layer
+        for (int i = 0; d.plain && i < n_lp; ++i) d.plain = 4 * min(dm[lp[i]], dm[lp[i] + 2]) <= kPlainRows;
         d.transposed = q32 && !d.plain && d.m > d.n;
         d.W0 = d.plain ? d.W : d.W0_staged;
         d.L = d.transposed ? d.m : d.n;
@@ -159,6 +153,8 @@ struct Chunk {
     int nops = 0;
     OpDesc* d_desc = nullptr;
     int *d_cta64 = nullptr, *d_cta32 = nullptr, *d_ctaqr = nullptr, *d_ctaq32 = nullptr;
+    int* d_lp = nullptr;   // path positions of the layer's ops
+    int n_lp = 0;
 };
 
 }  // namespace
@@ -183,7 +179,7 @@ void release(GraphState* g) {
     g->graph = nullptr;
     for (auto& L : g->chunks)
         for (auto& ch : L) {
-            void* ptrs[] = {ch.d_desc, ch.d_cta64, ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32};
+            void* ptrs[] = {ch.d_desc, ch.d_cta64, ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, ch.d_lp};
             for (void* p : ptrs)
                 if (p) cudaFree(p);
         }
@@ -206,8 +202,7 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
             plan_chunk_kernel<<<1, 256, 0, st>>>(ch.d_desc, nops, c->d_dims, c->N, g->Rj, g->Rq, ch.d_cta64,
                                                  ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, g->Rq32,
                                                  c->precond ? 1 : 0, q32 ? 1 : 0, c->mixed ? 1 : 0, blocked ? 1 : 0,
-                                                 c->d_jb_table, cap,
-                                                 g->d_error);
+                                                 c->d_jb_table, cap, ch.d_lp, ch.n_lp, g->d_error);
             CU(cudaGetLastError());
             CU(cudaMemsetAsync(c->d_sweeps, 0, sizeof(int) * nops, st));
             if (c->precond) {
@@ -274,6 +269,11 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
             ch.nops = nops;
             std::vector<OpDesc> h(nops);
             for (int s = 0; s < nops; ++s) fill_desc(c, items[s0 + s], s, false, h[s]);
+            std::vector<int> lp;
+            for (const Op& o : c->layers[li]) lp.push_back(o.p);
+            ch.n_lp = (int)lp.size();
+            CU(dalloc(&ch.d_lp, lp.size()));
+            CU(cudaMemcpyAsync(ch.d_lp, lp.data(), sizeof(int) * lp.size(), cudaMemcpyHostToDevice, c->st));
             CU(dalloc(&ch.d_desc, (size_t)nops));
             CU(dalloc(&ch.d_cta64, (size_t)2 * g->Rj + nops));
             CU(dalloc(&ch.d_ctaqr, (size_t)2 * g->Rq + nops));

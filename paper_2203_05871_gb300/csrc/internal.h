@@ -44,7 +44,7 @@ struct OpDesc {
     int cl, cm, cr;    // bond dims chi_{p-1}, chi_p, chi_{p+1}
     int m, n;          // 4*cl, 4*cr
     int transposed;    // 1 (m > n, preconditioning stages): the SVD is that of theta~^T, and Z carries its rotations
-    int plain;         // 1: of a chunk too small for the preconditioning stages (FP64 QR, then the FP64 Jacobi pass)
+    int plain;         // 1: too small for the preconditioning stages (FP64 QR, then the FP64 Jacobi pass)
     int c, L;          // Jacobi problem: c rows of length L
     int jb;            // Jacobi block size (rows per shared-memory block), FP64 pass
     int chi_max;
@@ -303,11 +303,12 @@ cudaError_t qrb_prepare();
 cudaError_t launch_qr_blocked(const OpDesc* d_desc, int nops, int chi_cap, OzProblem* probs,
                               unsigned long long timeout_ns, cudaStream_t st, int r_max);
 
-// A chunk of an FP64 context whose bonds all have at most this many rows leaves the
-// stages out: their 60 launches take longer than the FP64 QR and Jacobi pass of a few
-// rows (evolutions at their start: a chain of 7 over 11 steps 25.9 -> 17.9 ms, a grid of
-// 3 x 3 203 -> 192 ms).  One larger bond in the chunk and the small ones are in its
-// shadow (a limit bond by bond cost the chain of 8 at chi 32 a quarter).
+// A layer of an instance of an FP64 context whose bonds all have at most this many rows
+// leaves the stages out: their 60 launches take longer than the FP64 QR and Jacobi pass
+// of a few rows (evolutions at their start: a chain of 7 over 11 steps 25.9 -> 17.9 ms, a
+// grid of 3 x 3 203 -> 192 ms).  One larger bond in the layer and the small ones are in
+// its shadow (a limit bond by bond cost the chain of 8 at chi 32 a quarter).  The rule
+// looks at one instance, so that what becomes of it does not depend on its neighbours.
 constexpr int kPlainRows = 20;
 // FP32 Householder QR (qr32.cu) of the preconditioned SVD: Q^T (c x c) into U32, the
 // row order of W0 = Q^T theta~ (or Q^T theta~^T) graded.  Wider panels than one CTA

@@ -641,12 +641,14 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tslot;
     int lv = P.levels > 0 ? P.levels : kS;   // slice pairs t + u < lv
-    if (P.unit_d) {   // what A B adds to entries of a unit row of D is below 2^(e_i + f_j)
+    // What A B adds to entries of a unit row of D is below 2^(e_i + f_j).  Over blocks of
+    // 128 x 64 whatever TN is: TN follows from the launch's other problems, the result must not.
+    if (P.unit_d) {
         if (threadIdx.x < kTileM) {
             const int i = mt * kTileM + threadIdx.x;
             if (i < P.M) atomicMax(&s_ea, P.ea[i]);
-        } else if (threadIdx.x < kTileM + TN) {
-            const int j = nt * TN + threadIdx.x - kTileM;
+        } else if (threadIdx.x < kTileM + kTileN) {
+            const int j = nt * TN / kTileN * kTileN + threadIdx.x - kTileM;
             if (j < N) atomicMax(&s_eb, P.eb[j]);
         }
         __syncthreads();
