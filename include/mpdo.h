@@ -180,7 +180,8 @@ int mpdo_renyi2(mpdo_ctx *ctx, double *out, int out_on_device);
  * its exact Schmidt values s_k: Gram matrices X, Y of the two halves (batched
  * products of FP64 accuracy), X = F_X^T F_X and Y = F_Y^T F_Y from SVDs at the strict
  * FP64 tolerance, s_k the singular values of F_X F_Y^T (a third SVD).  Independent of the
- * gauge of the stored tensors.  out as for mpdo_renyi2.  A Jacobi SVD that hits
+ * gauge of the stored tensors as far as FP64 resolves the Gram matrices, which square it
+ * (MPDO_FP64: a bond whose columns span six decades).  out as for mpdo_renyi2.  A Jacobi SVD that hits
  * cfg.jacobi_max_sweeps sets MPDO_ST_NOCONV for its instance (mpdo_status).
  * EINVAL (bond), ESTATE, ECUDA. */
 int mpdo_osee(mpdo_ctx *ctx, int bond, double *out, int out_on_device);
@@ -194,7 +195,9 @@ int mpdo_status(mpdo_ctx *ctx, int *status, double *max_discarded, int *chi, dou
 /* Replace instance b's state: dims[N+1] bond dimensions (dims[0] = dims[N] = 1,
  * each <= chi_max of b), tensors = the N site tensors (dims[p], 4, dims[p+1])
  * packed one after another, row-major, host memory.  Schmidt weights are set
- * to 1.  Used to start from a prepared (e.g. saturated) state. */
+ * to 1.  Used to start from a prepared (e.g. saturated) state.  MPDO_FP64: a bond
+ * whose gauge would cost a contraction more than four bits (A D and D^-1 B with D over
+ * many decades) takes FP64 dot products until its next op. */
 int mpdo_set_state(mpdo_ctx *ctx, int b, const int *dims, const double *tensors);
 
 /* Copy instance b's state out: dims[N+1] and the packed site tensors (at most

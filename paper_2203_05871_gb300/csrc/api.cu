@@ -280,6 +280,7 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, bool plain, OpDesc& d) {
     d.n = 4 * d.cr;
     d.c = std::min(d.m, d.n);
     d.plain = plain;
+    d.dot64 = !c->precond;
     d.transposed = use_qr32(c) && !d.plain && d.m > d.n;
     d.L = d.transposed ? d.m : d.n;   // rows of theta~^T, of Q^T theta~ or of R
     d.chi_max = c->chi_max[b];
@@ -496,10 +497,14 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
               bool log_ranks) {
     const int nops = (int)items.size();
     const int N = c->N, cap = c->cap, ld = c->ld;
+    bool wide = false;
     for (int s = 0; s < nops; ++s) {
         const Item& it = items[s];
         OpDesc& d = c->h_desc[s];
-        fill_desc(c, it, s, plain_layer(c, it.b, it.layer), d);
+        const bool w = wide_op(c, it.b, c->layers[it.layer][it.idx].p);
+        fill_desc(c, it, s, w || plain_layer(c, it.b, it.layer), d);
+        if (w) d.dot64 = 1;
+        wide = wide || w;
         int fk = forced ? forced[s] : 0;
         if (!forced && step < c->forced_steps)
             fk = c->forced[((size_t)d.b * c->forced_steps + step) * c->n_ops + d.op];
@@ -541,9 +546,8 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     if (c->precond) {
         CU(launch_oz_ops(c->d_desc, nops, OZ_MERGE, cap, c->oz_s, false, timeout_ns, c->st));
         CU(launch_gate_weight(c->d_desc, nops, cap, c->st));
-    } else {
-        CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
     }
+    if (!c->precond || wide) CU(launch_merge_gate(c->d_desc, nops, cap, c->st));
     p_merge.stop();
     if (tape) {
         int nc = 0, max_rows = 1;
@@ -562,11 +566,11 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     CU(launch_truncate(c->d_desc, nops, cap, c->st));
     p_tr.stop();
     ProfScope p_rec(c, K_RECON);
-    if (c->precond)
-        CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_s, false, timeout_ns, c->st));
-    else
-        CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
+    if (c->precond) CU(launch_oz_ops(c->d_desc, nops, OZ_RECON, cap, c->oz_s, false, timeout_ns, c->st));
+    if (!c->precond || wide) CU(launch_reconstruct(c->d_desc, nops, cap, c->st));
     p_rec.stop();
+    // the ops' bonds have a gauge of their own SVD now
+    for (const Item& it : items) c->wide[(size_t)it.b * (N + 1) + c->layers[it.layer][it.idx].p + 1] = 0;
     // new bond dimensions back to the host (the next chunk's shapes depend on them)
     CU(cudaMemcpyAsync(c->h_dims.data(), c->d_dims, sizeof(int) * c->h_dims.size(), cudaMemcpyDeviceToHost,
                        c->st));
@@ -592,7 +596,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
     }
     // kernels per stage: a tensor-core product is two (slicing, slice
     // products), the merge adds the gate/weight kernel
-    prof_collect(c, K_MERGE, fl_merge, c->precond ? kOzKernels + 1 : 1);
+    prof_collect(c, K_MERGE, fl_merge, c->precond ? kOzKernels + 1 + wide : 1);
     prof_collect(c, K_QR, svd.qr_flops, svd.qr_kernels);
     prof_collect(c, K_JACOBI, fl_svd, 1);
     if (svd.staged) {
@@ -600,7 +604,7 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         prof_collect(c, K_GEMM, svd.gemm_flops, svd_products_kernels(c));
     }
     prof_collect(c, K_TRUNC, 0.0, 1);
-    prof_collect(c, K_RECON, fl_rec, c->precond ? kOzKernels : 1);
+    prof_collect(c, K_RECON, fl_rec, c->precond ? kOzKernels + wide : 1);
     for (int s = 0; s < nops && log_ranks; ++s) {
         const Item& it = items[s];
         const Op& op = c->layers[it.layer][it.idx];
@@ -609,6 +613,19 @@ int run_chunk(mpdo_ctx* c, const std::vector<Item>& items, int step, const int* 
         c->rank_log[(size_t)it.b * per_b + (size_t)step * c->n_ops + c->layer_op0[it.layer] + it.idx] = k;
     }
     return MPDO_OK;
+}
+
+int host_step(mpdo_ctx* c, int step) {
+    for (int li = 0; li < (int)c->layers.size(); ++li) {
+        const std::vector<Item> items = layer_items(c, li);
+        const size_t cs = (size_t)chunk_ops(c);
+        for (size_t s0 = 0; s0 < items.size(); s0 += cs) {
+            std::vector<Item> chunk(items.begin() + s0, items.begin() + std::min(items.size(), s0 + cs));
+            int rc = run_chunk(c, chunk, step, nullptr, nullptr, true);
+            if (rc) return rc;
+        }
+    }
+    return normalize_trace(c);
 }
 
 int normalize_trace(mpdo_ctx* c) {
@@ -771,6 +788,7 @@ int mpdo_init(mpdo_ctx** out, const mpdo_config* cfg, void* cuda_stream) {
             return bail(MPDO_ECUDA);
         }
     c->h_dims.assign((size_t)B * (N + 1), 1);
+    clear_gauge(c);
     *out = c;
     return MPDO_OK;
 }
@@ -881,6 +899,7 @@ int mpdo_build_gates(mpdo_ctx* c, const mpdo_model* m, double dt) {
     CU(cudaMemsetAsync(c->d_trace, 0, sizeof(double) * B, c->st));
     CU(cudaStreamSynchronize(c->st));
     c->built = true;
+    clear_gauge(c);
     ++c->gen;
     ++c->layout;
     c->forced.clear();
@@ -913,6 +932,7 @@ int mpdo_init_graph_state(mpdo_ctx* c, const int* pairs, int n_pairs) {
     CU(cudaMemsetAsync(c->d_status, 0, sizeof(int) * B, c->st));
     CU(cudaMemsetAsync(c->d_maxdisc, 0, sizeof(double) * B, c->st));
     CU(cudaStreamSynchronize(c->st));
+    clear_gauge(c);
     ++c->gen;
     if (n_pairs == 0) return MPDO_OK;
     // Pauli-basis superoperators: CZ (rho -> CZ rho CZ, by traces of Pauli products)
@@ -1002,19 +1022,10 @@ int mpdo_trotter_step(mpdo_ctx* c, int n_steps) {
     c->rank_steps = n_steps;
     c->rank_log.assign((size_t)c->B * n_steps * c->n_ops, 0);
     ++c->gen;
-    for (int step = 0; step < n_steps; ++step) {
-        for (int li = 0; li < (int)c->layers.size(); ++li) {
-            const std::vector<Item> items = layer_items(c, li);
-            const size_t cs = (size_t)chunk_ops(c);
-            for (size_t s0 = 0; s0 < items.size(); s0 += cs) {
-                std::vector<Item> chunk(items.begin() + s0, items.begin() + std::min(items.size(), s0 + cs));
-                int rc = run_chunk(c, chunk, step, nullptr, nullptr, true);
-                if (rc) return rc;
-            }
-        }
-        int rc = normalize_trace(c);
-        if (rc) return rc;
-    }
+    int rc = refresh_gauge(c);
+    if (rc) return rc;
+    for (int step = 0; step < n_steps; ++step)
+        if ((rc = host_step(c, step))) return rc;
     return check_status_code(c);
 }
 
@@ -1143,6 +1154,8 @@ int mpdo_set_state(mpdo_ctx* c, int b, const int* dims, const double* tensors) {
     for (int p = 0; p <= N; ++p) c->h_dims[(size_t)b * (N + 1) + p] = dims[p];
     CU(cudaMemcpyAsync(c->d_dims, c->h_dims.data(), sizeof(int) * c->h_dims.size(), cudaMemcpyHostToDevice, c->st));
     CU(cudaStreamSynchronize(c->st));
+    c->loaded[b] = 1;
+    std::fill_n(c->wide.begin() + (size_t)b * (N + 1), N + 1, 0);
     ++c->gen;
     return MPDO_OK;
 }

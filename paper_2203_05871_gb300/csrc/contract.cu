@@ -1,4 +1,6 @@
-// FP64 two-site contractions of one op (App. B update of |rho>> per bond):
+// FP64 two-site contractions of one op (App. B update of |rho>> per bond), as dot
+// products: contexts without the tensor-core products (oz_gemm.cu), and ops next to a
+// bond whose gauge those would not resolve (gauge.cu); ops of the other kind are skipped:
 //   merge + gate + weight:
 //     Theta [l,s1,s2,r] = sum_m A[l,s1,m] B[m,s2,r]
 //     Theta'[l,s1',s2',r] = sum_{s1,s2} G[s1's2', s1s2] Theta[l,s1,s2,r]
@@ -24,7 +26,7 @@ constexpr int KT = 16;   // m per k-step
 __global__ void __launch_bounds__(256) merge_gate_kernel(const OpDesc* descs, int chi_cap) {
     const OpDesc& d = descs[blockIdx.z];
     const int l0 = blockIdx.y * TL, r0 = blockIdx.x * TR;
-    if (l0 >= d.cl || r0 >= d.cr) return;
+    if (!d.dot64 || l0 >= d.cl || r0 >= d.cr) return;
     const int ld = 4 * chi_cap;
     __shared__ double As[TL][4][KT + 1];
     __shared__ double Bs[KT][4][TR];
@@ -80,6 +82,7 @@ constexpr int RK = 16;
 
 __global__ void __launch_bounds__(256) reconstruct_kernel(const OpDesc* descs, int chi_cap) {
     const OpDesc& d = descs[blockIdx.z];
+    if (!d.dot64) return;
     const int k = *d.k_out;
     const int i0 = blockIdx.y * RT, j0 = blockIdx.x * RT;
     if (i0 >= d.m || j0 >= k) return;

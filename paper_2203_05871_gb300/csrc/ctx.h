@@ -116,6 +116,8 @@ struct mpdo_ctx {
     int *d_q = nullptr, *d_pairs = nullptr;
     // host mirrors
     std::vector<int> h_dims;
+    std::vector<unsigned char> loaded;   // [B] the tensors came from outside and have not been looked at (gauge.cu)
+    std::vector<unsigned char> wide;     // [B][N+1] bonds whose gauge slice products would not resolve
     std::vector<int> rank_log;    // [B][steps*n_ops] of the last trotter_step call
     int rank_steps = 0;
     // imposed truncation ranks (mpdo_force_ranks): [B][forced_steps][n_ops]
@@ -190,6 +192,23 @@ int plan_jacobi(mpdo_ctx* c, const OpDesc* h, int nops, bool fp32, int* hbase, i
 // that the large ops of a chunk get their share of CTAs instead of one each.
 std::vector<Item> layer_items(mpdo_ctx* c, int li);
 int chunk_ops(mpdo_ctx* c);
+
+// Bond gauges of loaded states (gauge.cu): the flags brought up to date; whether an
+// instance, an op of it, or any instance has a flagged bond.
+int refresh_gauge(mpdo_ctx* c);
+bool wide_instance(const mpdo_ctx* c, int b);
+inline bool wide_op(const mpdo_ctx* c, int b, int p) {
+    const unsigned char* w = &c->wide[(size_t)b * (c->N + 1) + p];
+    return w[0] || w[1] || w[2];
+}
+bool wide_any(const mpdo_ctx* c);
+inline void clear_gauge(mpdo_ctx* c) {
+    c->loaded.assign(c->B, 0);
+    c->wide.assign((size_t)c->B * (c->N + 1), 0);
+}
+
+// One host-planned Trotter step, its ranks logged as those of `step`.
+int host_step(mpdo_ctx* c, int step);
 
 // Descriptor of item `it` in workspace slot s, with the bond dimensions of
 // c->h_dims (forced rank and tape cleared).

@@ -18,7 +18,8 @@
 // sv(F_X F_Y^T)^2, so a third Jacobi SVD, of C = F_X F_Y^T, gives the Schmidt
 // values s_k and OSEE = -sum_k p_k ln p_k with p_k = s_k^2 / sum s^2.
 // FP64 throughout.  The Gram sweeps are batched products: on FP64 contexts exact
-// slice products on the tensor cores (oz_gemm.cu, seven slices), else FP64 GEMMs
+// slice products on the tensor cores (oz_gemm.cu, seven slices), else, and for states
+// in a bond gauge that those do not resolve (gauge.cu), FP64 GEMMs
 // (gemm.cu: 0.68 ms for X' at chi 256, where 16 CTAs share it, against 0.07 ms).
 // The SVDs end at the strict tolerance sqrt(L) eps, through a step's stages where
 // staged_svd says so, else in the FP64 pass of jacobi.cu alone.  Squaring
@@ -150,9 +151,10 @@ struct GqPlan {
     }
 };
 
-// Left Gram sweep over sites 0..last of the chunk's instances: X (slot 2i) is
+// Left Gram sweep over sites 0..last of the chunk's instances, those with a bond gauge that
+// slice products do not resolve (gauge.cu) or the others: X (slot 2i) is
 // chi x chi with chi = dims[last + 1] at the end.  T (thetap slot 2i) holds X B.
-void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
+void plan_left(mpdo_ctx* c, int b0, int m, int last, bool wide, GqPlan& P) {
     const int N = c->N, cap = c->cap, ld = c->ld;
     const size_t mat = (size_t)ld * ld;
     const int f32 = sites_f32(c);
@@ -160,6 +162,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
         P.begin();
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
+            if (wide_instance(c, b) != wide) continue;
             const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
             double* X = c->d_Z + (size_t)(2 * i) * mat;
             double* T = c->d_thetap + (size_t)(2 * i) * mat;
@@ -170,6 +173,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
         P.begin();
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
+            if (wide_instance(c, b) != wide) continue;
             const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
             double* X = c->d_Z + (size_t)(2 * i) * mat;
             double* T = c->d_thetap + (size_t)(2 * i) * mat;
@@ -181,7 +185,7 @@ void plan_left(mpdo_ctx* c, int b0, int m, int last, GqPlan& P) {
 }
 
 // Right Gram sweep over sites N-1..first: Y (slot 2i + 1), U (thetap slot 2i + 1) holds B Y.
-void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
+void plan_right(mpdo_ctx* c, int b0, int m, int first, bool wide, GqPlan& P) {
     const int N = c->N, cap = c->cap, ld = c->ld;
     const size_t mat = (size_t)ld * ld;
     const int f32 = sites_f32(c);
@@ -189,6 +193,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
         P.begin();
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
+            if (wide_instance(c, b) != wide) continue;
             const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
             double* Y = c->d_Z + (size_t)(2 * i + 1) * mat;
             double* U = c->d_thetap + (size_t)(2 * i + 1) * mat;
@@ -200,6 +205,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
             P.begin();
             for (int i = 0; i < m; ++i) {
                 const int b = b0 + i;
+                if (wide_instance(c, b) != wide) continue;
                 const int l = c->h_dims[(size_t)b * (N + 1) + q], r = c->h_dims[(size_t)b * (N + 1) + q + 1];
                 double* Y = c->d_Z + (size_t)(2 * i + 1) * mat;
                 double* U = c->d_thetap + (size_t)(2 * i + 1) * mat;
@@ -212,7 +218,7 @@ void plan_right(mpdo_ctx* c, int b0, int m, int first, GqPlan& P) {
     }
 }
 
-int run_plan(mpdo_ctx* c, GqPlan& P) {
+int run_plan(mpdo_ctx* c, bool wide, GqPlan& P) {
     if (P.g.empty()) return MPDO_OK;
     if (c->gq_cap < P.g.size()) {
         if (c->d_gq) cudaFree(c->d_gq);
@@ -222,7 +228,7 @@ int run_plan(mpdo_ctx* c, GqPlan& P) {
         c->gq_cap = P.g.size();
     }
     CU(cudaMemcpyAsync(c->d_gq, P.g.data(), sizeof(GemmDesc) * P.g.size(), cudaMemcpyHostToDevice, c->st));
-    const bool tc = c->precond && c->oz_s == 7;
+    const bool tc = c->precond && c->oz_s == 7 && !wide;
     const OzScratch scr{static_cast<unsigned char*>(c->d_oz_as), static_cast<unsigned char*>(c->d_oz_bs), c->d_oz_ea,
                         c->d_oz_eb, c->d_oz, c->oz_slot_bytes, oz_exp_ints(c->ld)};
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
@@ -315,7 +321,7 @@ int global_prepare(mpdo_ctx* c, double* out) {
     if (c->slots < 2) return fail(MPDO_ECAPACITY, "needs at least two workspace slots");
     CU(cudaMemcpyAsync(c->h_dims.data(), c->d_dims, sizeof(int) * c->h_dims.size(), cudaMemcpyDeviceToHost, c->st));
     CU(cudaStreamSynchronize(c->st));
-    return MPDO_OK;
+    return refresh_gauge(c);
 }
 
 int finish(mpdo_ctx* c, double* out, int out_on_device) {
@@ -342,10 +348,12 @@ extern "C" int mpdo_renyi2(mpdo_ctx* c, double* out, int out_on_device) {
         const int m = std::min(per, B - b0);
         gram_unit_kernel<<<(2 * m + 127) / 128, 128, 0, c->st>>>(c->d_Z, mat, m);
         CU(cudaGetLastError());
-        GqPlan P;
-        plan_left(c, b0, m, N - 1, P);
-        rc = run_plan(c, P);
-        if (rc) return rc;
+        for (bool wide : {false, true}) {
+            GqPlan P;
+            plan_left(c, b0, m, N - 1, wide, P);
+            rc = run_plan(c, wide, P);
+            if (rc) return rc;
+        }
         renyi2_kernel<<<(m + 127) / 128, 128, 0, c->st>>>(c->d_Z, mat, c->d_envL, N, c->cap, b0, m, dst);
         CU(cudaGetLastError());
     }
@@ -367,18 +375,20 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
         const int m = std::min(std::min(per, per_chi), B - b0);
         gram_unit_kernel<<<(2 * m + 127) / 128, 128, 0, c->st>>>(c->d_Z, mat, m);
         CU(cudaGetLastError());
-        GqPlan P;
-        plan_left(c, b0, m, bond, P);
-        plan_right(c, b0, m, bond + 1, P);
-        rc = run_plan(c, P);
-        if (rc) return rc;
+        for (bool wide : {false, true}) {
+            GqPlan P;
+            plan_left(c, b0, m, bond, wide, P);
+            plan_right(c, b0, m, bond + 1, wide, P);
+            rc = run_plan(c, wide, P);
+            if (rc) return rc;
+        }
         // the instances of each route: [0] the FP64 Jacobi alone, [1] the stages
         std::vector<int> slots[2], chis[2], inst[2], chi2(2 * m), route(2 * m);
         int maxchi = 1;
         for (int i = 0; i < m; ++i) {
             const int b = b0 + i;
             const int chi = c->h_dims[(size_t)b * (N + 1) + bond + 1];
-            const int st = staged_svd(c, chi) ? 1 : 0;
+            const int st = staged_svd(c, chi) && !wide_instance(c, b) ? 1 : 0;
             maxchi = std::max(maxchi, chi);
             for (int h = 0; h < 2; ++h) {
                 slots[st].push_back(2 * i + h);
@@ -404,17 +414,20 @@ extern "C" int mpdo_osee(mpdo_ctx* c, int bond, double* out, int out_on_device) 
         CU(cudaGetLastError());
         // C_i = (rows of X) (rows of Y)^T into thetap slot 2i, then scaled to F_X F_Y^T
         // (staged: its transpose into slot 2i + 1)
-        GqPlan Pc;
-        Pc.begin();
+        GqPlan Pc[2];   // [1]: flagged instances
+        Pc[0].begin();
+        Pc[1].begin();
         for (int s = 0; s < 2 * m; ++s) {
             if ((s & 1) && !route[s]) continue;
             double* F = route[s] ? c->d_W : c->d_Z;
-            Pc.add(GemmDesc{chi2[s], chi2[s], chi2[s], F + (size_t)s * mat, ld, 0, F + (size_t)(s ^ 1) * mat, ld, 0,
+            Pc[wide_instance(c, b0 + s / 2)].add(GemmDesc{chi2[s], chi2[s], chi2[s], F + (size_t)s * mat, ld, 0, F + (size_t)(s ^ 1) * mat, ld, 0,
                             1, c->d_thetap + (size_t)s * mat, ld, 1.0, 0.0, nullptr, 0, 0, 0, 0, 0},
                    c->d_status + b0 + s / 2);
         }
-        rc = run_plan(c, Pc);
-        if (rc) return rc;
+        for (bool wide : {false, true}) {
+            rc = run_plan(c, wide, Pc[wide]);
+            if (rc) return rc;
+        }
         scale_kernel<<<dim3(64, 2 * m), 256, 0, c->st>>>(c->d_thetap, mat, ld, d_chi, d_staged, c->d_snorm);
         CU(cudaGetLastError());
         if (any) {

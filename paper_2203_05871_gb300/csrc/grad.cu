@@ -61,6 +61,7 @@ struct Arena {
 
 struct StepRecord {
     std::vector<int> dims;   // [B][N+1] at the start of the step
+    std::vector<unsigned char> wide;   // the context's gauge flags then: the recompute takes the same routes
     double* sites = nullptr; // compact site tensors, (b, p) in order
     double* lam = nullptr;   // copy of d_lam
 };
@@ -134,6 +135,7 @@ int ensure_copy_descs(mpdo_ctx* c, GradState* g, int need) {
 int save_state(mpdo_ctx* c, GradState* g, StepRecord& r) {
     const int B = c->B, N = c->N, cap = c->cap;
     r.dims = c->h_dims;
+    r.wide = c->wide;
     size_t total = 0;
     for (int b = 0; b < B; ++b)
         for (int p = 0; p < N; ++p) total += (size_t)4 * r.dims[b * (N + 1) + p] * r.dims[b * (N + 1) + p + 1];
@@ -175,6 +177,7 @@ int restore_state(mpdo_ctx* c, GradState* g, const StepRecord& r) {
     CU(launch_copy2d(g->d_cp, nc, max_rows, c->st));
     CU(cudaMemcpyAsync(c->d_lam, r.lam, sizeof(double) * B * N * cap, cudaMemcpyDeviceToDevice, c->st));
     c->h_dims = r.dims;
+    c->wide = r.wide;
     CU(cudaMemcpyAsync(c->d_dims, c->h_dims.data(), sizeof(int) * c->h_dims.size(), cudaMemcpyHostToDevice,
                        c->st));
     CU(cudaStreamSynchronize(c->st));
@@ -490,8 +493,10 @@ int mpdo_grad_forward(mpdo_ctx* c, int n_steps) {
     CU(dalloc(&g->d_traces, (size_t)n_steps * c->B));
     c->rank_steps = n_steps;
     c->rank_log.assign((size_t)c->B * n_steps * c->n_ops, 0);
+    int rc = refresh_gauge(c);
+    if (rc) return rc;
     for (int step = 0; step < n_steps; ++step) {
-        int rc = save_state(c, g, g->steps[step]);
+        rc = save_state(c, g, g->steps[step]);
         if (rc) return rc;
         for (int li = 0; li < (int)c->layers.size(); ++li) {
             std::vector<Item> items = layer_items(c, li);
@@ -507,7 +512,7 @@ int mpdo_grad_forward(mpdo_ctx* c, int n_steps) {
         CU(cudaMemcpyAsync(g->d_traces + (size_t)step * c->B, c->d_trace, sizeof(double) * c->B,
                            cudaMemcpyDeviceToDevice, c->st));
     }
-    int rc = save_state(c, g, g->steps[n_steps]);
+    rc = save_state(c, g, g->steps[n_steps]);
     if (rc) return rc;
     g->ranks = c->rank_log;
     rc = check_status_code(c);

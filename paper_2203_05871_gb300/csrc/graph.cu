@@ -326,10 +326,21 @@ extern "C" int mpdo_trotter_step_graph(mpdo_ctx* c, int n_steps) {
         int rc = build_graph(c, g);
         if (rc) return rc;
     }
+    // The captured step has the slice products alone: a loaded state whose gauge they would
+    // not resolve takes host-planned steps until its bonds have been through an SVD (one
+    // step, unless a bond has no op).
+    int first = 0;
+    int rc = refresh_gauge(c);
+    if (rc) return rc;
+    ++c->gen;
+    c->rank_steps = n_steps;
+    c->rank_log.assign((size_t)c->B * n_steps * c->n_ops, 0);
+    for (; first < n_steps && wide_any(c); ++first)
+        if ((rc = host_step(c, first))) return rc;
     const size_t per = (size_t)c->B * c->n_ops;
     int* d_all = nullptr;
-    CU(dalloc(&d_all, std::max<size_t>(1, per * n_steps)));
-    for (int step = 0; step < n_steps; ++step) {
+    CU(dalloc(&d_all, std::max<size_t>(1, per * (n_steps - first))));
+    for (int step = 0; step < n_steps - first; ++step) {
         cudaError_t e = cudaGraphLaunch(g->exec, c->st);
         if (e != cudaSuccess) {
             cudaFree(d_all);
@@ -341,7 +352,7 @@ extern "C" int mpdo_trotter_step_graph(mpdo_ctx* c, int n_steps) {
             return fail(MPDO_ECUDA, std::string("rank copy: ") + cudaGetErrorString(e));
         }
     }
-    std::vector<int> all(per * n_steps), err(1);
+    std::vector<int> all(per * (n_steps - first)), err(1);
     cudaError_t e1 = cudaMemcpyAsync(all.data(), d_all, sizeof(int) * all.size(), cudaMemcpyDeviceToHost, c->st);
     cudaError_t e2 = cudaMemcpyAsync(err.data(), g->d_error, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     cudaError_t e3 = cudaMemcpyAsync(c->h_dims.data(), c->d_dims, sizeof(int) * c->h_dims.size(),
@@ -351,12 +362,10 @@ extern "C" int mpdo_trotter_step_graph(mpdo_ctx* c, int n_steps) {
     for (cudaError_t e : {e1, e2, e3, e4})
         if (e != cudaSuccess) return fail(MPDO_ECUDA, std::string("graph step: ") + cudaGetErrorString(e));
     if (err[0]) return fail(MPDO_ECAPACITY, "graph step: more ops in flight than co-resident CTAs");
-    c->rank_steps = n_steps;
-    c->rank_log.assign(per * n_steps, 0);
-    for (int step = 0; step < n_steps; ++step)
+    for (int step = first; step < n_steps; ++step)
         for (int b = 0; b < c->B; ++b)
             for (int op = 0; op < c->n_ops; ++op)
-                c->rank_log[((size_t)b * n_steps + step) * c->n_ops + op] = all[per * step + (size_t)b * c->n_ops + op];
-    ++c->gen;
+                c->rank_log[((size_t)b * n_steps + step) * c->n_ops + op] =
+                    all[per * (step - first) + (size_t)b * c->n_ops + op];
     return check_status_code(c);
 }

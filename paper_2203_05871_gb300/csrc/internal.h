@@ -44,7 +44,8 @@ struct OpDesc {
     int cl, cm, cr;    // bond dims chi_{p-1}, chi_p, chi_{p+1}
     int m, n;          // 4*cl, 4*cr
     int transposed;    // 1 (m > n, preconditioning stages): the SVD is that of theta~^T, and Z carries its rotations
-    int plain;         // 1: too small for the preconditioning stages (FP64 QR, then the FP64 Jacobi pass)
+    int plain;         // 1: without the preconditioning stages (FP64 QR, then the FP64 Jacobi pass)
+    int dot64;         // 1: contractions as FP64 dot products (contract.cu), not slice products
     int c, L;          // Jacobi problem: c rows of length L
     int jb;            // Jacobi block size (rows per shared-memory block), FP64 pass
     int chi_max;
@@ -283,6 +284,10 @@ cudaError_t launch_refine(const OpDesc* d_desc, int nops, int chi_cap, int S, bo
 constexpr int kRefineIters = 4;
 // kernels of one launch_refine
 constexpr int kRefineKernels = kRefineIters * (3 + 4 * kOzKernels);
+
+// loss[b (n + 1) + m]: bits that products along bond m lose to its gauge (gauge.cu)
+cudaError_t launch_gauge(const void* sites, int sites_f32, const int* dims, int n, int B, int chi_cap, int* loss,
+                         cudaStream_t st);
 
 // Theta' = G Theta in place in thetap and theta~ = lambda_l Theta' (column-major, Acm)
 cudaError_t launch_gate_weight(const OpDesc* d_desc, int nops, int chi_cap, cudaStream_t st);

@@ -337,7 +337,7 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap, bool z) {
     const bool first = (kind & OZ_FIRST) != 0;
     kind &= OZ_FIRST - 1;
     if (z && !d.transposed) kind = -1;
-    if (d.plain && kind != OZ_MERGE && kind != OZ_RECON) kind = -1;
+    if (d.dot64 || (d.plain && kind != OZ_MERGE && kind != OZ_RECON)) kind = -1;
     auto rowmajor = [](const void* base, int f32, long long ld_) {   // (r, k) at r * ld + k
         return OzOperand{base, f32, ld_, 1, 0, 1, 1, nullptr, nullptr, 0};
     };
@@ -832,6 +832,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
 // lambda_{p-1}[l] Theta' (transposed: theta~^T) column-major in Acm; one thread per (l, r).
 __global__ void __launch_bounds__(256) gate_weight_kernel(const OpDesc* descs, int chi_cap) {
     const OpDesc& d = descs[blockIdx.y];
+    if (d.dot64) return;
     __shared__ double Gs[256];
     Gs[threadIdx.x] = d.G[threadIdx.x];
     __syncthreads();
