@@ -311,12 +311,16 @@ void fill_desc(mpdo_ctx* c, const Item& it, int s, bool plain, OpDesc& d) {
 
 cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, bool with_z, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
-    // E = U U^T - I (~1e-6), then one orthogonalisation step: second order
-    // (Q = U - E U / 2, defect 3 E^2 / 4) on the mixed path, fourth order (defect
-    // 35 E^4 / 64, below FP64 rounding; the third order's 5 E^3 / 8 showed as 2e-13 in
-    // the entropies at chi 256) on the FP64 path
-    std::vector<int> kinds = {OZ_E, OZ_Q, OZ_W};
-    if (!c->mixed) kinds = {OZ_E, OZ_T4, OZ_T3, OZ_T2, OZ_W};
+    // E = U U^T - I (~1e-6 per entry, 1e-5 in norm), then one orthogonalisation step.  FP64
+    // path: fourth order (defect 35 E^4 / 64, below FP64 rounding; the third order's
+    // 5 E^3 / 8 showed as 2e-13 in the entropies at chi 256).  Mixed path: third order
+    // after the Jacobi pass, whose rotations become the right vectors of transposed
+    // bonds (the second order's 3 E^2 / 4 left those 5e-9 from orthonormal and observables
+    // of the chi 173 step 1.5e-10 off, now 1e-11 and 5e-12; chi 256 step 103.9 -> 106.4 ms
+    // together with the refinement's aim below), second order (Q = U - E U / 2) after the
+    // QR, whose E is smaller: a higher one there changed no error
+    std::vector<int> kinds = {OZ_E, OZ_T4, OZ_T3, OZ_T2, OZ_W};
+    if (c->mixed) kinds = first ? std::vector<int>{OZ_E, OZ_Q, OZ_W} : std::vector<int>{OZ_E, OZ_U3, OZ_T2, OZ_W};
     for (int kind : kinds) {
         const cudaError_t e =
             launch_oz_ops(d_desc, nops, first + kind, c->cap, c->oz_s, with_z && !first && kind == OZ_W, timeout_ns, st);
@@ -325,7 +329,7 @@ cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, in
     return cudaSuccess;
 }
 
-int orthogonalise_kernels(const mpdo_ctx* c) { return (c->mixed ? 3 : 5) * kOzKernels; }
+int orthogonalise_kernels(const mpdo_ctx* c, int first) { return (c->mixed ? (first ? 3 : 4) : 5) * kOzKernels; }
 
 cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, bool with_z, cudaStream_t st) {
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
@@ -334,11 +338,17 @@ cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, dou
     if (!refine_on(c)) return cudaSuccess;
     // 6 slices resolve a Gram matrix to ~1e-14: a stricter tolerance is left to the Jacobi pass
     const bool can = c->oz_s == 7 || tol >= 1e-12;
-    return launch_refine(d_desc, nops, c->cap, c->oz_s, with_z, can ? tol : 1e-12, can, timeout_ns, st);
+    // The Jacobi pass ends far inside its tolerance (its last sweep starts from the square of
+    // the one before), the refinement wherever its prediction allows, so it aims at a tenth
+    // of the tolerance (tf32 batch of six chains: observables 2.6e-10 and 7e-11 off the
+    // exact ones on two inputs, 5e-11 and 2e-10 with the Jacobi pass, 1e-11 and 3e-11 now)
+    const double least = c->oz_s == 7 ? 1e-14 : 1e-12;
+    const double aim = !can ? 1e-12 : tol > 0.0 ? std::min(tol, std::max(0.1 * tol, least)) : tol;
+    return launch_refine(d_desc, nops, c->cap, c->oz_s, with_z, aim, can, timeout_ns, st);
 }
 
 int svd_products_kernels(const mpdo_ctx* c) {
-    return orthogonalise_kernels(c) + (refine_on(c) ? kRefineKernels : 0);
+    return orthogonalise_kernels(c, 0) + (refine_on(c) ? kRefineKernels : 0);
 }
 
 // The SVDs of the nops ops whose descriptors are in h_desc and d_desc: theta~ (Acm)
@@ -448,7 +458,7 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
             if (total > 0) {
                 CU(launch_qr32(c->d_desc, db, db + total, db + 2 * total, c->d_sync, total, timeout_ns, ld, c->st));
                 CU(launch_orthogonalise(c, c->d_desc, nops, OZ_FIRST, false, c->st));
-                out.qr_kernels += 1 + orthogonalise_kernels(c);
+                out.qr_kernels += 1 + orthogonalise_kernels(c, OZ_FIRST);
             }
             p_qr.stop();
         }

@@ -243,7 +243,7 @@ inline bool refine_on(const mpdo_ctx* c) { return c->precond && c->cfg.jacobi_ma
 // From the FP32-orthogonal U32: Q, orthogonal to FP64 accuracy, and W = Q W0; with
 // first = OZ_FIRST from the QR's Q^T: W0 = Q theta~.
 cudaError_t launch_orthogonalise(mpdo_ctx* c, const OpDesc* d_desc, int nops, int first, bool with_z, cudaStream_t st);
-int orthogonalise_kernels(const mpdo_ctx* c);
+int orthogonalise_kernels(const mpdo_ctx* c, int first);
 // The stages between the FP32 preconditioning pass and the FP64 Jacobi pass:
 // Q, the orthogonalised U32, W = Q W0, and the refinement of W's rows.
 cudaError_t launch_svd_products(mpdo_ctx* c, const OpDesc* d_desc, int nops, double tol, bool with_z, cudaStream_t st);

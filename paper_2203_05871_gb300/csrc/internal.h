@@ -249,13 +249,14 @@ cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int m
 // share them): kind OZ_MERGE Theta = A B (then launch_gate_weight applies the
 // gate and the left weights), OZ_RECON B_p' = Theta' Yk^T, OZ_E E = U U^T - I,
 // OZ_Q Q = U - E U / 2, OZ_W W = Q W0; OZ_T4 T = U - 5 E U / 6, OZ_T3 T = U - 3 E T / 4
-// and OZ_T2 Q = U - E T / 2 (fourth-order orthogonalisation); OZ_G G = W W^T and
+// and OZ_T2 Q = U - E T / 2 (fourth-order orthogonalisation; third order: OZ_U3
+// T = U - 3 E U / 4 in place of OZ_T4 and OZ_T3); OZ_G G = W W^T and
 // OZ_R3, OZ_R2, OZ_R1 the refinement's rotation (refine.cu).
 // OZ_FIRST + OZ_E, OZ_Q, OZ_T4, OZ_T3, OZ_T2, OZ_W: the same on the QR's Q^T, OZ_W then
 // being W0 = Q theta~ (transposed ops: theta~^T, and Q is Z's first value).
 // with_z: the products that turn W (OZ_W, OZ_R*) also turn Z of the transposed ops.
 enum { OZ_FIRST = 16, OZ_MERGE = 0, OZ_RECON = 1, OZ_E = 2, OZ_Q = 3, OZ_W = 4, OZ_T4 = 5, OZ_T3 = 6, OZ_G = 7, OZ_R3 = 8, OZ_R2 = 9,
-       OZ_R1 = 10, OZ_T2 = 11 };
+       OZ_R1 = 10, OZ_T2 = 11, OZ_U3 = 12 };
 cudaError_t launch_oz_ops(const OpDesc* d_desc, int nops, int kind, int chi_cap, int S, bool with_z,
                           unsigned long long timeout_ns, cudaStream_t st);
 constexpr int kOzKernels = 2;   // kernels of one launch_oz_ops

@@ -377,13 +377,14 @@ __device__ OzProblem op_problem(const OpDesc& d, int kind, int cap, bool z) {
         case OZ_Q:       // Q = U - E U / 2
         case OZ_T4:      // T = U - 5 E U / 6 (in W, free until OZ_W)
         case OZ_T3:      // T = U - 3 E T / 4
+        case OZ_U3:      // T = U - 3 E U / 4
         case OZ_T2:      // Q = U - E T / 2
             P.M = P.N = P.K = d.c;
             P.A = rowmajor(d.E, 0, ld);
             P.B = kind == OZ_T3 || kind == OZ_T2 ? colmajor(d.W, 0, ld) : colmajor(d.U32, 1, ld);
-            P.C = kind == OZ_T4 || kind == OZ_T3 ? d.W : first && d.transposed ? d.Z : d.Q;
+            P.C = kind == OZ_T4 || kind == OZ_T3 || kind == OZ_U3 ? d.W : first && d.transposed ? d.Z : d.Q;
             P.ldc = ld;
-            P.alpha = kind == OZ_T4 ? -5.0 / 6.0 : kind == OZ_T3 ? -0.75 : -0.5;
+            P.alpha = kind == OZ_T4 ? -5.0 / 6.0 : kind == OZ_T3 || kind == OZ_U3 ? -0.75 : -0.5;
             P.beta = 1.0;
             P.unit_d = 1;
             P.D = d.U32;

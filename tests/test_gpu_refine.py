@@ -79,3 +79,32 @@ def test_rank_deficient_and_degenerate(precision):
     for pairs in ([(0, 1), (1, 2), (2, 3), (3, 4), (4, 5)], []):
         a, b = both(wl, 16, lambda s: s.init_graph_state(pairs), 2, precision=prec)
         assert np.abs(a - b).max() <= tol
+
+
+@pytest.mark.parametrize("chi", [96, 160])
+@pytest.mark.parametrize("order", ["wide", "tall"])
+def test_mixed_right_vectors_are_orthonormal(chi, order):
+    """The right sites of a mixed step's last layer are the right singular vectors of their
+    bonds.  The refinement leaves pairs of rows at a tenth of the mixed tolerance, 1e-11,
+    at most, the rotations that become the vectors of a transposed bond are orthogonal to
+    the third order of the FP32 pass's defect (1e-5: 1e-15), and the products add 2^-46 per
+    term and sqrt(c) of them (4e-13): 2e-11 covers both."""
+    from paper_2203_05871_gb300 import MIXED_TF32, Solver
+    n = 9
+    wl = W.random_model(n, W.chain_bonds(n), 91, chi_max=chi, cutoff=1e-14, dt=0.02)
+    dims, tens = W.random_mpo_state(n, chi, seed=92, decay=0.04)
+    if order == "tall":   # mirrored: the bonds that were wide are tall
+        tens = [t.transpose(2, 1, 0) for t in tens[::-1]]
+        tens = [np.ascontiguousarray(t) for t in tens]
+        dims = [1] + [t.shape[2] for t in tens]
+    s = Solver(n, batch=1, chi_cap=chi, precision=MIXED_TF32)
+    s.build_gates(wl)
+    s.set_state(0, dims, tens)
+    s.step(1)
+    _, out = s.get_state(0)
+    worst = 0.0
+    for p in (1, 3, 5, 7):
+        v = out[p].reshape(out[p].shape[0], -1)
+        worst = max(worst, np.abs(v @ v.T - np.eye(len(v))).max())
+    assert worst <= 2e-11, worst
+    s.close()
