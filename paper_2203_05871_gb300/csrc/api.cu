@@ -113,12 +113,17 @@ int alloc_slots(mpdo_ctx* c, int want) {
     }
     size_t free_b = 0, total_b = 0;
     CU(cudaMemGetInfo(&free_b, &total_b));
-    if (!c->mixed && 2 * per_slot_bytes > free_b) {   // an FP64 context can do without the stages' buffers
+    const size_t budget = free_b / 2;
+    auto slots_of = [&](size_t bytes) { return std::max(1, std::min(want, (int)std::min<size_t>(budget / bytes, 1 << 20))); };
+    // An FP64 context does without the stages' buffers where they would not fit, or would
+    // leave it one slot and no entropies, which need two.
+    if (!c->mixed && (per_slot_bytes > budget || slots_of(per_slot_bytes) < std::min(2, slots_of(plain_bytes)))) {
         c->precond = false;
         per_slot_bytes = plain_bytes;
     }
-    const size_t budget = free_b / 2;
-    int s = std::max(1, std::min(want, (int)std::min<size_t>(budget / per_slot_bytes, 1 << 20)));
+    int s = slots_of(per_slot_bytes);
+    // for the second slot a mixed one goes up to three quarters of the free memory
+    if (s < 2 && want >= 2 && 2 * per_slot_bytes <= free_b / 4 * 3) s = 2;
     if (c->cfg.max_slots > 0) s = std::min(s, c->cfg.max_slots);
     s = std::min(s, c->jacobi_resident);   // every op of a chunk needs at least one co-resident Jacobi CTA
     if ((size_t)s * per_slot_bytes > free_b) return fail(MPDO_ENOMEM, "not enough device memory for one op slot");
@@ -132,7 +137,7 @@ int alloc_slots(mpdo_ctx* c, int want) {
     CU(dalloc(&c->d_pre_ok, (size_t)s));
     c->h_sweeps.assign(s, 0);
     CU(dalloc(&c->d_desc, (size_t)s));
-    const int gcap = std::max(std::max(c->jacobi_resident, c->qr_resident), s);
+    const int gcap = std::max({c->jacobi_resident, c->qr_resident, c->qr32_resident, s});
     CU(dalloc(&c->d_cta, (size_t)4 * (2 * gcap + s)));
     CU(dalloc(&c->d_sync, jacobi_sync_words(s)));
     CU(cudaMallocHost((void**)&c->h_desc, sizeof(OpDesc) * s));
@@ -361,7 +366,7 @@ int run_svd(mpdo_ctx* c, int nops, double tol, SvdWork& out) {
         const OpDesc& d = c->h_desc[s];
         qwork[s] = (double)d.m * d.n * d.c;
     }
-    const int gcap = std::max(std::max(c->jacobi_resident, c->qr_resident), c->slots);
+    const int gcap = std::max({c->jacobi_resident, c->qr_resident, c->qr32_resident, c->slots});
     // Jacobi launch plan: share the co-resident CTAs among the ops in
     // proportion to their work; h_cta/d_cta hold [op of each CTA | rank | CTAs per op]
     auto plan = [&](bool fp32, int* hbase, int& total) -> int {
