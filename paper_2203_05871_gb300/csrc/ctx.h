@@ -83,6 +83,7 @@ struct mpdo_ctx {
     mpdo::GateSpec* d_specs = nullptr;   // [B][n_ops]
     // per-slot workspaces
     int slots = 0;
+    unsigned char* d_slots = nullptr;   // the allocation that the slots' device buffers are parts of
     double *d_thetap = nullptr, *d_W = nullptr, *d_Z = nullptr, *d_Yk = nullptr, *d_snorm = nullptr;
     int* d_sweeps = nullptr;      // [slots] Jacobi sweeps of the last chunk
     int* d_pre_ok = nullptr;      // [slots] mixed path: the FP32 pass ended by its off-orthogonality rule
@@ -96,8 +97,6 @@ struct mpdo_ctx {
     size_t oz_slot_bytes = 0;
     double *d_W0 = nullptr, *d_E = nullptr, *d_Q = nullptr, *d_Zrot = nullptr;
     float *d_W32 = nullptr, *d_U32 = nullptr, *d_D32 = nullptr;
-    mpdo::GemmDesc* d_gemm = nullptr;
-    mpdo::GemmDesc* h_gemm = nullptr;   // pinned, [3][slots]
     mpdo::Copy2D* d_copy = nullptr;     // [4][slots] tape copies of a chunk
     mpdo::Copy2D* h_copy = nullptr;     // pinned
     std::vector<int> h_sweeps;
