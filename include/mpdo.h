@@ -321,7 +321,8 @@ int mpdo_measure_1q_noalloc(const double *sites, const int *dims, int n_qubits, 
  *   C  device, M x N (ldc >= N), overwritten.
  * Allocates its slice scratch (cudaMalloc) per call and synchronises the
  * stream.  A non-finite entry makes its row of C (A) or column (B) NaN.
- * EINVAL (sizes, kind), ENOMEM, ECUDA. */
+ * Keeps up to 256 MB of scratch per device between calls, which mpdo_destroy gives
+ * back.  EINVAL (sizes, kind), ENOMEM, ECUDA. */
 int mpdo_gemm_tc(int M, int N, int K, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
                  int kind, void *cuda_stream);
 
@@ -367,7 +368,8 @@ int mpdo_grad(mpdo_ctx *ctx, int n_steps, const double *zbar, const double *wbar
 /* Message of the last error on this thread ("" if none). */
 const char *mpdo_last_error(void);
 
-/* Free every device buffer of the context (NULL is a no-op). */
+/* Free every device buffer of the context (NULL: none), and give back the scratch
+ * that mpdo_gemm_tc keeps on its device (NULL: on the current device). */
 void mpdo_destroy(mpdo_ctx *ctx);
 
 #ifdef __cplusplus

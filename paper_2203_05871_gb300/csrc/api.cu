@@ -105,6 +105,7 @@ int alloc_slots(mpdo_ctx* c, int want) {
                           4 * oz_exp_ints(c->ld) * sizeof(int);
     }
     size_t free_b = 0, total_b = 0;
+    gemm_pool_trim();
     CU(cudaMemGetInfo(&free_b, &total_b));
     const size_t budget = free_b / 2;
     auto slots_of = [&](size_t bytes) { return std::max(1, std::min(want, (int)std::min<size_t>(budget / bytes, 1 << 20))); };
@@ -1341,8 +1342,12 @@ int mpdo_profile_sweeps_critical(mpdo_ctx* c, long long* crit, long long* crit_f
 }
 
 void mpdo_destroy(mpdo_ctx* c) {
-    if (!c) return;
+    if (!c) {
+        gemm_pool_trim();
+        return;
+    }
     cudaSetDevice(c->dev);
+    gemm_pool_trim();
     if (c->st) cudaStreamSynchronize(c->st);
     else cudaDeviceSynchronize();
     free_all(c);

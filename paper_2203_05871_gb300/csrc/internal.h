@@ -244,6 +244,9 @@ cudaError_t oz_prepare();
 cudaError_t launch_oz_gemm(const OzProblem* d_probs, int count, int max_m, int max_n, int max_rows_sliced,
                            int S, unsigned long long timeout_ns, cudaStream_t st);
 
+// Gives back the scratch that mpdo_gemm_tc keeps on the current device.
+void gemm_pool_trim();
+
 // The mixed path's tensor-core products of a chunk of ops, built on the
 // device from the op descriptors (so the host-planned and the graph step
 // share them): kind OZ_MERGE Theta = A B (then launch_gate_weight applies the

@@ -1000,6 +1000,8 @@ cudaError_t launch_gemm_tc(const GemmDesc* d_desc, int count, int max_m, int max
 // ---------------------------------------------------------------------------
 // mpdo_gemm_tc: the same product on caller matrices (include/mpdo.h)
 // ---------------------------------------------------------------------------
+#include <cuda.h>
+
 #include <mutex>
 #include <string>
 
@@ -1007,22 +1009,56 @@ namespace mpdo {
 namespace {
 
 // The scratch of mpdo_gemm_tc comes from a pool of its own per device, which keeps
-// up to 256 MB between calls (the slices of a 4096 x 4096 x 2048 product) and
-// returns the rest when a call's stream is synchronised; CUDA also takes
-// it back when another allocation runs out.  Allocation is in stream order, so calls
-// on several streams and threads do not share a buffer.
+// up to 256 MB between calls (the slices of a 4096 x 4096 x 2048 product) and returns
+// the rest when a call's stream is synchronised; gemm_pool_trim returns all of it.  Allocation is in stream
+// order, so calls on several streams and threads do not share a buffer.  A pool ends with
+// its device context: the context's id says whether the one at hand is still that
+// (after cudaDeviceReset it is not).
 constexpr unsigned long long kGemmPoolKeep = 256ull << 20;
 constexpr int kMaxPools = 64;
 
-cudaError_t gemm_pool(cudaMemPool_t* out) {
-    static std::mutex mu;
-    static cudaMemPool_t pools[kMaxPools] = {};
+struct GemmPool {
+    cudaMemPool_t pool = nullptr;
+    unsigned long long context = 0;
+};
+std::mutex g_pool_mu;
+GemmPool g_pools[kMaxPools];
+
+// id of the calling thread's current context, which is unique in the process
+cudaError_t context_id(unsigned long long* id) {
+    using GetCurrent = CUresult (*)(CUcontext*);
+    using GetId = CUresult (*)(CUcontext, unsigned long long*);
+    static GetCurrent current = nullptr;
+    static GetId get = nullptr;
+    static const cudaError_t found = [] {
+        cudaDriverEntryPointQueryResult r;
+        void *a = nullptr, *b = nullptr;
+        cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &r);
+        if (e == cudaSuccess) e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &r);
+        current = reinterpret_cast<GetCurrent>(a);
+        get = reinterpret_cast<GetId>(b);
+        return e != cudaSuccess ? e : a && b ? cudaSuccess : cudaErrorNotSupported;
+    }();
+    if (found != cudaSuccess) return found;
+    CUcontext c = nullptr;
+    if (current(&c) != CUDA_SUCCESS || !c || get(c, id) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
+    return cudaSuccess;
+}
+
+// the current device's pool of the context at hand (with make, a new one if there is none)
+cudaError_t gemm_pool(cudaMemPool_t* out, bool make) {
+    *out = nullptr;
     int dev = 0;
+    unsigned long long id = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && make) e = cudaSetDevice(dev);   // the context exists and is current
+    if (e == cudaSuccess) e = context_id(&id);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxPools) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!pools[dev]) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    GemmPool& g = g_pools[dev];
+    if (g.pool && g.context != id) g.pool = nullptr;   // gone with its context
+    if (!g.pool && make) {
         if ((e = oz_prepare()) != cudaSuccess) return e;
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
@@ -1036,13 +1072,21 @@ cudaError_t gemm_pool(cudaMemPool_t* out) {
             cudaMemPoolDestroy(p);
             return e;
         }
-        pools[dev] = p;
+        g.pool = p;
+        g.context = id;
     }
-    *out = pools[dev];
+    *out = g.pool;
     return cudaSuccess;
 }
 
 }  // namespace
+
+void gemm_pool_trim() {
+    cudaMemPool_t p = nullptr;
+    if (gemm_pool(&p, false) == cudaSuccess && p) cudaMemPoolTrimTo(p, 0);
+    cudaGetLastError();
+}
+
 }  // namespace mpdo
 
 extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,
@@ -1072,7 +1116,7 @@ extern "C" int mpdo_gemm_tc(int M, int N, int K, const double* A, int lda, const
     const size_t bytes = sa + sb + sizeof(int) * (ia + ib);
     unsigned char* buf = nullptr;
     cudaMemPool_t pool = nullptr;
-    cudaError_t e = gemm_pool(&pool);
+    cudaError_t e = gemm_pool(&pool, true);
     if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&buf, bytes, pool, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
