@@ -155,6 +155,7 @@ struct Chunk {
     int *d_cta64 = nullptr, *d_cta32 = nullptr, *d_ctaqr = nullptr, *d_ctaq32 = nullptr;
     int* d_lp = nullptr;   // path positions of the layer's ops
     int n_lp = 0;
+    bool stages = true;    // whether any of its bonds can grow over kPlainRows rows
 };
 
 }  // namespace
@@ -195,10 +196,11 @@ void release(GraphState* g) {
 int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
     const int cap = c->cap, ld = c->ld;
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
-    const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap), q32 = use_qr32(c);
+    const bool blocked = c->mixed && c->cfg.qr_blocked && qrb_fits(cap);
     for (auto& L : g->chunks)
         for (auto& ch : L) {
             const int nops = ch.nops;
+            const bool q32 = use_qr32(c), staged = c->precond && ch.stages;
             plan_chunk_kernel<<<1, 256, 0, st>>>(ch.d_desc, nops, c->d_dims, c->N, g->Rj, g->Rq, ch.d_cta64,
                                                  ch.d_cta32, ch.d_ctaqr, ch.d_ctaq32, g->Rq32,
                                                  c->precond ? 1 : 0, q32 ? 1 : 0, c->mixed ? 1 : 0, blocked ? 1 : 0,
@@ -219,14 +221,14 @@ int enqueue_step(mpdo_ctx* c, GraphState* g, cudaStream_t st) {
                 if (!q32 || !c->mixed)   // mixed contexts have no plain ops
                     CU(launch_qr(ch.d_desc, ch.d_ctaqr, ch.d_ctaqr + g->Rq, ch.d_ctaqr + 2 * g->Rq, c->d_sync, g->Rq,
                                  timeout_ns, ld, st));
-                if (q32) {
+                if (q32 && staged) {
                     CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
                     CU(launch_qr32(ch.d_desc, ch.d_ctaq32, ch.d_ctaq32 + g->Rq32, ch.d_ctaq32 + 2 * g->Rq32, c->d_sync,
                                    g->Rq32, timeout_ns, ld, st));
                     CU(launch_orthogonalise(c, ch.d_desc, nops, OZ_FIRST, false, st));
                 }
             }
-            if (c->precond) {
+            if (staged) {
                 CU(cudaMemsetAsync(c->d_sync, 0, sync_bytes, st));
                 CU(launch_jacobi(ch.d_desc, nops, ch.d_cta32, ch.d_cta32 + g->Rj, ch.d_cta32 + 2 * g->Rj, c->d_sync,
                                  g->Rj, kMaxSweepsCap / 2, 0.0, timeout_ns, ld, true, st, precond_rho(c)));
@@ -272,6 +274,13 @@ int build_graph(mpdo_ctx* c, GraphState* g) {
             std::vector<int> lp;
             for (const Op& o : c->layers[li]) lp.push_back(o.p);
             ch.n_lp = (int)lp.size();
+            // Instances of chi_max <= kPlainRows / 4 leave the stages out whatever their bonds
+            // are: a chunk of them is captured without (chi 4, one chain of 10: 5.1 -> 4.6 ms
+            // for two steps, sixteen: 6.3 -> 5.3 ms).
+            ch.stages = c->mixed;
+            for (int s = 0; s < nops; ++s)
+                for (int p : lp)
+                    ch.stages = ch.stages || (p > 0 && p + 2 < c->N && 4 * c->chi_max[items[s0 + s].b] > kPlainRows);
             CU(dalloc(&ch.d_lp, lp.size()));
             CU(cudaMemcpyAsync(ch.d_lp, lp.data(), sizeof(int) * lp.size(), cudaMemcpyHostToDevice, c->st));
             CU(dalloc(&ch.d_desc, (size_t)nops));
@@ -328,14 +337,22 @@ extern "C" int mpdo_trotter_step_graph(mpdo_ctx* c, int n_steps) {
     }
     // The captured step has the slice products alone: a loaded state whose gauge they would
     // not resolve takes host-planned steps until its bonds have been through an SVD (one
-    // step, unless a bond has no op).
+    // step, unless a bond has no op).  So do steps all of whose bonds leave the SVD's stages
+    // out, while those are captured: the host-planned step does not launch them (see
+    // build_graph for what that takes).
     int first = 0;
+    auto small = [&] {
+        bool any = false;
+        for (const auto& L : g->chunks)
+            for (const Chunk& ch : L) any = any || ch.stages;
+        return any && !c->mixed && use_qr32(c) && 4 * *std::max_element(c->h_dims.begin(), c->h_dims.end()) <= kPlainRows;
+    };
     int rc = refresh_gauge(c);
     if (rc) return rc;
     ++c->gen;
     c->rank_steps = n_steps;
     c->rank_log.assign((size_t)c->B * n_steps * c->n_ops, 0);
-    for (; first < n_steps && wide_any(c); ++first)
+    for (; first < n_steps && (wide_any(c) || small()); ++first)
         if ((rc = host_step(c, first))) return rc;
     const size_t per = (size_t)c->B * c->n_ops;
     int* d_all = nullptr;
