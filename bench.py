@@ -43,7 +43,6 @@ import time
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-FP64_PEAK_NOMINAL_TFLOPS = 1.25   # GB300 FP64 (recipe table, nominal)
 
 
 def parse():
@@ -458,15 +457,13 @@ def contraction_roofline(prof):
                     + ("" if bf16 else ", of fallback")}
 
 
-def qr_roofline(prof):
-    """The QR stage (FP32 Householder QR, its orthogonalisation and W0 = Q^T theta~ on
-    the tensor cores) against the nominal FP64 peak of a QR in FP64."""
+def qr_rate(prof):
+    """The QR stage (FP32 Householder QR, its orthogonalisation and W0 = Q^T theta~ on the
+    tensor cores) in the flops of a Householder QR."""
     q = prof["qr"]
-    achieved = q["flops"] / (q["ms"] / 1e3) / 1e12 if q["ms"] > 0 else None
-    return {"kernel": "qr32_kernel and its products", "bound": "alu", "achieved": achieved,
-            "peak": FP64_PEAK_NOMINAL_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_NOMINAL_TFLOPS if achieved else None, "traffic": None,
-            "note": "flops 4 m n r - 2 (m + n) r^2 + 4/3 r^3 per op (r = min(m, n)); peak = nominal FP64"}
+    return {"stage": "qr32_kernel and its products", "ms": q["ms"],
+            "algorithmic_tflops": q["flops"] / (q["ms"] / 1e3) / 1e12 if q["ms"] > 0 else None,
+            "note": "flops 4 m n r - 2 (m + n) r^2 + 4/3 r^3 per op (r = min(m, n))"}
 
 
 def run_observables(args, local, reps=5):
@@ -604,24 +601,68 @@ def arm_summary(r, world):
     return out
 
 
-def truncation_roofline(prof, precision):
-    """The truncation stage (QR + SVD, about 95% of the step) against the FP64
-    peak, with the fixed algorithmic convention of 21 n^3 flops per n x n SVD."""
+def op_shapes(wl, chi):
+    """(rows c, row length L) of every SVD of one step: c = 4 min, L = 4 max of the bonds
+    left and right of the op (chi: [B][N - 1] bond dimensions)."""
+    import ctypes
+    from paper_2203_05871_gb300.mpdo import load_library
+    bi = (ctypes.c_int * len(wl.bonds))(*[b[0] for b in wl.bonds])
+    bj = (ctypes.c_int * len(wl.bonds))(*[b[1] for b in wl.bonds])
+    n = ctypes.c_int(0)
+    lib = load_library()
+    lib.mpdo_schedule(wl.n, len(wl.bonds), bi, bj, None, ctypes.c_longlong(0), ctypes.byref(n))
+    ops = (ctypes.c_int * (7 * n.value))()
+    lib.mpdo_schedule(wl.n, len(wl.bonds), bi, bj, ops, ctypes.c_longlong(7 * n.value), ctypes.byref(n))
+    out = []
+    for row in chi:
+        d = [1] + [int(x) for x in row] + [1]
+        for k in range(n.value):
+            p = ops[7 * k + 2]
+            out.append((4 * min(d[p], d[p + 2]), 4 * max(d[p], d[p + 2])))
+    return out
+
+
+def jacobi32_roofline(arm):
+    """The FP32 Jacobi pass, the largest kernel of a step, in the tf32 work that its block
+    pairs execute, against the tensor cores' tf32 rate.  Per sweep every two of the c / 32
+    row blocks meet once: their cross Gram block (32 x 32 x L multiply-adds) and the
+    product of the 64 x 64 rotation with the pair's rows of W32 and U32 (64 x 64 x (L + c)),
+    three tf32 products each (operands split in two); every block's own Gram matrix is
+    formed once a sweep."""
+    prof = arm["prof"]
+    jac, ms = prof["jacobi_svd"], prof["jacobi_fp32"]["ms"]
+    if not prof["jacobi_fp32"]["launches"] or not jac["svds"]:
+        return None
+    work = 0.0
+    for c, L in op_shapes(arm["wl"], arm["status"]["chi"]):
+        nb = -(-c // 32)
+        work += 3 * 2.0 * (nb * (nb - 1) / 2 * (32 * 32 * L + 64 * 64 * (L + c)) + nb * 32 * 32 * L)
+    work *= arm["steps"] * jac["sweeps_fp32"] / jac["svds"]
+    achieved = work / (ms / 1e3) / 1e12 if ms > 0 else None
+    bf16 = measured_peaks().get("bf16_tflops")
+    peak = (bf16 if bf16 else 1900.0) * 1.1 / 2.25
+    return {"kernel": "jacobi32_kernel", "bound": "latency", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak if achieved else None, "traffic": None,
+            "note": "achieved = tf32 work of the mean FP32 sweeps over the step's bonds (every block pair counted as "
+                    "turned) / CUDA-event time of the pass; peak = measured bf16 burst"
+                    + ("" if bf16 else ", of fallback") + " x 1.1/2.25 (nominal tf32/bf16); the pass is a chain of "
+                    "rotation steps, and mma.sync, which it uses, reaches about a third of that rate; traffic: null, "
+                    "the rows stay in L2"}
+
+
+def truncation_rate(prof):
+    """The truncation stage (QR + SVD, about 95% of the step) in the fixed algorithmic
+    convention of 21 n^3 flops per n x n SVD: a rate to compare runs by, not a fraction of a
+    peak (the kernels do little of that work in FP64)."""
     jac = prof["jacobi_svd"]
     parts = ["qr", "jacobi_svd"] + [k for k in ("jacobi_fp32", "precond_gemm") if prof[k]["launches"]]
     ms = sum(prof[k]["ms"] for k in parts)
     achieved = jac["flops"] / (ms / 1e3) / 1e12 if ms > 0 else None
     names = {"qr": "qr32_kernel and its products", "jacobi_svd": "jacobi_kernel", "jacobi_fp32": "jacobi32_kernel",
              "precond_gemm": "oz_slice/oz_gemm/refine kernels (orthogonalisation and refinement)"}
-    return {"kernel": "truncation stage: " + " + ".join(names[k] for k in parts),
-            "bound": "alu", "achieved": achieved, "peak": FP64_PEAK_NOMINAL_TFLOPS, "unit": "TFLOP/s",
-            "frac": (achieved / FP64_PEAK_NOMINAL_TFLOPS) if achieved else None,
-            "traffic": None,
-            "note": "achieved = 21 n^3 flops per n x n SVD (n = 4 max(chi_l, chi_r)), the FP64 work of an ideal "
-                    "Golub-Kahan SVD, over the summed CUDA-event time of the listed kernels (QR included); peak = "
-                    "nominal FP64 of GB300 (2 DFMA/SM/clk x 152 SMs x 2.07 GHz; MEASURED_PEAKS.json has no "
-                    "FP64 figure), of nominal (the kernels do little of it in FP64, so the fraction can pass 1); "
-                    "traffic: null, the stage is several kernels whose rows stay in L2"}
+    return {"stage": " + ".join(names[k] for k in parts), "ms": ms, "algorithmic_tflops": achieved,
+            "note": "21 n^3 flops per n x n SVD (n = 4 max(chi_l, chi_r)), the work of an ideal Golub-Kahan SVD, "
+                    "over the summed CUDA-event time of the listed kernels"}
 
 
 def main():
@@ -655,9 +696,8 @@ def main():
     e2e_value = world * n_ops * args.e2e_steps / (head["e2e_ms"] / 1e3) if args.e2e_steps > 0 else None
     prof = head["prof"]
     launches = sum(v["launches"] for v in prof.values())      # kernels, as counted by the library
-    dtype = (("mixed: tcgen05 %s slice products (six 8-bit slices, exact level sums, fp64 re-accumulated) for the "
-              "contractions and SVD products, fp32 QR and Jacobi refined to fp64 accuracy" % args.mixed_kind)
-             if hp == "mixed" else "f64")
+    dtype = ("mixed: tcgen05 bf16 slice products (six 8-bit slices, exact level sums, fp64 re-accumulated) for the "
+             "contractions and SVD products, fp32 QR and Jacobi refined to 1e-11" if hp == "mixed" else "f64")
     line = {
         "metric": "gate_applications_per_sec", "value": hs["value"], "unit": "gate-applications/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": hs["ms_per_step"],
@@ -682,9 +722,10 @@ def main():
         "jacobi_critical_sweeps": ([prof["jacobi_svd"]["critical_sweeps"] / prof["jacobi_svd"]["chunks"],
                                     prof["jacobi_svd"]["critical_sweeps_fp32"] / prof["jacobi_svd"]["chunks"]]
                                    if prof["jacobi_svd"].get("chunks") else None),
-        "roofline": truncation_roofline(prof, hp),
+        "roofline": jacobi32_roofline(head),
         "roofline_contraction": contraction_roofline(prof) if hp == "mixed" else None,
-        "roofline_qr": qr_roofline(prof),
+        "truncation": truncation_rate(prof),
+        "qr": qr_rate(prof),
         "autotune": {"jacobi_rows_per_block": head["tuned"],
                      "note": "(chi_l x chi_r): [FP64 pass, FP32 pass], measured before the timed steps"},
         "graph_step": ({"ms_per_step": head["graph_ms"] / args.steps,
@@ -696,7 +737,7 @@ def main():
     if "fp64" in res and hp != "fp64":
         f = arm_summary(res["fp64"], world)
         f["dtype"] = "f64"
-        f["note"] = "the same workload, steps and start on the FP64 path (FP64 contractions, FP64 QR + Jacobi)"
+        f["note"] = "the same workload, steps and start on the FP64 path (seven slices, the SVD refined to FP64)"
         line["fp64_path"] = f
         line["speedup_mixed_vs_fp64"] = res["fp64"]["ms"] / res["fp64"]["steps"] / hs["ms_per_step"]
     if args.per_gate_steps > 0:

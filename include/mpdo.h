@@ -86,12 +86,14 @@ typedef struct {
     int device;              /* CUDA device ordinal; < 0: the calling thread's current device */
     int qr_blocked;          /* mixed path only: 1 = blocked Householder QR (window-pivoted panels of
                                 16 columns, trailing updates on the tensor cores); 0 (default) =
-                                the column-by-column QR, measured faster on this GPU */
-    double precond_rho;      /* mixed path only: the FP32 preconditioning sweeps stop after a sweep
-                                whose largest rotation (relative off-orthogonality |g|/sqrt(a b) of
-                                a rotated pair) was at most this (<= 0: 1e-3); a smaller value
-                                trades FP32 sweeps for fewer FP64 finishing sweeps.  Accuracy is
-                                unchanged: the FP64 sweeps finish to the FP64 tolerance. */
+                                the FP32 Householder QR made orthogonal by products, measured
+                                faster on this GPU */
+    double precond_rho;      /* the FP32 preconditioning sweeps (mixed contexts, FP64 ones with
+                                jacobi_max_sweeps >= 16) stop after a sweep whose largest rotation
+                                (relative off-orthogonality |g|/sqrt(a b) of a rotated pair) was at
+                                most this (<= 0: 1e-3); a smaller value trades FP32 sweeps for
+                                less work in the stages after them.  The tolerance that those
+                                finish to is unchanged. */
 } mpdo_config;
 
 typedef struct {
@@ -136,9 +138,11 @@ int mpdo_build_gates(mpdo_ctx *ctx, const mpdo_model *model, double dt);
 int mpdo_init_graph_state(mpdo_ctx *ctx, const int *pairs, int n_pairs);
 
 /* Advance every instance by n_steps Trotter steps (cfg.trotter_order).  Per op:
- * merge the two sites, apply the gate, weight by the left Schmidt values,
- * Householder QR (only R is kept), SVD of R (FP64 one-sided Jacobi on its
- * rows), truncate, write the two new sites.  After each
+ * merge the two sites, apply the gate, weight by the left Schmidt values, SVD
+ * (rows graded by a QR, one-sided Jacobi in FP32, refined to the tolerance through
+ * the rows' Gram matrix, an FP64 Jacobi pass for what that leaves; bonds of a few
+ * rows, and small sweep limits, take an FP64 QR and the FP64 pass alone), truncate,
+ * write the two new sites.  After each
  * step the trace is forced to 1 when cfg.force_trace.  Returns ENOCONV /
  * ENONFINITE / ETIMEOUT when some instance reported that status (the other
  * instances are still advanced), ESTATE before mpdo_build_gates. */
@@ -148,7 +152,9 @@ int mpdo_trotter_step(mpdo_ctx *ctx, int n_steps);
  * after mpdo_build_gates captures one step (planner kernels read the bond
  * dimensions on the device and size every launch there, so nothing returns
  * to the host inside a step) and every call replays it n_steps times, then
- * synchronises once.  Same results, rank log and status errors as
+ * synchronises once.  MPDO_FP64: steps from a loaded state in an unbalanced gauge
+ * (mpdo_set_state) and steps all of whose bonds are small are planned by the
+ * host as mpdo_trotter_step does.  Same results, rank log and status errors as
  * mpdo_trotter_step; kernel profiling is not collected; EINVAL while forced
  * ranks are set; ECAPACITY if a chunk holds more ops than co-resident CTAs. */
 int mpdo_trotter_step_graph(mpdo_ctx *ctx, int n_steps);
@@ -168,7 +174,7 @@ int mpdo_measure_2q(mpdo_ctx *ctx, const int *pairs, int np, const char comp[2],
  * S2 = -ln tr(rho^2) of the normalised rho.  In the orthonormal basis
  * P_a/sqrt2 tr(rho^2) = <<rho|rho>> / (tr rho)^2, the squared norm of the
  * coefficient MPS over the squared trace, computed by a left-to-right sweep of
- * Gram matrices (batched FP64 GEMMs).  out is [B] doubles, host (out_on_device
+ * Gram matrices (batched products of FP64 accuracy).  out is [B] doubles, host (out_on_device
  * = 0; the call synchronises) or device.  Uses the per-op workspaces (the state
  * is untouched).  ESTATE before mpdo_build_gates. */
 int mpdo_renyi2(mpdo_ctx *ctx, double *out, int out_on_device);
@@ -227,8 +233,10 @@ int mpdo_force_ranks(mpdo_ctx *ctx, const int *k, int n_steps);
  * largest layer), and the fastest is kept (FP64 pass; the FP32 pass has one block
  * size; bonds with chi_l > chi_r whose SVD is that of the transposed matrix keep the
  * default rule).  Later steps (plain and graph) use the table; classes not tuned
- * keep the default rule (largest block that fits).  chosen (host, may be NULL)
- * receives [n_classes][2] = (FP64 block, FP32 block or 0).  Uses the per-op
+ * keep the default rule (largest block that fits).  With the SVD's stages only what
+ * they leave reaches the FP64 pass, so the table matters for contexts without them
+ * (MPDO_FP64, jacobi_max_sweeps < 16).  chosen (host, may be NULL)
+ * receives [n_classes][2] = (FP64 block, the mixed path's FP32 block or 0).  Uses the per-op
  * workspaces only (the state is untouched); synchronises.  EINVAL, ESTATE, ECUDA. */
 int mpdo_autotune(mpdo_ctx *ctx, const int *classes, int n_classes, int *chosen);
 /* Copy instance b's gate matrices out: [n_ops][16][16] row-major doubles in

@@ -86,8 +86,8 @@ struct mpdo_ctx {
     unsigned char* d_slots = nullptr;   // the allocation that the slots' device buffers are parts of
     double *d_thetap = nullptr, *d_W = nullptr, *d_Z = nullptr, *d_Yk = nullptr, *d_snorm = nullptr;
     int* d_sweeps = nullptr;      // [slots] Jacobi sweeps of the last chunk
-    int* d_pre_ok = nullptr;      // [slots] mixed path: the FP32 pass ended by its off-orthogonality rule
-    bool mixed = false;           // mixed-precision SVD (FP32 preconditioning + FP64 finish)
+    int* d_pre_ok = nullptr;      // [slots] the FP32 pass ended by its off-orthogonality rule
+    bool mixed = false;           // mixed path: six slices, the SVD finished at kMixedFinishTol
     bool precond = false;         // SVD with FP32 preconditioning and Gram-matrix refinement (mixed and FP64 paths)
     int oz_s = 6;                 // slices per operand of the SVD's products: 6 (mixed path), 7 (FP64 path)
     mpdo::RefineOp* d_refine = nullptr;   // [slots]
@@ -104,7 +104,7 @@ struct mpdo_ctx {
     long long prof_crit = 0, prof_crit32 = 0, prof_chunks = 0;   // per chunk: largest sweeps of any op
     mpdo::OpDesc* d_desc = nullptr;
     mpdo::OpDesc* h_desc = nullptr;     // pinned
-    int *d_cta = nullptr, *h_cta = nullptr;   // [3][grid cap]: op, rank, then group [slots]
+    int *d_cta = nullptr, *h_cta = nullptr;   // [4][grid cap]: op, rank, then group [slots]
     unsigned* d_sync = nullptr;
     int jacobi_resident = 0;
     int qr_resident = 0, qr32_resident = 0;

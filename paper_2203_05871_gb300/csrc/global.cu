@@ -237,7 +237,7 @@ int run_plan(mpdo_ctx* c, bool wide, GqPlan& P) {
         if (tc)
             CU(launch_gemm_tc(c->d_gq + L.first, L.count, L.max_m, L.max_n, c->ld, scr, 7, timeout_ns, c->st));
         else
-            CU(launch_gemm(c->d_gq + L.first, L.count, L.max_m, L.max_n, false, c->st));
+            CU(launch_gemm(c->d_gq + L.first, L.count, L.max_m, L.max_n, c->st));
     }
     CU(cudaStreamSynchronize(c->st));   // the host descriptors are rebuilt by the next plan
     return MPDO_OK;

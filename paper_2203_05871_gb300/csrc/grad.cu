@@ -374,7 +374,7 @@ int run_bwd_chunk(mpdo_ctx* c, GradState* g, const std::vector<const TapeRec*>& 
         const bool tc = c->mixed && (q == 4 || q >= 6);
         return tc ? launch_gemm_tc(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], mx[q][2], g->oz,
                                    6, timeout_ns, c->st)
-                  : launch_gemm(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], false, c->st);
+                  : launch_gemm(g->d_bg + (size_t)q * S, nops, mx[q][0], mx[q][1], c->st);
     };
     CU(launch_copy2d(g->d_bc, 2 * nops, max_pack, c->st));
     CU(gemm(0));

@@ -346,14 +346,13 @@ struct GemmDesc {
     int ldd, d_f32;
     int sub_identity;
     int a_trans;      // A stored K x M (default 0)
-    int sym;          // 1: C is symmetric (A B with B = A^T, D = nullptr): only the tiles on and
-                      // above the diagonal are computed, each written to both triangles
+    int sym;          // 1: C is symmetric (D = nullptr): the part on and above the diagonal is
+                      // computed, the rest mirrored
     int* status;      // tensor-core route: MPDO_ST_TIMEOUT lands here (or nullptr)
 };
-cudaError_t launch_gemm(const GemmDesc* d_desc, int count, int max_m, int max_n, bool fp32_compute,
-                        cudaStream_t st);
-// The batched GemmDesc products (f64 operands; S slices) on the tensor cores: problem s takes slot s of the scratch (slices of slot_bytes per
-// operand, exponents of exp_ints per operand, oz_slice_bytes / oz_exp_ints of
+cudaError_t launch_gemm(const GemmDesc* d_desc, int count, int max_m, int max_n, cudaStream_t st);
+// The batched GemmDesc products (S slices) on the tensor cores: problem s takes slot s of
+// the scratch (slices of slot_bytes per operand, exponents of exp_ints per operand, oz_slice_bytes / oz_exp_ints of
 // the largest dimension) and probs[s]; max_m, max_n, max_k bound every product.
 struct OzScratch {
     unsigned char *as, *bs;

@@ -1,5 +1,5 @@
-// FP64-accurate batched GEMM on the tcgen05 tensor cores (the mixed path's
-// contractions and its SVD-preconditioner products).
+// FP64-accurate batched GEMM on the tcgen05 tensor cores (the contractions, the SVD's
+// products and, on FP64 contexts, the Gram sweeps of the entropies).
 //
 //   C = alpha * A B + beta * D  (- I when sub_identity),  A: M x K, B: K x N,
 // FP64 (or f32) in and out, computed from exact products of narrow slices of

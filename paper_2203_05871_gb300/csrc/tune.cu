@@ -9,7 +9,10 @@
 // tuner fills as many workspace slots as a layer has ops in flight with a
 // seeded graded matrix of the class's shape (rows scaled like the rows of a
 // pivoted R; at most 16 slots), and times the FP64 Jacobi launch for every b that
-// fits, keeping the fastest.  The FP32 pass has a fixed block of 32 rows.  The winners go
+// fits, keeping the fastest.  The FP32 pass has a fixed block of 32 rows.  In contexts
+// with the SVD's stages only what the refinement leaves reaches the FP64 pass, so there
+// the table decides little of a step's time; it is for contexts whose sweep limit leaves
+// the stages out.  The winners go
 // to a (chi_l, chi_r) table that both the host-planned and the graph step
 // read.  Different b change the order of the rotations, so results change at
 // rounding level only.
@@ -39,11 +42,9 @@ int time_jacobi(mpdo_ctx* c, std::vector<OpDesc>& h, int b, double* ms_out) {
                              cudaMemcpyDeviceToDevice, c->st));
     CU(cudaMemcpyAsync(c->d_desc, h.data(), sizeof(OpDesc) * nops, cudaMemcpyHostToDevice, c->st));
     int total = 0;
-    const int gcap = std::max(std::max(c->jacobi_resident, c->qr_resident), c->slots);
     int rc = plan_jacobi(c, h.data(), nops, false, c->h_cta, total);
     if (rc) return rc;
     CU(cudaMemcpyAsync(c->d_cta, c->h_cta, sizeof(int) * (2 * total + nops), cudaMemcpyHostToDevice, c->st));
-    (void)gcap;
     const unsigned long long timeout_ns = (unsigned long long)c->cfg.barrier_timeout_ms * 1000000ull;
     cudaEvent_t e0, e1;
     CU(cudaEventCreate(&e0));

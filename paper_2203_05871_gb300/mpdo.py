@@ -184,9 +184,8 @@ class Solver:
     STORE_F64 or STORE_F32; ``trotter_order`` 2 or 4; ``jacobi_tol`` and
     ``jacobi_max_sweeps`` of the SVD; ``barrier_timeout_ms`` bounding every
     device-side wait; ``max_slots`` (ops in flight, 0 = automatic);
-    ``qr_blocked`` (mixed path: the blocked QR instead of the column QR);
-    ``precond_rho`` (mixed path: the FP32 preconditioning sweeps' stop
-    threshold, 0 = 1e-3); ``stream`` a torch stream or a raw cudaStream_t.
+    ``qr_blocked`` (mixed path: the blocked QR instead of the FP32 one);
+    ``precond_rho`` (the FP32 preconditioning sweeps' stop threshold, 0 = 1e-3); ``stream`` a torch stream or a raw cudaStream_t.
     """
 
     def __init__(self, n_qubits: int, batch: int = 1, chi_cap: int = 32, precision: int = FP64,
