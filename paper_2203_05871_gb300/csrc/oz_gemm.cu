@@ -615,8 +615,9 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
     if (P.sym && (nt + 1) * TN <= mt * kTileM) return;   // mirrored from above the diagonal
     const int Kt = P.Kt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ int s_ea, s_eb;
-    if (threadIdx.x == 0) s_ea = s_eb = -(1 << 20);
+    constexpr int kGroup = 16, kGroups = TN / kGroup;   // columns that share a number of levels
+    __shared__ int s_ea, s_eb[kGroups];
+    if (threadIdx.x <= kGroups) *(threadIdx.x ? s_eb + threadIdx.x - 1 : &s_ea) = -(1 << 20);
 
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + kStages * kStageBytes + 128);
@@ -642,18 +643,21 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tslot;
     int lv = P.levels > 0 ? P.levels : kS;   // slice pairs t + u < lv
-    // What A B adds to entries of a unit row of D is below 2^(e_i + f_j).  Over blocks of
-    // 128 x 64 whatever TN is: TN follows from the launch's other problems, the result must not.
+    // What A B adds to entries of a unit row of D is below 2^(e_i + f_j).  The levels that
+    // count are those of 128 rows and 16 columns whatever TN is (lv is their largest, the
+    // epilogue takes each group's own): TN follows from the launch's other problems, the
+    // result must not.
     if (P.unit_d) {
         if (threadIdx.x < kTileM) {
             const int i = mt * kTileM + threadIdx.x;
             if (i < P.M) atomicMax(&s_ea, P.ea[i]);
-        } else if (threadIdx.x < kTileM + kTileN) {
-            const int j = nt * TN / kTileN * kTileN + threadIdx.x - kTileM;
-            if (j < N) atomicMax(&s_eb, P.eb[j]);
+        } else if (threadIdx.x < kTileM + TN) {
+            const int j = nt * TN + threadIdx.x - kTileM;
+            if (j < N) atomicMax(&s_eb[(threadIdx.x - kTileM) / kGroup], P.eb[j]);
         }
         __syncthreads();
-        lv = oz_levels(kS, s_ea + s_eb);
+        lv = 0;
+        for (int g = 0; g < kGroups; ++g) lv = max(lv, oz_levels(kS, s_ea + s_eb[g]));
     }
     const int nrange = (Kt + kRangeTiles - 1) / kRangeTiles;
 
@@ -752,6 +756,10 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
         unsigned nan = 0;
 #pragma unroll
         for (int j = 0; j < CP; ++j) hi[j] = lo[j] = 0;
+        int lg[(CP + kGroup - 1) / kGroup];   // the levels of this warp's column groups
+#pragma unroll
+        for (int g = 0; g < (CP + kGroup - 1) / kGroup; ++g)
+            lg[g] = P.unit_d ? oz_levels(kS, s_ea + s_eb[half * CP / kGroup + g]) : lv;
         bool ok = true;
         for (int r = 0; r < nrange; ++r) {
             if (!mbar_wait(smem_u32(bar + kBarAccFull), r & 1, abort_flag, timeout_ns)) {
@@ -765,6 +773,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(OzSource src,
                 const float scale = __int_as_float((127 + 8 * lvl) << 23);   // 2^8d
 #pragma unroll
                 for (int c = 0; c < CP; c += 8) {
+                    if (lvl >= lg[c / kGroup]) continue;   // uniform
                     float v[8];
                     tmem_ld8(taddr + (uint32_t)(lvl * TN + c), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
