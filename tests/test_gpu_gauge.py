@@ -32,12 +32,12 @@ def gauged(tens, bond, decades):
     return out
 
 
-def solver(states):
+def solver(states, **kw):
     from paper_2203_05871_gb300 import Solver
     B = len(states)
     wl = W.random_model(N, W.chain_bonds(N), 77, chi_max=CAP, cutoff=0.0)
     two = {f: np.repeat(getattr(wl, f), B, 0) for f in ("h_x", "h_y", "h_z", "g0", "g1", "g2", "J", "Jz", "cutoff", "chi_max")}
-    s = Solver(N, batch=B, chi_cap=CAP)
+    s = Solver(N, batch=B, chi_cap=CAP, **kw)
     s.build_gates(wl.with_(**two))
     for b, st in enumerate(states):
         s.set_state(b, *st)
@@ -88,4 +88,17 @@ def test_gradient():
     s.grad_forward(1)
     g, loss = s.grad_backward(zbar, wbar)
     assert abs(loss[0] - loss[1]) <= 1e-10 and np.all(np.isfinite(g))
+    s.close()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_float_storage(graph):
+    """Float site tensors: the entries round to 6e-8 of themselves in any gauge, so the two
+    instances agree within the storage's 1e-5."""
+    from paper_2203_05871_gb300 import STORE_F32
+    dims, tens = W.random_mpo_state(N, CHI0, seed=82)
+    s = solver([(dims, gauged(tens, 2, 8)), (dims, tens)], storage=STORE_F32)
+    s.step(1, graph=graph)
+    z = observables(s)
+    assert np.abs(z[0] - z[1]).max() <= 1e-5 * max(1.0, np.abs(z).max())
     s.close()
