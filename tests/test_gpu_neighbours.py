@@ -39,16 +39,19 @@ def same(a, b):
 
 @pytest.mark.parametrize("graph", [False, True])
 @pytest.mark.parametrize("poison", [False, True])
-def test_step(graph, poison):
+@pytest.mark.parametrize("precision", ["FP64", "MIXED_TF32"])
+def test_step(graph, poison, precision):
+    import paper_2203_05871_gb300 as M
+    precision = getattr(M, precision)
     chis = [64, 4, 5, 24]
     wl = W.random_model(N, W.chain_bonds(N), 401, batch=4, chi_max=64, cutoff=1e-12)
     states = [W.random_mpo_state(N, c, seed=402 + b) for b, c in enumerate(chis)]
     if poison:
         states[0][1][3][0, 1, 0] = np.nan
-    s = solver(chis, wl, states, [0, 1, 2, 3])
+    s = solver(chis, wl, states, [0, 1, 2, 3], precision)
     s.step(STEPS, graph=graph, check=False)
     for b in (1, 2, 3):
-        alone = solver(chis, wl, states, [b])
+        alone = solver(chis, wl, states, [b], precision)
         alone.step(STEPS, graph=graph)
         assert same(s.get_state(b), alone.get_state(0)), b
         alone.close()
